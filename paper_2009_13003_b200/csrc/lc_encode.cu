@@ -28,8 +28,8 @@
 // index, and this kernel takes its offsets from there instead of looking back. Same bytes, one more pass over
 // the key plane.
 //
-// Rare cases take a compact two-pass path (lengths, then bits ORed in place): the ragged last chunk,
-// codes longer than 32 bits, a lane or chunk that outgrows its shared-memory area, and vectors with an
+// The vector's partial last chunk takes a masked form of A. Rare cases take a compact two-pass path (lengths, then bits
+// ORed in place): codes longer than 32 bits, a lane or chunk that outgrows its shared-memory area, and vectors with an
 // exponent field >= 128, for which the one-byte key plane is not enough and keys come from base and cur.
 //
 // Bound: reads 1 byte and writes about 0.5 bytes per element, so this pass is limited by the integer
@@ -95,8 +95,7 @@ struct OrPacker {
 
 // Slow, compact path (see the header). With dst == nullptr it only returns the lane's bit count;
 // otherwise it ORs the lane's bits into the zeroed chunk image at dst, starting at bit lane_start.
-// The plane bytes of four steps are read as one 16-byte vector, the way the fast path reads them (this path also
-// codes the vector's partial last chunk, alone in its warp). Codes come from the per-key table in global memory:
+// The plane bytes of four steps are read as one 16-byte vector, the way the fast path reads them. Codes come from the per-key table in global memory:
 // passing the CTA's shared tables in as well was measured to cost the kernel's main loop 4 %.
 __device__ __noinline__ uint32_t chunk_slow(const EncEntry* __restrict__ enc, KeySource ks, uint64_t c,
                                             uint32_t lane, uint64_t n, uint32_t* dst, uint32_t lane_start) {
@@ -176,6 +175,76 @@ struct ColumnPacker {
   }
 };
 
+// Packed table entries (shared address packed_addr) of the four plane bytes of `word`.
+__device__ __forceinline__ void lookup4(uint32_t packed_addr, uint32_t word, uint32_t (&g)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const uint32_t b = __byte_perm(word, 0u, 0x4440 + e);  // plane byte of slot e
+    // volatile: keeps the loads where they are written, one row ahead of their use
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(g[e]) : "r"(packed_addr + b * 4u));
+  }
+}
+
+// Appends four codes whose packed entries are g, none of them the marker of a long code. Packed codes have at most 16
+// bits, so two neighbours are joined into one append of at most 32 bits (half the accumulator and flush work).
+__device__ __forceinline__ void put4_packed(ColumnPacker& pk, const uint32_t (&g)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; e += 2) {
+    const uint32_t l0 = g[e] >> kPackedLenShift, l1 = g[e + 1] >> kPackedLenShift;
+    const uint32_t c0 = g[e] & kPackedCodeMask, c1 = g[e + 1] & kPackedCodeMask;
+    pk.put((c0 << l1) | c1, l0 + l1);
+  }
+}
+
+// Ends a lane's column: writes the pending bits and returns the lane's bit count, or ~0 if the column was too small.
+__device__ __forceinline__ uint32_t finish_column(const ColumnPacker& pk, uint32_t col0) {
+  if (pk.nb >= 32 || (pk.nb > 0 && pk.dst >= pk.lim)) return 0xffffffffu;
+  if (pk.nb > 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(pk.dst), "r"(pk.lo << (32 - pk.nb)) : "memory");
+  return ((pk.dst - col0) >> 7) * 32 + pk.nb;
+}
+
+// Phase A for the vector's partial last chunk of `rem` elements: as for a whole chunk, with the slots beyond the end
+// masked to empty codes and only the steps that hold elements visited. A kernel of its own size in miniature: one warp
+// runs it once per call, and on vectors of a few thousand chunks everything else waits for that warp, so it must not
+// take the element-by-element path (which took 20 us for the codes and 60 us for the tracked state). Out of line, so
+// that it does not weigh on the registers of the main loop. Returns the lane's bit count, ~0 if a column overflowed.
+__device__ __noinline__ uint32_t code_partial(const Tables* tb, const uint4* ep, uint32_t rem, uint32_t lane,
+                                              uint32_t col0, uint32_t lane_words) {
+  ColumnPacker pk{0u, 0u, 0u, col0, col0 + lane_words * 128};
+  const uint32_t packed_addr = smem_addr(tb->packed);
+  const uint32_t rows = (rem + 127) / 128;
+  uint4 nxt = __ldg(ep);
+#pragma unroll 1
+  for (uint32_t q = 0; 4 * q < rows; ++q) {
+    const uint32_t words[4] = {nxt.x, nxt.y, nxt.z, nxt.w};
+    if (q + 1 < kSteps / 4) nxt = __ldg(ep + 32 * (q + 1));
+    uint32_t g[4][4];
+#pragma unroll
+    for (uint32_t r = 0; r < 4; ++r) {
+      lookup4(packed_addr, words[r], g[r]);
+      const uint32_t first = (4 * q + r) * 128 + 4 * lane;
+      const uint32_t have = first < rem ? rem - first : 0u;  // elements from this slot group on
+#pragma unroll
+      for (uint32_t e = 0; e < 4; ++e)
+        if (e >= have) g[r][e] = 0u;  // no element: an empty code
+    }
+#pragma unroll
+    for (uint32_t r = 0; r < 4; ++r) {
+      if ((int)(g[r][0] | g[r][1] | g[r][2] | g[r][3]) < 0) {
+#pragma unroll
+        for (uint32_t e = 0; e < 4; ++e) {
+          if (g[r][e] == 0u) continue;
+          const uint2 f = tb->full[__byte_perm(words[r], 0u, 0x4440 + e)];
+          pk.put(f.x, f.y);
+        }
+      } else {
+        put4_packed(pk, g[r]);
+      }
+    }
+  }
+  return finish_column(pk, col0);
+}
+
 // UPDATE: the kernel also writes the tracked state of Algorithm 1 step 7, tracked_out = base + quantized delta
 // (fp32, the representative of the zero bucket, +0, added like any other): inside the coding loop for the chunks
 // whose coding never reads base, otherwise chunk by chunk once a chunk's coding no longer needs base.
@@ -232,19 +301,9 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   uint32_t* image = column + image_words;
   const uint32_t packed_addr = smem_addr(tb.packed);
 
-  // Packed table entries of the four plane bytes of `word`.
-  auto lookup4 = [&](uint32_t word, uint32_t (&g)[4]) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const uint32_t b = __byte_perm(word, 0u, 0x4440 + e);  // plane byte of slot e
-      // volatile: keeps the loads where they are written, one row ahead of their use
-      asm volatile("ld.shared.u32 %0, [%1];" : "=r"(g[e]) : "r"(packed_addr + b * 4u));
-    }
-  };
-  // Appends the four codes of `word`, whose packed entries are g. Packed codes have at most 16 bits, so two
-  // neighbours are joined into one append of at most 32 bits (half the accumulator and flush work). Only the
-  // marker has bit 31 set, so one test per row finds the rare longer codes; that row then appends its four
-  // codes one by one from `full`.
+  // Appends the four codes of `word`, whose packed entries are g. Only the marker of a code of more than 16 bits has
+  // bit 31 set, so one test per row finds the rare longer codes; that row then appends its four codes one by one from
+  // `full`.
   auto put4 = [&](ColumnPacker& pk, uint32_t word, const uint32_t (&g)[4]) {
     if (__any_sync(0xffffffffu, (int)(g[0] | g[1] | g[2] | g[3]) < 0)) {
 #pragma unroll
@@ -253,12 +312,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
         pk.put(f.x, f.y);
       }
     } else {
-#pragma unroll
-      for (int e = 0; e < 4; e += 2) {
-        const uint32_t l0 = g[e] >> kPackedLenShift, l1 = g[e + 1] >> kPackedLenShift;
-        const uint32_t c0 = g[e] & kPackedCodeMask, c1 = g[e + 1] & kPackedCodeMask;
-        pk.put((c0 << l1) | c1, l0 + l1);
-      }
+      put4_packed(pk, g);
     }
   };
   auto fast_chunk = [&](uint64_t cc) { return cc < nchunks && (cc + 1) * kChunkElems <= n && !long_codes && !ks.wide; };
@@ -300,7 +354,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
       ColumnPacker pk{0u, 0u, 0u, col0, col0 + lane_words * 128};
       uint32_t g0[4], g1[4];
       uint4 cur4 = __ldg(ep);
-      lookup4(cur4.x, g0);
+      lookup4(packed_addr, cur4.x, g0);
       // UPDATE: the tracked state of this chunk is written here, where its plane bytes are in registers; the
       // memory traffic of the update then runs under the coding, which is bound by instruction issue. A chunk on
       // this path never reads base for its coding (not even when it is coded again the slow way), so base may be
@@ -338,28 +392,27 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
 #pragma unroll 1
       for (int q = 0; q < 8; ++q) {
         const uint4 nxt = __ldg(ep + 32 * (q + 1 < 8 ? q + 1 : q));  // next 16 plane bytes, one step ahead
-        lookup4(cur4.y, g1);
+        lookup4(packed_addr, cur4.y, g1);
         put4(pk, cur4.x, g0);
         if (UPDATE) update_row(cur4.x, 4 * q);
-        lookup4(cur4.z, g0);
+        lookup4(packed_addr, cur4.z, g0);
         put4(pk, cur4.y, g1);
         if (UPDATE) update_row(cur4.y, 4 * q + 1);
-        lookup4(cur4.w, g1);
+        lookup4(packed_addr, cur4.w, g1);
         put4(pk, cur4.z, g0);
         if (UPDATE) update_row(cur4.z, 4 * q + 2);
-        lookup4(nxt.x, g0);  // first row of the next step (unused after the last step)
+        lookup4(packed_addr, nxt.x, g0);  // first row of the next step (unused after the last step)
         put4(pk, cur4.w, g1);
         if (UPDATE) update_row(cur4.w, 4 * q + 3);
         cur4 = nxt;
       }
-      const bool overflow = pk.nb >= 32 || (pk.nb > 0 && pk.dst >= pk.lim);
-      if (__any_sync(0xffffffffu, overflow)) {
-        fast = false;  // some lane outgrew its column: redo the chunk the slow way
-      } else {
-        if (pk.nb > 0) column[((pk.dst - col0) >> 7) * 32 + lane] = pk.lo << (32 - pk.nb);
-        lane_bits = ((pk.dst - col0) >> 7) * 32 + pk.nb;
-      }
+      lane_bits = finish_column(pk, col0);
+    } else if (valid && !long_codes && !ks.wide) {
+      lane_bits = code_partial(&tb, reinterpret_cast<const uint4*>(plane + c * kChunkElems) + lane, (uint32_t)(n - c * kChunkElems),
+                               lane, smem_addr(column) + lane * 4, lane_words);
+      fast = true;
     }
+    if (fast && __any_sync(0xffffffffu, lane_bits == 0xffffffffu)) fast = false;  // some lane outgrew its column: redo the chunk the slow way
     if (!fast && valid) lane_bits = chunk_slow(ctl->enc, ks, c, lane, n, nullptr, 0);
 
     // ---- B: lane offsets, lane index, chunk size; the tile's size is published as early as possible
@@ -512,8 +565,34 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
               o4[32 * (4 * q + r)] = x;
             }
           }
+        } else if (!ks.wide) {
+          // partial last chunk: four steps' loads at a time, the slots beyond the end left out
+          const uint32_t rem = (uint32_t)(n - p_c * kChunkElems);
+          const uint4* ep = reinterpret_cast<const uint4*>(plane + p_c * kChunkElems) + lane;
+          const float* b1 = base + p_c * kChunkElems;
+          float* o1 = tracked_out + p_c * kChunkElems;
+#pragma unroll 1
+          for (uint32_t q = 0; q * 512 < rem; ++q) {
+            const uint4 w4 = __ldg(ep + 32 * q);
+            const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+            float b[4][4];
+#pragma unroll
+            for (uint32_t r = 0; r < 4; ++r)
+#pragma unroll
+              for (uint32_t e = 0; e < 4; ++e) {
+                const uint32_t i = (4 * q + r) * 128 + 4 * lane + e;
+                if (i < rem) b[r][e] = b1[i];
+              }
+#pragma unroll
+            for (uint32_t r = 0; r < 4; ++r)
+#pragma unroll
+              for (uint32_t e = 0; e < 4; ++e) {
+                const uint32_t i = (4 * q + r) * 128 + 4 * lane + e;
+                if (i < rem) o1[i] = __fadd_rn(b[r][e], __uint_as_float(s_rep[__byte_perm(w[r], 0u, 0x4440 + e)]));
+              }
+          }
         } else {
-          // ragged last chunk, or exponents the one-byte plane does not hold: element by element
+          // exponents the one-byte plane does not hold: element by element
           for (uint32_t j = 0; j < kSteps; ++j) {
             for (uint32_t e = 0; e < kGroup; ++e) {
               const uint64_t i = p_c * kChunkElems + 128ull * j + 4 * lane + e;
