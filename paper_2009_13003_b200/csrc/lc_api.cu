@@ -190,7 +190,6 @@ static int recover_impl(const float* base, const void* const* streams, const uin
     if (!streams[j] || !aligned(streams[j], 16)) return LC_ERR_ARG;
   if (workspace_bytes < workspace_layout(0).total) return LC_ERR_CAPACITY;
   Control* ctl = static_cast<Control*>(workspace);
-  void* images = static_cast<uint8_t*>(workspace) + workspace_layout(0).decode_off;
   if (reset_status && cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
   // up to four streams per launch; later launches continue in place from `out`.
   const float* src = base;
@@ -202,7 +201,7 @@ static int recover_impl(const float* base, const void* const* streams, const uin
       ds.ptr[j] = static_cast<const uint8_t*>(streams[first + j]);
       ds.bytes[j] = stream_bytes[first + j];
     }
-    if (launch_decode(src, ds, kk, n, out, &ctl->status, images, cs) != cudaSuccess) return LC_ERR_CUDA;
+    if (launch_decode(src, ds, kk, n, out, &ctl->status, cs) != cudaSuccess) return LC_ERR_CUDA;
     src = out;
   }
   return LC_OK;
@@ -514,7 +513,6 @@ extern "C" int lc_recover_host(const float* base_host, const void* const* stream
   HostPipeline pipe;
   if (!pipe.create()) return LC_ERR_CUDA;
   Control* ctl = reinterpret_cast<Control*>(a);
-  void* images = a + workspace_layout(0).decode_off;
   if (cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
   const int groups = (k + 3) / 4;
   for (int i = 0; i < kHostSlices; ++i) {
@@ -532,10 +530,7 @@ extern "C" int lc_recover_host(const float* base_host, const void* const* stream
         ds.ptr[j] = static_cast<const uint8_t*>(d_streams[first + j]);
         ds.bytes[j] = stream_bytes[first + j];
       }
-      // the decode tables of a group of four streams are built once if there is one group; two groups share the
-      // table area and rebuild theirs for every slice
-      const bool prepare = groups > 1 || i == 0;
-      if (launch_decode(d_x, ds, kk, n, d_x, &ctl->status, images, cs, c0, c1, prepare) != cudaSuccess) return LC_ERR_CUDA;
+      if (launch_decode(d_x, ds, kk, n, d_x, &ctl->status, cs, c0, c1) != cudaSuccess) return LC_ERR_CUDA;
     }
     if (cudaEventRecord(pipe.decoded[i], cs) != cudaSuccess) return LC_ERR_CUDA;
     if (cudaStreamWaitEvent(pipe.out, pipe.decoded[i], 0) != cudaSuccess) return LC_ERR_CUDA;

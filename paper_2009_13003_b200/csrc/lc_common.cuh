@@ -91,14 +91,12 @@ struct ShardStats {
 static_assert(sizeof(ShardStats) == LC_STATS_BYTES, "size promised by the header");
 static_assert(sizeof(Control) % 256 == 0, "control block must keep the planes 256-byte aligned");
 
-// lc_recover keeps the decode tables of the (at most four) streams of one launch behind the control block, at an
-// offset that does not depend on n: the prepare kernel builds them there once, every CTA of the decode kernel copies
-// them into its shared memory.
-constexpr uint32_t kDecodeImageBytes = 24 * 1024;  // per stream
-constexpr uint32_t kDecodeRegionBytes = 4 * kDecodeImageBytes;
+// A region behind the control block whose size does not depend on n. Nothing uses it at present (the decode kernel's
+// CTAs build their tables in shared memory); it stays so that the sizes lc_workspace_bytes returns stay.
+constexpr uint32_t kSpareRegionBytes = 96 * 1024;
 
 struct WorkspaceLayout {
-  uint64_t control_off, decode_off, tiles_off, plane_off, total;
+  uint64_t control_off, spare_off, tiles_off, plane_off, total;
   uint64_t nchunks, nunits;
 };
 
@@ -107,8 +105,8 @@ __host__ __device__ constexpr inline WorkspaceLayout workspace_layout(uint64_t n
   W.nchunks = (n + kChunkElems - 1) / kChunkElems;
   W.nunits = W.nchunks * kUnitsPerChunk;
   W.control_off = 0;
-  W.decode_off = sizeof(Control);
-  W.tiles_off = W.decode_off + kDecodeRegionBytes;              // one 8-byte descriptor per chunk
+  W.spare_off = sizeof(Control);
+  W.tiles_off = W.spare_off + kSpareRegionBytes;              // one 8-byte descriptor per chunk
   W.plane_off = align_up(W.tiles_off + 8 * W.nchunks, 256);
   W.total = align_up(W.plane_off + W.nchunks * kChunkElems, 256);  // 1 byte per element, whole chunks
   return W;
@@ -169,11 +167,8 @@ struct DecodeStreams {
   const uint8_t* ptr[4];
   uint64_t bytes[4];
 };
-// images: kDecodeRegionBytes of device scratch for the streams' decode tables (built by a first small kernel)
-// Decodes the chunks [chunk_begin, chunk_end) only (clipped to the vector's chunks). prepare: build the images first
-// (false: an earlier launch for the same streams has left them there).
+// Decodes the chunks [chunk_begin, chunk_end) only (clipped to the vector's chunks).
 cudaError_t launch_decode(const float* base, const DecodeStreams& streams, int k, uint64_t n, float* out,
-                          int32_t* status, void* images, cudaStream_t cs, uint64_t chunk_begin = 0,
-                          uint64_t chunk_end = ~0ull, bool prepare = true);
+                          int32_t* status, cudaStream_t cs, uint64_t chunk_begin = 0, uint64_t chunk_end = ~0ull);
 
 }  // namespace lc

@@ -61,270 +61,224 @@ constexpr uint32_t kTableBytes = 8192;
 constexpr uint32_t kTablePad = 128;  // the tables start on a 128-byte boundary (a lane's copy of an entry is chosen by OR)
 static_assert((1 << kL1Bits) * kL1Rep * 8 == kTableBytes, "table sizes");
 
+// Where device-detected errors go: the first one stays.
+struct Status {
+  int32_t* word;
+  __device__ __forceinline__ void set(int32_t code) const { set_status(word, code); }
+};
+
 struct alignas(16) StreamState {
-  uint2* l1;  // [(1 << kL1Bits) * kL1Rep] {bit pattern of rep, code length}; length kLongCode = not resolved here
-  uint2* sub; // 8 KB of sub-tables of (1 << sub_bits) entries: {rep, length} or length kLongCode = longer code
-  uint32_t sorted_rep[kMaxSymbols];   // representatives in canonical (len, id) order
-  unsigned long long first_code[64];  // first canonical code of each length
+  const uint8_t* ptr;  // the stream
+  uint32_t l1_addr;    // shared address of the first level: [(1 << kL1Bits) * kL1Rep] {bit pattern of rep, code length};
+                       // length kLongCode = not resolved here. The second level follows it at kTableBytes: sub-tables of
+                       // (1 << sub_bits) entries: {rep, length} or length kLongCode = longer code
+  int32_t err;         // outcome of the validation
+  unsigned long long payload_off, payload_size, chunk_index_off, lane_index_off;
+  uint32_t max_len, nused, only_rep;
+  uint32_t nsub;        // first-level prefixes that belong to longer codes: the last nsub of them (codes are canonical)
+  uint32_t sub_bits;    // depth of the sub-tables, kSubBitsMin..kSubBitsMax: as many as 8 KB hold at that depth
+  uint32_t end31[20];   // [L], L = 1..16: end of the range that codes of at most L bits fill, left-aligned to 31 bits
+  uint32_t sorted_rep[kMaxSymbols];    // representatives in canonical (len, id) order
+  unsigned long long first_code[64];   // first canonical code of each length
   unsigned long long last_aligned[64]; // largest left-aligned 64-bit window whose code has at most this length
-  uint32_t len_count[64];             // codes of each length
-  uint32_t len_offset[64];            // index of the first of them in sorted_rep
-  // header
-  unsigned long long n, payload_bits, total_bytes, payload_off, payload_size;
-  unsigned long long chunk_index_off, lane_index_off;
-  uint32_t nsym, max_len, nchunks, only_rep;
-  uint32_t fixed;  // fixed-width codes (format section 1.5): every symbol is coded, used or not
-  uint32_t shared_table;  // the table comes from a larger vector (format section 1.6): unused symbols may have codes
-  // validation accumulators
-  unsigned long long kraft, count_sum, bit_sum;
-  uint32_t seen_max, nused, nsub;
-  uint32_t sub_bits;  // depth of the sub-tables, kSubBitsMin..kSubBitsMax: as many as 8 KB hold at that depth
-  uint8_t sub_of_prefix[1 << kL1Bits], prefix_of_sub[1 << kL1Bits];
-  uint8_t sym_len[kMaxSymbols];  // code length by symbol id
-  uint32_t miss_count[2];  // first-level prefixes without a short code, per warp of 32 prefixes
-  alignas(16) uint8_t hdr[kHeaderBytes];  // the stream header, staged
+  uint32_t len_count[64];              // codes of each length
+  uint32_t len_offset[64];             // index of the first of them in sorted_rep
+  uint32_t len_next[64];               // index of the next of them while sorted_rep is filled
 };
 
 static_assert(sizeof(StreamState) % 16 == 0, "the staging areas behind the tables take 16-byte accesses");
 
-// Canonical decode of the top `width` bits `idx`: (index into sorted_rep, length) or length 0 if the code
-// is longer than `width`.
-__device__ __forceinline__ uint2 canonical_lookup(const StreamState& S, uint32_t idx, uint32_t width) {
-  for (uint32_t L = 1; L <= width; ++L) {
-    const unsigned long long c = idx >> (width - L);
-    if (c >= S.first_code[L] && c - S.first_code[L] < S.len_count[L])
-      return make_uint2(S.len_offset[L] + (uint32_t)(c - S.first_code[L]), L);
-  }
-  return make_uint2(0u, 0u);
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
 }
 
-// Parses and validates stream `s`, then builds its decode tables in shared memory. All threads of the
-// CTA call this; returns 0 or the error to report.
-__device__ __noinline__ int prepare_stream(StreamState& S, unsigned char* tables, const uint8_t* __restrict__ s,
-                              uint64_t bytes, uint64_t n, int* s_err) {
-  const int tid = threadIdx.x, nthreads = blockDim.x;
-  if (tid < 4 && bytes >= kHeaderBytes)
-    reinterpret_cast<uint4*>(S.hdr)[tid] = __ldg(reinterpret_cast<const uint4*>(s) + tid);
-  __syncthreads();
-  if (tid == 0) {
-    int err = 0;
-    const uint8_t* h = S.hdr;
-    S.l1 = reinterpret_cast<uint2*>(tables);
-    S.sub = reinterpret_cast<uint2*>(tables + kTableBytes);
-    S.kraft = 0; S.count_sum = 0; S.bit_sum = 0; S.seen_max = 0; S.nused = 0; S.only_rep = 0;
-    if (bytes < kHeaderBytes) {
-      err = LC_ERR_FORMAT;
-    } else {
-      const uint32_t nbits = h[6];
-      S.n = load_le(h + 8, 8);
-      S.nsym = (uint32_t)load_le(h + 16, 4);
-      S.max_len = (uint32_t)load_le(h + 20, 4);
-      S.nchunks = (uint32_t)load_le(h + 32, 4);
-      S.payload_bits = load_le(h + 40, 8);
-      S.total_bytes = load_le(h + 48, 8);
-      S.payload_off = load_le(h + 56, 8);
-      const bool magic = h[0] == 'L' && h[1] == 'C' && h[2] == 'C' && h[3] == '1';
-      S.fixed = h[7] & 1u;
-      S.shared_table = (h[7] >> 1) & 1u;
-      if (!magic || load_le(h + 4, 2) != 1 || nbits < 1 || nbits > (uint32_t)kMaxNbits || (h[7] > 4 && h[7] != 8)) err = LC_ERR_FORMAT;  // bits 2 (cached lengths) and 3 (mean) go alone
-      else if (S.nsym < 1 || S.nsym > (1u << nbits) || S.max_len > 63) err = LC_ERR_FORMAT;
-      else if (load_le(h + 24, 4) != kChunkElems || load_le(h + 28, 2) != kLanes ||
-               load_le(h + 30, 2) != kGroup || load_le(h + 36, 4) != kPayloadAlign) err = LC_ERR_FORMAT;
-      else if (S.n != n) err = S.n < (1ull << 32) ? LC_ERR_MISMATCH : LC_ERR_FORMAT;
-      if (!err) {
-        const StreamLayout L = stream_layout(S.n, S.nsym);
-        S.chunk_index_off = L.chunk_index_off;
-        S.lane_index_off = L.lane_index_off;
-        if (S.nchunks != L.nchunks || S.payload_off != L.payload_off || S.total_bytes > bytes ||
-            S.total_bytes < L.payload_off) {
-          err = LC_ERR_FORMAT;
-        } else {
-          S.payload_size = S.total_bytes - S.payload_off;
-          if (load_le(s + L.chunk_index_off, 8) != 0 ||
-              load_le(s + L.chunk_index_off + 8 * L.nchunks, 8) != S.payload_size)
-            err = LC_ERR_FORMAT;
-        }
-      }
-    }
-    *s_err = err;
-  }
-  for (int L = tid; L < 64; L += nthreads) S.len_count[L] = 0;
-  __syncthreads();
-  if (*s_err) return *s_err;
+// Parses and validates stream `s` and derives its canonical code, all in one warp: every CTA of the decode kernel runs
+// this for its streams at once, a warp each, before it fills its tables. `scratch`: 5 * kMaxSymbols bytes of shared
+// memory. Returns 0 or the error to report (the same for all lanes).
+// Bound: latency. Two dependent reads of the stream (header, then symbol table and chunk index) and no block barrier;
+// 64-bit sums go through shuffles (a 64-bit shared-memory atomic is a compare-and-swap loop) and the per-length
+// quantities through one scan over the lengths instead of a serial loop of one thread. As a kernel of its own that built
+// the tables once per launch this step took 12 to 20 us, ahead of a decode kernel that takes as long for a small vector.
+__device__ __noinline__ int prepare_stream(StreamState& S, unsigned char* scratch, const uint8_t* __restrict__ s,
+                                           uint64_t bytes, uint64_t n, uint32_t lane) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  uint32_t* sym_rep = reinterpret_cast<uint32_t*>(scratch);
+  uint8_t* sym_len = scratch + 4 * kMaxSymbols;
+  if (bytes < kHeaderBytes) return LC_ERR_FORMAT;
+  const uint4 hv = __ldg(reinterpret_cast<const uint4*>(s) + (lane & 3));
+  const auto u32_at = [&](int off) {
+    const uint32_t v = (off & 12) == 0 ? hv.x : (off & 12) == 4 ? hv.y : (off & 12) == 8 ? hv.z : hv.w;
+    return __shfl_sync(kAll, v, off >> 4);
+  };
+  const auto u64_at = [&](int off) { return (unsigned long long)u32_at(off + 4) << 32 | u32_at(off); };
+  const uint32_t magic = u32_at(0), ver = u32_at(4), nsym = u32_at(16), max_len = u32_at(20);
+  const uint32_t nbits = (ver >> 16) & 255u, flags = ver >> 24;
+  const unsigned long long hdr_n = u64_at(8), payload_bits = u64_at(40), total_bytes = u64_at(48), payload_off = u64_at(56);
+  const uint32_t chunk_elems = u32_at(24), lanes_group = u32_at(28), nchunks = u32_at(32), payload_align = u32_at(36);
+  const bool fixed = (flags & 1u) != 0, shared_table = (flags & 2u) != 0;  // format sections 1.5 and 1.6
+  if (magic != 0x3143434Cu || (ver & 0xffffu) != 1 || nbits < 1 || nbits > (uint32_t)kMaxNbits || (flags > 4 && flags != 8))
+    return LC_ERR_FORMAT;  // flag bits 2 (cached lengths) and 3 (mean) go alone
+  if (nsym < 1 || nsym > (1u << nbits) || max_len > 63) return LC_ERR_FORMAT;
+  if (chunk_elems != kChunkElems || lanes_group != (kLanes | kGroup << 16) || payload_align != kPayloadAlign) return LC_ERR_FORMAT;
+  if (hdr_n != n) return hdr_n < (1ull << 32) ? LC_ERR_MISMATCH : LC_ERR_FORMAT;
+  const StreamLayout L = stream_layout(n, nsym);
+  if (nchunks != L.nchunks || payload_off != L.payload_off || total_bytes > bytes || total_bytes < payload_off)
+    return LC_ERR_FORMAT;
+  const unsigned long long payload_size = total_bytes - payload_off;
+  // first and last entry of the chunk index, read beside the symbol table
+  const unsigned long long index_end =
+      __ldg(reinterpret_cast<const unsigned long long*>(s + L.chunk_index_off) + ((lane & 1) ? L.nchunks : 0));
 
-  // ---- table entries: a thread per symbol (up to 509 symbols, CTAs of 256 threads and more)
-  const uint32_t nsym = S.nsym;
-  const bool fixed = S.fixed != 0, shared_table = S.shared_table != 0;
+  for (uint32_t l = lane; l < 64; l += 32) S.len_count[l] = 0;
+  __syncwarp();
   uint32_t fixed_width = 0;
   while ((1u << fixed_width) < nsym) fixed_width += 1;
-  bool entry_bad = false;
-  for (uint32_t sym = tid; sym < nsym; sym += nthreads) {
-    const uint4 e = __ldg(reinterpret_cast<const uint4*>(s + kHeaderBytes) + sym);  // key:16 len:8 pad:8 | rep | count
-    const uint32_t my_len = (e.x >> 16) & 255u, my_rep = e.y;
-    const unsigned long long my_count = ((unsigned long long)e.w << 32) | e.z;
-    entry_bad |= (e.x >> 24) != 0 || my_len > 63;
-    entry_bad |= fixed ? (my_len != fixed_width) : (!shared_table && my_count == 0 && my_len != 0);
-    entry_bad |= my_count != 0 && my_len == 0 && shared_table && S.max_len != 0;  // a used symbol needs its code
-    S.sym_len[sym] = (uint8_t)my_len;
-    atomicMax(&S.seen_max, my_len);
-    if (my_count != 0) {
-      atomicAdd(&S.count_sum, my_count);
-      atomicAdd(&S.bit_sum, my_count * my_len);
+  // ---- table entries, 32 symbols at a time
+  bool bad = index_end != ((lane & 1) ? payload_size : 0ull);
+  unsigned long long kraft = 0, count_sum = 0, bit_sum = 0;
+  uint32_t nused = 0, seen_max = 0, only_rep = 0;
+  for (uint32_t first = 0; first < nsym; first += 32) {
+    const uint32_t sym = first + lane;
+    const bool have = sym < nsym;
+    uint4 e = make_uint4(0u, 0u, 0u, 0u);
+    if (have) e = __ldg(reinterpret_cast<const uint4*>(s + kHeaderBytes) + sym);  // key:16 len:8 pad:8 | rep | count
+    const uint32_t len = (e.x >> 16) & 255u;
+    const unsigned long long count = ((unsigned long long)e.w << 32) | e.z;
+    if (have) {
+      bad |= (e.x >> 24) != 0 || len > 63;
+      bad |= fixed ? (len != fixed_width) : (!shared_table && count == 0 && len != 0);
+      bad |= count != 0 && len == 0 && shared_table && max_len != 0;  // a used symbol needs its code
+      sym_len[sym] = (uint8_t)len;
+      sym_rep[sym] = e.y;
     }
-    if (!fixed && my_count != 0) S.only_rep = my_rep;  // meaningful only when no symbol has a code length
-    if (fixed ? (fixed_width > 0 || sym == 0) : (shared_table && S.max_len != 0 ? my_len != 0 : my_count != 0)) {
-      // the symbols that have a code
-      atomicAdd(&S.nused, 1u);
-      if (fixed && sym == 0) S.only_rep = my_rep;
-      if (my_len > 0 && my_len <= 63) {
-        atomicAdd(&S.kraft, 1ull << (63 - my_len));
-        atomicAdd(&S.len_count[my_len], 1u);
-      }
+    seen_max = max(seen_max, len);
+    count_sum += count;
+    bit_sum += count * len;
+    // the symbols that have a code
+    const bool coded = have && (fixed ? (fixed_width > 0 || sym == 0) : (shared_table && max_len != 0 ? len != 0 : count != 0));
+    if (coded && len > 0 && len <= 63) {
+      kraft += 1ull << (63 - len);
+      atomicAdd(&S.len_count[len], 1u);
     }
+    nused += __popc(__ballot_sync(kAll, coded));
+    // meaningful only when no symbol has a code length
+    const uint32_t single = __ballot_sync(kAll, fixed ? have && sym == 0 : count != 0);
+    const uint32_t rep = __shfl_sync(kAll, e.y, single ? __ffs(single) - 1 : 0);
+    if (single) only_rep = rep;
   }
-  if (__syncthreads_or(entry_bad)) return LC_ERR_FORMAT;
-  if (tid == 0) {
-    int err = 0;
-    if (S.count_sum != S.n || S.bit_sum != S.payload_bits) err = LC_ERR_FORMAT;
-    if (S.fixed) {
-      uint32_t width = 0;
-      while ((1u << width) < S.nsym) width += 1;
-      if (S.max_len != width) err = LC_ERR_FORMAT;  // every entry's length was compared with the width above
-    } else {
-      if (S.seen_max != S.max_len) err = LC_ERR_FORMAT;
-      if (S.nused >= 2) {
-        if (S.kraft != (1ull << 63)) err = LC_ERR_FORMAT;
-      } else if (S.max_len != 0) {
-        err = LC_ERR_FORMAT;
-      }
-    }
-    // canonical first codes per length
-    unsigned long long code = 0;
-    uint32_t offset = 0;
-    for (int L = 1; L < 64; ++L) {
-      S.first_code[L] = code;
-      S.len_offset[L] = offset;
-      code = (code + S.len_count[L]) << 1;
-      offset += S.len_count[L];
-    }
-    S.first_code[0] = 0;
-    S.len_offset[0] = 0;
-    // codes of length <= L fill the left-aligned range [0, (first_code[L] + count[L]) << (64 - L))
-    for (int L = 1; L < 64; ++L) {
-      const unsigned long long end = (S.first_code[L] + S.len_count[L]) << (64 - L);  // 0 when the range is everything
-      S.last_aligned[L] = end - 1;
-    }
-    *s_err = err;
+  if (__any_sync(kAll, bad)) return LC_ERR_FORMAT;
+  seen_max = __reduce_max_sync(kAll, seen_max);
+  if (warp_sum(count_sum) != n || warp_sum(bit_sum) != payload_bits) return LC_ERR_FORMAT;
+  if (fixed) {
+    if (max_len != fixed_width) return LC_ERR_FORMAT;  // every entry's length was compared with the width above
+  } else {
+    if (seen_max != max_len) return LC_ERR_FORMAT;
+    if (nused >= 2 ? warp_sum(kraft) != (1ull << 63) : max_len != 0) return LC_ERR_FORMAT;
   }
-  __syncthreads();
-  if (*s_err) return *s_err;
-  if (S.nused >= 2) {
-    for (uint32_t sym = tid; sym < nsym; sym += nthreads) {
-      const uint32_t my_len = S.sym_len[sym];
-      if (my_len == 0) continue;  // a symbol without a code (unused, in a Huffman-coded stream)
-      // rank among the symbols of the same length with smaller id
-      uint32_t r = 0;
-      for (uint32_t j = 0; j < sym; ++j) r += (S.sym_len[j] == my_len) ? 1u : 0u;
-      S.sorted_rep[S.len_offset[my_len] + r] = __ldg(reinterpret_cast<const uint32_t*>(s + kHeaderBytes + 16 * sym + 4));
-    }
-  }
-  if (S.nused < 2 && tid == 0) S.sorted_rep[0] = S.only_rep;
-  __syncthreads();
+  __syncwarp();  // len_count is complete
 
-  // ---- lookup tables: canonical decode of each entry's own index
-  // First-level prefixes that belong to longer codes get a sub-table each. Sub-tables are as deep as
-  // their number allows (8 KB in all).
-  {
-    const bool miss = tid < (1 << kL1Bits) && S.nused >= 2 && canonical_lookup(S, tid, kL1Bits).y == 0;
-    const uint32_t ballot = __ballot_sync(0xffffffffu, miss);
-    if (tid < (1 << kL1Bits) && (tid & 31) == 0) S.miss_count[tid >> 5] = __popc(ballot);
-    __syncthreads();
-    if (tid < (1 << kL1Bits)) {
-      const uint32_t misses = S.miss_count[0] + S.miss_count[1];
-      uint32_t sub_bits = kSubBitsMax;
-      while (sub_bits > kSubBitsMin && misses > (kTableBytes >> (sub_bits + 3))) sub_bits -= 1;
-      const uint32_t usable = kTableBytes >> (sub_bits + 3);  // >= misses: every such prefix gets a table
-      const uint32_t rank = __popc(ballot & ((1u << (tid & 31)) - 1)) + (tid >= 32 ? S.miss_count[0] : 0u);
-      uint32_t sub = 0;
-      if (miss && rank < usable) {
-        sub = rank;
-        S.prefix_of_sub[sub] = (uint8_t)tid;
-      }
-      S.sub_of_prefix[tid] = (uint8_t)sub;
-      if (tid == 0) {
-        S.nsub = misses < usable ? misses : usable;
-        S.sub_bits = sub_bits;
-      }
-    }
+  // ---- canonical code: codes of length <= L fill the left-aligned range [0, sum over l <= L of count[l] << (63 - l)) of
+  // 2^63, so one inclusive scan over the lengths (two per lane) gives every first code, range end and table offset
+  const uint32_t l0 = 2 * lane, l1 = l0 + 1;
+  const uint32_t c0 = S.len_count[l0], c1 = S.len_count[l1];  // length 0 counts nothing
+  const unsigned long long r0 = (unsigned long long)c0 << (63 - l0), r1 = (unsigned long long)c1 << (63 - l1);
+  unsigned long long range = r0 + r1;
+  uint32_t offset = c0 + c1;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned long long rv = __shfl_up_sync(kAll, range, d);
+    const uint32_t ov = __shfl_up_sync(kAll, offset, d);
+    if ((int)lane >= d) range += rv, offset += ov;
   }
-  __syncthreads();
-  const uint32_t sub_bits = S.sub_bits;
-  for (uint32_t k = tid; k < (1u << kL1Bits) * kL1Rep; k += nthreads) {
-    const uint32_t idx = k / kL1Rep;
-    uint2 ent;
-    if (S.nused < 2) {
-      ent = make_uint2(S.only_rep, 0u);
-    } else {
-      const uint2 r = canonical_lookup(S, idx, kL1Bits);
-      if (r.y) ent = make_uint2(S.sorted_rep[r.x], r.y);
-      // address of the prefix's sub-table, less the offset that the prefix bits add when the lookup indexes it
-      // with prefix and sub-table bits together (32-bit wrap-around arithmetic)
-      else ent = make_uint2(smem_addr(S.sub) + ((uint32_t)S.sub_of_prefix[idx] << (sub_bits + 3)) -
-                                ((idx << sub_bits) << 3), kLongCode);
-    }
-    S.l1[k] = ent;
+  const unsigned long long end1 = range, end0 = range - r1, begin0 = end0 - r0;
+  S.first_code[l0] = begin0 >> (63 - l0);
+  S.first_code[l1] = end0 >> (63 - l1);
+  S.last_aligned[l0] = (end0 << 1) - 1;
+  S.last_aligned[l1] = (end1 << 1) - 1;
+  S.len_offset[l0] = S.len_next[l0] = offset - c1 - c0;
+  S.len_offset[l1] = S.len_next[l1] = offset - c1;
+  if (l0 <= 16) S.end31[l0] = (uint32_t)(end0 >> 32);
+  if (l1 <= 16) S.end31[l1] = (uint32_t)(end1 >> 32);
+  // first-level prefixes behind the codes of at most kL1Bits bits get a sub-table each, as deep as their number allows
+  const uint32_t short_end = (uint32_t)(__shfl_sync(kAll, (kL1Bits & 1) ? end1 : end0, kL1Bits / 2) >> (63 - kL1Bits));
+  const uint32_t misses = nused >= 2 ? (1u << kL1Bits) - min(short_end, 1u << kL1Bits) : 0u;
+  uint32_t sub_bits = kSubBitsMax;
+  while (sub_bits > kSubBitsMin && misses > (kTableBytes >> (sub_bits + 3))) sub_bits -= 1;
+  if (lane == 0) {
+    S.payload_off = payload_off;
+    S.payload_size = payload_size;
+    S.chunk_index_off = L.chunk_index_off;
+    S.lane_index_off = L.lane_index_off;
+    S.max_len = max_len;
+    S.nused = nused;
+    S.only_rep = only_rep;
+    S.nsub = misses;
+    S.sub_bits = sub_bits;
   }
-  for (uint32_t k = tid; k < kTableBytes / 8; k += nthreads) {
-    const uint32_t sub = k >> sub_bits, j = k & ((1u << sub_bits) - 1);
-    uint2 ent = make_uint2(0u, kLongCode);
-    if (sub < S.nsub) {
-      const uint2 r = canonical_lookup(S, ((uint32_t)S.prefix_of_sub[sub] << sub_bits) | j, kL1Bits + sub_bits);
-      if (r.y) ent = make_uint2(S.sorted_rep[r.x], r.y);
+  __syncwarp();
+
+  // ---- representatives in canonical order: a symbol's place among those of its length is by id
+  if (nused >= 2) {
+    for (uint32_t first = 0; first < nsym; first += 32) {
+      const uint32_t sym = first + lane;
+      const uint32_t len = sym < nsym ? sym_len[sym] : 0u;  // 0: a symbol without a code (unused, in a Huffman-coded stream)
+      const uint32_t same = __match_any_sync(kAll, len);
+      const uint32_t place = S.len_next[len] + __popc(same & ((1u << lane) - 1));
+      if (len) S.sorted_rep[min(place, kMaxSymbols - 1)] = sym_rep[sym];
+      __syncwarp();
+      if (len && (int)lane == __ffs(same) - 1) S.len_next[len] += __popc(same);
+      __syncwarp();
     }
-    S.sub[k] = ent;
+  } else if (lane == 0) {
+    S.sorted_rep[0] = only_rep;
   }
-  __syncthreads();
   return 0;
 }
 
-// What the prepare kernel leaves in global memory for one stream and every CTA of the decode kernel copies: the two
-// lookup tables, the stream's state, and the outcome of the validation. First-level entries that point to a sub-table
-// hold that table's offset from the start of the sub-table area there (the shared address is added by the copy).
-struct DecodeImage {
-  uint2 l1[kTableBytes / 8];
-  uint2 sub[kTableBytes / 8];
-  StreamState state;
-  int32_t err;
-  int32_t pad_[3];
-};
-static_assert(sizeof(DecodeImage) <= kDecodeImageBytes, "the workspace region holds four of these");
-static_assert(sizeof(DecodeImage) % 16 == 0 && sizeof(StreamState) % 16 == 0, "copied with 16-byte accesses");
+// {representative, length} of the code at the top of the 31-bit left-aligned window `v`, length 0 if no code of at most
+// `width` (<= 16) bits is there.
+__device__ __forceinline__ uint2 canonical_lookup(const StreamState& S, uint32_t v, uint32_t width) {
+  uint32_t L = 1;
+#pragma unroll
+  for (int l = 1; l <= kL2Bits; ++l) L += v >= S.end31[l] ? 1u : 0u;
+  if (L > width) return make_uint2(0u, 0u);
+  const uint32_t r = (v >> (31 - L)) - (uint32_t)S.first_code[L];
+  if (r >= S.len_count[L]) return make_uint2(0u, 0u);  // only with damaged lengths
+  return make_uint2(S.sorted_rep[min(S.len_offset[L] + r, kMaxSymbols - 1)], L);
+}
 
-constexpr int kPrepThreads = 512;
-constexpr uint32_t kPrepSmem = kTableBytes + 2 * kTableBytes + sizeof(StreamState);
-
-// One CTA per stream: parse, validate, build the tables (in this CTA's shared memory, as the decode kernel would),
-// then write the image.
-__global__ void __launch_bounds__(kPrepThreads)
-decode_prepare_kernel(DecodeStreams streams, uint64_t n, DecodeImage* __restrict__ images) {
-  extern __shared__ __align__(16) unsigned char p_raw[];
-  unsigned char* tables = p_raw + ((kTableBytes - (smem_addr(p_raw) & (kTableBytes - 1))) & (kTableBytes - 1));
-  StreamState& S = *reinterpret_cast<StreamState*>(p_raw + kTableBytes + 2 * kTableBytes);
-  __shared__ int s_err;
-  DecodeImage& img = images[blockIdx.x];
-  const int err = prepare_stream(S, tables, streams.ptr[blockIdx.x], streams.bytes[blockIdx.x], n, &s_err);
-  if (threadIdx.x == 0) img.err = err;
-  if (err) return;
-  const uint32_t sub_addr = smem_addr(S.sub);
-  for (uint32_t k = threadIdx.x; k < kTableBytes / 8; k += kPrepThreads) {
-    uint2 e = S.l1[k];
-    if (e.y == kLongCode) e.x -= sub_addr;
-    img.l1[k] = e;
-    img.sub[k] = S.sub[k];
+// Fills the two table levels of all KS streams; all threads of the CTA.
+template <int KS>
+__device__ __forceinline__ void fill_tables(const StreamState* S, unsigned char* tables) {
+  for (uint32_t k = threadIdx.x; k < KS * (1u << kL1Bits) * (kL1Rep / 2); k += blockDim.x) {  // two copies of an entry each
+    const uint32_t s = k / ((1u << kL1Bits) * (kL1Rep / 2)), pair = k % (kL1Rep / 2);
+    const uint32_t idx = k / (kL1Rep / 2) % (1u << kL1Bits);
+    const StreamState& T = S[s];
+    uint2 ent = make_uint2(T.only_rep, 0u);
+    if (T.nused >= 2) {
+      const uint2 r = canonical_lookup(T, idx << (31 - kL1Bits), kL1Bits);
+      // else the address of the prefix's sub-table, less the offset that the prefix bits add when the lookup indexes it
+      // with prefix and sub-table bits together (32-bit wrap-around arithmetic)
+      const uint32_t sub = idx - ((1u << kL1Bits) - T.nsub);
+      ent = r.y ? r : make_uint2(T.l1_addr + kTableBytes + (sub << (T.sub_bits + 3)) - ((idx << T.sub_bits) << 3), kLongCode);
+    }
+    uint4* l1 = reinterpret_cast<uint4*>(tables + s * 2 * kTableBytes);
+    l1[idx * (kL1Rep / 2) + pair] = make_uint4(ent.x, ent.y, ent.x, ent.y);
   }
-  const uint4* src = reinterpret_cast<const uint4*>(&S);
-  uint4* dst = reinterpret_cast<uint4*>(&img.state);
-  for (uint32_t k = threadIdx.x; k < sizeof(StreamState) / 16; k += kPrepThreads) dst[k] = src[k];
+  for (uint32_t k = threadIdx.x; k < KS * (kTableBytes / 8); k += blockDim.x) {
+    const uint32_t s = k / (kTableBytes / 8), i = k % (kTableBytes / 8);
+    const StreamState& T = S[s];
+    const uint32_t sub = i >> T.sub_bits, j = i & ((1u << T.sub_bits) - 1);
+    uint2 ent = make_uint2(0u, kLongCode);
+    if (sub < T.nsub) {
+      const uint32_t idx = (1u << kL1Bits) - T.nsub + sub, width = kL1Bits + T.sub_bits;
+      const uint2 r = canonical_lookup(T, ((idx << T.sub_bits) | j) << (31 - width), width);
+      if (r.y) ent = r;
+    }
+    reinterpret_cast<uint2*>(tables + s * 2 * kTableBytes + kTableBytes)[i] = ent;
+  }
 }
 
 // Two-level table lookup of the code at the top of `hi`: {representative, length}, length kLongCode if
@@ -356,21 +310,21 @@ __device__ __forceinline__ uint2 lookup_code(uint32_t hi, uint32_t l1lane, uint3
 // the lane's bit buffer behind the code. Returns the representative.
 template <bool STAGED>
 __device__ __forceinline__ uint32_t long_code(LaneBits<STAGED>& B, const StreamState& S, const Source& W,
-                                              int32_t* status) {
+                                              Status status) {
   const uint32_t pos = B.bitpos(W);
   const uint32_t idx = pos >> 5, sh = pos & 31;
   const uint32_t w0 = B.word(W, idx), w1 = B.word(W, idx + 1), w2 = B.word(W, idx + 2);
   const unsigned long long window =
       ((unsigned long long)__funnelshift_l(w1, w0, sh) << 32) | __funnelshift_l(w2, w1, sh);
-  // the first level resolves shorter codes, and so does the prefix's sub-table if it has a real one
-  uint32_t L = kL1Bits + 1 + (S.sub_of_prefix[window >> (64 - kL1Bits)] < S.nsub ? S.sub_bits : 0u);
+  // the first level resolves shorter codes, and so does the prefix's sub-table
+  uint32_t L = kL1Bits + 1 + (S.nsub ? S.sub_bits : 0u);
   while (L < S.max_len && (S.len_count[L] == 0 || window > S.last_aligned[L])) L += 1;
   const unsigned long long code = window >> (64 - L);
   uint32_t rep = 0;
   if (L <= S.max_len && code >= S.first_code[L] && code - S.first_code[L] < S.len_count[L]) {
     rep = S.sorted_rep[S.len_offset[L] + (uint32_t)(code - S.first_code[L])];
   } else {
-    set_status(status, LC_ERR_FORMAT);  // no code matches: damaged payload
+    status.set(LC_ERR_FORMAT);  // no code matches: damaged payload
   }
   B.seek(W, pos + L);
   return rep;
@@ -389,13 +343,28 @@ __device__ __forceinline__ uint32_t long_code(LaneBits<STAGED>& B, const StreamS
 // started, one code at a time with a top-up before each (a top-up makes 32 bits valid, a table-resolved code
 // takes at most 16). Whatever the quick pass did to their buffers in
 // between stays inside the staged chunk (a top-up moves one word per step) and is discarded.
-template <int KS, bool STAGED>
+// PARTIAL: the vector's last chunk. Only the steps that hold elements are visited, and of a step's four slots only
+// the first `have` are loaded, checked and stored. (The lane's codes end with its last element, so what the quick pass
+// decodes behind it are codes of the next lane or the chunk's zero slack; nothing is reported for them.)
+template <bool PARTIAL>
+__device__ __forceinline__ float4 load_row(const float* p, int have) {
+  if (!PARTIAL || have >= 4) return ldg_stream_v4(p);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (have > 0) v.x = p[0];
+  if (have > 1) v.y = p[1];
+  if (have > 2) v.z = p[2];
+  return v;
+}
+
+template <int KS, bool STAGED, bool PARTIAL>
 __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const Source* W, const uint32_t* start,
-                                                    const float* base, float* out, uint64_t c, uint32_t lane,
-                                                    const float* next_rows, int32_t* status) {
+                                                    const float* base, float* out, uint64_t c, uint64_t n, uint32_t lane,
+                                                    const float* next_rows, Status status) {
   LaneBits<STAGED> bits[KS];
+  const int rem = PARTIAL ? (int)(n - c * kChunkElems) - 4 * (int)lane : 0;  // elements from this lane's first slot on
+  const uint32_t steps = PARTIAL ? (uint32_t)(n - c * kChunkElems + 127) / 128 : kSteps;
   // the streams' tables follow each other at 2 * kTableBytes: one base address, the rest as immediate offsets
-  const uint32_t l1lane = smem_addr(S[0].l1) | ((lane & (kL1Rep - 1)) * 8u);
+  const uint32_t l1lane = S[0].l1_addr | ((lane & (kL1Rep - 1)) * 8u);
   uint32_t sub_shift[KS];
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
@@ -403,30 +372,31 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
     sub_shift[s] = 32 - kL1Bits - S[s].sub_bits;
   }
   const uint64_t e0 = c * kChunkElems + 4 * lane;
-  float4 b = ldg_stream_v4(base + e0);
+  float4 b = load_row<PARTIAL>(base + e0, rem);
   // With one stream a step is short, and one row of base in registers ahead of its use leaves too few bytes in flight
   // for the L2's latency (0.80 of the copy rate); a second row brings that to 0.92. With two or more streams the
   // second row makes the kernel slower (measured for 2, 3 and 4 streams), so they keep one.
   float4 b2 = b;
-  if (KS == 1) b2 = ldg_stream_v4(base + e0 + 128);
+  if (KS == 1) b2 = load_row<PARTIAL>(base + e0 + 128, rem - 128);
   // Rows of base are asked into the L2 kPrefetchRows steps before they are loaded: a warp has one row in
   // registers ahead of its use, which alone leaves far too few bytes in flight per SM for the DRAM latency.
   // Behind this chunk's last row the requests go on with the first rows of the chunk this warp decodes next
   // (`next_rows`: this lane's part of that chunk's first row, or of this chunk's first row if there is none).
   const float* pf = base + e0 + 128 * kPrefetchRows<KS>;
 #pragma unroll 1
-  for (uint32_t j = 0; j < kSteps; ++j) {
+  for (uint32_t j = 0; j < steps; ++j) {
     const uint64_t i = e0 + 128ull * j;
+    const int have = rem - 128 * (int)j;  // PARTIAL: slots of this step that hold elements, if fewer than four
     float x[4] = {b.x, b.y, b.z, b.w};
     // the 16 bytes of base of a later step, requested one step ahead (one stream: two steps); the last steps
     // re-read their own
     if (KS == 1) {
       b = b2;
-      b2 = ldg_stream_v4(base + i + (j + 2 < kSteps ? 256 : 0));
+      b2 = PARTIAL ? load_row<PARTIAL>(base + i + 256, have - 256) : ldg_stream_v4(base + i + (j + 2 < kSteps ? 256 : 0));
     } else {
-      b = ldg_stream_v4(base + i + (j + 1 < kSteps ? 128 : 0));
+      b = PARTIAL ? load_row<PARTIAL>(base + i + 128, have - 128) : ldg_stream_v4(base + i + (j + 1 < kSteps ? 128 : 0));
     }
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
+    if (!PARTIAL) asm volatile("prefetch.global.L2 [%0];" ::"l"(pf));
     pf = (j == kSteps - kPrefetchRows<KS> - 1) ? next_rows : pf + 128;
     int cnt0[KS];
     uint32_t flags = 0;
@@ -461,9 +431,10 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
     }
 #pragma unroll
     for (int s = 0; s < KS; ++s) flags |= (uint32_t)bits[s].cnt;
+    if (PARTIAL && have <= 0) flags = 0;
     if (__builtin_expect(__any_sync(0xffffffffu, (int)flags < 0), 0)) {
       if ((int)flags < 0) {
-        const float4 b0 = ldg_stream_v4(base + i);
+        const float4 b0 = load_row<PARTIAL>(base + i, have);
         x[0] = b0.x; x[1] = b0.y; x[2] = b0.z; x[3] = b0.w;
 #pragma unroll
         for (int s = 0; s < KS; ++s) {
@@ -474,6 +445,10 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
 #pragma unroll 1
         for (int e = 0; e < 4; ++e) {
           float v = x[0];
+          if (PARTIAL && e >= have) {
+            x[0] = x[1]; x[1] = x[2]; x[2] = x[3];
+            continue;
+          }
           uint2 ent[KS];
 #pragma unroll
           for (int s = 0; s < KS; ++s) bits[s].refill(W[s]);
@@ -491,184 +466,151 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
         }
       }
     }
-    *reinterpret_cast<float4*>(out + i) = make_float4(x[0], x[1], x[2], x[3]);
+    if (!PARTIAL || have >= 4) {
+      *reinterpret_cast<float4*>(out + i) = make_float4(x[0], x[1], x[2], x[3]);
+    } else {
+      if (have > 0) out[i] = x[0];
+      if (have > 1) out[i + 1] = x[1];
+      if (have > 2) out[i + 2] = x[2];
+    }
   }
 }
 static_assert(kL1Rep * 8 == 128, "first-level entries of one index span 128 bytes");
 
-// The vector's last, partial chunk: element by element (indices beyond n are skipped), each code with a top-up, a
-// table lookup and, if the tables do not resolve it, the canonical search. Out of line: it runs once per call, in one
-// warp, and must not weigh on the registers of the loop above. The chunk's words come from the staging areas if
-// they fit there (a single warp waiting for global memory at every code would take several times as long as all the
-// other chunks of a medium-sized vector together), else from global memory.
-struct PartialChunk {
-  Source W[4];
-  uint32_t start[4];
-  uint32_t sub_shift[4];
-};
-template <int KS, bool STAGED>
-__device__ __noinline__ void decode_chunk_partial(const StreamState* S, PartialChunk P, uint32_t l1lane,
-                                                  const float* base, float* out, uint64_t c, uint64_t n, uint32_t lane,
-                                                  int32_t* status) {
-  LaneBits<STAGED> bits[KS];
+// Chunk `c` of every stream: where its payload is and the lanes' bit counts. An entry that is not a valid range of the
+// payload is reported and taken as empty.
+template <int KS>
+__device__ __forceinline__ bool stage_chunk(const StreamState* S, uint64_t c, uint32_t lane, unsigned char* stage0,
+                                            uint32_t stage_bytes, Source* W, uint32_t* start, Status status) {
+  uint32_t bytes[KS];
+  unsigned long long off0[KS], off1[KS];
+  bool fits = true;
+  // all index loads of all streams first, so that their latencies overlap
 #pragma unroll
-  for (int s = 0; s < KS; ++s) bits[s].seek(P.W[s], P.start[s]);
-#pragma unroll 1
-  for (uint32_t j = 0; j < kSteps; ++j) {
-#pragma unroll 1
-    for (uint32_t e = 0; e < kGroup; ++e) {
-      const uint64_t i = c * kChunkElems + 128ull * j + 4 * lane + e;
-      if (i >= n) continue;
-      float x = base[i];
+  for (int s = 0; s < KS; ++s) {
+    const uint8_t* sp = S[s].ptr;
+    const unsigned long long* ci = reinterpret_cast<const unsigned long long*>(sp + S[s].chunk_index_off);
+    off0[s] = __ldg(ci + c);
+    off1[s] = __ldg(ci + c + 1);
+    const uint16_t* li = reinterpret_cast<const uint16_t*>(sp + S[s].lane_index_off);
+    start[s] = __ldg(li + c * kLanes + lane);
+  }
+  // then the asynchronous copies of the payloads into the staging areas
 #pragma unroll
-      for (int s = 0; s < KS; ++s) {
-        bits[s].refill(P.W[s]);
-        uint2 ent = lookup_code<0>(bits[s].hi, l1lane + s * 2 * kTableBytes, P.sub_shift[s]);
-        if (ent.y > 63u) ent = make_uint2(long_code<STAGED>(bits[s], S[s], P.W[s], status), 0u);  // consumed
-        x = __fadd_rn(x, __uint_as_float(ent.x));
-        bits[s].consume(ent.y);
-      }
-      out[i] = x;
+  for (int s = 0; s < KS; ++s) {
+    if (off0[s] > off1[s] || off1[s] > S[s].payload_size || (off0[s] & 15) || (off1[s] & 15)) {
+      status.set(LC_ERR_FORMAT);
+      off0[s] = off1[s] = 0;
+    }
+    bytes[s] = (uint32_t)min(off1[s] - off0[s], (unsigned long long)kChunkElems * 8);
+    const uint8_t* g = S[s].ptr + S[s].payload_off + off0[s];
+    unsigned char* st = stage0 + (size_t)s * stage_bytes;
+    W[s].g = reinterpret_cast<const uint32_t*>(g);
+    W[s].nw = bytes[s] >> 2;
+    W[s].sbase = smem_addr(st);
+    W[s].slim = W[s].sbase + bytes[s] + 12;
+    // 16 bytes of zero slack after the chunk must fit too
+    if (bytes[s] + 16 <= stage_bytes) {
+      for (uint32_t k = lane * 16; k < bytes[s]; k += 32 * 16) cp_async_16(W[s].sbase + k, g + k);
+      if (lane == 0) *reinterpret_cast<uint4*>(st + bytes[s]) = make_uint4(0, 0, 0, 0);
+    } else {
+      fits = false;
     }
   }
+  cp_async_commit();
+  // lane start offsets (exclusive scan of the lane bit counts) while the copies are in flight
+#pragma unroll
+  for (int s = 0; s < KS; ++s) {
+    const uint32_t lane_bits = start[s];
+    uint32_t incl = lane_bits;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d);
+      if ((int)lane >= d) incl += v;
+    }
+    start[s] = min(incl - lane_bits, bytes[s] * 8u);
+  }
+  cp_async_wait_all();
+  __syncwarp();
+  return fits;
 }
 
+// The vector's last, partial chunk, out of line and outside the main loop: it runs once per call, in one warp, and must
+// not weigh on the registers of the others. On vectors of a few thousand chunks the whole launch waits for that warp, so
+// it runs the same straight-line steps as a whole chunk (one code at a time it took 15 us with one stream and 60 us
+// with four).
+template <int KS>
+__device__ __noinline__ void decode_last_chunk(const StreamState* S, const float* base, float* out, uint64_t c, uint64_t n,
+                                               uint32_t lane, unsigned char* stage0, uint32_t stage_bytes, Status status) {
+  Source W[KS];
+  uint32_t start[KS];
+  __syncwarp();  // the previous chunk's reads of the staging area are done
+  if (stage_chunk<KS>(S, c, lane, stage0, stage_bytes, W, start, status))
+    decode_chunk_fast<KS, true, true>(S, W, start, base, out, c, n, lane, base, status);
+  else
+    decode_chunk_fast<KS, false, true>(S, W, start, base, out, c, n, lane, base, status);
+}
+
+// Chunks [chunk_begin, chunk_end) of one vector, by `ctas` CTAs of which this is number `cta`.
 // stage_bytes: bytes of staging area per warp and stream (a multiple of 16, at least 32).
 template <int KS>
-__global__ void __launch_bounds__(kDecMaxThreads, 1)
-decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status,
-              const DecodeImage* __restrict__ images, uint32_t stage_bytes, uint64_t chunk_begin, uint64_t chunk_end) {
+__device__ __forceinline__ void decode_vector(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
+                                              Status status, uint32_t stage_bytes, uint64_t chunk_begin,
+                                              uint64_t chunk_end, uint32_t cta, uint32_t ctas) {
   // dynamic shared memory: [pad to 128 bytes | 2 tables per stream | StreamState per stream | staging areas]
   extern __shared__ __align__(16) unsigned char s_raw[];
   unsigned char* tables = s_raw + ((kTablePad - (smem_addr(s_raw) & (kTablePad - 1))) & (kTablePad - 1));
   StreamState* S = reinterpret_cast<StreamState*>(s_raw + kTablePad + KS * 2 * kTableBytes);
-  // A launch of a single CTA (a vector of a few chunks) validates the streams and builds their tables itself, which
-  // saves the prepare kernel's launch; `images` is null then.
-  __shared__ int s_err;
-  if (images == nullptr) {
-    for (int s = 0; s < KS; ++s) {
-      const int err = prepare_stream(S[s], tables + s * 2 * kTableBytes, streams.ptr[s], streams.bytes[s], n, &s_err);
-      if (err) {  // the same value for every thread
-        if (threadIdx.x == 0) set_status(status, err);
-        return;
-      }
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  static_assert(KS <= 4 && 5 * kMaxSymbols <= kTableBytes, "a warp per stream; the second level is the scratch");
+  if (warp < KS) {
+    const int err = prepare_stream(S[warp], tables + warp * 2 * kTableBytes + kTableBytes, streams.ptr[warp],
+                                   streams.bytes[warp], n, lane);
+    if (lane == 0) {
+      S[warp].err = err;
+      S[warp].ptr = streams.ptr[warp];
+      S[warp].l1_addr = smem_addr(tables + warp * 2 * kTableBytes);
     }
   }
-  // otherwise the streams were validated and their tables built by decode_prepare_kernel: report a rejected stream
-  // (the same words for every thread) or copy the images in
+  __syncthreads();
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
-    const int err = images ? images[s].err : 0;
-    if (err) {
-      if (threadIdx.x == 0) set_status(status, err);
+    const int err = S[s].err;
+    if (err) {  // the same words for every thread
+      if (threadIdx.x == 0) status.set(err);
       return;
     }
   }
-#pragma unroll
-  for (int s = 0; s < KS && images != nullptr; ++s) {
-    uint2* l1 = reinterpret_cast<uint2*>(tables + s * 2 * kTableBytes);
-    uint2* sub = l1 + kTableBytes / 8;
-    const uint32_t sub_addr = smem_addr(sub);
-    for (uint32_t k = threadIdx.x; k < kTableBytes / 8; k += blockDim.x) {
-      uint2 e = __ldg(&images[s].l1[k]);
-      if (e.y == kLongCode) e.x += sub_addr;
-      l1[k] = e;
-      sub[k] = __ldg(&images[s].sub[k]);
-    }
-    const uint4* src = reinterpret_cast<const uint4*>(&images[s].state);
-    uint4* dst = reinterpret_cast<uint4*>(&S[s]);
-    for (uint32_t k = threadIdx.x; k < sizeof(StreamState) / 16; k += blockDim.x) dst[k] = __ldg(src + k);
-  }
-  __syncthreads();
-  if (threadIdx.x < KS) {
-    S[threadIdx.x].l1 = reinterpret_cast<uint2*>(tables + threadIdx.x * 2 * kTableBytes);
-    S[threadIdx.x].sub = S[threadIdx.x].l1 + kTableBytes / 8;
-  }
+  fill_tables<KS>(S, tables);
   __syncthreads();
 
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   unsigned char* stage0 = reinterpret_cast<unsigned char*>(S + KS) + (size_t)warp * KS * stage_bytes;
-  const uint64_t warp0 = chunk_begin + (uint64_t)blockIdx.x * warps + warp;  // this launch decodes [chunk_begin, chunk_end)
-  const uint64_t nwarps = (uint64_t)gridDim.x * warps;
-
-  for (uint64_t c = warp0; c < chunk_end; c += nwarps) {
+  const uint64_t nwarps = (uint64_t)ctas * warps;
+  const uint64_t whole_end = min(chunk_end, n / kChunkElems);  // the chunks that are full
+  uint64_t c = chunk_begin + (uint64_t)cta * warps + warp;
+  for (; c < whole_end; c += nwarps) {
     Source W[KS];
-    uint32_t start[KS], bytes[KS];
-    unsigned long long off0[KS], off1[KS];
-    bool fits = true;
+    uint32_t start[KS];
     __syncwarp();  // the previous chunk's reads of the staging area are done
-    // all index loads of all streams first, so that their latencies overlap
-#pragma unroll
-    for (int s = 0; s < KS; ++s) {
-      const uint8_t* sp = streams.ptr[s];
-      const unsigned long long* ci = reinterpret_cast<const unsigned long long*>(sp + S[s].chunk_index_off);
-      off0[s] = __ldg(ci + c);
-      off1[s] = __ldg(ci + c + 1);
-      const uint16_t* li = reinterpret_cast<const uint16_t*>(sp + S[s].lane_index_off);
-      start[s] = __ldg(li + c * kLanes + lane);
-    }
-    // then the asynchronous copies of the payloads into the staging areas
-#pragma unroll
-    for (int s = 0; s < KS; ++s) {
-      if (off0[s] > off1[s] || off1[s] > S[s].payload_size || (off0[s] & 15) || (off1[s] & 15)) {
-        set_status(status, LC_ERR_FORMAT);
-        off0[s] = off1[s] = 0;
-      }
-      bytes[s] = (uint32_t)min(off1[s] - off0[s], (unsigned long long)kChunkElems * 8);
-      const uint8_t* g = streams.ptr[s] + S[s].payload_off + off0[s];
-      unsigned char* st = stage0 + (size_t)s * stage_bytes;
-      W[s].g = reinterpret_cast<const uint32_t*>(g);
-      W[s].nw = bytes[s] >> 2;
-      W[s].sbase = smem_addr(st);
-      W[s].slim = W[s].sbase + bytes[s] + 12;
-      // 16 bytes of zero slack after the chunk must fit too
-      if (bytes[s] + 16 <= stage_bytes) {
-        for (uint32_t k = lane * 16; k < bytes[s]; k += 32 * 16) cp_async_16(W[s].sbase + k, g + k);
-        if (lane == 0) *reinterpret_cast<uint4*>(st + bytes[s]) = make_uint4(0, 0, 0, 0);
-      } else {
-        fits = false;
-      }
-    }
-    cp_async_commit();
-    // lane start offsets (exclusive scan of the lane bit counts) while the copies are in flight
-#pragma unroll
-    for (int s = 0; s < KS; ++s) {
-      const uint32_t lane_bits = start[s];
-      uint32_t incl = lane_bits;
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d);
-        if ((int)lane >= d) incl += v;
-      }
-      start[s] = min(incl - lane_bits, bytes[s] * 8u);
-    }
-    cp_async_wait_all();
-    __syncwarp();
-    if ((c + 1) * kChunkElems <= n) {
-      // where the L2 prefetch goes on behind this chunk: the next chunk of this warp, if it is a full one
-      const uint64_t cn = c + nwarps;
-      const float* next_rows = base + (cn < chunk_end && (cn + 1) * kChunkElems <= n ? cn : c) * kChunkElems + 4 * lane;
-      if (fits) decode_chunk_fast<KS, true>(S, W, start, base, out, c, lane, next_rows, status);
-      else decode_chunk_fast<KS, false>(S, W, start, base, out, c, lane, next_rows, status);
-    } else {
-      PartialChunk P;
-#pragma unroll
-      for (int s = 0; s < KS; ++s) {
-        P.W[s] = W[s];
-        P.start[s] = start[s];
-        P.sub_shift[s] = 32 - kL1Bits - S[s].sub_bits;
-      }
-      const uint32_t l1lane = smem_addr(S[0].l1) | ((lane & (kL1Rep - 1)) * 8u);
-      if (fits) decode_chunk_partial<KS, true>(S, P, l1lane, base, out, c, n, lane, status);
-      else decode_chunk_partial<KS, false>(S, P, l1lane, base, out, c, n, lane, status);
-    }
+    const bool fits = stage_chunk<KS>(S, c, lane, stage0, stage_bytes, W, start, status);
+    // where the L2 prefetch goes on behind this chunk: the next full chunk of this warp, if there is one
+    const float* next_rows = base + (c + nwarps < whole_end ? c + nwarps : c) * kChunkElems + 4 * lane;
+    if (fits) decode_chunk_fast<KS, true, false>(S, W, start, base, out, c, n, lane, next_rows, status);
+    else decode_chunk_fast<KS, false, false>(S, W, start, base, out, c, n, lane, next_rows, status);
   }
+  if (c < chunk_end) decode_last_chunk<KS>(S, base, out, c, n, lane, stage0, stage_bytes, status);
+}
+
+template <int KS>
+__global__ void __launch_bounds__(kDecMaxThreads, 1)
+decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status,
+              uint32_t stage_bytes, uint64_t chunk_begin, uint64_t chunk_end) {
+  decode_vector<KS>(base, streams, n, out, Status{status}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
 }
 
 template <int KS>
 cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
-                             int32_t* status, DecodeImage* images, uint64_t chunk_begin, uint64_t chunk_end,
-                             bool prepare, cudaStream_t cs) {
+                             int32_t* status, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
   static int sms_of[kMaxDevices] = {};  // by device ordinal; non-zero once the kernel's attributes are set there
   constexpr uint32_t kTables = kTablePad + KS * (2 * kTableBytes + sizeof(StreamState));
   constexpr uint32_t kMaxDyn = kSmemPerSm - 1024 - kOverrunBytes;  // room for static __shared__ and the padding
@@ -746,45 +688,23 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
     if (cudaFuncSetAttribute(decode_kernel<KS>, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess)
       return cudaErrorUnknown;
   }
-  // The streams' tables: built by one CTA per stream ahead of a launch of many CTAs, by the decoding CTA itself when
-  // there is only one (`images` null), or left from an earlier launch over the same streams (`prepare` false).
-  const DecodeImage* use = images;
-  if (prepare) {
-    if (grid == 1) {
-      use = nullptr;
-    } else {
-      decode_prepare_kernel<<<KS, kPrepThreads, kPrepSmem, cs>>>(streams, n, images);
-      if (cudaGetLastError() != cudaSuccess) return cudaErrorLaunchFailure;
-    }
-  }
-  decode_kernel<KS><<<grid, warps * 32, dyn, cs>>>(base, streams, n, out, status, use, stage, chunk_begin, chunk_end);
+  decode_kernel<KS><<<grid, warps * 32, dyn, cs>>>(base, streams, n, out, status, stage, chunk_begin, chunk_end);
   return cudaGetLastError();
 }
 
 }  // namespace
 
 cudaError_t launch_decode(const float* base, const DecodeStreams& streams, int k, uint64_t n, float* out,
-                          int32_t* status, void* images, cudaStream_t cs, uint64_t chunk_begin, uint64_t chunk_end,
-                          bool prepare) {
+                          int32_t* status, cudaStream_t cs, uint64_t chunk_begin, uint64_t chunk_end) {
   if (k < 1 || k > 4) return cudaErrorInvalidValue;
   const uint64_t all_chunks = (n + kChunkElems - 1) / kChunkElems;
   if (chunk_end > all_chunks) chunk_end = all_chunks;
   if (chunk_begin > chunk_end) chunk_begin = chunk_end;
-  static bool prep_ready[kMaxDevices] = {};  // by device ordinal
-  const int dev = current_device_index();
-  if (dev < 0) return cudaErrorInvalidDevice;
-  if (!prep_ready[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(decode_prepare_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)kPrepSmem);
-    if (e != cudaSuccess) return e;
-    prep_ready[dev] = true;
-  }
-  DecodeImage* img = static_cast<DecodeImage*>(images);
   switch (k) {
-    case 1: return launch_decode_ks<1>(base, streams, n, out, status, img, chunk_begin, chunk_end, prepare, cs);
-    case 2: return launch_decode_ks<2>(base, streams, n, out, status, img, chunk_begin, chunk_end, prepare, cs);
-    case 3: return launch_decode_ks<3>(base, streams, n, out, status, img, chunk_begin, chunk_end, prepare, cs);
-    case 4: return launch_decode_ks<4>(base, streams, n, out, status, img, chunk_begin, chunk_end, prepare, cs);
+    case 1: return launch_decode_ks<1>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
+    case 2: return launch_decode_ks<2>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
+    case 3: return launch_decode_ks<3>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
+    case 4: return launch_decode_ks<4>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
     default: return cudaErrorInvalidValue;
   }
 }
