@@ -179,10 +179,8 @@ int lc_compress_timed(const float* base, const float* cur, uint64_t n, int nbits
   return ok ? LC_OK : LC_ERR_CUDA;
 }
 
-// lc_recover; reset_status: false when an earlier part of the same call may already have set the status word
-static int recover_impl(const float* base, const void* const* streams, const uint64_t* stream_bytes, int k,
-                        uint64_t n, float* out, void* workspace, uint64_t workspace_bytes, lc_cuda_stream_t cs,
-                        bool reset_status) {
+int lc_recover(const float* base, const void* const* streams, const uint64_t* stream_bytes, int k,
+               uint64_t n, float* out, void* workspace, uint64_t workspace_bytes, lc_cuda_stream_t cs) {
   if (k < 1 || k > LC_MAX_CHAIN || n >= (1ull << 32)) return LC_ERR_ARG;
   if (!streams || !stream_bytes || !workspace || (n > 0 && (!base || !out))) return LC_ERR_ARG;
   if (!aligned(base, 16) || !aligned(out, 16) || !aligned(workspace, 256)) return LC_ERR_ARG;
@@ -190,7 +188,7 @@ static int recover_impl(const float* base, const void* const* streams, const uin
     if (!streams[j] || !aligned(streams[j], 16)) return LC_ERR_ARG;
   if (workspace_bytes < workspace_layout(0).total) return LC_ERR_CAPACITY;
   Control* ctl = static_cast<Control*>(workspace);
-  if (reset_status && cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
+  if (cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
   // up to four streams per launch; later launches continue in place from `out`.
   const float* src = base;
   for (int first = 0; first < k; first += 4) {
@@ -201,15 +199,10 @@ static int recover_impl(const float* base, const void* const* streams, const uin
       ds.ptr[j] = static_cast<const uint8_t*>(streams[first + j]);
       ds.bytes[j] = stream_bytes[first + j];
     }
-    if (launch_decode(src, ds, kk, n, out, &ctl->status, cs) != cudaSuccess) return LC_ERR_CUDA;
+    if (launch_decode(src, ds, kk, n, out, &ctl->status, first > 0, cs) != cudaSuccess) return LC_ERR_CUDA;
     src = out;
   }
   return LC_OK;
-}
-
-int lc_recover(const float* base, const void* const* streams, const uint64_t* stream_bytes, int k,
-               uint64_t n, float* out, void* workspace, uint64_t workspace_bytes, lc_cuda_stream_t cs) {
-  return recover_impl(base, streams, stream_bytes, k, n, out, workspace, workspace_bytes, cs, true);
 }
 
 // ---- per-layer granularity: one stream per segment of the vector --------------------------------------------
@@ -264,20 +257,30 @@ int lc_recover_segments(const float* base, const void* const* streams, int k, co
     return LC_ERR_ARG;
   for (int j = 0; j < k; ++j)
     if (!streams[j] || !aligned(streams[j], 256)) return LC_ERR_ARG;
+  if (!workspace || !aligned(workspace, 256) || (seg_begin[nseg] > 0 && (!base || !out)) || !aligned(base, 16) || !aligned(out, 16))
+    return LC_ERR_ARG;
+  if (workspace_bytes < workspace_layout(0).total) return LC_ERR_CAPACITY;
+  Control* ctl = static_cast<Control*>(workspace);
+  if (cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
+  SegBatch batch;
   uint64_t off = 0;
-  for (int i = 0; i < nseg; ++i) {
-    const uint64_t lo = seg_begin[i], ni = seg_begin[i + 1] - lo;
-    const uint64_t cap = align_up(lc_stream_bound(ni, nbits), 256);
-    const void* seg_streams[LC_MAX_CHAIN];
-    uint64_t seg_bytes[LC_MAX_CHAIN];
-    for (int j = 0; j < k; ++j) {
-      seg_streams[j] = static_cast<const uint8_t*>(streams[j]) + off;
-      seg_bytes[j] = cap;
+  for (int i = 0; i < nseg;) {
+    batch.first = (uint32_t)i;
+    for (batch.nseg = 0; batch.nseg < kSegBatch && i < nseg; ++batch.nseg, ++i) {
+      batch.elem_begin[batch.nseg] = seg_begin[i];
+      batch.stream_begin[batch.nseg] = off;
+      off += align_up(lc_stream_bound(seg_begin[i + 1] - seg_begin[i], nbits), 256);
     }
-    const int rc = recover_impl(base + lo, seg_streams, seg_bytes, k, ni, out + lo, workspace, workspace_bytes, cs,
-                                /*reset_status=*/i == 0);
-    if (rc != LC_OK) return rc;
-    off += cap;
+    batch.elem_begin[batch.nseg] = seg_begin[i];
+    batch.stream_begin[batch.nseg] = off;
+    // up to four streams of every segment per launch; later launches continue in place from `out`
+    for (int first = 0; first < k; first += 4) {
+      const uint8_t* group[4];
+      const int kk = (k - first) < 4 ? (k - first) : 4;
+      for (int j = 0; j < kk; ++j) group[j] = static_cast<const uint8_t*>(streams[first + j]);
+      if (launch_decode_segments(first == 0 ? base : out, group, kk, batch, nbits, out, &ctl->status, first > 0, cs) != cudaSuccess)
+        return LC_ERR_CUDA;
+    }
   }
   return LC_OK;
 }
@@ -530,7 +533,7 @@ extern "C" int lc_recover_host(const float* base_host, const void* const* stream
         ds.ptr[j] = static_cast<const uint8_t*>(d_streams[first + j]);
         ds.bytes[j] = stream_bytes[first + j];
       }
-      if (launch_decode(d_x, ds, kk, n, d_x, &ctl->status, cs, c0, c1) != cudaSuccess) return LC_ERR_CUDA;
+      if (launch_decode(d_x, ds, kk, n, d_x, &ctl->status, g > 0, cs, c0, c1) != cudaSuccess) return LC_ERR_CUDA;
     }
     if (cudaEventRecord(pipe.decoded[i], cs) != cudaSuccess) return LC_ERR_CUDA;
     if (cudaStreamWaitEvent(pipe.out, pipe.decoded[i], 0) != cudaSuccess) return LC_ERR_CUDA;

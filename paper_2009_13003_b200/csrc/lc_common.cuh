@@ -68,7 +68,7 @@ struct EncEntry {
 // Control block at the start of the workspace. Zeroed at the start of every lc_compress.
 struct Control {
   int32_t status;         // first device-detected error, 0 if none
-  uint32_t ticket;        // next chunk of the encode pass
+  uint32_t ticket;        // next chunk of the encode pass; in a recovery, the rank of the error (set_status_ranked)
   uint32_t nsym;          // written by the table kernel
   uint32_t max_len;       // written by the table kernel
   uint64_t payload_bits;  // written by the table kernel
@@ -114,6 +114,19 @@ __host__ __device__ constexpr inline WorkspaceLayout workspace_layout(uint64_t n
 
 // ---- device helpers ----------------------------------------------------------------------------
 __device__ inline void set_status(int32_t* status, int32_t code) { atomicCAS(status, 0, code); }
+
+// For a launch that does in parallel what is defined as a sequence (the segments of a vector, a chain's streams): of
+// several failures the one with the smallest rank stays. The rank stands in the word behind the status word, and means
+// something only once the status is set.
+static __device__ __noinline__ void set_status_ranked(int32_t* status, uint32_t rank, int32_t code) {
+  unsigned long long* w = reinterpret_cast<unsigned long long*>(status);  // the control block is 256-byte aligned
+  unsigned long long old = *reinterpret_cast<volatile unsigned long long*>(w);
+  while ((uint32_t)old == 0 || (uint32_t)(old >> 32) > rank) {
+    const unsigned long long seen = atomicCAS(w, old, (unsigned long long)rank << 32 | (uint32_t)code);
+    if (seen == old) return;
+    old = seen;
+  }
+}
 
 // ---- per-device launch parameters ---------------------------------------------------------------------
 // Occupancy figures, SM counts and the "attributes are set" marks that the launchers cache are properties of a
@@ -167,8 +180,23 @@ struct DecodeStreams {
   const uint8_t* ptr[4];
   uint64_t bytes[4];
 };
-// Decodes the chunks [chunk_begin, chunk_end) only (clipped to the vector's chunks).
+// The segments of one launch of the per-layer recovery, passed by value (within the 4 KB that kernel parameters may
+// take): where each begins in the vector and in every streams buffer, and which CTAs work on it.
+constexpr uint32_t kSegBatch = 160;
+struct SegBatch {
+  uint32_t nseg;
+  uint32_t first;                       // number of the first of them among the segments of the call
+  uint32_t cta_begin[kSegBatch + 1];    // filled in by the launcher
+  uint64_t elem_begin[kSegBatch + 1];
+  uint64_t stream_begin[kSegBatch + 1]; // segment i's stream has the bytes up to stream_begin[i + 1]
+};
+// Decodes every segment's k <= 4 streams onto its part of base, in one launch; second: later streams of the same chains.
+// The streams of segment i start at streams[j] + stream_begin[i].
+cudaError_t launch_decode_segments(const float* base, const uint8_t* const* streams, int k, SegBatch& batch, int nbits,
+                                   float* out, int32_t* status, bool second, cudaStream_t cs);
+
+// Decodes the chunks [chunk_begin, chunk_end) only (clipped to the vector's chunks). second: as above.
 cudaError_t launch_decode(const float* base, const DecodeStreams& streams, int k, uint64_t n, float* out,
-                          int32_t* status, cudaStream_t cs, uint64_t chunk_begin = 0, uint64_t chunk_end = ~0ull);
+                          int32_t* status, bool second, cudaStream_t cs, uint64_t chunk_begin = 0, uint64_t chunk_end = ~0ull);
 
 }  // namespace lc

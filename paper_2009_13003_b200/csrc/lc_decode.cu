@@ -61,10 +61,11 @@ constexpr uint32_t kTableBytes = 8192;
 constexpr uint32_t kTablePad = 128;  // the tables start on a 128-byte boundary (a lane's copy of an entry is chosen by OR)
 static_assert((1 << kL1Bits) * kL1Rep * 8 == kTableBytes, "table sizes");
 
-// Where device-detected errors go: the first one stays.
+// Where device-detected errors go.
 struct Status {
   int32_t* word;
-  __device__ __forceinline__ void set(int32_t code) const { set_status(word, code); }
+  uint32_t rank;
+  __device__ __forceinline__ void set(int32_t code) const { set_status_ranked(word, rank, code); }
 };
 
 struct alignas(16) StreamState {
@@ -564,11 +565,15 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   static_assert(KS <= 4 && 5 * kMaxSymbols <= kTableBytes, "a warp per stream; the second level is the scratch");
   if (warp < KS) {
-    const int err = prepare_stream(S[warp], tables + warp * 2 * kTableBytes + kTableBytes, streams.ptr[warp],
-                                   streams.bytes[warp], n, lane);
+    const uint8_t* ptr = streams.ptr[0];
+    uint64_t bytes = streams.bytes[0];
+#pragma unroll
+    for (int s = 1; s < KS; ++s)
+      if (warp == s) ptr = streams.ptr[s], bytes = streams.bytes[s];
+    const int err = prepare_stream(S[warp], tables + warp * 2 * kTableBytes + kTableBytes, ptr, bytes, n, lane);
     if (lane == 0) {
       S[warp].err = err;
-      S[warp].ptr = streams.ptr[warp];
+      S[warp].ptr = ptr;
       S[warp].l1_addr = smem_addr(tables + warp * 2 * kTableBytes);
     }
   }
@@ -603,108 +608,188 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
 
 template <int KS>
 __global__ void __launch_bounds__(kDecMaxThreads, 1)
-decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status,
+decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status, uint32_t rank,
               uint32_t stage_bytes, uint64_t chunk_begin, uint64_t chunk_end) {
-  decode_vector<KS>(base, streams, n, out, Status{status}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
+  decode_vector<KS>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
 }
 
+// Per-layer recovery: the CTAs [cta_begin[i], cta_begin[i + 1]) decode segment i. One launch instead of one per segment
+// (a segment of a few chunks occupies one SM for the 15 us that a chunk takes; 62 of them in a row took 870 us).
 template <int KS>
-cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
-                             int32_t* status, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
-  static int sms_of[kMaxDevices] = {};  // by device ordinal; non-zero once the kernel's attributes are set there
+__global__ void __launch_bounds__(kDecMaxThreads, 1)
+decode_segments_kernel(const float* base, const __grid_constant__ DecodeStreams buffers, float* out,
+                       int32_t* __restrict__ status, uint32_t second, uint32_t stage_bytes,
+                       const __grid_constant__ SegBatch batch) {
+  uint32_t lo = 0, hi = batch.nseg;  // cta_begin[lo] <= blockIdx.x < cta_begin[hi]
+  while (hi - lo > 1) {
+    const uint32_t mid = (lo + hi) / 2;
+    if (batch.cta_begin[mid] <= blockIdx.x) lo = mid;
+    else hi = mid;
+  }
+  const uint64_t first = batch.elem_begin[lo], n = batch.elem_begin[lo + 1] - first;
+  const uint64_t off = batch.stream_begin[lo], bytes = batch.stream_begin[lo + 1] - off;
+  DecodeStreams streams;
+#pragma unroll
+  for (int s = 0; s < KS; ++s) {
+    streams.ptr[s] = buffers.ptr[s] + off;
+    streams.bytes[s] = bytes;
+  }
+  decode_vector<KS>(base + first, streams, n, out + first, Status{status, 2 * (batch.first + lo) + second}, stage_bytes, 0,
+                    (n + kChunkElems - 1) / kChunkElems, blockIdx.x - batch.cta_begin[lo],
+                    batch.cta_begin[lo + 1] - batch.cta_begin[lo]);
+}
+
+// Launch shape: CTAs of `warps` warps, `per_sm` of them on an SM, `stage` bytes of staging area per warp and stream.
+struct Shape {
+  uint32_t warps, stage, dyn, per_sm, sms;
+};
+
+// What bounds the CTAs on an SM: registers (allocated in units of 256 per warp), shared memory (1 KB per CTA is the
+// system's) and 64 warps. Computed here because the occupancy query costs the host about a microsecond a call.
+inline uint32_t ctas_on_sm(uint32_t warps, uint32_t dyn, uint32_t regs) {
+  const uint32_t per_warp = (regs * 32 + 255) / 256 * 256;
+  const uint32_t by_regs = 65536 / per_warp / 4 * 4 / warps;  // warps are spread over four schedulers
+  const uint32_t by_smem = 228 * 1024 / (dyn + 1024), by_warps = 64 / warps;
+  return min(min(by_regs, by_smem), by_warps);
+}
+
+// want_stage: staging bytes that hold an average chunk with some room. Among CTAs of 16, 12 and 8 warps, takes the shape
+// that puts most warps on an SM (with four streams that is one CTA of 16 warps, with one stream several smaller ones),
+// then gives the staging areas whatever shared memory that shape leaves (chunk sizes vary around the average).
+template <int KS>
+cudaError_t decode_shape(const void* fn, uint64_t want_stage, uint32_t (&regs_of)[kMaxDevices], Shape& best) {
   constexpr uint32_t kTables = kTablePad + KS * (2 * kTableBytes + sizeof(StreamState));
   constexpr uint32_t kMaxDyn = kSmemPerSm - 1024 - kOverrunBytes;  // room for static __shared__ and the padding
+  constexpr uint32_t kMaxStage = kChunkElems * 8 + 16;
+  static int sms_of[kMaxDevices] = {};
   const int dev = current_device_index();
   if (dev < 0) return cudaErrorInvalidDevice;
-  if (sms_of[dev] == 0) {
+  if (regs_of[dev] == 0) {  // by device ordinal; non-zero once the kernel's attributes are set there
     int v = 0;
+    cudaFuncAttributes at;
     cudaError_t e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(decode_kernel<KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kMaxDyn + kOverrunBytes));
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, fn);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxDyn + kOverrunBytes));
     if (e != cudaSuccess) return e;
     sms_of[dev] = v;
+    regs_of[dev] = (uint32_t)at.numRegs;
   }
-  const int sms = sms_of[dev];
-  const uint64_t nchunks = (n + kChunkElems - 1) / kChunkElems;
-  // Staging per warp and stream: 1.03 x the largest average chunk of the streams (from the buffer sizes,
-  // which bound the payload). Among CTAs of 16, 12 and 8 warps, take the shape that puts most warps on an
-  // SM (shared memory and registers both count; with four streams that is one CTA of 16 warps, with one
-  // stream several smaller CTAs).
-  uint64_t avg = 0;
-  for (int s = 0; s < KS; ++s) {
-    const uint64_t index_bytes = 72 * nchunks;  // lane and chunk index entries are not staged
-    const uint64_t a = (streams.bytes[s] > index_bytes ? streams.bytes[s] - index_bytes : 0) / (nchunks ? nchunks : 1);
-    avg = a > avg ? a : avg;
-  }
-  uint64_t want_stage = align_up(avg + avg / 32 + 48, 16);
-  if (want_stage > kChunkElems * 8 + 16) want_stage = kChunkElems * 8 + 16;
-  uint32_t warps = 8, stage = 0, dyn = 0, best_warps_per_sm = 0, ctas_per_sm = 1;
+  const uint32_t regs = regs_of[dev];
+  if (want_stage > kMaxStage) want_stage = kMaxStage;
+  best = Shape{0, 0, 0, 0, (uint32_t)sms_of[dev]};
   for (uint32_t w = 16; w >= 8; w -= 4) {
     uint32_t st = (uint32_t)want_stage;
     if (kTables + (uint64_t)w * KS * st > kMaxDyn) {
       if (w > 8) continue;                               // try fewer warps first
       st = ((kMaxDyn - kTables) / (w * KS)) / 16 * 16;   // last resort: what fits; large chunks decode from global
     }
-    const uint32_t d = kTables + w * KS * st + kOverrunBytes;
-    int bps = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, decode_kernel<KS>, (int)(w * 32), d) != cudaSuccess)
-      return cudaErrorUnknown;
-    if (bps < 1) continue;
-    if ((uint32_t)bps * w > best_warps_per_sm) {
-      best_warps_per_sm = (uint32_t)bps * w;
-      warps = w;
-      stage = st;
-      dyn = d;
-      ctas_per_sm = (uint32_t)bps;
+    const uint32_t d = kTables + w * KS * st + kOverrunBytes, bps = ctas_on_sm(w, d, regs);
+    if (bps * w > best.per_sm * best.warps) {
+      best.warps = w;
+      best.stage = st;
+      best.dyn = d;
+      best.per_sm = bps;
     }
   }
-  if (best_warps_per_sm == 0) return cudaErrorLaunchOutOfResources;
-  // chunk sizes vary around the average: give the staging areas whatever shared memory this shape leaves
-  {
-    const uint32_t budget = kSmemPerSm / ctas_per_sm - 1024 - 64;
-    if (budget > kTables + kOverrunBytes) {
-      uint32_t st = ((budget - kTables - kOverrunBytes) / (warps * KS)) / 16 * 16;
-      if (st > kChunkElems * 8 + 16) st = kChunkElems * 8 + 16;
-      const uint32_t d = kTables + warps * KS * st + kOverrunBytes;
-      int bps = 0;
-      if (st > stage && d <= kMaxDyn + kOverrunBytes &&
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, decode_kernel<KS>, (int)(warps * 32), d) == cudaSuccess &&
-          (uint32_t)bps >= ctas_per_sm) {
-        stage = st;
-        dyn = d;
-      }
+  if (best.per_sm == 0) return cudaErrorLaunchOutOfResources;
+  const uint32_t budget = kSmemPerSm / best.per_sm - 1024 - 64;
+  if (budget > kTables + kOverrunBytes) {
+    uint32_t st = ((budget - kTables - kOverrunBytes) / (best.warps * KS)) / 16 * 16;
+    if (st > kMaxStage) st = kMaxStage;
+    const uint32_t d = kTables + best.warps * KS * st + kOverrunBytes;
+    if (st > best.stage && d <= kMaxDyn + kOverrunBytes && ctas_on_sm(best.warps, d, regs) >= best.per_sm) {
+      best.stage = st;
+      best.dyn = d;
     }
   }
-  uint64_t want = (chunk_end - chunk_begin + warps - 1) / warps;
+  // shared-memory carve-out in percent of the SM's 228 KB: what the resident CTAs use (dynamic, static and the
+  // 1 KB per CTA that the system reserves), so that whatever is left serves as L1
+  const int carve = (int)(((uint64_t)best.per_sm * (best.dyn + 2048) * 100 + 228 * 1024 - 1) / (228 * 1024)) + 1;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve < 100 ? carve : 100);
+}
+
+template <int KS>
+cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
+                             int32_t* status, bool second, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
+  static uint32_t regs_of[kMaxDevices] = {};
+  const uint64_t nchunks = (n + kChunkElems - 1) / kChunkElems;
+  // 1.03 x the largest average chunk of the streams (from the buffer sizes, which bound the payload)
+  uint64_t avg = 0;
+  for (int s = 0; s < KS; ++s) {
+    const uint64_t index_bytes = 72 * nchunks;  // lane and chunk index entries are not staged
+    const uint64_t a = (streams.bytes[s] > index_bytes ? streams.bytes[s] - index_bytes : 0) / (nchunks ? nchunks : 1);
+    avg = a > avg ? a : avg;
+  }
+  Shape sh;
+  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_kernel<KS>), align_up(avg + avg / 32 + 48, 16),
+                                         regs_of, sh);
+  if (e != cudaSuccess) return e;
+  uint64_t want = (chunk_end - chunk_begin + sh.warps - 1) / sh.warps;
   if (want == 0) want = 1;  // still reports a rejected stream
-  const uint64_t full = (uint64_t)sms * ctas_per_sm;
+  const uint64_t full = (uint64_t)sh.sms * sh.per_sm;
   const unsigned grid = (unsigned)(want < full ? want : full);
-  {
-    // shared-memory carve-out in percent of the SM's 228 KB: what the resident CTAs use (dynamic, static and the
-    // 1 KB per CTA that the system reserves), so that whatever is left serves as L1
-    int carve = (int)(((uint64_t)ctas_per_sm * (dyn + 2048) * 100 + 228 * 1024 - 1) / (228 * 1024)) + 1;
-    if (carve > 100) carve = 100;
-    if (cudaFuncSetAttribute(decode_kernel<KS>, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess)
-      return cudaErrorUnknown;
+  decode_kernel<KS><<<grid, sh.warps * 32, sh.dyn, cs>>>(base, streams, n, out, status, second ? 1u : 0u, sh.stage, chunk_begin,
+                                                         chunk_end);
+  return cudaGetLastError();
+}
+
+template <int KS>
+cudaError_t launch_segments_ks(const float* base, const uint8_t* const* streams, SegBatch& batch, int nbits, float* out,
+                               int32_t* status, bool second, cudaStream_t cs) {
+  static uint32_t regs_of[kMaxDevices] = {};
+  // the buffers are sized for nbits bits per element, which no chunk exceeds by much
+  Shape sh;
+  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_segments_kernel<KS>),
+                                         align_up((uint64_t)nbits * (kChunkElems / 8) + 64, 16), regs_of, sh);
+  if (e != cudaSuccess) return e;
+  DecodeStreams buffers;
+  for (int s = 0; s < 4; ++s) buffers.ptr[s] = s < KS ? streams[s] : nullptr, buffers.bytes[s] = 0;
+  // Chunks per CTA: one per warp while all CTAs fit on the device at once, else as many more as it takes for that
+  // (a second wave of CTAs would cost their preparation again and leave the SMs idle at its end).
+  const uint64_t slots = (uint64_t)sh.sms * sh.per_sm;
+  uint64_t ctas = 0;
+  for (uint64_t per_cta = sh.warps;; per_cta += sh.warps) {
+    ctas = 0;
+    uint64_t longest = 0;
+    for (uint32_t i = 0; i < batch.nseg; ++i) {
+      const uint64_t chunks = (batch.elem_begin[i + 1] - batch.elem_begin[i] + kChunkElems - 1) / kChunkElems;
+      batch.cta_begin[i] = (uint32_t)ctas;
+      ctas += chunks ? (chunks + per_cta - 1) / per_cta : 1;  // an empty segment's stream is validated too
+      longest = chunks > longest ? chunks : longest;
+    }
+    if (ctas <= slots || per_cta >= longest) break;
   }
-  decode_kernel<KS><<<grid, warps * 32, dyn, cs>>>(base, streams, n, out, status, stage, chunk_begin, chunk_end);
+  batch.cta_begin[batch.nseg] = (uint32_t)ctas;
+  decode_segments_kernel<KS><<<(unsigned)ctas, sh.warps * 32, sh.dyn, cs>>>(base, buffers, out, status, second ? 1u : 0u, sh.stage,
+                                                                           batch);
   return cudaGetLastError();
 }
 
 }  // namespace
 
+cudaError_t launch_decode_segments(const float* base, const uint8_t* const* streams, int k, SegBatch& batch, int nbits,
+                                   float* out, int32_t* status, bool second, cudaStream_t cs) {
+  switch (k) {
+    case 1: return launch_segments_ks<1>(base, streams, batch, nbits, out, status, second, cs);
+    case 2: return launch_segments_ks<2>(base, streams, batch, nbits, out, status, second, cs);
+    case 3: return launch_segments_ks<3>(base, streams, batch, nbits, out, status, second, cs);
+    case 4: return launch_segments_ks<4>(base, streams, batch, nbits, out, status, second, cs);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 cudaError_t launch_decode(const float* base, const DecodeStreams& streams, int k, uint64_t n, float* out,
-                          int32_t* status, cudaStream_t cs, uint64_t chunk_begin, uint64_t chunk_end) {
+                          int32_t* status, bool second, cudaStream_t cs, uint64_t chunk_begin, uint64_t chunk_end) {
   if (k < 1 || k > 4) return cudaErrorInvalidValue;
   const uint64_t all_chunks = (n + kChunkElems - 1) / kChunkElems;
   if (chunk_end > all_chunks) chunk_end = all_chunks;
   if (chunk_begin > chunk_end) chunk_begin = chunk_end;
   switch (k) {
-    case 1: return launch_decode_ks<1>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
-    case 2: return launch_decode_ks<2>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
-    case 3: return launch_decode_ks<3>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
-    case 4: return launch_decode_ks<4>(base, streams, n, out, status, chunk_begin, chunk_end, cs);
+    case 1: return launch_decode_ks<1>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+    case 2: return launch_decode_ks<2>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+    case 3: return launch_decode_ks<3>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+    case 4: return launch_decode_ks<4>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
     default: return cudaErrorInvalidValue;
   }
 }
