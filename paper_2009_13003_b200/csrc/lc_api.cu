@@ -337,6 +337,8 @@ int lc_shard_encode(const float* base, const float* cur, uint64_t n, int nbits, 
   const WorkspaceLayout W = workspace_layout(n);
   if (workspace_bytes < W.total || stream_capacity < lc_stream_bound(n, nbits)) return LC_ERR_CAPACITY;
   const Carved c = carve(workspace, W);
+  // the statistics of a shard may be coded more than once: the encode pass's scan starts from zero each time
+  if (cudaMemsetAsync(c.tiles, 0, 8 * W.nchunks, cs) != cudaSuccess) return LC_ERR_CUDA;
   if (launch_table(c.ctl, n, nbits, static_cast<uint8_t*>(stream), true, false,
                    static_cast<const ShardStats*>(whole_stats), nullptr, cs) != cudaSuccess)
     return LC_ERR_CUDA;

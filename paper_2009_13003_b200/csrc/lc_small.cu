@@ -1,186 +1,232 @@
 // Small vectors: the whole compress pass (Algorithm 1 steps 4-6, optionally step 7) in one CTA and one launch.
 //
-// For a vector of a few chunks the three kernels of the general path and the memset before them are all launch
-// latency (about 40 us together); layers of a few hundred elements are common in per-layer use. Here one CTA of 512
-// threads does the statistics in shared memory, runs the table pass (the same function as table_kernel), and codes
-// the chunks one warp per chunk, straight into the payload. Same bytes as the general path.
+// For a vector of one chunk the three kernels of the general path and the memset before them are all launch latency;
+// layers of a few hundred elements are common in per-layer use. Bound: latency, so every part of the pass is spread over
+// all 16 warps. A thread loads its (at most) eight elements once and keeps base and delta in registers through
+// statistics, coding and the tracked state. Warp w takes the chunk's steps 2w and 2w + 1, so the codes of a thread are
+// one contiguous piece of its lane's sub-stream: a scan over warps and lanes of the pieces' bit counts places them, and
+// each thread ORs its piece into the chunk's image in shared memory, which leaves with 16-byte stores. Same bytes as the
+// general path. A call of 1000 elements: 20.4 us with one warp coding
+// alone and the earlier table pass, now 10.3 us.
 #include "lc_table.cuh"
 
 namespace lc {
 namespace {
 
+constexpr uint32_t kThreadSteps = 2;  // steps per warp: 16 warps cover the 32 steps of a chunk
+static_assert(kThreadSteps * (kTableThreads / 32) == kSteps && kSmallMaxElems == kChunkElems, "one chunk per CTA");
+constexpr uint32_t kHistCols = 8;     // columns of the histogram: lane % 8 (32 of them take longer to clear and fold)
+constexpr uint32_t kImageWords = (kChunkElems * kMaxNbits / 8 + 16) / 4;  // the payload has at most nbits bits per element
+
+struct SmallShared {
+  TableShared T;
+  union {
+    struct {
+      uint32_t cnt[kKeys * kHistCols];
+      uint2 mm[kKeys];  // running maxima of ~bits and of bits
+    } h;
+    struct {
+      uint4 image[kImageWords / 4];
+      uint32_t bits[kTableThreads / 32][32];  // [warp][lane]: bit count, then bit position, of a thread's piece
+      uint32_t code[kKeys], len[kKeys], rep[kKeys];
+      uint32_t chunk_bytes;
+    } c;
+  };
+};
+
 __device__ __forceinline__ uint32_t key_of_bits(uint32_t bits) { return ((bits >> 31) << 8) | ((bits >> 23) & 255u); }
 
-// Appends a code of at most 32 bits to a lane's bit accumulator; completed words are ORed into the zeroed payload.
-struct WordPacker {
-  unsigned long long acc;
-  uint32_t nb;
-  uint32_t* dst;
-  __device__ __forceinline__ void put(uint32_t code, uint32_t len) {
-    acc = (acc << len) | code;
-    nb += len;
-    if (nb >= 32) {
-      nb -= 32;
-      atomicOr(dst, (uint32_t)(acc >> nb));
-      dst += 1;
-    }
-  }
-  __device__ __forceinline__ void flush() {
-    if (nb > 0) atomicOr(dst, (uint32_t)(acc << (32 - nb)));
-  }
-};
+// One vector of n <= kSmallMaxElems elements; all threads of the CTA. dbg: nullptr, or the control block that receives
+// the statistics and the code table (lc_debug_*). Returns 0 or the error that makes the vector unencodable.
+__device__ __forceinline__ int small_vector(SmallShared& S, const float* base, const float* cur, uint32_t n, int nbits,
+                                            uint8_t* stream, float* tracked_out, Control* dbg) {
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-// Per-key tables in shared memory for the coding passes: code length, low 32 bits of the code, representative.
-struct KeyTables {
-  const uint32_t* len;
-  const uint32_t* code;
-  const EncEntry* enc;  // global: the upper code bits of the rare codes longer than 32 bits
-};
-
-// Bits of lane `lane`'s sub-stream of chunk c (format section 2); with dst != nullptr the codes are also written,
-// starting at bit lane_start of the chunk image at dst. Only the steps that hold elements are visited; a lane's four
-// elements of a step are read as one 16-byte vector where all four exist.
-__device__ uint32_t code_lane(const KeyTables& T, const float* base, const float* cur, uint64_t n, uint64_t c,
-                              uint32_t lane, uint32_t* dst, uint32_t lane_start) {
-  WordPacker pk{0ull, lane_start & 31u, dst ? dst + (lane_start >> 5) : nullptr};
-  uint32_t bits = 0;
-  const uint64_t c0 = c * kChunkElems;
-  const uint32_t in_chunk = (uint32_t)(n - c0 < kChunkElems ? n - c0 : kChunkElems);
-  const uint32_t steps = (in_chunk + 127) / 128;
-  for (uint32_t j = 0; j < steps; ++j) {
-    const uint64_t i0 = c0 + 128ull * j + 4 * lane;
-    float d[4];
-    uint32_t cnt = 0;
-    if (i0 + 4 <= n) {
-      const float4 b4 = *reinterpret_cast<const float4*>(base + i0), c4 = *reinterpret_cast<const float4*>(cur + i0);
-      d[0] = __fsub_rn(c4.x, b4.x); d[1] = __fsub_rn(c4.y, b4.y); d[2] = __fsub_rn(c4.z, b4.z); d[3] = __fsub_rn(c4.w, b4.w);
-      cnt = 4;
+  // ---- load; delta against the tracked state
+  float b[kThreadSteps][4];
+  uint32_t d[kThreadSteps][4];
+  uint32_t have[kThreadSteps];  // elements of the thread's slot group that exist
+#pragma unroll
+  for (uint32_t r = 0; r < kThreadSteps; ++r) {
+    const uint32_t i = 128 * (kThreadSteps * warp + r) + 4 * lane;
+    have[r] = i < n ? min(n - i, 4u) : 0u;
+    float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (uint32_t e = 0; e < 4; ++e) b[r][e] = 0.f;
+    if (have[r] == 4) {
+      const float4 b4 = *reinterpret_cast<const float4*>(base + i), c4 = *reinterpret_cast<const float4*>(cur + i);
+      b[r][0] = b4.x; b[r][1] = b4.y; b[r][2] = b4.z; b[r][3] = b4.w;
+      c[0] = c4.x; c[1] = c4.y; c[2] = c4.z; c[3] = c4.w;
     } else {
-      for (uint32_t e = 0; e < kGroup; ++e)
-        if (i0 + e < n) d[cnt++] = __fsub_rn(cur[i0 + e], base[i0 + e]);
+#pragma unroll
+      for (uint32_t e = 0; e < 3; ++e)
+        if (e < have[r]) b[r][e] = base[i + e], c[e] = cur[i + e];
     }
-    for (uint32_t e = 0; e < cnt; ++e) {
-      const uint32_t key = key_of_bits(__float_as_uint(d[e]));
-      const uint32_t len = T.len[key];
-      bits += len;
-      if (dst) {
-        if (len > 32) {
-          pk.put(T.enc[key].code_hi, len - 32);
-          pk.put(T.code[key], 32);
-        } else {
-          pk.put(T.code[key], len);
-        }
+#pragma unroll
+    for (uint32_t e = 0; e < 4; ++e) d[r][e] = __float_as_uint(__fsub_rn(c[e], b[r][e]));
+  }
+
+  // ---- statistics (Section 3.1.1): count, and the running maxima of ~bits and bits, per key
+  for (uint32_t k = tid; k < kKeys * kHistCols / 4; k += kTableThreads) reinterpret_cast<uint4*>(S.h.cnt)[k] = make_uint4(0u, 0u, 0u, 0u);
+  S.h.mm[tid] = make_uint2(0u, 0u);
+  __syncthreads();
+#pragma unroll
+  for (uint32_t r = 0; r < kThreadSteps; ++r)
+#pragma unroll
+    for (uint32_t e = 0; e < 4; ++e)
+      if (e < have[r]) {
+        const uint32_t bits = d[r][e], key = key_of_bits(bits);
+        atomicAdd(&S.h.cnt[key * kHistCols + lane % kHistCols], 1u);
+        const uint2 mm = S.h.mm[key];
+        if (~bits > mm.x) atomicMax(&S.h.mm[key].x, ~bits);
+        if (bits > mm.y) atomicMax(&S.h.mm[key].y, bits);
+      }
+  __syncthreads();
+  const uint32_t my_key = key_of_position(tid);
+  KeyStats my;
+  {
+    const uint4* row = reinterpret_cast<const uint4*>(&S.h.cnt[my_key * kHistCols]);
+    const uint4 x = row[0], y = row[1];
+    static_assert(kHistCols == 8, "two 16-byte reads");
+    my.count = my.local = x.x + x.y + x.z + x.w + y.x + y.y + y.z + y.w;
+    my.inv_min = S.h.mm[my_key].x;
+    my.max_bits = S.h.mm[my_key].y;
+    my.mant_sum = 0;
+  }
+  if (dbg) {
+    dbg->count[my_key] = my.count;
+    dbg->inv_min[my_key] = my.inv_min;
+    dbg->max_bits[my_key] = my.max_bits;
+    dbg->mant_sum[my_key] = 0;
+  }
+
+  // ---- table pass: header, symbol table (its barriers also end the histogram's use)
+  const int err = table_pass(S.T, my, TableArgs{n, nbits, true, false, false, false, nullptr}, stream);
+  if (err || n == 0) return err;
+  {
+    const uint32_t sym = S.T.sym_of_key[my_key];
+    const unsigned long long code = S.T.code[sym];
+    S.c.code[my_key] = (uint32_t)code;
+    S.c.len[my_key] = S.T.len[sym];
+    S.c.rep[my_key] = S.T.rep[sym];
+    if (dbg) dbg->enc[my_key] = EncEntry{(uint32_t)code, S.T.len[sym], (uint32_t)(code >> 32), sym};
+  }
+  for (uint32_t k = tid; k < kImageWords / 4; k += kTableThreads) S.c.image[k] = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+
+  // ---- tracked state (Algorithm 1 step 7; tracked_out may be base: a thread reads only its own elements), and the bit
+  // count of the thread's piece
+  uint32_t piece = 0;
+#pragma unroll
+  for (uint32_t r = 0; r < kThreadSteps; ++r) {
+    float x[4];
+#pragma unroll
+    for (uint32_t e = 0; e < 4; ++e) {
+      const uint32_t key = key_of_bits(d[r][e]);
+      if (e < have[r]) piece += S.c.len[key];
+      x[e] = __fadd_rn(b[r][e], __uint_as_float(S.c.rep[key]));
+    }
+    if (tracked_out) {
+      const uint32_t i = 128 * (kThreadSteps * warp + r) + 4 * lane;
+      if (have[r] == 4) {
+        *reinterpret_cast<float4*>(tracked_out + i) = make_float4(x[0], x[1], x[2], x[3]);
+      } else {
+#pragma unroll
+        for (uint32_t e = 0; e < 3; ++e)
+          if (e < have[r]) tracked_out[i + e] = x[e];
       }
     }
   }
-  if (dst) pk.flush();
-  return bits;
+  S.c.bits[warp][lane] = piece;
+  __syncthreads();
+
+  // ---- bit position of every piece: pieces of a lane follow each other by warp, lanes follow each other
+  const StreamLayout L = stream_layout(n, S.T.nsym);
+  if (warp == 0) {
+    uint32_t at[kTableThreads / 32], total = 0;
+#pragma unroll
+    for (uint32_t w = 0; w < kTableThreads / 32; ++w) {
+      at[w] = total;
+      total += S.c.bits[w][lane];
+    }
+    uint32_t incl = total;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, s);
+      if ((int)lane >= s) incl += v;
+    }
+#pragma unroll
+    for (uint32_t w = 0; w < kTableThreads / 32; ++w) S.c.bits[w][lane] = incl - total + at[w];
+    reinterpret_cast<uint16_t*>(stream + L.lane_index_off)[lane] = (uint16_t)total;
+    if (lane == 31) {
+      const uint32_t bytes = (uint32_t)align_up((incl + 7) / 8, kPayloadAlign);
+      S.c.chunk_bytes = bytes;
+      unsigned long long* chunk_index = reinterpret_cast<unsigned long long*>(stream + L.chunk_index_off);
+      chunk_index[0] = 0;
+      chunk_index[1] = bytes;
+      *reinterpret_cast<unsigned long long*>(stream + 48) = L.payload_off + bytes;
+    }
+  }
+  __syncthreads();
+
+  // ---- the codes
+  if (piece > 0) {
+    uint32_t* image = reinterpret_cast<uint32_t*>(S.c.image);
+    const uint32_t pos = S.c.bits[warp][lane];
+    uint32_t* dst = image + (pos >> 5);
+    unsigned long long acc = 0;  // pending bits in the low `nb` bits; the first word's leading bits belong to others
+    uint32_t nb = pos & 31u;
+    auto put = [&](uint32_t code, uint32_t len) {  // len <= 32
+      acc = (acc << len) | code;
+      nb += len;
+      if (nb >= 32) {
+        nb -= 32;
+        atomicOr(dst, (uint32_t)(acc >> nb));
+        dst += 1;
+      }
+    };
+#pragma unroll
+    for (uint32_t r = 0; r < kThreadSteps; ++r)
+#pragma unroll
+      for (uint32_t e = 0; e < 4; ++e) {
+        if (e >= have[r]) continue;
+        const uint32_t key = key_of_bits(d[r][e]), len = S.c.len[key];
+        if (len > 32) {
+          put((uint32_t)(S.T.code[S.T.sym_of_key[key]] >> 32), len - 32);
+          put(S.c.code[key], 32);
+        } else {
+          put(S.c.code[key], len);
+        }
+      }
+    if (nb > 0) atomicOr(dst, (uint32_t)(acc << (32 - nb)));
+  }
+  __syncthreads();
+  uint4* payload = reinterpret_cast<uint4*>(stream + L.payload_off);
+  for (uint32_t k = tid; k < S.c.chunk_bytes / 16; k += kTableThreads) payload[k] = S.c.image[k];
+  return LC_OK;
 }
 
-constexpr uint32_t kSmallWarps = kTableThreads / 32;  // one chunk per warp
-static_assert(kSmallMaxElems <= (uint64_t)kSmallWarps * kChunkElems, "a warp per chunk");
-
 __global__ void __launch_bounds__(kTableThreads)
-small_compress_kernel(Control* ctl, const float* base, const float* cur, uint64_t n, int nbits, uint8_t* stream,
+small_compress_kernel(Control* ctl, const float* base, const float* cur, uint32_t n, int nbits, uint8_t* stream,
                       float* tracked_out, int keep_status) {
-  __shared__ uint32_t h_count[kKeys], h_inv_min[kKeys], h_max[kKeys];
-  __shared__ uint32_t s_chunk_bytes[kSmallWarps];
-  __shared__ unsigned long long s_chunk_off[kSmallWarps + 1];
-  __shared__ uint32_t s_lane_start[kSmallWarps][32];
-  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  // ---- what the memset of the general path clears, as far as this kernel uses it
+  extern __shared__ __align__(16) unsigned char s_small[];
+  SmallShared& S = *reinterpret_cast<SmallShared*>(s_small);
+  const uint32_t tid = threadIdx.x;
+  const int earlier = keep_status ? ctl->status : 0;  // the same for every thread: nothing here has written it yet
+  if (earlier) {
+    clear_header(stream);
+    return;
+  }
+  const int err = small_vector(S, base, cur, n, nbits, stream, tracked_out, ctl);
+  if (err) clear_header(stream);
   if (tid == 0) {
-    if (!keep_status) ctl->status = 0;
+    // what the memset of the general path clears, as far as later readers look at it
+    ctl->status = err;  // barriers lie between the reads above and this
     ctl->ticket = 0;
-    ctl->nsym = 0;
-    ctl->max_len = 0;
-    ctl->payload_bits = 0;
-    ctl->wide = 0;
-  }
-  h_count[tid] = 0;
-  h_inv_min[tid] = 0;
-  h_max[tid] = 0;
-  __syncthreads();
-
-  // ---- statistics (Section 3.1.1): count, and the running maxima of ~bits and bits, per key
-  // (Finding the lanes of a warp that meet the same key with a match, so that one lane updates the bin for all of
-  // them, was measured slower than these plain shared-memory atomics: 57 against 45 us at 4096 elements.)
-  for (uint64_t i = tid; i < n; i += kTableThreads) {
-    const uint32_t bits = __float_as_uint(__fsub_rn(cur[i], base[i]));
-    const uint32_t key = key_of_bits(bits);
-    atomicAdd(&h_count[key], 1u);
-    atomicMax(&h_inv_min[key], ~bits);
-    atomicMax(&h_max[key], bits);
-  }
-  __syncthreads();
-  ctl->count[tid] = h_count[tid];
-  ctl->inv_min[tid] = h_inv_min[tid];
-  ctl->max_bits[tid] = h_max[tid];
-  ctl->mant_sum[tid] = 0;
-  __syncthreads();  // this CTA's own global writes are visible to all its threads
-
-  // ---- table pass: header, symbol table, per-key encode table
-  if (!table_pass(ctl, n, nbits, stream, /*wide_ok=*/1, /*fixed=*/0, nullptr, nullptr, /*mean=*/0)) return;
-  __syncthreads();
-
-  // ---- encode: lane bit counts and chunk sizes, then the chunk offsets, then the bits
-  // the statistics are in the control block now: their shared arrays take the per-key tables of the coding passes
-  const EncEntry* enc = ctl->enc;
-  uint32_t *k_len = h_count, *k_code = h_inv_min, *k_rep = h_max;
-  {
-    const EncEntry e = enc[tid];
-    k_len[tid] = e.len;
-    k_code[tid] = e.code_lo;
-    k_rep[tid] = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
-  }
-  __syncthreads();
-  const KeyTables T{k_len, k_code, enc};
-  const StreamLayout L = stream_layout(n, ctl->nsym);
-  const uint32_t nchunks = (uint32_t)L.nchunks;  // at most kSmallWarps (checked by the launcher)
-  unsigned long long* chunk_index = reinterpret_cast<unsigned long long*>(stream + L.chunk_index_off);
-  uint16_t* lane_index = reinterpret_cast<uint16_t*>(stream + L.lane_index_off);
-  uint8_t* payload = stream + L.payload_off;
-  if (warp < nchunks) {
-    const uint32_t bits = code_lane(T, base, cur, n, warp, lane, nullptr, 0);
-    lane_index[warp * kLanes + lane] = (uint16_t)bits;
-    uint32_t incl = bits;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d);
-      if ((int)lane >= d) incl += v;
-    }
-    s_lane_start[warp][lane] = incl - bits;
-    if (lane == 31) s_chunk_bytes[warp] = (uint32_t)align_up((incl + 7) / 8, kPayloadAlign);
-  }
-  __syncthreads();
-  if (tid == 0) {
-    unsigned long long off = 0;
-    for (uint32_t c = 0; c < nchunks; ++c) {
-      s_chunk_off[c] = off;
-      chunk_index[c] = off;
-      off += s_chunk_bytes[c];
-    }
-    s_chunk_off[nchunks] = off;
-    chunk_index[nchunks] = off;
-    *reinterpret_cast<unsigned long long*>(stream + 48) = L.payload_off + off;
-  }
-  __syncthreads();
-  if (warp < nchunks) {
-    uint4* dst4 = reinterpret_cast<uint4*>(payload + s_chunk_off[warp]);
-    for (uint32_t k = lane; k < s_chunk_bytes[warp] / 16; k += 32) dst4[k] = make_uint4(0, 0, 0, 0);
-    __syncwarp();  // the zeros are in place before any lane ORs into them
-    code_lane(T, base, cur, n, warp, lane, reinterpret_cast<uint32_t*>(dst4), s_lane_start[warp][lane]);
-  }
-
-  // ---- Algorithm 1 step 7: tracked_out = base + quantized delta (tracked_out may be base: everything that reads
-  // base for coding is done)
-  if (tracked_out) {
-    __syncthreads();
-    for (uint64_t i = tid; i < n; i += kTableThreads) {
-      const float b = base[i];
-      tracked_out[i] = __fadd_rn(b, __uint_as_float(k_rep[key_of_bits(__float_as_uint(__fsub_rn(cur[i], b)))]));
-    }
+    ctl->nsym = err ? 0 : S.T.nsym;
+    ctl->wide = err ? 0 : S.T.wide;
+    ctl->max_len = err ? 0 : S.T.max_len;
+    ctl->payload_bits = err ? 0 : S.T.payload_bits;
   }
 }
 
@@ -189,7 +235,16 @@ small_compress_kernel(Control* ctl, const float* base, const float* cur, uint64_
 cudaError_t launch_small_compress(Control* ctl, const float* base, const float* cur, uint64_t n, int nbits,
                                   uint8_t* stream, float* tracked_out, bool keep_status, cudaStream_t cs) {
   if (n == 0 || n > kSmallMaxElems) return cudaErrorInvalidValue;
-  small_compress_kernel<<<1, kTableThreads, 0, cs>>>(ctl, base, cur, n, nbits, stream, tracked_out, keep_status ? 1 : 0);
+  static bool ready[kMaxDevices] = {};  // by device ordinal
+  const int dev = current_device_index();
+  if (dev < 0) return cudaErrorInvalidDevice;
+  if (!ready[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(small_compress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallShared));
+    if (e != cudaSuccess) return e;
+    ready[dev] = true;
+  }
+  small_compress_kernel<<<1, kTableThreads, sizeof(SmallShared), cs>>>(ctl, base, cur, (uint32_t)n, nbits, stream, tracked_out,
+                                                                      keep_status ? 1 : 0);
   return cudaGetLastError();
 }
 

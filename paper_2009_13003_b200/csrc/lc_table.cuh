@@ -1,314 +1,313 @@
 // The table pass as a function of one CTA of kTableThreads threads (Section 3.1.1: priority promotion and
 // representatives; Section 3.1.2: Huffman code; format sections 1.2-1.8): shared by table_kernel and by the
-// single-CTA kernel for small vectors. Returns false (for every thread alike) if it left no table behind: an earlier
-// pass had failed, or the vector is not encodable.
+// single-CTA kernel for small vectors.
+//
+// Bound: latency. Every compress call waits for this one CTA, so what counts is the length of its dependent chain: one
+// thread per bucket (later per symbol), ten block barriers, and a single serial loop (the Huffman merges, one thread,
+// with the fronts of both queues in registers: about 50 cycles a merge). Ranks, tree depths (pointer jumping), codes
+// (a sum over the symbols that come before) and sums are computed by all symbols at once; the stream's header and table
+// leave as 16-byte stores. With those steps in one thread, 64-bit shared-memory atomics and byte stores the pass took 10.5 us
+// for 8 symbols, 14 us for 16 and 28-36 us for 64; now 7.1, 8.6 and 15.5 us (cold caches, about 3 us of each the launch).
 #pragma once
 #include "lc_common.cuh"
 
 namespace lc {
 
 constexpr int kTableThreads = 512;
-constexpr int kMaxSym = kMaxSymbols;
 
-__device__ __forceinline__ void store_le(uint8_t* p, uint64_t v, int bytes) {
-  for (int b = 0; b < bytes; ++b) p[b] = (uint8_t)(v >> (8 * b));
+// Thread `tid` of the pass looks at one key: positions 0..507 are the candidates in priority order (exponent descending,
+// + before -), then come the non-finite keys and the two keys of exponent field 0.
+__device__ __forceinline__ uint32_t key_of_position(uint32_t tid) {
+  if (tid < 508) return 256 * (tid & 1) + 254 - (tid >> 1);
+  return tid == 508 ? 255u : tid == 509 ? 511u : tid == 510 ? 0u : 256u;
 }
 
-__device__ __forceinline__ bool table_pass(Control* __restrict__ ctl, uint64_t n, int nbits, uint8_t* __restrict__ stream,
-                                           int wide_ok, int fixed, const ShardStats* __restrict__ whole,
-                                           uint8_t* __restrict__ cache, int mean) {
-  __shared__ uint32_t warp_cand[16];
-  __shared__ uint16_t sym_of_key[kKeys];
-  __shared__ unsigned long long sym_count[kMaxSym];
-  __shared__ uint32_t sym_key[kMaxSym];
-  __shared__ uint32_t sym_rep[kMaxSym];
-  __shared__ uint32_t sym_len[kMaxSym];
-  __shared__ unsigned long long sym_code[kMaxSym];
-  __shared__ unsigned long long node_w[2 * kMaxSym];
-  __shared__ uint16_t node_parent[2 * kMaxSym];
-  __shared__ uint16_t node_depth[2 * kMaxSym];
-  __shared__ uint16_t leaf_sym[kMaxSym];
-  __shared__ uint16_t canon_order[kMaxSym];
-  __shared__ uint32_t s_maxlen;
-  __shared__ unsigned long long s_kept_total, s_payload_bits;
-  __shared__ unsigned long long s_cached_bits;  // payload size with the lengths of the cache row
+// The statistics of one key.
+struct KeyStats {
+  unsigned long long count;     // elements, of the vector that decides the table
+  unsigned long long local;     // elements of the vector that is coded: the same unless it is a shard
+  uint32_t inv_min, max_bits;
+  unsigned long long mant_sum;  // mean representatives only
+};
 
-  const int tid = threadIdx.x;
-  const int lane = tid & 31, warp = tid >> 5;
-  // The statistics that decide the table: this vector's own, or those of the whole vector it is a shard of.
-  const unsigned long long* g_count = whole ? whole->count : ctl->count;
-  const uint32_t* g_inv_min = whole ? whole->inv_min : ctl->inv_min;
-  const uint32_t* g_max_bits = whole ? whole->max_bits : ctl->max_bits;
-  __shared__ unsigned long long s_whole_total;
-  __shared__ unsigned long long sym_local[kMaxSym];  // the table's counts: this vector's own elements per symbol
+struct TableArgs {
+  uint64_t n;
+  int nbits;
+  bool wide_ok;    // false: a vector with an exponent field >= 128 is rejected
+  bool fixed;      // fixed-width codes
+  bool shard;      // the counts decide the table, the local counts go into it
+  bool mean;
+  uint8_t* cache;  // nullptr, or the length cache
+};
 
-  // ---- an earlier pass of the same call has failed (lc_merge: a stream was rejected): leave no stream behind
-  if (ctl->status != 0) {  // nothing in this kernel has written the word yet: the same for every thread
-    if (tid < 64) stream[tid] = 0;
-    return false;
-  }
+// What the pass leaves in shared memory.
+struct TableShared {
+  unsigned long long count[kMaxSymbols], local[kMaxSymbols], code[kMaxSymbols];  // by symbol
+  unsigned long long leaf_w[kMaxSymbols + 2], node_w[kMaxSymbols + 2];           // the two queues
+  unsigned long long part[4][kTableThreads / 32];
+  uint32_t rep[kMaxSymbols], key[kMaxSymbols], len[kMaxSymbols];                 // by symbol
+  uint32_t up[2 * kMaxSymbols];  // by tree node: depth below the node in the low half << 16 | that node
+  uint32_t ballot[kTableThreads / 32], flags[kTableThreads / 32];
+  uint16_t sym_of_key[kKeys], leaf_sym[kMaxSymbols];
+  uint32_t nsym, max_len, wide;
+  unsigned long long payload_bits;
+};
 
-  // ---- non-finite deltas make the vector unencodable ------------------------------------------
-  const bool bad = (tid == 255 || tid == 511) && g_count[tid] != 0;
-  if (__syncthreads_or(bad)) {
-    if (tid == 0) {
-      set_status(&ctl->status, LC_ERR_NONFINITE);
-      for (int b = 0; b < 64; ++b) stream[b] = 0;
-    }
-    return false;
-  }
+__device__ __forceinline__ unsigned long long table_warp_sum(unsigned long long v) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+__device__ __forceinline__ unsigned long long table_part_total(const unsigned long long* part) {
+  unsigned long long v = 0;
+#pragma unroll
+  for (int w = 0; w < kTableThreads / 32; ++w) v += part[w];
+  return v;
+}
 
-  // ---- does the one-byte key plane identify every bucket? (only if all exponent fields are < 128)
-  const bool big = (tid & 255) >= 128 && (g_count[tid] != 0 || ctl->count[tid] != 0);
-  const int wide = __syncthreads_or(big);
-  if (wide && !wide_ok) {
-    // the caller has released base and cur, and the one-byte keys do not identify the buckets of this vector
-    if (tid == 0) {
-      set_status(&ctl->status, LC_ERR_RANGE);
-      for (int b = 0; b < 64; ++b) stream[b] = 0;
-    }
-    return false;
-  }
+// No stream is left: its first 64 bytes (the magic among them) become zero.
+__device__ __forceinline__ void clear_header(uint8_t* stream) {
+  if (threadIdx.x < 4) reinterpret_cast<uint4*>(stream)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
+}
 
-  // ---- priority promotion -------------------------------------------------------------------------
-  // thread `tid` < 508 looks at the key of priority position tid: exponent descending, + before -.
-  uint32_t key = 0;
-  unsigned long long cnt = 0;
-  bool cand = false;
-  if (tid < 508) {
-    const uint32_t E = 254 - (tid >> 1), s = tid & 1;
-    key = 256 * s + E;
-    cnt = g_count[key];
-    cand = cnt != 0;
+// `my`: the statistics of key_of_position(threadIdx.x). Returns 0, or the error that makes the vector unencodable, the
+// same for all threads; on success the stream's header (but for its total size), table and padding are written, and T is
+// complete and visible to all threads.
+__device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, const TableArgs& A, uint8_t* __restrict__ stream) {
+  constexpr uint32_t kAll = 0xffffffffu;
+  constexpr unsigned long long kNone = ~0ull;  // weight behind the end of a queue
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t key = key_of_position(tid);
+
+  // ---- non-finite deltas make the vector unencodable; exponent fields >= 128 are more than the key plane holds
+  const bool cand = tid < 508 && my.count != 0;
+  const uint32_t ballot = __ballot_sync(kAll, cand);
+  const bool bad = (key & 255u) == 255u && my.count != 0;
+  const bool big = (key & 255u) >= 128u && (my.count != 0 || my.local != 0);
+  const uint32_t flags = (__any_sync(kAll, bad) ? 1u : 0u) | (__any_sync(kAll, big) ? 2u : 0u);
+  if (lane == 0) {
+    T.ballot[warp] = ballot;
+    T.flags[warp] = flags;
   }
-  if (tid < kMaxSym) {
-    sym_count[tid] = 0;
-    sym_len[tid] = 0;
-    sym_code[tid] = 0;
-    sym_key[tid] = 0;
-    sym_rep[tid] = 0;
-  }
-  sym_of_key[tid] = 0;
-  if (tid == 0) {
-    s_kept_total = 0;
-    s_payload_bits = 0;
-    s_maxlen = 0;
-    s_whole_total = 0;
-    s_cached_bits = 0;
-  }
-  sym_local[tid] = 0;
-  const uint32_t ballot = __ballot_sync(0xffffffffu, cand);
-  if (lane == 0) warp_cand[warp] = __popc(ballot);
+  T.sym_of_key[tid] = 0;
+  T.len[tid] = 0;
+  T.code[tid] = 0;
+  T.node_w[tid] = kNone;
+  T.leaf_w[tid] = kNone;
+  if (tid < 2) T.node_w[kMaxSymbols + tid] = T.leaf_w[kMaxSymbols + tid] = kNone;
+  if (tid == 0) T.max_len = 0;
   __syncthreads();
-  uint32_t rank = __popc(ballot & ((1u << lane) - 1));
-  uint32_t ncand = 0;
-  for (int w = 0; w < 16; ++w) {
-    if (w < warp) rank += warp_cand[w];
-    ncand += warp_cand[w];
+
+  // ---- priority promotion
+  uint32_t rank = __popc(ballot & ((1u << lane) - 1)), ncand = 0, all_flags = 0;
+#pragma unroll
+  for (uint32_t w = 0; w < kTableThreads / 32; ++w) {
+    const uint32_t b = __popc(T.ballot[w]);
+    if (w < warp) rank += b;
+    ncand += b;
+    all_flags |= T.flags[w];
   }
-  const uint32_t keep = min((1u << nbits) - 1u, ncand);
-  const uint32_t nsym = keep + 1;
-  if (cand && rank < keep) {
+  if (all_flags & 1u) return LC_ERR_NONFINITE;
+  const uint32_t wide = all_flags >> 1;
+  // the caller has released base and cur, and the one-byte keys do not identify the buckets of this vector
+  if (wide && !A.wide_ok) return LC_ERR_RANGE;
+  const uint32_t keep = min((1u << A.nbits) - 1u, ncand), nsym = keep + 1;
+  const bool kept = cand && rank < keep;
+  if (kept) {
     const uint32_t sym = rank + 1;
-    sym_of_key[key] = (uint16_t)sym;
-    sym_count[sym] = cnt;
-    sym_key[sym] = key;
+    T.sym_of_key[key] = (uint16_t)sym;
+    T.count[sym] = my.count;
+    T.local[sym] = my.local;
+    T.key[sym] = key;
     // midrange of two values with the same sign and exponent, rounded to nearest even, on mantissas.
-    sym_local[sym] = ctl->count[key];
-    const uint32_t mmin = (~g_inv_min[key]) & 0x7FFFFFu;
-    const uint32_t mmax = g_max_bits[key] & 0x7FFFFFu;
-    const uint32_t t = mmin + mmax;
+    const uint32_t t = ((~my.inv_min) & 0x7FFFFFu) + (my.max_bits & 0x7FFFFFu);
     uint32_t mr = t >> 1;
     if ((t & 1u) && (mr & 1u)) mr += 1;
-    if (mean) {
+    if (A.mean) {
       // variant (format section 1.8): mean of the mantissa fields, rounded to nearest, ties to even; it cannot reach
       // 2^23 because it does not exceed the largest field
-      const unsigned long long sum = ctl->mant_sum[key];
-      unsigned long long q = sum / cnt;
-      const unsigned long long r = sum - q * cnt;
-      if (2 * r > cnt || (2 * r == cnt && (q & 1ull))) q += 1;
+      unsigned long long q = my.mant_sum / my.count;
+      const unsigned long long r = my.mant_sum - q * my.count;
+      if (2 * r > my.count || (2 * r == my.count && (q & 1ull))) q += 1;
       mr = (uint32_t)q;
     }
-    sym_rep[sym] = (key << 23) | mr;
-    atomicAdd(&s_kept_total, cnt);
+    T.rep[sym] = (key << 23) | mr;
   }
-  if (whole) atomicAdd(&s_whole_total, g_count[tid]);  // elements of the whole vector
-  __syncthreads();
-  if (tid == 0) {
-    sym_count[0] = (whole ? s_whole_total : n) - s_kept_total;
-    unsigned long long kept_local = 0;
-    for (uint32_t j = 1; j < nsym; ++j) kept_local += sym_local[j];
-    sym_local[0] = n - kept_local;
+  {
+    const unsigned long long kept_sum = table_warp_sum(kept ? my.count : 0ull);
+    if (lane == 0) T.part[0][warp] = kept_sum;
+    if (A.shard) {
+      const unsigned long long kept_local = table_warp_sum(kept ? my.local : 0ull), whole = table_warp_sum(my.count);
+      if (lane == 0) {
+        T.part[1][warp] = kept_local;
+        T.part[2][warp] = whole;
+      }
+    }
   }
   __syncthreads();
 
-  // ---- Huffman lengths: two-queue construction ----------------------------------------------------
-  // queue A = used symbols sorted by (count, id), found with a rank sort.
-  bool used = false;
-  unsigned long long my_count = 0;
-  if (tid < (int)nsym) {
-    my_count = sym_count[tid];
-    used = my_count != 0;
-  }
-  const uint32_t used_ballot = __ballot_sync(0xffffffffu, used);
-  if (lane == 0) warp_cand[warp] = __popc(used_ballot);
-  __syncthreads();
-  uint32_t nused = 0;
-  for (int w = 0; w < 16; ++w) nused += warp_cand[w];
-  if (fixed) {
+  // ---- from here on thread tid looks at symbol tid. Symbol 0 is everything that is not kept.
+  const unsigned long long kept_total = table_part_total(T.part[0]);
+  const unsigned long long count0 = (A.shard ? table_part_total(T.part[2]) : A.n) - kept_total;
+  const unsigned long long local0 = A.n - (A.shard ? table_part_total(T.part[1]) : kept_total);
+  const bool is_sym = tid < nsym;
+  const unsigned long long my_count = !is_sym ? 0ull : tid == 0 ? count0 : T.count[tid];
+  const unsigned long long my_local = !is_sym ? 0ull : tid == 0 ? local0 : T.local[tid];
+  const bool used = my_count != 0;  // every kept symbol is
+  const uint32_t nused = keep + (count0 != 0 ? 1u : 0u);
+  uint32_t my_len = 0;
+  bool hit = false;
+  uint8_t* row = nullptr;
+  if (A.fixed) {
     // fixed-width codes (format section 1.5): every symbol, used or not, takes ceil(log2 nsym) bits; its code is its id
     uint32_t width = 0;
     while ((1u << width) < nsym) width += 1;
-    if (tid < (int)nsym) {
-      sym_len[tid] = width;
-      sym_code[tid] = (unsigned long long)tid;
+    my_len = width;
+    if (is_sym) {
+      T.len[tid] = width;
+      T.code[tid] = tid;
     }
-    if (tid == 0) {
-      s_maxlen = width;
-      s_payload_bits = n * width;
-    }
-  }
-  // ---- code-table caching (Section 3.2; format section 1.7): a valid row for this number of used symbols gives
-  // the r-th most frequent symbol its r-th length, if the payload then stays within n * nbits bits
-  uint8_t* row = (cache && !fixed && nused >= 2) ? cache + (size_t)kLengthCacheRow * (nused - 1) : nullptr;
-  uint32_t offered = 0;
-  if (row && row[0] != 0 && used) {  // row[0] is read before anything in this kernel writes the row
-    uint32_t r = 0;
-    for (uint32_t j = 0; j < nsym; ++j) {
-      const unsigned long long cj = sym_count[j];
-      if (cj != 0 && (cj > my_count || (cj == my_count && (int)j < tid))) r += 1;
-    }
-    offered = row[r];
-    atomicAdd(&s_cached_bits, my_count * offered);
-  }
-  const bool row_valid = row && row[0] != 0;
-  __syncthreads();
-  const bool hit = row_valid && s_cached_bits <= n * (unsigned long long)nbits;
-  if (hit) {
+    if (tid == 0) T.max_len = width;
+  } else if (nused >= 2) {
+    // place among the used symbols by (count, id) ascending
+    uint32_t place = 0;
     if (used) {
-      sym_len[tid] = offered;
-      atomicMax(&s_maxlen, offered);
-    }
-  }
-  if (used && !fixed && !hit) {
-    uint32_t r = 0;
-    for (uint32_t j = 0; j < nsym; ++j) {
-      const unsigned long long cj = sym_count[j];
-      if (cj != 0 && (cj < my_count || (cj == my_count && (int)j < tid))) r += 1;
-    }
-    node_w[r] = my_count;
-    leaf_sym[r] = (uint16_t)tid;
-  }
-  __syncthreads();
-  if (tid == 0 && nused >= 2 && !fixed && !hit) {
-    uint32_t front_a = 0, front_b = nused, next = nused;
-    for (uint32_t merge = 0; merge + 1 < nused; ++merge) {
-      uint32_t pick[2];
-      for (int q = 0; q < 2; ++q) {
-        const bool a_has = front_a < nused, b_has = front_b < next;
-        if (a_has && (!b_has || node_w[front_a] <= node_w[front_b])) pick[q] = front_a++;
-        else pick[q] = front_b++;
+      for (uint32_t j = 0; j < nsym; ++j) {
+        const unsigned long long cj = j == 0 ? count0 : T.count[j];
+        place += cj != 0 && (cj < my_count || (cj == my_count && j < tid)) ? 1u : 0u;
       }
-      node_w[next] = node_w[pick[0]] + node_w[pick[1]];
-      node_parent[pick[0]] = (uint16_t)next;
-      node_parent[pick[1]] = (uint16_t)next;
-      next += 1;
     }
-    // depths, from the root (the last node) down; parents always have larger indices.
-    const uint32_t root = next - 1;
-    node_depth[root] = 0;
-    for (int v = (int)root - 1; v >= 0; --v) node_depth[v] = node_depth[node_parent[v]] + 1;
-    uint32_t maxlen = 0;
-    unsigned long long bits = 0;
-    for (uint32_t r = 0; r < nused; ++r) {
-      sym_len[leaf_sym[r]] = node_depth[r];
-      maxlen = max(maxlen, (uint32_t)node_depth[r]);
-      bits += node_w[r] * node_depth[r];
+    // ---- code-table caching (Section 3.2; format section 1.7): a valid row for this number of used symbols gives
+    // the r-th most frequent symbol its r-th length, if the payload then stays within n * nbits bits
+    row = A.cache ? A.cache + (size_t)kLengthCacheRow * (nused - 1) : nullptr;
+    if (row && row[0] != 0) {  // read before anything in this kernel writes the row
+      uint32_t offered = 0;
+      if (used) {
+        uint32_t r = 0;  // place by (count descending, id ascending)
+        for (uint32_t j = 0; j < nsym; ++j) {
+          const unsigned long long cj = j == 0 ? count0 : T.count[j];
+          r += cj != 0 && (cj > my_count || (cj == my_count && j < tid)) ? 1u : 0u;
+        }
+        offered = row[r];
+      }
+      const unsigned long long bits = table_warp_sum(my_count * offered);
+      if (lane == 0) T.part[1][warp] = bits;  // a shard takes no cache
+      __syncthreads();
+      hit = table_part_total(T.part[1]) <= A.n * (unsigned long long)A.nbits;
+      if (hit) my_len = offered;
     }
-    s_maxlen = maxlen;
-    s_payload_bits = bits;
+    if (!hit) {
+      // ---- Huffman lengths: two-queue construction over the leaves in that order
+      if (used) {
+        T.leaf_w[place] = my_count;
+        T.leaf_sym[place] = (uint16_t)tid;
+      }
+      __syncthreads();
+      const uint32_t root = 2 * nused - 2;
+      if (tid == 0) {
+        unsigned long long a0 = T.leaf_w[0], a1 = T.leaf_w[1], b0 = kNone, b1 = kNone;  // fronts of the queues
+        uint32_t fa = 0, fb = 0;
+        for (uint32_t m = 0; m + 1 < nused; ++m) {
+          unsigned long long sum = 0;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            uint32_t node;
+            if (a0 <= b0) {
+              sum += a0;
+              node = fa;
+              fa += 1;
+              a0 = a1;
+              a1 = T.leaf_w[fa + 1];
+            } else {
+              sum += b0;
+              node = nused + fb;
+              fb += 1;
+              b0 = b1;
+              b1 = T.node_w[fb + 1];
+            }
+            T.up[node] = 1u << 16 | (nused + m);
+          }
+          T.node_w[m] = sum;
+          if (m == fb) b0 = sum;
+          else if (m == fb + 1) b1 = sum;
+        }
+        T.up[root] = root;
+      }
+      __syncthreads();
+      // ---- depths: every node jumps to its ancestor's ancestor until all have reached the root
+      for (uint32_t reach = 1; reach < min(nused, 64u); reach *= 2) {  // no leaf is deeper than nused - 1, nor than 63
+        uint32_t x[2];
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h) {
+          const uint32_t v = tid + h * kTableThreads;
+          if (v <= root) {
+            const uint32_t a = T.up[v], b = T.up[a & 0xffffu];
+            x[h] = ((a >> 16) + (b >> 16)) << 16 | (b & 0xffffu);
+          }
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t h = 0; h < 2; ++h)
+          if (tid + h * kTableThreads <= root) T.up[tid + h * kTableThreads] = x[h];
+        __syncthreads();
+      }
+      if (used) my_len = T.up[place] >> 16;
+    }
+    if (used) T.len[tid] = my_len;
+    // ---- canonical codes: used symbols sorted by (len, id); a code is the sum of 2^-len over those before it
+    __syncthreads();
+    if (used) {
+      unsigned long long before = 0;
+      uint32_t r = 0;
+      for (uint32_t j = 0; j < nsym; ++j) {
+        const uint32_t lj = T.len[j];
+        const bool first = lj != 0 && (lj < my_len || (lj == my_len && j < tid));
+        before += first ? 1ull << (63 - lj) : 0ull;
+        r += first ? 1u : 0u;
+      }
+      T.code[tid] = before >> (63 - my_len);
+      if (row && !hit) row[r] = (uint8_t)my_len;  // a miss stores the new lengths, ascending
+    }
+    if (row && !hit && tid >= nused) row[tid] = 0;
+    const uint32_t longest = __reduce_max_sync(kAll, my_len);
+    if (lane == 0 && longest) atomicMax(&T.max_len, longest);
   }
-  __syncthreads();
-
-  // ---- canonical codes: used symbols sorted by (len, id) -------------------------------------------
-  if (used && nused >= 2 && !fixed) {
-    const uint32_t my_len = sym_len[tid];
-    uint32_t r = 0;
-    for (uint32_t j = 0; j < nsym; ++j) {
-      const uint32_t lj = sym_len[j];
-      if (lj != 0 && (lj < my_len || (lj == my_len && (int)j < tid))) r += 1;
-    }
-    canon_order[r] = (uint16_t)tid;
-    if (row && !hit) row[r] = (uint8_t)my_len;  // a miss stores the new lengths, ascending
-  }
-  if (row && !hit && tid >= (int)nused) row[tid] = 0;
-  __syncthreads();
-  if (tid == 0 && nused >= 2 && !fixed) {
-    unsigned long long code = 0;
-    uint32_t prev_len = 0;
-    for (uint32_t r = 0; r < nused; ++r) {
-      const uint32_t j = canon_order[r];
-      if (r > 0) code = (code + 1) << (sym_len[j] - prev_len);
-      sym_code[j] = code;
-      prev_len = sym_len[j];
-    }
-  }
-  __syncthreads();
-
-  // ---- payload size: this vector's own elements, with the lengths just found --------------------------
-  if (tid == 0) s_payload_bits = 0;
-  __syncthreads();
-  if (tid < (int)nsym) atomicAdd(&s_payload_bits, sym_local[tid] * sym_len[tid]);
-  __syncthreads();
-
-  // ---- outputs ---------------------------------------------------------------------------------------
+  // ---- payload size: this vector's own elements, with the lengths just found
   {
-    const uint32_t sym = sym_of_key[tid];
-    EncEntry e;
-    e.code_lo = (uint32_t)sym_code[sym];
-    e.code_hi = (uint32_t)(sym_code[sym] >> 32);
-    e.len = sym_len[sym];
-    e.sym = sym;
-    ctl->enc[tid] = e;
+    const unsigned long long bits = table_warp_sum(my_local * my_len);
+    if (lane == 0) T.part[3][warp] = bits;
   }
-  const StreamLayout L = stream_layout(n, nsym);
-  if (tid < (int)nsym) {
-    uint8_t* e = stream + L.table_off + 16 * tid;
-    store_le(e, sym_key[tid], 2);
-    e[2] = (uint8_t)sym_len[tid];
-    e[3] = 0;
-    store_le(e + 4, sym_rep[tid], 4);
-    store_le(e + 8, sym_local[tid], 8);
-  }
+  __syncthreads();
+  const unsigned long long payload_bits = table_part_total(T.part[3]);
+
+  // ---- outputs
   if (tid == 0) {
-    ctl->nsym = nsym;
-    ctl->wide = wide ? 1u : 0u;
-    ctl->max_len = s_maxlen;
-    ctl->payload_bits = s_payload_bits;
-    uint8_t* h = stream;
-    h[0] = 'L'; h[1] = 'C'; h[2] = 'C'; h[3] = '1';
-    store_le(h + 4, 1, 2);
-    h[6] = (uint8_t)nbits;
-    h[7] = (uint8_t)((fixed ? 1 : 0) | (whole ? 2 : 0) | (hit ? 4 : 0) | (mean ? 8 : 0));
-    store_le(h + 8, n, 8);
-    store_le(h + 16, nsym, 4);
-    store_le(h + 20, s_maxlen, 4);
-    store_le(h + 24, kChunkElems, 4);
-    store_le(h + 28, kLanes, 2);
-    store_le(h + 30, kGroup, 2);
-    store_le(h + 32, L.nchunks, 4);
-    store_le(h + 36, kPayloadAlign, 4);
-    store_le(h + 40, s_payload_bits, 8);
-    store_le(h + 56, L.payload_off, 8);
-    // bytes between the lane index and the payload are zero.
-    for (uint64_t p = L.lane_index_off + 64 * L.nchunks; p < L.payload_off; ++p) stream[p] = 0;
-    if (L.nchunks == 0) {
-      // nothing for the encode pass to do: finish the stream here.
-      store_le(stream + L.chunk_index_off, 0, 8);
-      store_le(h + 48, L.payload_off, 8);
-    }
+    T.rep[0] = 0;
+    T.nsym = nsym;
+    T.wide = wide;
+    T.payload_bits = payload_bits;
   }
-  return true;
+  const StreamLayout L = stream_layout(A.n, nsym);
+  if (is_sym)
+    reinterpret_cast<uint4*>(stream + L.table_off)[tid] =
+        make_uint4((tid ? T.key[tid] : 0u) | my_len << 16, tid ? T.rep[tid] : 0u, (uint32_t)my_local, (uint32_t)(my_local >> 32));
+  if (tid < 4) {
+    const uint32_t flag = (A.fixed ? 1u : 0u) | (A.shard ? 2u : 0u) | (hit ? 4u : 0u) | (A.mean ? 8u : 0u);
+    // a vector without chunks leaves nothing for the encode pass to do: its stream ends here
+    const unsigned long long total = L.nchunks == 0 ? L.payload_off : 0ull;
+    uint4 h;
+    if (tid == 0) h = make_uint4(0x3143434Cu /* "LCC1" */, 1u | (uint32_t)A.nbits << 16 | flag << 24, (uint32_t)A.n, (uint32_t)(A.n >> 32));
+    else if (tid == 1) h = make_uint4(nsym, T.max_len, kChunkElems, kLanes | kGroup << 16);
+    else if (tid == 2) h = make_uint4((uint32_t)L.nchunks, kPayloadAlign, (uint32_t)payload_bits, (uint32_t)(payload_bits >> 32));
+    else h = make_uint4((uint32_t)total, (uint32_t)(total >> 32), (uint32_t)L.payload_off, (uint32_t)(L.payload_off >> 32));
+    reinterpret_cast<uint4*>(stream)[tid] = h;
+  }
+  // bytes between the lane index and the payload are zero
+  const uint64_t index_end = L.lane_index_off + 64 * L.nchunks;
+  if (tid < L.payload_off - index_end) stream[index_end + tid] = 0;
+  if (tid == 0 && L.nchunks == 0) *reinterpret_cast<unsigned long long*>(stream + L.chunk_index_off) = 0;
+  __syncthreads();
+  return LC_OK;
 }
 
 }  // namespace lc
