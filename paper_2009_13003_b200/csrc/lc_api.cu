@@ -232,21 +232,48 @@ int lc_compress_segments(const float* base, const float* cur, const uint64_t* se
   if (!segments_ok(seg_begin, nseg) || nbits < 1 || nbits > kMaxNbits || !streams || !aligned(streams, 256))
     return LC_ERR_ARG;
   if (streams_capacity < lc_segments_layout(seg_begin, nseg, nbits, nullptr)) return LC_ERR_CAPACITY;
+  uint64_t longest = 0;
+  for (int i = 0; i < nseg; ++i) longest = seg_begin[i + 1] - seg_begin[i] > longest ? seg_begin[i + 1] - seg_begin[i] : longest;
+  if (!workspace || !aligned(workspace, 256) || (longest > 0 && (!base || !cur)) || !aligned(base, 16) || !aligned(cur, 16))
+    return LC_ERR_ARG;
+  if (tracked_out && (!aligned(tracked_out, 16) || (longest > 0 && tracked_out == cur))) return LC_ERR_ARG;
+  if (workspace_bytes < workspace_layout(longest).total) return LC_ERR_CAPACITY;
+  // Of the control block only the words up to `count` are used here; the segments' blocks and scan descriptors take the
+  // place of everything behind them. A group is as many segments as the workspace and the kernel parameters hold (one
+  // always fits: a workspace for n elements has 100 KB more than a block and n elements' descriptors).
+  constexpr uint64_t kScratch = offsetof(Control, count);
+  Control* ctl = static_cast<Control*>(workspace);
+  uint8_t* scratch = static_cast<uint8_t*>(workspace) + kScratch;
+  const uint64_t capacity = workspace_bytes - kScratch;
+  SegGroup g;
   uint64_t off = 0;
-  for (int i = 0; i < nseg; ++i) {
-    const uint64_t lo = seg_begin[i], ni = seg_begin[i + 1] - lo;
-    const uint64_t cap = align_up(lc_stream_bound(ni, nbits), 256);
-    float* t = tracked_out ? tracked_out + lo : nullptr;
-    if (t) {
-      const int rc = check_tracked_out(cur + lo, ni, t);
-      if (rc != LC_OK) return rc;
+  for (int i = 0; i < nseg;) {
+    const bool first_group = i == 0;
+    g.first = (uint32_t)i;
+    uint32_t blocks = 0, tiles = 0;
+    for (g.nseg = 0; g.nseg < kSegGroup && i < nseg; ++g.nseg, ++i) {
+      const uint64_t ni = seg_begin[i + 1] - seg_begin[i];
+      const bool small = ni <= kSmallMaxElems;
+      const uint32_t t = small ? 0 : (uint32_t)((ni + kEncWarps * kChunkElems - 1) / (kEncWarps * kChunkElems));
+      if (!small && sizeof(SegBlock) * (blocks + 1) + 8ull * (tiles + t) > capacity) break;
+      g.block[g.nseg] = (uint16_t)blocks;
+      g.tile_begin[g.nseg] = tiles;
+      g.elem_begin[g.nseg] = seg_begin[i];
+      g.stream_begin[g.nseg] = off;
+      blocks += small ? 0 : 1;
+      tiles += t;
+      off += align_up(lc_stream_bound(ni, nbits), 256);
     }
-    // the status word is cleared before the first segment only: a segment the device rejects makes the table and
-    // encode passes of all later ones leave their streams invalid, and the word keeps the first failure
-    const int rc = compress_impl(base + lo, cur + lo, ni, nbits, static_cast<uint8_t*>(streams) + off, cap, t, workspace,
-                                 workspace_bytes, EncodeOptions(), cs, /*keep_status=*/i > 0);
-    if (rc != LC_OK) return rc;
-    off += cap;
+    g.tile_begin[g.nseg] = tiles;
+    g.elem_begin[g.nseg] = seg_begin[i];
+    g.stream_begin[g.nseg] = off;
+    const uint64_t used = sizeof(SegBlock) * blocks + 8ull * tiles;
+    uint8_t* clear = first_group ? static_cast<uint8_t*>(workspace) : scratch;  // status and failure word once per call
+    if (cudaMemsetAsync(clear, 0, (size_t)(scratch + used - clear), cs) != cudaSuccess) return LC_ERR_CUDA;
+    if (launch_compress_segments(ctl, reinterpret_cast<SegBlock*>(scratch),
+                                 reinterpret_cast<unsigned long long*>(scratch + sizeof(SegBlock) * blocks), base, cur, g, nbits,
+                                 static_cast<uint8_t*>(streams), tracked_out, cs) != cudaSuccess)
+      return LC_ERR_CUDA;
   }
   return LC_OK;
 }

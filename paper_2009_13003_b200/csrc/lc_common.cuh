@@ -73,8 +73,10 @@ struct Control {
   uint32_t max_len;       // written by the table kernel
   uint64_t payload_bits;  // written by the table kernel
   uint32_t wide;          // written by the table kernel: some delta has an exponent field >= 128
+  uint32_t seg_ticket;    // per-layer compress: next tile of the launch
+  uint32_t seg_fail;      // per-layer compress: ~number of the first segment that failed, 0 if none
   uint32_t pad32_;
-  uint64_t pad_[28];
+  uint64_t pad_[27];
   unsigned long long count[kKeys];  // elements per key
   uint32_t inv_min[kKeys];          // max over the bucket of ~bits (zero-initialised running minimum)
   uint32_t max_bits[kKeys];         // max over the bucket of bits
@@ -179,6 +181,35 @@ struct DecodeStreams {
   const uint8_t* ptr[4];
   uint64_t bytes[4];
 };
+// ---- per-layer compress ---------------------------------------------------------------------------------
+// A group of segments goes through three launches (statistics, tables, encode). Passed by value, within the 4 KB that
+// kernel parameters may take.
+constexpr uint32_t kSegGroup = 128;
+struct SegGroup {
+  uint32_t nseg;
+  uint32_t first;                        // number of the first of them among the segments of the call
+  uint32_t cta_begin[kSegGroup + 1];     // statistics CTAs of each segment (filled in by the launcher)
+  uint32_t tile_begin[kSegGroup + 1];    // tiles of kEncWarps chunks of each segment (0 for one of a single chunk)
+  uint16_t block[kSegGroup];             // its SegBlock, if it has tiles
+  uint64_t elem_begin[kSegGroup + 1];
+  uint64_t stream_begin[kSegGroup + 1];  // segment i's stream starts there in the streams buffer
+};
+// What the passes hand each other about one segment of more than one chunk; zero at the start of the group.
+struct SegBlock {
+  uint32_t nsym;  // 0: no stream (the segment, or one before it, has failed)
+  uint32_t max_len, wide, pad_;
+  uint64_t payload_bits, pad64_[5];
+  union {
+    ShardStats stats;     // until the table pass has read them
+    EncEntry enc[kKeys];  // after it
+  };
+};
+static_assert(sizeof(SegBlock) == 64 + 8192, "two arrays of the same size share the block");
+// `blocks`, then the scan descriptors of the tiles (one u64 each), both zeroed by the caller, lie in the workspace
+cudaError_t launch_compress_segments(Control* ctl, SegBlock* blocks, unsigned long long* tiles, const float* base,
+                                     const float* cur, SegGroup& group, int nbits, uint8_t* streams, float* tracked_out,
+                                     cudaStream_t cs);
+
 // The segments of one launch of the per-layer recovery, passed by value (within the 4 KB that kernel parameters may
 // take): where each begins in the vector and in every streams buffer, and which CTAs work on it.
 constexpr uint32_t kSegBatch = 160;

@@ -23,79 +23,12 @@
 //    plain load and only issues an atomic when its value would improve it, which after the first few
 //    elements almost never happens;
 //  * counts are integers and min / max are order-free, so the result is deterministic.
-#include "lc_common.cuh"
+#include "lc_stats.cuh"
 
 namespace lc {
 namespace {
 
-constexpr int kStatsThreads = 384;
-constexpr int kRows = 8;  // steps per unit
-constexpr uint32_t kCntWords = kKeys * 32;
-constexpr uint32_t kStatsSmem = (kCntWords + 2 * kKeys) * 4;  // 64 KB + 4 KB
-// Mean-representative variant (format section 1.8): two more tables of the same shape hold, per key and lane, the
-// sums of the low 12 and of the high 11 bits of the mantissa fields. A column receives at most 32 elements per warp
-// and unit, so 32-bit sums hold for kMeanMaxUnitsPerWarp units per warp: 12 warps * 32 * 4095 * 2731 < 2^32.
-constexpr uint32_t kStatsSmemMean = (3 * kCntWords + 2 * kKeys) * 4;  // 192 KB + 4 KB: one CTA per SM
-constexpr uint64_t kMeanMaxUnitsPerWarp = 2731;
-
-__device__ __forceinline__ float4 ld_stream(const float4* p) {
-  float4 v;
-  asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "l"(p));
-  return v;
-}
-
-// Slot of a delta's bucket in the shared-memory tables: (exponent field << 1) | sign. The two signs of one
-// exponent are neighbours and 8 consecutive exponents fill the 16 bank pairs of a 64-bit access exactly once,
-// so the few hot buckets of a vector (neighbouring exponents, both signs) rarely meet in a bank. The low byte
-// of the slot is the element's byte in the key plane.
-__device__ __forceinline__ uint32_t slot_of(uint32_t bits) { return ((bits >> 22) & 0x1FEu) | (bits >> 31); }
-__device__ __forceinline__ uint32_t key_of_slot(uint32_t slot) { return ((slot & 1u) << 8) | (slot >> 1); }
-
-template <bool MEAN>
-struct Acc {
-  uint32_t* cnt_lane;  // &cnt[lane]
-  uint2* mm;
-  __device__ __forceinline__ void sum(uint32_t bits, uint32_t slot) {
-    if (MEAN) {
-      atomicAdd(cnt_lane + kCntWords + slot * 32, bits & 0xFFFu);
-      atomicAdd(cnt_lane + 2 * kCntWords + slot * 32, (bits >> 12) & 0x7FFu);
-    }
-  }
-  __device__ __forceinline__ void improve(uint32_t bits, uint32_t slot, uint2 cur) {
-    if (~bits > cur.x) atomicMax(&mm[slot].x, ~bits);
-    if (bits > cur.y) atomicMax(&mm[slot].y, bits);
-  }
-  __device__ __forceinline__ void add(uint32_t bits) {
-    const uint32_t slot = slot_of(bits);
-    atomicAdd(cnt_lane + slot * 32, 1u);
-    sum(bits, slot);
-    improve(bits, slot, mm[slot]);
-  }
-  // Four elements at once: the four reads of the running min / max pairs go out together, and one test
-  // covers all eight comparisons, because after the first few elements none of them ever holds.
-  __device__ __forceinline__ void add4(uint32_t d0, uint32_t d1, uint32_t d2, uint32_t d3, uint32_t k0, uint32_t k1,
-                                       uint32_t k2, uint32_t k3) {
-    const uint2 c0 = mm[k0], c1 = mm[k1], c2 = mm[k2], c3 = mm[k3];
-    atomicAdd(cnt_lane + k0 * 32, 1u);
-    atomicAdd(cnt_lane + k1 * 32, 1u);
-    atomicAdd(cnt_lane + k2 * 32, 1u);
-    atomicAdd(cnt_lane + k3 * 32, 1u);
-    sum(d0, k0);
-    sum(d1, k1);
-    sum(d2, k2);
-    sum(d3, k3);
-    const bool any = (~d0 > c0.x) | (d0 > c0.y) | (~d1 > c1.x) | (d1 > c1.y) | (~d2 > c2.x) | (d2 > c2.y) |
-                     (~d3 > c3.x) | (d3 > c3.y);
-    if (any) {
-      improve(d0, k0, c0);
-      improve(d1, k1, c1);
-      improve(d2, k2, c2);
-      improve(d3, k3, c3);
-    }
-  }
-};
+using namespace stats;
 
 template <bool MEAN>
 __global__ void __launch_bounds__(kStatsThreads, MEAN ? 1 : 2)
@@ -114,74 +47,9 @@ stats_kernel(const float* __restrict__ base, const float* __restrict__ cur, uint
   const uint64_t nwarps = (uint64_t)gridDim.x * (kStatsThreads / 32);
   Acc<MEAN> acc{cnt + lane, mm};
 
-  for (uint64_t u = warp; u < nunits; u += nwarps) {
-    const uint64_t i0 = u * kUnitElems;
-    uint32_t ew[kRows];
-    if (i0 + kUnitElems <= n) {
-      const float4* b4 = reinterpret_cast<const float4*>(base + i0) + lane;
-      const float4* c4 = reinterpret_cast<const float4*>(cur + i0) + lane;
-      float4 b[kRows], c[kRows];
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) {
-        b[r] = ld_stream(b4 + 32 * r);
-        c[r] = ld_stream(c4 + 32 * r);
-      }
-#pragma unroll
-      for (int r = 0; r < kRows; ++r) {
-        const uint32_t d0 = __float_as_uint(__fsub_rn(c[r].x, b[r].x));
-        const uint32_t d1 = __float_as_uint(__fsub_rn(c[r].y, b[r].y));
-        const uint32_t d2 = __float_as_uint(__fsub_rn(c[r].z, b[r].z));
-        const uint32_t d3 = __float_as_uint(__fsub_rn(c[r].w, b[r].w));
-        const uint32_t k0 = slot_of(d0), k1 = slot_of(d1), k2 = slot_of(d2), k3 = slot_of(d3);
-        acc.add4(d0, d1, d2, d3, k0, k1, k2, k3);
-        // plane byte = low byte of the slot; gather the four into one word, element e in byte e.
-        const uint32_t lo = __byte_perm(k0, k1, 0x0040);
-        const uint32_t hi = __byte_perm(k2, k3, 0x0040);
-        ew[r] = __byte_perm(lo, hi, 0x5410);
-      }
-    } else {
-      // ragged tail: the last units of the vector, element by element.
-#pragma unroll 1
-      for (int r = 0; r < kRows; ++r) {
-        uint32_t word = 0;
-        for (int e = 0; e < 4; ++e) {
-          const uint64_t i = i0 + 128 * r + 4 * lane + e;
-          uint32_t d = 0;
-          if (i < n) {
-            d = __float_as_uint(__fsub_rn(cur[i], base[i]));
-            acc.add(d);
-          }
-          word |= (slot_of(d) & 255u) << (8 * e);
-        }
-        ew[r] = word;
-      }
-    }
-    uint4* ep = reinterpret_cast<uint4*>(plane + i0) + lane;
-    ep[0] = make_uint4(ew[0], ew[1], ew[2], ew[3]);
-    ep[32] = make_uint4(ew[4], ew[5], ew[6], ew[7]);
-  }
+  stats_units<MEAN, true>(acc, base, cur, n, warp, nunits, nwarps, lane, plane);
   __syncthreads();
-
-  // fold the 32 lane columns of each key and merge into the global bins.
-  for (uint32_t slot = threadIdx.x; slot < kKeys; slot += kStatsThreads) {
-    uint32_t total = 0;
-#pragma unroll 8
-    for (uint32_t l = 0; l < 32; ++l) total += cnt[slot * 32 + ((l + threadIdx.x) & 31)];
-    if (total != 0) {
-      const uint32_t key = key_of_slot(slot);
-      atomicAdd(&ctl->count[key], (unsigned long long)total);
-      atomicMax(&ctl->inv_min[key], mm[slot].x);
-      atomicMax(&ctl->max_bits[key], mm[slot].y);
-      if (MEAN) {
-        unsigned long long lo = 0, hi = 0;
-        for (uint32_t l = 0; l < 32; ++l) {
-          lo += cnt[kCntWords + slot * 32 + ((l + threadIdx.x) & 31)];
-          hi += cnt[2 * kCntWords + slot * 32 + ((l + threadIdx.x) & 31)];
-        }
-        atomicAdd(&ctl->mant_sum[key], lo + (hi << 12));
-      }
-    }
-  }
+  fold_stats<MEAN>(cnt, mm, ctl->count, ctl->inv_min, ctl->max_bits, ctl->mant_sum);
 }
 
 }  // namespace

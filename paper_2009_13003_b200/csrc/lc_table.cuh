@@ -7,7 +7,7 @@
 // with the fronts of both queues in registers: about 50 cycles a merge). Ranks, tree depths (pointer jumping), codes
 // (a sum over the symbols that come before) and sums are computed by all symbols at once; the stream's header and table
 // leave as 16-byte stores. With those steps in one thread, 64-bit shared-memory atomics and byte stores the pass took 10.5 us
-// for 8 symbols, 14 us for 16 and 28-36 us for 64; now 7.1, 8.6 and 15.5 us (cold caches, about 3 us of each the launch).
+// for 8 symbols, 14 us for 16 and 28-36 us for 64; now 7.0, 8.3 and 13.4 us (cold caches, about 3 us of each the launch).
 #pragma once
 #include "lc_common.cuh"
 
@@ -211,25 +211,23 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
           unsigned long long sum = 0;
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
-            uint32_t node;
-            if (a0 <= b0) {
-              sum += a0;
-              node = fa;
-              fa += 1;
-              a0 = a1;
-              a1 = T.leaf_w[fa + 1];
-            } else {
-              sum += b0;
-              node = nused + fb;
-              fb += 1;
-              b0 = b1;
-              b1 = T.node_w[fb + 1];
-            }
+            // one select chain and one load: the fronts come from registers, the entry two behind the front taken from
+            // the queue it is taken from
+            const bool leaf = a0 <= b0;  // a leaf goes before an internal node of the same weight
+            sum += leaf ? a0 : b0;
+            const uint32_t node = leaf ? fa : nused + fb;
+            fa += leaf ? 1u : 0u;
+            fb += leaf ? 0u : 1u;
+            const unsigned long long next = leaf ? T.leaf_w[fa + 1] : T.node_w[fb + 1];
+            a0 = leaf ? a1 : a0;
+            a1 = leaf ? next : a1;
+            b0 = leaf ? b0 : b1;
+            b1 = leaf ? b1 : next;
             T.up[node] = 1u << 16 | (nused + m);
           }
           T.node_w[m] = sum;
-          if (m == fb) b0 = sum;
-          else if (m == fb + 1) b1 = sum;
+          b0 = m == fb ? sum : b0;
+          b1 = m == fb + 1 ? sum : b1;
         }
         T.up[root] = root;
       }

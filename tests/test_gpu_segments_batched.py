@@ -70,3 +70,81 @@ def test_first_of_several_damaged_segments_is_reported(lc):
     worse[off[3] + 8: off[3] + 10] = 1
     lc.recover_segments_async(base, [streams, bad, streams, streams, worse], begin, 4, torch.empty_like(base), ws)
     assert lc.last_status(ws) == lc.ERR_FORMAT
+
+
+def check_segments(lc, oracle, base, cur, begin, nbits):
+    """In place, against the oracle segment by segment."""
+    offsets, total = lc.segments_layout(begin, nbits)
+    bh, ch = to_np(base).copy(), to_np(cur)
+    tracked = base.clone()
+    streams = torch.full((total,), 0xA5, dtype=torch.uint8, device=DEV)
+    longest = max(b - a for a, b in zip(begin[:-1], begin[1:]))
+    wsb = lc.workspace_bytes(longest)  # no more than the call asks for: groups end where it is full
+    ws = torch.full((wsb + 256,), 0x5A, dtype=torch.uint8, device=DEV)
+    lc.compress_segments(tracked, cur, begin, nbits, streams=streams, workspace=ws[:wsb], tracked_out=tracked)
+    assert bool((ws[wsb:] == 0x5A).all()), "wrote past the workspace"
+    got, state = to_np(streams), to_np(tracked)
+    for i, (a, b) in enumerate(zip(begin[:-1], begin[1:])):
+        want = oracle.compress(bh[a:b], ch[a:b], nbits)
+        assert got[offsets[i]: offsets[i] + want.size].tobytes() == want.tobytes(), "segment %d of %d" % (i, b - a)
+        assert np.array_equal(state[a:b].view(np.uint32), oracle.recover(bh[a:b], [want]).view(np.uint32)), "segment %d" % i
+
+
+def to_begin(sizes):
+    return [int(v) for v in np.concatenate([[0], np.cumsum(sizes)])]
+
+
+@pytest.mark.parametrize("nbits", [1, 4, 8, 9])
+def test_segments_of_every_kind(lc, oracle, nbits):
+    """Exponents the key plane does not hold, codes beyond 16 and 32 bits, entropy beyond a lane's column."""
+    g = torch.Generator(device="cpu").manual_seed(nbits)
+
+    def exponents(n, lo, hi):  # every (sign, exponent) of the range equally often: the longest streams
+        e = torch.randint(lo, hi, (n,), generator=g, dtype=torch.int32)
+        m = torch.randint(0, 1 << 23, (n,), generator=g, dtype=torch.int32)
+        s = torch.randint(0, 2, (n,), generator=g, dtype=torch.int32)
+        return ((s << 31) | (e << 23) | m).view(torch.float32)
+
+    def fibonacci(k):
+        from test_gpu_parity import _fibonacci_case
+
+        x = _fibonacci_case(k, False)[1].cpu() * 2.0 ** -20
+        return x[: x.numel() // 4 * 4]
+
+    parts = [exponents(70_000, 1, 127), fibonacci(24), torch.zeros(50_000), exponents(4096, 1, 254), exponents(70_004, 60, 200),
+             torch.cat([exponents(36_000, 1, 127), torch.full((300_000,), 1e-3)]), fibonacci(26), exponents(8, 100, 127)]
+    cur = torch.cat(parts).to(DEV)
+    check_segments(lc, oracle, torch.zeros_like(cur), cur, to_begin([p.numel() for p in parts]), nbits)
+
+
+def test_groups_that_the_workspace_limits(lc, oracle):
+    # many segments just above one chunk: a workspace for one of them holds the blocks of a dozen
+    sizes = [4100, 4096, 8192, 4, 6000] * 40
+    base, curs, begin = layered_case(sizes, 4100, 1)
+    check_segments(lc, oracle, base, curs[0], begin, 5)
+
+
+@pytest.mark.parametrize("failed", [0, 2, 3, 150, 199])
+def test_segments_behind_a_failure_have_no_stream(lc, oracle, failed):
+    sizes = [4096, 40_000, 1000, 12_292] * 50
+    base, curs, begin = layered_case(sizes, 5, 1)
+    cur, nbits = curs[0].clone(), 4
+    for f in (failed, min(failed + 3, len(sizes) - 1)):
+        cur[begin[f] + 7] = float("nan")
+    offsets, total = lc.segments_layout(begin, nbits)
+    ws = lc.alloc_workspace(max(sizes), DEV)
+    tracked = base.clone()
+    streams, _ = lc.compress_segments(base, curs[0], begin, nbits)  # valid streams of another call stand there
+    good = to_np(streams).copy()
+    lc.compress_segments_async(tracked, cur, begin, nbits, streams, ws, tracked)
+    assert lc.last_status(ws) == lc.ERR_NONFINITE
+    got = to_np(streams)
+    for i in range(len(sizes)):
+        if i < failed:
+            assert got[offsets[i]: offsets[i] + 64].tobytes() == good[offsets[i]: offsets[i] + 64].tobytes()
+        else:
+            assert lc.stream_info(streams[offsets[i]:]).valid == 0
+    assert torch.equal(tracked[begin[failed]:], base[begin[failed]:])
+    if failed:
+        want = lc.recover_segments(base[: begin[failed]].contiguous(), [streams], begin[: failed + 1], nbits)
+        assert torch.equal(tracked[: begin[failed]], want)
