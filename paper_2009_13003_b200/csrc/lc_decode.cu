@@ -36,7 +36,12 @@ namespace {
 
 using namespace dec;
 
-constexpr int kDecMaxThreads = 512;
+// Threads per CTA at most, and CTAs per SM that the registers must allow: with one stream 24 warps fit on an SM as two CTAs
+// of 12 (80 registers); with more streams a thread holds more state and one CTA of 16 warps takes the SM.
+template <int KS>
+constexpr int kDecThreads = KS == 1 ? 384 : 512;
+template <int KS>
+constexpr int kDecCtas = KS == 1 ? 2 : 1;
 constexpr int kL1Bits = 6;
 constexpr int kL1Rep = 16;
 // Second level: one sub-table per 6-bit prefix that belongs to longer codes, all of one depth: the next 10 bits if a
@@ -607,7 +612,7 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
 }
 
 template <int KS>
-__global__ void __launch_bounds__(kDecMaxThreads, 1)
+__global__ void __launch_bounds__(kDecThreads<KS>, kDecCtas<KS>)
 decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status, uint32_t rank,
               uint32_t stage_bytes, uint64_t chunk_begin, uint64_t chunk_end) {
   decode_vector<KS>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
@@ -616,7 +621,7 @@ decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, 
 // Per-layer recovery: the CTAs [cta_begin[i], cta_begin[i + 1]) decode segment i. One launch instead of one per segment
 // (a segment of a few chunks occupies one SM for the 15 us that a chunk takes; 62 of them in a row took 870 us).
 template <int KS>
-__global__ void __launch_bounds__(kDecMaxThreads, 1)
+__global__ void __launch_bounds__(kDecThreads<KS>, kDecCtas<KS>)
 decode_segments_kernel(const float* base, const __grid_constant__ DecodeStreams buffers, float* out,
                        int32_t* __restrict__ status, uint32_t second, uint32_t stage_bytes,
                        const __grid_constant__ SegBatch batch) {
@@ -678,7 +683,7 @@ cudaError_t decode_shape(const void* fn, uint64_t want_stage, uint32_t (&regs_of
   const uint32_t regs = regs_of[dev];
   if (want_stage > kMaxStage) want_stage = kMaxStage;
   best = Shape{0, 0, 0, 0, (uint32_t)sms_of[dev]};
-  for (uint32_t w = 16; w >= 8; w -= 4) {
+  for (uint32_t w = kDecThreads<KS> / 32; w >= 8; w -= 4) {
     uint32_t st = (uint32_t)want_stage;
     if (kTables + (uint64_t)w * KS * st > kMaxDyn) {
       if (w > 8) continue;                               // try fewer warps first
@@ -709,6 +714,18 @@ cudaError_t decode_shape(const void* fn, uint64_t want_stage, uint32_t (&regs_of
   return cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve < 100 ? carve : 100);
 }
 
+// A warp decodes whole chunks, so `chunks` of them take a whole number of rounds over the CTAs that fit on the device.
+// With as few warps as do them in the same number of rounds all rounds are equally full; with all warps the last one can
+// be nearly empty, and takes nearly as long as the others (11.7 M elements, four streams: 19.3 chunks per SM in rounds of
+// 16 and 3.3, or of 10 and 9.3). Four warps at least: fewer take longer over the tables than they save.
+template <int KS>
+uint32_t balanced_warps(uint64_t chunks, uint64_t ctas, uint32_t most) {
+  const uint64_t rounds = (chunks + ctas * most - 1) / (ctas * most);
+  if (rounds == 0) return 4;
+  const uint64_t w = (chunks + ctas * rounds - 1) / (ctas * rounds);
+  return w < 4 ? 4 : (uint32_t)w;
+}
+
 template <int KS>
 cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
                              int32_t* status, bool second, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
@@ -725,11 +742,12 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
   const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_kernel<KS>), align_up(avg + avg / 32 + 48, 16),
                                          regs_of, sh);
   if (e != cudaSuccess) return e;
-  uint64_t want = (chunk_end - chunk_begin + sh.warps - 1) / sh.warps;
+  const uint64_t chunks = chunk_end - chunk_begin, full = (uint64_t)sh.sms * sh.per_sm;
+  const uint32_t warps = balanced_warps<KS>(chunks, full, sh.warps);
+  uint64_t want = (chunks + warps - 1) / warps;
   if (want == 0) want = 1;  // still reports a rejected stream
-  const uint64_t full = (uint64_t)sh.sms * sh.per_sm;
   const unsigned grid = (unsigned)(want < full ? want : full);
-  decode_kernel<KS><<<grid, sh.warps * 32, sh.dyn, cs>>>(base, streams, n, out, status, second ? 1u : 0u, sh.stage, chunk_begin,
+  decode_kernel<KS><<<grid, warps * 32, sh.dyn - (sh.warps - warps) * KS * sh.stage, cs>>>(base, streams, n, out, status, second ? 1u : 0u, sh.stage, chunk_begin,
                                                          chunk_end);
   return cudaGetLastError();
 }
