@@ -38,13 +38,12 @@ int compress_impl(const float* base, const float* cur, uint64_t n, int nbits, vo
   if (workspace_bytes < W.total || stream_capacity < lc_stream_bound(n, nbits)) return LC_ERR_CAPACITY;
   const Carved c = carve(workspace, W);
 
-  // a small vector with the default options: one CTA does everything in one launch (no memset either)
+  // a small vector with the default options: one CTA or cluster does everything in one launch (no memset either)
   if (n > 0 && n <= kSmallMaxElems && !opt.two_pass_scan && !opt.fixed_width && !opt.mean_rep && !opt.length_cache &&
       opt.ticket_bias == 0 && opt.spin_limit == EncodeOptions().spin_limit) {
-    if (launch_small_compress(c.ctl, base, cur, n, nbits, static_cast<uint8_t*>(stream), tracked_out, keep_status, cs) !=
-        cudaSuccess)
-      return LC_ERR_CUDA;
-    return LC_OK;
+    const cudaError_t e = launch_small_compress(c.ctl, base, cur, n, nbits, static_cast<uint8_t*>(stream), tracked_out, keep_status, cs);
+    if (e == cudaSuccess) return LC_OK;
+    if (e != cudaErrorNotSupported) return LC_ERR_CUDA;
   }
 
   // control block and tile descriptors start at zero (keep_status: all but the status word, which holds the
@@ -253,7 +252,7 @@ int lc_compress_segments(const float* base, const float* cur, const uint64_t* se
     uint32_t blocks = 0, tiles = 0;
     for (g.nseg = 0; g.nseg < kSegGroup && i < nseg; ++g.nseg, ++i) {
       const uint64_t ni = seg_begin[i + 1] - seg_begin[i];
-      const bool small = ni <= kSmallMaxElems;
+      const bool small = ni <= kChunkElems;
       const uint32_t t = small ? 0 : (uint32_t)((ni + kEncWarps * kChunkElems - 1) / (kEncWarps * kChunkElems));
       if (!small && sizeof(SegBlock) * (blocks + 1) + 8ull * (tiles + t) > capacity) break;
       g.block[g.nseg] = (uint16_t)blocks;

@@ -154,12 +154,13 @@ struct EncodeOptions {
 constexpr uint32_t kLengthCacheRow = 512;                            // bytes per row: one row per number of used symbols
 constexpr uint64_t kLengthCacheBytes = 512ull * kLengthCacheRow;
 
-// Vectors of at most this many elements (one chunk, which the CTA holds in registers) take the single-CTA, single-launch
-// compress path: 10 us a call at 1000 elements, where the memset and three launches of the general path took 44-48 us.
-constexpr uint64_t kSmallMaxElems = kChunkElems;
+// Vectors of at most this many elements take the single-launch compress path: one CTA for one chunk, a cluster of up to
+// 16 CTAs (the most that the hardware schedules together) with one or two chunks each beyond that.
+constexpr uint64_t kSmallMaxElems = 32 * kChunkElems;
 
 // ---- launchers (each defined next to its kernel) ---------------------------------------------------
-// the whole compress pass of a small vector (0 < n <= kSmallMaxElems) in one launch; tracked_out may be null
+// the whole compress pass of a small vector (0 < n <= kSmallMaxElems) in one launch; tracked_out may be null.
+// cudaErrorNotSupported, with nothing launched: the device has no room for a cluster of that size.
 cudaError_t launch_small_compress(Control* ctl, const float* base, const float* cur, uint64_t n, int nbits,
                                   uint8_t* stream, float* tracked_out, bool keep_status, cudaStream_t cs);
 // mean: also accumulate the mantissa sums the mean-representative variant needs (a slower kernel variant)

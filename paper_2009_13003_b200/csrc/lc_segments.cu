@@ -39,7 +39,7 @@ segments_stats_kernel(const float* base, const float* __restrict__ cur, Control*
   const uint32_t s = find_segment(group.cta_begin, group.nseg, blockIdx.x);
   const uint64_t lo = group.elem_begin[s], n = group.elem_begin[s + 1] - lo;
   bool bad = false;
-  if (n <= kSmallMaxElems) {
+  if (n <= kChunkElems) {
     for (uint32_t i = threadIdx.x; i < n; i += kStatsThreads)
       bad |= (__float_as_uint(__fsub_rn(cur[lo + i], base[lo + i])) & 0x7f800000u) == 0x7f800000u;
   } else {
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kTableThreads)
 segments_table_kernel(const float* base, const float* cur, Control* __restrict__ ctl, SegBlock* __restrict__ blocks, int nbits,
                       uint8_t* __restrict__ streams, float* tracked_out, const __grid_constant__ SegGroup group) {
   extern __shared__ __align__(16) unsigned char s_small[];
-  small::SmallShared& S = *reinterpret_cast<small::SmallShared*>(s_small);
+  small::SmallShared<1>& S = *reinterpret_cast<small::SmallShared<1>*>(s_small);
   const uint32_t s = blockIdx.x, tid = threadIdx.x;
   const uint64_t lo = group.elem_begin[s], n = group.elem_begin[s + 1] - lo;
   uint8_t* stream = streams + group.stream_begin[s];
@@ -76,8 +76,8 @@ segments_table_kernel(const float* base, const float* cur, Control* __restrict__
     if (tid == 0 && group.first + s == ~fail) set_status_ranked(&ctl->status, ~fail, LC_ERR_NONFINITE);
     return;
   }
-  if (n <= kSmallMaxElems) {
-    small::small_vector(S, base + lo, cur + lo, (uint32_t)n, nbits, stream, tracked_out ? tracked_out + lo : nullptr, nullptr);
+  if (n <= kChunkElems) {
+    small::small_vector<1, false>(S, base + lo, cur + lo, (uint32_t)n, nbits, stream, tracked_out ? tracked_out + lo : nullptr, nullptr);
     return;
   }
   SegBlock& B = blocks[group.block[s]];
@@ -402,7 +402,7 @@ cudaError_t launch_compress_segments(Control* ctl, SegBlock* blocks, unsigned lo
     if (e == cudaSuccess) e = cudaFuncSetAttribute(segments_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStatsSmem);
     // the carve-out that two resident CTAs need, as for the kernel for one vector (the rest serves as L1)
     if (e == cudaSuccess) e = cudaFuncSetAttribute(segments_stats_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 61);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(segments_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(small::SmallShared));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(segments_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(small::SmallShared<1>));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(segments_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(kEncWarps * (seg_lane_words(kMaxNbits) * 128 + seg_image_bytes(kMaxNbits))));
@@ -420,14 +420,14 @@ cudaError_t launch_compress_segments(Control* ctl, SegBlock* blocks, unsigned lo
     for (uint32_t i = 0; i < group.nseg; ++i) {
       const uint64_t n = group.elem_begin[i + 1] - group.elem_begin[i], units = (n + kUnitElems - 1) / kUnitElems;
       group.cta_begin[i] = (uint32_t)ctas;
-      ctas += n <= kSmallMaxElems ? (n > 0 ? 1 : 0) : (units + per_cta - 1) / per_cta;
+      ctas += n <= kChunkElems ? (n > 0 ? 1 : 0) : (units + per_cta - 1) / per_cta;
       longest = units > longest ? units : longest;
     }
     if (ctas <= slots || per_cta >= longest) break;
   }
   group.cta_begin[group.nseg] = (uint32_t)ctas;
   if (ctas > 0) segments_stats_kernel<<<(unsigned)ctas, kStatsThreads, kStatsSmem, cs>>>(base, cur, ctl, blocks, group);
-  segments_table_kernel<<<group.nseg, kTableThreads, sizeof(small::SmallShared), cs>>>(base, cur, ctl, blocks, nbits, streams, tracked_out, group);
+  segments_table_kernel<<<group.nseg, kTableThreads, sizeof(small::SmallShared<1>), cs>>>(base, cur, ctl, blocks, nbits, streams, tracked_out, group);
   const uint32_t ntiles = group.tile_begin[group.nseg];
   if (ntiles > 0) {
     const uint32_t lane_words = seg_lane_words(nbits), image_bytes = seg_image_bytes(nbits);

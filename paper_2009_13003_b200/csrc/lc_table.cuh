@@ -71,9 +71,10 @@ __device__ __forceinline__ void clear_header(uint8_t* stream) {
 }
 
 // `my`: the statistics of key_of_position(threadIdx.x). Returns 0, or the error that makes the vector unencodable, the
-// same for all threads; on success the stream's header (but for its total size), table and padding are written, and T is
-// complete and visible to all threads.
-__device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, const TableArgs& A, uint8_t* __restrict__ stream) {
+// same for all threads; on success the stream's header (but for its total size), table and padding are written (unless
+// !write), and T is complete and visible to all threads.
+__device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, const TableArgs& A, uint8_t* __restrict__ stream,
+                                          bool write = true) {
   constexpr uint32_t kAll = 0xffffffffu;
   constexpr unsigned long long kNone = ~0ull;  // weight behind the end of a queue
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -286,10 +287,10 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
     T.payload_bits = payload_bits;
   }
   const StreamLayout L = stream_layout(A.n, nsym);
-  if (is_sym)
+  if (is_sym && write)
     reinterpret_cast<uint4*>(stream + L.table_off)[tid] =
         make_uint4((tid ? T.key[tid] : 0u) | my_len << 16, tid ? T.rep[tid] : 0u, (uint32_t)my_local, (uint32_t)(my_local >> 32));
-  if (tid < 4) {
+  if (tid < 4 && write) {
     const uint32_t flag = (A.fixed ? 1u : 0u) | (A.shard ? 2u : 0u) | (hit ? 4u : 0u) | (A.mean ? 8u : 0u);
     // a vector without chunks leaves nothing for the encode pass to do: its stream ends here
     const unsigned long long total = L.nchunks == 0 ? L.payload_off : 0ull;
@@ -302,8 +303,8 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
   }
   // bytes between the lane index and the payload are zero
   const uint64_t index_end = L.lane_index_off + 64 * L.nchunks;
-  if (tid < L.payload_off - index_end) stream[index_end + tid] = 0;
-  if (tid == 0 && L.nchunks == 0) *reinterpret_cast<unsigned long long*>(stream + L.chunk_index_off) = 0;
+  if (write && tid < L.payload_off - index_end) stream[index_end + tid] = 0;
+  if (write && tid == 0 && L.nchunks == 0) *reinterpret_cast<unsigned long long*>(stream + L.chunk_index_off) = 0;
   __syncthreads();
   return LC_OK;
 }
