@@ -186,6 +186,16 @@ def stream_info(stream) -> LCInfo:
     return info
 
 
+def _finished(stream, workspace, what) -> int:
+    """Waits for a compress pass on the current stream and returns its stream's size. One read of the header is enough
+    when the pass has succeeded: a pass that fails takes the magic away or never writes the size, and only then is the
+    status word read as well."""
+    info = stream_info(stream)
+    if not info.valid or info.total_bytes == 0:
+        _check(last_status(workspace), what)
+    return info.total_bytes
+
+
 def compress(base, cur, nbits, stream=None, workspace=None, fixed=False, mean=False):
     """stream <- LC(cur - base). Returns the stream trimmed to its size (a view of ``stream``). ``fixed``: fixed-width
     bucket indices instead of the Huffman code (LC_OPT_FIXED_WIDTH). ``mean``: bucket means as representatives
@@ -199,9 +209,7 @@ def compress(base, cur, nbits, stream=None, workspace=None, fixed=False, mean=Fa
         compress_opt_async(base, cur, nbits, stream, workspace, (OPT_FIXED_WIDTH if fixed else 0) | (OPT_MEAN_REP if mean else 0))
     else:
         compress_async(base, cur, nbits, stream, workspace)
-    _check(last_status(workspace), "lc_compress (device)")
-    info = stream_info(stream)
-    return stream[: info.total_bytes]
+    return stream[: _finished(stream, workspace, "lc_compress (device)")]
 
 
 LENGTH_CACHE_BYTES = 262144
@@ -229,8 +237,7 @@ def compress_cached(base, cur, nbits, length_cache, stream=None, workspace=None,
     if workspace is None:
         workspace = alloc_workspace(n, base.device)
     compress_cached_async(base, cur, nbits, stream, workspace, length_cache, tracked_out)
-    _check(last_status(workspace), "lc_compress_cached (device)")
-    return stream[: stream_info(stream).total_bytes]
+    return stream[: _finished(stream, workspace, "lc_compress_cached (device)")]
 
 
 def segments_layout(seg_begin, nbits):
@@ -300,9 +307,7 @@ def compress_update(base, cur, nbits, tracked_out=None, stream=None, workspace=N
     if tracked_out is None:
         tracked_out = torch.empty_like(base)
     compress_update_async(base, cur, nbits, stream, tracked_out, workspace)
-    _check(last_status(workspace), "lc_compress_update (device)")
-    info = stream_info(stream)
-    return stream[: info.total_bytes], tracked_out
+    return stream[: _finished(stream, workspace, "lc_compress_update (device)")], tracked_out
 
 
 def recover_async(base, streams, out, workspace):
@@ -386,8 +391,7 @@ def shard_encode(base, cur, nbits, whole_stats, workspace, stream=None):
     _check(lib().lc_shard_encode(base.data_ptr(), cur.data_ptr(), n, nbits, whole_stats.data_ptr(), stream.data_ptr(),
                                  stream.numel(), workspace.data_ptr(), workspace.numel(), _cs(base.device)),
            "lc_shard_encode")
-    _check(last_status(workspace), "lc_shard_encode (device)")
-    return stream[: stream_info(stream).total_bytes]
+    return stream[: _finished(stream, workspace, "lc_shard_encode (device)")]
 
 
 def merge_async(base, streams, nbits, stream, scratch, workspace):
@@ -412,8 +416,7 @@ def merge(base, streams, nbits, stream=None, scratch=None, workspace=None):
     if workspace is None:
         workspace = alloc_workspace(n, base.device)
     merge_async(base, streams, nbits, stream, scratch, workspace)
-    _check(last_status(workspace), "lc_merge (device)")
-    return stream[: stream_info(stream).total_bytes]
+    return stream[: _finished(stream, workspace, "lc_merge (device)")]
 
 
 def host_arena_bytes(n, nbits, k) -> int:
