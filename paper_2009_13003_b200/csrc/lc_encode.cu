@@ -6,11 +6,10 @@
 //
 // A CTA takes a tile of 8 consecutive chunks, one per warp; lane t owns lane sub-stream t. Per chunk:
 //   A. every lane codes its 128 elements into its own column of a warp-private word matrix in shared
-//      memory (word k of lane t at k*32 + t: plain stores, no bank conflicts, no atomics). Code and
-//      length come packed in one 32-bit table entry (a 16-byte entry made the lookups saturate the
-//      shared-memory pipe) and two neighbouring codes are appended as one; the rare codes of 17..32 bits
-//      sit behind one vote per four elements. Emitting a finished word is a handful of predicated
-//      instructions;
+//      memory (word k of lane t at k*32 + t: plain stores, no bank conflicts, no atomics). Two elements are looked up at
+//      once in a table of pairs whose index is formed for all four elements of a step together (lc_encode_bits.cuh),
+//      and the step's codes are appended as one, so a step of four elements costs two lookups and one append. With a
+//      lookup per element and an append per two this pass took 0.99 ms for 1.3 G elements (a 5-bit code); now 0.68 ms;
 //   B. a warp shuffle scan of the lane bit counts gives every lane its bit offset in the chunk (the
 //      lane index of the stream) and the chunk its size, which is published at once;
 //   C. the lanes' words are shifted to their bit offsets and ORed into the chunk image (shared memory);
@@ -32,8 +31,8 @@
 // ORed in place): codes longer than 32 bits, a lane or chunk that outgrows its shared-memory area, and vectors with an
 // exponent field >= 128, for which the one-byte key plane is not enough and keys come from base and cur.
 //
-// Bound: reads 1 byte and writes about 0.5 bytes per element, so this pass is limited by the integer
-// work per element, not by HBM.
+// Bound: reads 1 byte and writes about 0.5 bytes per element, so this pass is limited by the integer work per element,
+// not by HBM: logic, shifts, permutes and compares issue at 64 lanes per clock and SM, half the rate of multiply-adds.
 #include "lc_encode_bits.cuh"
 
 namespace lc {
@@ -42,9 +41,9 @@ namespace {
 using namespace enc;
 
 constexpr int kEncThreads = kEncWarps * 32;
-// 48 KB of dynamic shared memory per CTA (four CTAs per SM), split evenly between the warps that work:
-// all 8 while an average chunk fits half of a 6 KB share (column matrix + chunk image), else 4, 2 or 1.
-constexpr uint32_t kEncSmem = 48 * 1024;
+// 44 KB of dynamic shared memory per CTA (four CTAs per SM, beside 8 KB of tables), split evenly between the warps that work:
+// all 8 while an average chunk fits half of a 5.5 KB share (column matrix + chunk image), else 4, 2 or 1.
+constexpr uint32_t kEncSmem = 44 * 1024;
 constexpr int kUpdRows = 4;  // rows of base in flight per warp in the kernel that also writes the tracked state
 constexpr uint32_t kUpdSmem = kEncWarps * kUpdRows * 512;  // its ring, behind the kEncSmem bytes of coding areas
 constexpr int kLookBack = 8;  // look-back sub-windows of 32 tile descriptors read per round
@@ -80,11 +79,12 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   for (uint32_t b = tid; b < 256; b += kEncThreads) {
     const EncEntry e = ctl->enc[((b & 1u) << 8) | (b >> 1)];
     tb.full[b] = make_uint2(e.code_lo, e.len);
-    tb.packed[b] = e.len <= kPackedMaxLen ? (e.len << kPackedLenShift) | e.code_lo : kPackedLong << kPackedLenShift;
     // the table pass has written the stream's symbol table: entry of symbol s at 64 + 16 s, representative at +4
     if (UPDATE) s_rep[b] = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
   }
   __syncthreads();
+  static_assert(kEncThreads == 256, "a thread per plane byte");
+  build_tables(tb, ctl->enc[0].len, [&](uint32_t b) { return ctl->enc[((b & 1u) << 8) | (b >> 1)].sym != 0; });
 
   const uint32_t nsym = ctl->nsym;
   const bool long_codes = ctl->max_len > 32;
@@ -103,22 +103,9 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   const uint32_t lane_words = image_words / 32;        // rows of the column matrix
   uint32_t* column = s_dyn + (warp % active) * (2 * image_words);  // word k of lane t at column[k*32 + t]
   uint32_t* image = column + image_words;
-  const uint32_t packed_addr = smem_addr(tb.packed);
+  const uint32_t neg_base = (uint32_t)(-tb.base) & 0xffffu, neg_base2 = neg_base << 16 | neg_base;
+  const bool use_pair = tb.use_pair != 0;
 
-  // Appends the four codes of `word`, whose packed entries are g. Only the marker of a code of more than 16 bits has
-  // bit 31 set, so one test per row finds the rare longer codes; that row then appends its four codes one by one from
-  // `full`.
-  auto put4 = [&](ColumnPacker& pk, uint32_t word, const uint32_t (&g)[4]) {
-    if (__any_sync(0xffffffffu, (int)(g[0] | g[1] | g[2] | g[3]) < 0)) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint2 f = tb.full[__byte_perm(word, 0u, 0x4440 + e)];
-        pk.put(f.x, f.y);
-      }
-    } else {
-      put4_packed(pk, g);
-    }
-  };
   auto fast_chunk = [&](uint64_t cc) { return cc < nchunks && (cc + 1) * kChunkElems <= n && !long_codes && !ks.wide; };
 
   const uint64_t ntiles = (nchunks + active - 1) / active;
@@ -155,10 +142,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     if (fast) {
       const uint4* ep = reinterpret_cast<const uint4*>(plane + c * kChunkElems) + lane;
       const uint32_t col0 = smem_addr(column) + lane * 4;
-      ColumnPacker pk{0u, 0u, 0u, col0, col0 + lane_words * 128};
-      uint32_t g0[4], g1[4];
-      uint4 cur4 = __ldg(ep);
-      lookup4(packed_addr, cur4.x, g0);
+      ColumnPacker pk{0u, 0u, col0, col0 + lane_words * 128};
       // UPDATE: the tracked state of this chunk is written here, where its plane bytes are in registers; the
       // memory traffic of the update then runs under the coding, which is bound by instruction issue. A chunk on
       // this path never reads base for its coding (not even when it is coded again the slow way), so base may be
@@ -193,23 +177,12 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
         o4[32 * j] = x;
         issue_row(j + kUpdRows);
       };
-#pragma unroll 1
-      for (int q = 0; q < 8; ++q) {
-        const uint4 nxt = __ldg(ep + 32 * (q + 1 < 8 ? q + 1 : q));  // next 16 plane bytes, one step ahead
-        lookup4(packed_addr, cur4.y, g1);
-        put4(pk, cur4.x, g0);
-        if (UPDATE) update_row(cur4.x, 4 * q);
-        lookup4(packed_addr, cur4.z, g0);
-        put4(pk, cur4.y, g1);
-        if (UPDATE) update_row(cur4.y, 4 * q + 1);
-        lookup4(packed_addr, cur4.w, g1);
-        put4(pk, cur4.z, g0);
-        if (UPDATE) update_row(cur4.z, 4 * q + 2);
-        lookup4(packed_addr, nxt.x, g0);  // first row of the next step (unused after the last step)
-        put4(pk, cur4.w, g1);
-        if (UPDATE) update_row(cur4.w, 4 * q + 3);
-        cur4 = nxt;
-      }
+      auto load = [&](int q) { return __ldg(ep + 32 * q); };
+      auto row = [&](uint32_t word, int j) {
+        if (UPDATE) update_row(word, j);
+      };
+      if (use_pair) code_rows<true>(pk, tb, neg_base2, load, row);
+      else code_rows<false>(pk, tb, neg_base2, load, row);
       lane_bits = finish_column(pk, col0);
     } else if (valid && !long_codes && !ks.wide) {
       lane_bits = code_partial(&tb, reinterpret_cast<const uint4*>(plane + c * kChunkElems) + lane, (uint32_t)(n - c * kChunkElems),

@@ -6,15 +6,97 @@
 namespace lc {
 namespace enc {
 
-constexpr uint32_t kPackedLenShift = 26;                      // packed entry: length << 26 | code
-constexpr uint32_t kPackedCodeMask = (1u << kPackedLenShift) - 1;
-constexpr uint32_t kPackedMaxLen = 16;                        // two packed codes make one append of <= 32 bits
-constexpr uint32_t kPackedLong = 63;                          // length field of a code that does not fit
+// ---- code tables ---------------------------------------------------------------------------------------------
+// A table entry holds its code left-aligned in the upper 24 bits and the length in the low byte: the code is then appended
+// with one shift by the number of pending bits, and adding two entries adds their lengths.
+constexpr uint32_t kEntryLenMask = 255u;
+constexpr uint32_t kEntryMaxLen = 24;
+constexpr uint32_t kEntryLong = 100u;      // length of an entry without a code: it takes every sum of two beyond 32
+constexpr uint32_t kSingleMaxLen = 16;     // codes in `single`: two of them make one append of at most 32 bits
+constexpr int kPairSpan = 32;              // values a byte takes in the index of a pair
 
 struct Tables {
-  uint32_t packed[256];  // by plane byte: length << 26 | code for codes of up to 16 bits, else length field 63
-  uint2 full[256];       // by plane byte: {code, length} for codes of up to 32 bits
+  union {
+    uint32_t pair[kPairSpan * kPairSpan];  // both codes of two neighbouring elements
+    uint32_t single[256];                  // by plane byte
+  };
+  uint2 full[256];     // by plane byte: {code, length} for codes of up to 32 bits
+  uint32_t scan[256];  // while the table is built
+  uint32_t best, below, above;
+  int32_t base;        // see build_tables
+  uint32_t use_pair;
 };
+
+__device__ __forceinline__ uint32_t make_entry(uint32_t code, uint32_t len, uint32_t longest) {
+  return len > longest ? kEntryLong : (len ? code << (32 - len) : 0u) | len;
+}
+
+// Builds the table the coding loop looks codes up in; `full` is there, `sym0_len` is the zero bucket's code length and
+// kept(b) tells whether plane byte b's bucket has a symbol of its own. All threads of a CTA of 256; ends with a barrier.
+//
+// Two neighbouring elements are looked up together: a plane byte b counts as clamp(b - base, 0, 31), and the two make an
+// index of 10 bits. The clamped values cover 16 exponents of both signs, which is all that 2^5 - 1 kept buckets usually
+// span; all bytes below are the zero bucket then. If more than that is kept, the 32 values go where most elements are, and
+// a pair with an element outside is marked and coded the long way. Unless less than one element in 256 is outside, single
+// bytes are looked up instead (one row of 128 elements in three would take the long way, which costs as much as it saves).
+template <class Kept>
+__device__ __forceinline__ void build_tables(Tables& tb, uint32_t sym0_len, Kept kept) {
+  const uint32_t b = threadIdx.x, lane = b & 31, warp = b >> 5;
+  const bool is_kept = kept(b);
+  const uint32_t my_len = tb.full[b].y;
+  // the share of the elements that a code of this length stands for, out of 2^22
+  const auto share = [](uint32_t len) { return len == 0 || len > 22 ? 0u : 1u << (22 - len); };
+  const uint32_t mine = is_kept ? share(my_len) : 0u;
+  uint32_t incl = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d);
+    if ((int)lane >= d) incl += v;
+  }
+  const uint32_t ballot = __ballot_sync(0xffffffffu, is_kept);
+  if (b == 0) tb.best = 0, tb.below = 255, tb.above = 0;
+  __syncthreads();
+  tb.scan[b] = incl;
+  if (lane == 0 && ballot) {
+    atomicMin(&tb.below, 32 * warp + __ffs(ballot) - 1);
+    atomicMax(&tb.above, 32 * warp + 31 - __clz(ballot));
+  }
+  __syncthreads();
+  for (uint32_t w = 0; w < warp; ++w) incl += tb.scan[32 * w + 31];
+  __syncthreads();
+  tb.scan[b] = incl;  // share of the kept bytes up to b
+  __syncthreads();
+  const uint32_t lowest = tb.below, highest = tb.above;  // of the kept bytes; 255 and 0 if there are none
+  // candidate: base = b. Values 1..30 are bytes of their own; 0 and 31 stand for all beyond, if those are of one kind.
+  {
+    const uint32_t upto = tb.scan[min(b + 30, 255u)];
+    uint32_t covered = upto - incl;
+    if (lowest > b || lowest > highest) covered += share(sym0_len);
+    if (highest <= b + 31 && b + 31 < 256) covered += tb.scan[b + 31] - upto;
+    const uint32_t score = __reduce_max_sync(0xffffffffu, covered << 8 | b);  // covered <= 2^22
+    if (lane == 0) atomicMax(&tb.best, score);
+  }
+  __syncthreads();
+  const int32_t base = (int32_t)(tb.best & 255u);
+  const uint32_t covered = tb.best >> 8, all = tb.scan[255] + share(sym0_len);
+  const bool use_pair = lowest > highest || all - covered <= all >> 8;
+  if (b == 0) {
+    tb.base = base;
+    tb.use_pair = use_pair ? 1u : 0u;
+  }
+  if (use_pair) {
+    for (uint32_t k = b; k < kPairSpan * kPairSpan; k += 256) {
+      const uint32_t v0 = k % kPairSpan, v1 = k / kPairSpan;  // clamped bytes of the first and second element
+      const auto escapes = [&](uint32_t v) { return v == 0 ? lowest <= (uint32_t)base && lowest <= highest : v == 31 && highest > (uint32_t)base + 31; };
+      const uint2 f0 = tb.full[min(base + v0, 255u)], f1 = tb.full[min(base + v1, 255u)];
+      const uint32_t len = f0.y + f1.y;
+      tb.pair[k] = escapes(v0) || escapes(v1) || f0.y > 32 || f1.y > 32 ? kEntryLong : make_entry(f0.x << (f1.y & 31) | f1.x, len, kEntryMaxLen);
+    }
+  } else {
+    tb.single[b] = make_entry(tb.full[b].x, my_len, kSingleMaxLen);
+  }
+  __syncthreads();
+}
 
 // Where the slow path gets an element's key from.
 struct KeySource {
@@ -106,59 +188,130 @@ __device__ __forceinline__ void st_tile(unsigned long long* p, unsigned long lon
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Fast-path state of a lane: pending bits in hi:lo (low `nb` bits valid), next word slot in its column.
+// Fast-path state of a lane: pending bits at the top of `w` (`nb` < 32 of them), next word slot in its column.
 struct ColumnPacker {
-  uint32_t hi, lo, nb;
+  uint32_t w, nb;
   uint32_t dst;  // shared address of the next word of this lane's column (stride 128 bytes)
   uint32_t lim;  // shared address one past the column
+  // appends `len` <= 32 bits that stand left-aligned in `code` (zero below)
   __device__ __forceinline__ void put(uint32_t code, uint32_t len) {
-    // (hi:lo) = (hi:lo) << len | code, len <= 32
-    hi = __funnelshift_lc(lo, hi, len);
-    lo = __funnelshift_lc(0u, lo, len) | code;
-    nb += len;
-    // emit the oldest 32 pending bits once there are 32 or more, unless the column is full
+    // the word that is complete with 32 or more bits is emitted, unless the column is full: nb then stays at 32 or more
     asm volatile(
         "{\n\t"
         ".reg .pred q;\n\t"
-        ".reg .u32 w;\n\t"
-        "setp.ge.u32 q, %0, 32;\n\t"
-        "setp.lt.and.u32 q, %1, %4, q;\n\t"
-        "@q sub.u32 %0, %0, 32;\n\t"
-        "@q shf.r.clamp.b32 w, %3, %2, %0;\n\t"
-        "@q st.shared.u32 [%1], w;\n\t"
-        "@q add.u32 %1, %1, 128;\n\t"
+        ".reg .u32 t;\n\t"
+        "shr.u32 t, %4, %1;\n\t"
+        "or.b32 %0, %0, t;\n\t"
+        "shf.r.wrap.b32 t, 0, %4, %1;\n\t"  // the bits that do not fit: code << (32 - nb), 0 if nb is 0
+        "add.u32 %1, %1, %5;\n\t"
+        "setp.ge.u32 q, %1, 32;\n\t"
+        "setp.lt.and.u32 q, %2, %3, q;\n\t"
+        "@q st.shared.u32 [%2], %0;\n\t"
+        "@q mov.u32 %0, t;\n\t"
+        "@q add.u32 %2, %2, 128;\n\t"
+        "@q sub.u32 %1, %1, 32;\n\t"
         "}"
-        : "+r"(nb), "+r"(dst)
-        : "r"(hi), "r"(lo), "r"(lim)
+        : "+r"(w), "+r"(nb), "+r"(dst)
+        : "r"(lim), "r"(code), "r"(len)
         : "memory");
+  }
+  // a code of at most 32 bits as `full` has it
+  __device__ __forceinline__ void put_full(uint2 f) { put(f.y ? f.x << (32 - f.y) : 0u, f.y); }
+  // two entries, lengths together at most 32
+  __device__ __forceinline__ void put_two(uint32_t e0, uint32_t e1, uint32_t len) {
+    put((e0 & ~kEntryLenMask) | __funnelshift_r(e1 & ~kEntryLenMask, 0u, e0), len);  // shift by the low 5 bits: e0's length
   }
 };
 
-// Packed table entries (shared address packed_addr) of the four plane bytes of `word`.
-__device__ __forceinline__ void lookup4(uint32_t packed_addr, uint32_t word, uint32_t (&g)[4]) {
+// Entries of the two pairs of a row's plane bytes `word`: elements 0 and 1, elements 2 and 3. `neg_base`: -base in both
+// halves. The four bytes are clamped two at a time, in 16-bit halves.
+__device__ __forceinline__ uint2 lookup_pairs(const Tables& tb, uint32_t word, uint32_t neg_base) {
+  const uint32_t v0 = __viaddmin_s16x2_relu(__byte_perm(word, 0u, 0x4240), neg_base, 0x001f001fu);  // elements 0, 2
+  const uint32_t v1 = __viaddmin_s16x2_relu(__byte_perm(word, 0u, 0x4341), neg_base, 0x001f001fu);  // elements 1, 3
+  const uint32_t at = (v1 * kPairSpan + v0) * 4u;  // byte offsets of the two entries, one in each half
+  const volatile char* t = reinterpret_cast<const volatile char*>(tb.pair);  // volatile: one row ahead of the use
+  return make_uint2(*reinterpret_cast<const volatile uint32_t*>(t + (at & 0xffffu)),
+                    *reinterpret_cast<const volatile uint32_t*>(t + (at >> 16)));
+}
+// One row (four elements) of which e holds the pairs' entries. A pair that is marked, or two that are longer than 32 bits
+// together, send the warp the long way.
+__device__ __forceinline__ void put_pairs(ColumnPacker& pk, const Tables& tb, uint32_t word, uint2 e) {
+  const uint32_t len = (e.x + e.y) & kEntryLenMask;
+  if (__any_sync(0xffffffffu, len > 32)) {
 #pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    const uint32_t b = __byte_perm(word, 0u, 0x4440 + e);  // plane byte of slot e
-    // volatile: keeps the loads where they are written, one row ahead of their use
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(g[e]) : "r"(packed_addr + b * 4u));
+    for (int k = 0; k < 4; ++k) pk.put_full(tb.full[__byte_perm(word, 0u, 0x4440 + k)]);
+  } else {
+    pk.put_two(e.x, e.y, len);
   }
 }
 
-// Appends four codes whose packed entries are g, none of them the marker of a long code. Packed codes have at most 16
-// bits, so two neighbours are joined into one append of at most 32 bits (half the accumulator and flush work).
-__device__ __forceinline__ void put4_packed(ColumnPacker& pk, const uint32_t (&g)[4]) {
+// The same with single bytes: entries of the four plane bytes, two appends of two.
+__device__ __forceinline__ uint4 lookup_singles(const Tables& tb, uint32_t word) {
+  const volatile uint32_t* t = tb.single;
+  return make_uint4(t[word & 255u], t[(word >> 8) & 255u], t[(word >> 16) & 255u], t[word >> 24]);
+}
+__device__ __forceinline__ void put_singles(ColumnPacker& pk, const Tables& tb, uint32_t word, uint4 e) {
+  const uint32_t l0 = (e.x + e.y) & kEntryLenMask, l1 = (e.z + e.w) & kEntryLenMask;
+  if (__any_sync(0xffffffffu, max(l0, l1) > 32)) {
 #pragma unroll
-  for (int e = 0; e < 4; e += 2) {
-    const uint32_t l0 = g[e] >> kPackedLenShift, l1 = g[e + 1] >> kPackedLenShift;
-    const uint32_t c0 = g[e] & kPackedCodeMask, c1 = g[e + 1] & kPackedCodeMask;
-    pk.put((c0 << l1) | c1, l0 + l1);
+    for (int k = 0; k < 4; ++k) pk.put_full(tb.full[__byte_perm(word, 0u, 0x4440 + k)]);
+  } else {
+    pk.put_two(e.x, e.y, l0);
+    pk.put_two(e.z, e.w, l1);
+  }
+}
+
+// Codes a whole chunk's rows for one lane: `load(q)` gives the plane bytes of steps 4q .. 4q + 3, and row(word, j) is
+// called behind step j. Plane bytes are read one q ahead, lookups run one row ahead of the appends (which depend on each
+// other through the pending bits).
+template <bool PAIR, class Load, class Row>
+__device__ __forceinline__ void code_rows(ColumnPacker& pk, const Tables& tb, uint32_t neg_base, Load load, Row row) {
+  uint4 now = load(0);
+  if (PAIR) {
+    uint2 a = lookup_pairs(tb, now.x, neg_base), b;
+#pragma unroll 1
+    for (int q = 0; q < (int)kSteps / 4; ++q) {
+      const uint4 nxt = load(q + 1 < (int)kSteps / 4 ? q + 1 : q);
+      b = lookup_pairs(tb, now.y, neg_base);
+      put_pairs(pk, tb, now.x, a);
+      row(now.x, 4 * q);
+      a = lookup_pairs(tb, now.z, neg_base);
+      put_pairs(pk, tb, now.y, b);
+      row(now.y, 4 * q + 1);
+      b = lookup_pairs(tb, now.w, neg_base);
+      put_pairs(pk, tb, now.z, a);
+      row(now.z, 4 * q + 2);
+      a = lookup_pairs(tb, nxt.x, neg_base);  // first row of the next step (unused after the last step)
+      put_pairs(pk, tb, now.w, b);
+      row(now.w, 4 * q + 3);
+      now = nxt;
+    }
+  } else {
+    uint4 a = lookup_singles(tb, now.x), b;
+#pragma unroll 1
+    for (int q = 0; q < (int)kSteps / 4; ++q) {
+      const uint4 nxt = load(q + 1 < (int)kSteps / 4 ? q + 1 : q);
+      b = lookup_singles(tb, now.y);
+      put_singles(pk, tb, now.x, a);
+      row(now.x, 4 * q);
+      a = lookup_singles(tb, now.z);
+      put_singles(pk, tb, now.y, b);
+      row(now.y, 4 * q + 1);
+      b = lookup_singles(tb, now.w);
+      put_singles(pk, tb, now.z, a);
+      row(now.z, 4 * q + 2);
+      a = lookup_singles(tb, nxt.x);
+      put_singles(pk, tb, now.w, b);
+      row(now.w, 4 * q + 3);
+      now = nxt;
+    }
   }
 }
 
 // Ends a lane's column: writes the pending bits and returns the lane's bit count, or ~0 if the column was too small.
 __device__ __forceinline__ uint32_t finish_column(const ColumnPacker& pk, uint32_t col0) {
   if (pk.nb >= 32 || (pk.nb > 0 && pk.dst >= pk.lim)) return 0xffffffffu;
-  if (pk.nb > 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(pk.dst), "r"(pk.lo << (32 - pk.nb)) : "memory");
+  if (pk.nb > 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(pk.dst), "r"(pk.w) : "memory");
   return ((pk.dst - col0) >> 7) * 32 + pk.nb;
 }
 
@@ -169,37 +322,25 @@ __device__ __forceinline__ uint32_t finish_column(const ColumnPacker& pk, uint32
 // that it does not weigh on the registers of the main loop. Returns the lane's bit count, ~0 if a column overflowed.
 static __device__ __noinline__ uint32_t code_partial(const Tables* tb, const uint4* ep, uint32_t rem, uint32_t lane,
                                               uint32_t col0, uint32_t lane_words) {
-  ColumnPacker pk{0u, 0u, 0u, col0, col0 + lane_words * 128};
-  const uint32_t packed_addr = smem_addr(tb->packed);
+  ColumnPacker pk{0u, 0u, col0, col0 + lane_words * 128};
   const uint32_t rows = (rem + 127) / 128;
   uint4 nxt = *ep;
 #pragma unroll 1
   for (uint32_t q = 0; 4 * q < rows; ++q) {
     const uint32_t words[4] = {nxt.x, nxt.y, nxt.z, nxt.w};
     if (q + 1 < kSteps / 4) nxt = ep[32 * (q + 1)];
-    uint32_t g[4][4];
+    uint2 f[4][4];
 #pragma unroll
     for (uint32_t r = 0; r < 4; ++r) {
-      lookup4(packed_addr, words[r], g[r]);
       const uint32_t first = (4 * q + r) * 128 + 4 * lane;
-      const uint32_t have = first < rem ? rem - first : 0u;  // elements from this slot group on
 #pragma unroll
-      for (uint32_t e = 0; e < 4; ++e)
-        if (e >= have) g[r][e] = 0u;  // no element: an empty code
+      for (uint32_t e = 0; e < 4; ++e)  // no element: an empty code
+        f[r][e] = first + e < rem ? tb->full[__byte_perm(words[r], 0u, 0x4440 + e)] : make_uint2(0u, 0u);
     }
 #pragma unroll
-    for (uint32_t r = 0; r < 4; ++r) {
-      if ((int)(g[r][0] | g[r][1] | g[r][2] | g[r][3]) < 0) {
+    for (uint32_t r = 0; r < 4; ++r)
 #pragma unroll
-        for (uint32_t e = 0; e < 4; ++e) {
-          if (g[r][e] == 0u) continue;
-          const uint2 f = tb->full[__byte_perm(words[r], 0u, 0x4440 + e)];
-          pk.put(f.x, f.y);
-        }
-      } else {
-        put4_packed(pk, g[r]);
-      }
-    }
+      for (uint32_t e = 0; e < 4; ++e) pk.put_full(f[r][e]);
   }
   return finish_column(pk, col0);
 }

@@ -149,10 +149,11 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
   for (uint32_t b = tid; b < 256; b += kSegThreads) {
     const EncEntry e = B.enc[((b & 1u) << 8) | (b >> 1)];
     tb.full[b] = make_uint2(e.code_lo, e.len);
-    tb.packed[b] = e.len <= kPackedMaxLen ? (e.len << kPackedLenShift) | e.code_lo : kPackedLong << kPackedLenShift;
     s_rep[b] = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
   }
   __syncthreads();
+  static_assert(kSegThreads == 256, "a thread per plane byte");
+  build_tables(tb, B.enc[0].len, [&](uint32_t b) { return B.enc[((b & 1u) << 8) | (b >> 1)].sym != 0; });
 
   const StreamLayout L = stream_layout(n, nsym);
   const uint32_t first_tile = group.tile_begin[s], last_tile = group.tile_begin[s + 1] - 1;
@@ -212,35 +213,12 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
   if (fast) {
     const uint4* ep = reinterpret_cast<const uint4*>(plane) + lane;
     if (rem == kChunkElems) {
-      ColumnPacker pk{0u, 0u, 0u, col0, col0 + lane_words * 128};
-      const uint32_t packed_addr = smem_addr(tb.packed);
-      uint32_t g[2][4];
-      auto put4 = [&](uint32_t word, const uint32_t (&e4)[4]) {
-        if (__any_sync(0xffffffffu, (int)(e4[0] | e4[1] | e4[2] | e4[3]) < 0)) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const uint2 f = tb.full[__byte_perm(word, 0u, 0x4440 + e)];
-            pk.put(f.x, f.y);
-          }
-        } else {
-          put4_packed(pk, e4);
-        }
-      };
-      uint4 now = ep[0];
-      lookup4(packed_addr, now.x, g[0]);
-#pragma unroll 1
-      for (uint32_t q = 0; q < kSteps / 4; ++q) {
-        const uint4 nxt = ep[32 * (q + 1 < kSteps / 4 ? q + 1 : q)];
-        lookup4(packed_addr, now.y, g[1]);
-        put4(now.x, g[0]);
-        lookup4(packed_addr, now.z, g[0]);
-        put4(now.y, g[1]);
-        lookup4(packed_addr, now.w, g[1]);
-        put4(now.z, g[0]);
-        lookup4(packed_addr, nxt.x, g[0]);
-        put4(now.w, g[1]);
-        now = nxt;
-      }
+      ColumnPacker pk{0u, 0u, col0, col0 + lane_words * 128};
+      const uint32_t neg_base = (uint32_t)(-tb.base) & 0xffffu, neg_base2 = neg_base << 16 | neg_base;
+      auto load = [&](int q) { return ep[32 * q]; };
+      auto row = [](uint32_t, int) {};
+      if (tb.use_pair) code_rows<true>(pk, tb, neg_base2, load, row);
+      else code_rows<false>(pk, tb, neg_base2, load, row);
       lane_bits = finish_column(pk, col0);
     } else {
       lane_bits = code_partial(&tb, ep, rem, lane, col0, lane_words);
