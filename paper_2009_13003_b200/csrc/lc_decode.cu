@@ -37,9 +37,11 @@ namespace {
 using namespace dec;
 
 // Threads per CTA at most, and CTAs per SM that the registers must allow: with one stream 24 warps fit on an SM as two CTAs
-// of 12 (80 registers); with more streams a thread holds more state and one CTA of 16 warps takes the SM.
+// of 12 (80 registers); two streams fit one CTA of 20 (96 registers: 138 M elements 240 -> 220 us against 16 warps, 11.7 M
+// elements 46 -> 31 us, because their 19.3 chunks per SM are then one round); with three and four a thread holds more state
+// and one CTA of 16 takes the SM (bounded to 96 registers, four streams spill and take 1.4 times as long).
 template <int KS>
-constexpr int kDecThreads = KS == 1 ? 384 : 512;
+constexpr int kDecThreads = KS == 1 ? 384 : KS == 2 ? 640 : 512;
 template <int KS>
 constexpr int kDecCtas = KS == 1 ? 2 : 1;
 constexpr int kL1Bits = 6;
@@ -658,7 +660,7 @@ inline uint32_t ctas_on_sm(uint32_t warps, uint32_t dyn, uint32_t regs) {
   return min(min(by_regs, by_smem), by_warps);
 }
 
-// want_stage: staging bytes that hold an average chunk with some room. Among CTAs of 16, 12 and 8 warps, takes the shape
+// want_stage: staging bytes that hold an average chunk with some room. Among CTAs of 20 (two streams only), 16, 12 and 8 warps, takes the shape
 // that puts most warps on an SM (with four streams that is one CTA of 16 warps, with one stream several smaller ones),
 // then gives the staging areas whatever shared memory that shape leaves (chunk sizes vary around the average).
 template <int KS>
