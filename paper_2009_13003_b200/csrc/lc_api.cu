@@ -94,15 +94,16 @@ int compress_impl(const float* base, const float* cur, uint64_t n, int nbits, vo
 
   // control block and tile descriptors start at zero (keep_status: all but the status word, which holds the
   // outcome of the pass that produced `cur`; the table pass then leaves the vector alone if it is set)
-  const uint64_t skip = keep_status ? sizeof(int32_t) : 0;
-  cudaError_t e = cudaMemsetAsync(static_cast<uint8_t*>(workspace) + skip, 0, W.plane_off - skip, cs);
+  // The four kernels are launched so that each may begin before the one ahead of it has ended.
+  const uint64_t control = opt.mean_rep ? sizeof(Control) : offsetof(Control, enc);  // the sums of the variant lie behind enc
+  cudaError_t e = launch_clear(c.ctl, control, c.tiles, align_up(8 * W.nchunks, 16), keep_status, cs);
   if (e != cudaSuccess) return LC_ERR_CUDA;
-  if ((e = launch_stats(base, cur, n, c.ctl, c.plane, cs, opt.mean_rep)) != cudaSuccess) return LC_ERR_CUDA;
+  if ((e = launch_stats(base, cur, n, c.ctl, c.plane, cs, opt.mean_rep, true)) != cudaSuccess) return LC_ERR_CUDA;
   if ((e = launch_table(c.ctl, n, nbits, static_cast<uint8_t*>(stream), true, opt.fixed_width, nullptr, opt.length_cache, cs,
-                        opt.mean_rep)) != cudaSuccess)
+                        opt.mean_rep, true)) != cudaSuccess)
     return LC_ERR_CUDA;
-  if ((e = launch_encode(c.ctl, c.tiles, c.plane, base, cur, n, static_cast<uint8_t*>(stream), tracked_out, opt,
-                         cs)) != cudaSuccess)
+  if ((e = launch_encode(c.ctl, c.tiles, c.plane, base, cur, n, static_cast<uint8_t*>(stream), tracked_out, opt, cs, true)) !=
+      cudaSuccess)
     return LC_ERR_CUDA;
   return LC_OK;
 }
@@ -289,7 +290,7 @@ int lc_compress_segments(const float* base, const float* cur, const uint64_t* se
   constexpr uint64_t kScratch = offsetof(Control, count);
   Control* ctl = static_cast<Control*>(workspace);
   uint8_t* scratch = static_cast<uint8_t*>(workspace) + kScratch;
-  const uint64_t capacity = workspace_bytes - kScratch;
+  const uint64_t capacity = (workspace_bytes - kScratch) & ~15ull;
   SegGroup g;
   uint64_t off = 0;
   for (int i = 0; i < nseg;) {
@@ -314,7 +315,7 @@ int lc_compress_segments(const float* base, const float* cur, const uint64_t* se
     g.stream_begin[g.nseg] = off;
     const uint64_t used = sizeof(SegBlock) * blocks + 8ull * tiles;
     uint8_t* clear = first_group ? static_cast<uint8_t*>(workspace) : scratch;  // status and failure word once per call
-    if (cudaMemsetAsync(clear, 0, (size_t)(scratch + used - clear), cs) != cudaSuccess) return LC_ERR_CUDA;
+    if (launch_clear(clear, align_up((uint64_t)(scratch + used - clear), 16), nullptr, 0, false, cs) != cudaSuccess) return LC_ERR_CUDA;
     if (launch_compress_segments(ctl, reinterpret_cast<SegBlock*>(scratch),
                                  reinterpret_cast<unsigned long long*>(scratch + sizeof(SegBlock) * blocks), base, cur, g, nbits,
                                  static_cast<uint8_t*>(streams), tracked_out, cs) != cudaSuccess)

@@ -130,6 +130,32 @@ static __device__ __noinline__ void set_status_ranked(int32_t* status, uint32_t 
   }
 }
 
+// ---- overlapped launches -------------------------------------------------------------------------------
+// The kernels of a call follow each other closely and the small ones last as long as a launch. A kernel launched with
+// `overlap` may start once every CTA of the one before it in the stream has called begin_next(), and may touch what that
+// kernel (and those before it) wrote only behind wait_previous(). Every kernel of such a chain calls wait_previous(), so
+// that the guarantee reaches back to the first; the first of a call is launched without `overlap`, i.e. behind everything
+// the caller has enqueued. Without the attribute both are no-ops. With a memset and plain launches instead, a compress of
+// 11.7 M elements took 52 us on the GPU, with this 45 us. (Recovery has only a memset ahead of its kernel; there the launch of
+// a clearing kernel costs the host more than the overlap gains.)
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void begin_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_kernel(bool overlap, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t cs, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = cs;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- per-device launch parameters ---------------------------------------------------------------------
 // Occupancy figures, SM counts and the "attributes are set" marks that the launchers cache are properties of a
 // device (cudaFuncSetAttribute applies to the current device only), so every such cache is an array indexed by
@@ -158,6 +184,10 @@ constexpr uint64_t kLengthCacheBytes = 512ull * kLengthCacheRow;
 // 16 CTAs (the most that the hardware schedules together) with one or two chunks each beyond that.
 constexpr uint64_t kSmallMaxElems = 32 * kChunkElems;
 
+// Zeroes two ranges (16-byte aligned, multiples of 16 bytes; the first word of `a` is kept if keep_first) with a kernel, the
+// first of a chain of overlapped launches: unlike a memset it lets the next kernel begin beside it.
+cudaError_t launch_clear(void* a, uint64_t a_bytes, void* b, uint64_t b_bytes, bool keep_first, cudaStream_t cs);
+
 // ---- launchers (each defined next to its kernel) ---------------------------------------------------
 // the whole compress pass of a small vector (0 < n <= kSmallMaxElems) in one launch; tracked_out may be null.
 // cudaErrorNotSupported, with nothing launched: the device has no room for a cluster of that size.
@@ -165,18 +195,18 @@ cudaError_t launch_small_compress(Control* ctl, const float* base, const float* 
                                   uint8_t* stream, float* tracked_out, bool keep_status, cudaStream_t cs);
 // mean: also accumulate the mantissa sums the mean-representative variant needs (a slower kernel variant)
 cudaError_t launch_stats(const float* base, const float* cur, uint64_t n, Control* ctl, uint8_t* plane,
-                         cudaStream_t cs, bool mean = false);
+                         cudaStream_t cs, bool mean = false, bool overlap = false);
 // wide_ok: false if the encode pass will not be able to read base and cur (the table pass then rejects a vector
 // with an exponent field >= 128 with LC_ERR_RANGE)
 // fixed: fixed-width codes (format section 1.5) instead of the Huffman code
 // whole: nullptr, or the statistics of the whole vector of which this call codes a shard (format section 1.6):
 //        kept buckets, representatives and code then come from them, the table's counts from ctl's own
 cudaError_t launch_table(Control* ctl, uint64_t n, int nbits, uint8_t* stream, bool wide_ok, bool fixed,
-                         const ShardStats* whole, uint8_t* length_cache, cudaStream_t cs, bool mean = false);
+                         const ShardStats* whole, uint8_t* length_cache, cudaStream_t cs, bool mean = false, bool overlap = false);
 // tracked_out: nullptr, or where to write base + quantized delta (may be base itself)
 cudaError_t launch_encode(Control* ctl, unsigned long long* tiles, const uint8_t* plane, const float* base,
                           const float* cur, uint64_t n, uint8_t* stream, float* tracked_out, const EncodeOptions& opt,
-                          cudaStream_t cs);
+                          cudaStream_t cs, bool overlap = false);
 
 struct DecodeStreams {
   const uint8_t* ptr[4];

@@ -68,6 +68,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   __shared__ uint32_t s_arrived[2];  // warps that have coded their chunk of the tile in this half
   __shared__ uint32_t s_rep[UPDATE ? 256 : 1];  // UPDATE: representative (bit pattern) by plane byte
 
+  wait_previous();
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // The table pass may have rejected the vector, or another CTA may already have given up waiting: leave, all
   // threads together (one thread reads the word; a thread-by-thread test could split the CTA if the word changed
@@ -493,7 +494,7 @@ encode_scan_kernel(const Control* __restrict__ ctl, const unsigned long long* __
 
 cudaError_t launch_encode(Control* ctl, unsigned long long* tiles, const uint8_t* plane, const float* base,
                           const float* cur, uint64_t n, uint8_t* stream, float* tracked_out, const EncodeOptions& opt,
-                          cudaStream_t cs) {
+                          cudaStream_t cs, bool overlap) {
   const WorkspaceLayout W = workspace_layout(n);
   if (W.nchunks == 0) return cudaSuccess;
   static int blocks_per_sm[kMaxDevices][2] = {}, sms[kMaxDevices] = {};  // by device ordinal
@@ -523,13 +524,12 @@ cudaError_t launch_encode(Control* ctl, unsigned long long* tiles, const uint8_t
     if (cudaGetLastError() != cudaSuccess) return cudaErrorLaunchFailure;
   }
   const uint32_t two = opt.two_pass_scan ? 1u : 0u;
+  overlap = overlap && !opt.two_pass_scan;
   if (v)
-    encode_kernel<true><<<grid, kEncThreads, kEncSmem + kUpdSmem, cs>>>(ctl, tiles, plane, base, cur, n, stream, tracked_out,
-                                                                       opt.spin_limit, opt.ticket_bias, two);
-  else
-    encode_kernel<false><<<grid, kEncThreads, kEncSmem, cs>>>(ctl, tiles, plane, base, cur, n, stream, nullptr,
-                                                              opt.spin_limit, opt.ticket_bias, two);
-  return cudaGetLastError();
+    return launch_kernel(overlap, encode_kernel<true>, grid, kEncThreads, kEncSmem + kUpdSmem, cs, ctl, tiles, plane, base, cur, n, stream,
+                         tracked_out, opt.spin_limit, opt.ticket_bias, two);
+  return launch_kernel(overlap, encode_kernel<false>, grid, kEncThreads, kEncSmem, cs, ctl, tiles, plane, base, cur, n, stream,
+                       static_cast<float*>(nullptr), opt.spin_limit, opt.ticket_bias, two);
 }
 
 }  // namespace lc

@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(kStatsThreads, 2)
 segments_stats_kernel(const float* base, const float* __restrict__ cur, Control* __restrict__ ctl, SegBlock* __restrict__ blocks,
                       const __grid_constant__ SegGroup group) {
   extern __shared__ __align__(16) uint32_t smem[];
+  begin_next();
   const uint32_t s = find_segment(group.cta_begin, group.nseg, blockIdx.x);
   const uint64_t lo = group.elem_begin[s], n = group.elem_begin[s + 1] - lo;
   bool bad = false;
@@ -53,10 +54,12 @@ segments_stats_kernel(const float* base, const float* __restrict__ cur, Control*
     Acc<false> acc{cnt + lane, mm};
     stats_units<false, false>(acc, base + lo, cur + lo, n, (uint64_t)cta * (kStatsThreads / 32) + warp, (n + kUnitElems - 1) / kUnitElems,
                               (uint64_t)ctas * (kStatsThreads / 32), lane, nullptr);
+    wait_previous();  // the blocks are clear
     __syncthreads();
     ShardStats& out = blocks[group.block[s]].stats;
     bad = fold_stats<false>(cnt, mm, out.count, out.inv_min, out.max_bits, nullptr);
   }
+  wait_previous();
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicMax(&ctl->seg_fail, ~(group.first + s));
 }
 
@@ -65,6 +68,8 @@ segments_table_kernel(const float* base, const float* cur, Control* __restrict__
                       uint8_t* __restrict__ streams, float* tracked_out, const __grid_constant__ SegGroup group) {
   extern __shared__ __align__(16) unsigned char s_small[];
   small::SmallShared<1>& S = *reinterpret_cast<small::SmallShared<1>*>(s_small);
+  begin_next();
+  wait_previous();
   const uint32_t s = blockIdx.x, tid = threadIdx.x;
   const uint64_t lo = group.elem_begin[s], n = group.elem_begin[s + 1] - lo;
   uint8_t* stream = streams + group.stream_begin[s];
@@ -132,6 +137,7 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
   __shared__ uint32_t s_tile;
   __shared__ unsigned long long s_prefix;
   __shared__ int s_abort;
+  wait_previous();
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
     s_tile = atomicAdd(&ctl->seg_ticket, 1u);
@@ -404,15 +410,20 @@ cudaError_t launch_compress_segments(Control* ctl, SegBlock* blocks, unsigned lo
     if (ctas <= slots || per_cta >= longest) break;
   }
   group.cta_begin[group.nseg] = (uint32_t)ctas;
-  if (ctas > 0) segments_stats_kernel<<<(unsigned)ctas, kStatsThreads, kStatsSmem, cs>>>(base, cur, ctl, blocks, group);
-  segments_table_kernel<<<group.nseg, kTableThreads, sizeof(small::SmallShared<1>), cs>>>(base, cur, ctl, blocks, nbits, streams, tracked_out, group);
+  // overlapped launches, the first behind the caller's clear kernel
+  cudaError_t e = cudaSuccess;
+  if (ctas > 0)
+    e = launch_kernel(true, segments_stats_kernel, (unsigned)ctas, kStatsThreads, kStatsSmem, cs, base, cur, ctl, blocks, group);
+  if (e == cudaSuccess)
+    e = launch_kernel(true, segments_table_kernel, group.nseg, kTableThreads, sizeof(small::SmallShared<1>), cs, base, cur, ctl, blocks,
+                      nbits, streams, tracked_out, group);
   const uint32_t ntiles = group.tile_begin[group.nseg];
-  if (ntiles > 0) {
+  if (e == cudaSuccess && ntiles > 0) {
     const uint32_t lane_words = seg_lane_words(nbits), image_bytes = seg_image_bytes(nbits);
-    segments_encode_kernel<<<ntiles, kSegThreads, kEncWarps * (lane_words * 128 + image_bytes), cs>>>(
-        ctl, blocks, tiles, base, cur, streams, tracked_out, lane_words, image_bytes, EncodeOptions().spin_limit, group);
+    e = launch_kernel(true, segments_encode_kernel, ntiles, kSegThreads, kEncWarps * (lane_words * 128 + image_bytes), cs, ctl, blocks,
+                      tiles, base, cur, streams, tracked_out, lane_words, image_bytes, EncodeOptions().spin_limit, group);
   }
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace lc

@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(kStatsThreads, MEAN ? 1 : 2)
 stats_kernel(const float* __restrict__ base, const float* __restrict__ cur, uint64_t n, uint64_t nunits,
              Control* __restrict__ ctl, uint8_t* __restrict__ plane) {
   extern __shared__ __align__(16) uint32_t smem[];
+  begin_next();
   // MEAN: cnt, then the two sum tables, then mm
   constexpr uint32_t kTables = MEAN ? 3 : 1;
   uint32_t* cnt = smem;
@@ -48,6 +49,7 @@ stats_kernel(const float* __restrict__ base, const float* __restrict__ cur, uint
   Acc<MEAN> acc{cnt + lane, mm};
 
   stats_units<MEAN, true>(acc, base, cur, n, warp, nunits, nwarps, lane, plane);
+  wait_previous();  // the bins are clear
   __syncthreads();
   fold_stats<MEAN>(cnt, mm, ctl->count, ctl->inv_min, ctl->max_bits, ctl->mant_sum);
 }
@@ -55,7 +57,7 @@ stats_kernel(const float* __restrict__ base, const float* __restrict__ cur, uint
 }  // namespace
 
 cudaError_t launch_stats(const float* base, const float* cur, uint64_t n, Control* ctl, uint8_t* plane,
-                         cudaStream_t cs, bool mean) {
+                         cudaStream_t cs, bool mean, bool overlap) {
   const WorkspaceLayout W = workspace_layout(n);
   if (W.nunits == 0) return cudaSuccess;
   static int blocks_per_sm[kMaxDevices][2] = {}, sms[kMaxDevices] = {};  // by device ordinal and kernel variant
@@ -89,11 +91,9 @@ cudaError_t launch_stats(const float* base, const float* cur, uint64_t n, Contro
     // the 32-bit column sums of the variant hold for a bounded number of units per warp (see kMeanMaxUnitsPerWarp)
     const uint64_t nwarps = (uint64_t)grid * (kStatsThreads / 32);
     if ((W.nunits + nwarps - 1) / nwarps > kMeanMaxUnitsPerWarp) return cudaErrorInvalidConfiguration;
-    stats_kernel<true><<<grid, kStatsThreads, smem, cs>>>(base, cur, n, W.nunits, ctl, plane);
-  } else {
-    stats_kernel<false><<<grid, kStatsThreads, smem, cs>>>(base, cur, n, W.nunits, ctl, plane);
+    return launch_kernel(overlap, stats_kernel<true>, grid, kStatsThreads, smem, cs, base, cur, n, W.nunits, ctl, plane);
   }
-  return cudaGetLastError();
+  return launch_kernel(overlap, stats_kernel<false>, grid, kStatsThreads, smem, cs, base, cur, n, W.nunits, ctl, plane);
 }
 
 }  // namespace lc

@@ -16,6 +16,8 @@ __global__ void __launch_bounds__(kTableThreads)
 table_kernel(Control* __restrict__ ctl, uint64_t n, int nbits, uint8_t* __restrict__ stream, int wide_ok,
              int fixed, const ShardStats* __restrict__ whole, uint8_t* __restrict__ cache, int mean) {
   __shared__ TableShared T;
+  begin_next();
+  wait_previous();
   const uint32_t tid = threadIdx.x, key = key_of_position(tid);
   // an earlier pass of the same call has failed (lc_merge: a stream was rejected): leave no stream behind
   if (ctl->status != 0) {  // nothing in this kernel has written the word yet: the same for every thread
@@ -46,13 +48,35 @@ table_kernel(Control* __restrict__ ctl, uint64_t n, int nbits, uint8_t* __restri
   }
 }
 
+__device__ __forceinline__ void clear_range(uint4* p, uint64_t count, bool keep_first) {
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (uint64_t)gridDim.x * blockDim.x) {
+    if (i == 0 && keep_first) {
+      uint32_t* w = reinterpret_cast<uint32_t*>(p);
+      w[1] = w[2] = w[3] = 0;
+    } else {
+      p[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(256) clear_kernel(uint4* a, uint64_t a_count, uint4* b, uint64_t b_count, uint32_t keep_first) {
+  begin_next();
+  clear_range(a, a_count, keep_first != 0);
+  clear_range(b, b_count, false);
+}
+
 }  // namespace
 
+cudaError_t launch_clear(void* a, uint64_t a_bytes, void* b, uint64_t b_bytes, bool keep_first, cudaStream_t cs) {
+  const uint64_t items = (a_bytes > b_bytes ? a_bytes : b_bytes) / 16, ctas = (items + 255) / 256;
+  return launch_kernel(false, clear_kernel, (unsigned)(ctas < 1 ? 1 : ctas > 148 ? 148 : ctas), 256, 0, cs, static_cast<uint4*>(a),
+                       a_bytes / 16, static_cast<uint4*>(b), b_bytes / 16, keep_first ? 1u : 0u);
+}
+
 cudaError_t launch_table(Control* ctl, uint64_t n, int nbits, uint8_t* stream, bool wide_ok, bool fixed,
-                         const ShardStats* whole, uint8_t* cache, cudaStream_t cs, bool mean) {
-  table_kernel<<<1, kTableThreads, 0, cs>>>(ctl, n, nbits, stream, wide_ok ? 1 : 0, fixed ? 1 : 0, whole, cache,
-                                            mean ? 1 : 0);
-  return cudaGetLastError();
+                         const ShardStats* whole, uint8_t* cache, cudaStream_t cs, bool mean, bool overlap) {
+  return launch_kernel(overlap, table_kernel, 1, kTableThreads, 0, cs, ctl, n, nbits, stream, wide_ok ? 1 : 0, fixed ? 1 : 0, whole,
+                       cache, mean ? 1 : 0);
 }
 
 }  // namespace lc
