@@ -58,10 +58,11 @@ __global__ void read_back_kernel(const uint32_t* src, uint32_t* dst, uint32_t wo
   if (threadIdx.x < words) dst[threadIdx.x] = src[threadIdx.x];
 }
 
+thread_local ReadBack t_read_back;
+
 // Copies `words` (at most 32) 32-bit words from the device and waits for `cs`.
 bool read_back(void* dst, const void* device_src, uint32_t words, cudaStream_t cs) {
-  static thread_local ReadBack mine;
-  void *page = mine.get(), *mapped = nullptr;
+  void *page = t_read_back.get(), *mapped = nullptr;
   if (page && cudaHostGetDevicePointer(&mapped, page, 0) == cudaSuccess) {
     read_back_kernel<<<1, 32, 0, cs>>>(static_cast<const uint32_t*>(device_src), static_cast<uint32_t*>(mapped), words);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(cs) != cudaSuccess) return false;
