@@ -16,12 +16,11 @@
 //    first level is indexed by the next kL1Bits bits and replicated 16 times (entry for (index, lane)
 //    at index*16 + lane%16): a 64-bit shared load is served half a warp at a time, so the 16 lanes of
 //    a half-warp always hit 16 different bank pairs although their indices are data dependent.
-//    An entry whose 6-bit prefix belongs to longer codes points to a 64-entry sub-table indexed by the
-//    next 6 bits (one predicated load, no branch), which resolves codes of up to 12 bits; still longer
-//    codes are found by a canonical search behind a warp vote.
+//    Codes are canonical, so the 6-bit prefixes of longer codes are the last ones; from the first of them on a lane
+//    reads the second level instead, indexed by up to 10 more bits (the same load, no branch), which resolves codes of
+//    up to 16 bits; still longer codes are found by a canonical search behind a warp vote.
 //  * A lane keeps a 64-bit bit buffer per stream and tops it up with one predicated word load before
-//    every second symbol; that is enough because two table-resolved codes use at most 2*12 <= 33
-//    bits.
+//    every fourth symbol; a lane whose four codes take more bits than it held does the step again.
 //
 // Every read of a stream is bounds-checked against the caller's buffer size and every table is
 // validated before use, so a damaged stream yields LC_ERR_FORMAT (and unspecified output), never an
@@ -58,10 +57,10 @@ static_assert(((1 << kL1Bits) << (kSubBitsMin + 3)) <= 8192, "at the smallest de
 // which is how the hot loop notices: a step subtracts at most four of them per stream, and 1..4 times 2^29 (less a
 // few real lengths) leaves the sign bit of the 32-bit count set in every case.
 constexpr uint32_t kLongCode = 0x20000000u;
-// distance, in steps of 512 bytes per warp, of the L2 prefetch of base (measured: 4, 6, 8, 12 and 16 rows; chains of
-// two and more do not care between 4 and 12, a single stream is fastest at 6)
+// distance, in steps of 512 bytes per warp, of the L2 prefetch of base: chains of two and more do not care between 4 and 12;
+// a single stream of 138 M elements takes 194 us at 4, 207 at 6, 228 at 8 and 247 at 12
 template <int KS>
-constexpr int kPrefetchRows = KS == 1 ? 6 : 8;
+constexpr int kPrefetchRows = KS == 1 ? 4 : 8;
 
 // The two lookup tables of a stream are 8 KB each; the first starts on a 128-byte boundary of shared memory.
 constexpr uint32_t kTableBytes = 8192;
@@ -77,13 +76,14 @@ struct Status {
 
 struct alignas(16) StreamState {
   const uint8_t* ptr;  // the stream
-  uint32_t l1_addr;    // shared address of the first level: [(1 << kL1Bits) * kL1Rep] {bit pattern of rep, code length};
-                       // length kLongCode = not resolved here. The second level follows it at kTableBytes: sub-tables of
-                       // (1 << sub_bits) entries: {rep, length} or length kLongCode = longer code
+  uint32_t l1_addr;    // shared address of the first level: [(1 << kL1Bits) * kL1Rep] {bit pattern of rep, code length}.
+                       // The second level follows it at kTableBytes: nsub sub-tables of (1 << sub_bits) entries:
+                       // {rep, length} or length kLongCode = longer code
   int32_t err;         // outcome of the validation
   unsigned long long payload_off, payload_size, chunk_index_off, lane_index_off;
   uint32_t max_len, nused, only_rep;
-  uint32_t nsub;        // first-level prefixes that belong to longer codes: the last nsub of them (codes are canonical)
+  uint32_t misses;      // first-level prefixes that belong to longer codes: the last ones (codes are canonical)
+  uint32_t nsub;        // prefixes looked up in the second level: the most misses among the launch's streams
   uint32_t sub_bits;    // depth of the sub-tables, kSubBitsMin..kSubBitsMax: as many as 8 KB hold at that depth
   uint32_t end31[20];   // [L], L = 1..16: end of the range that codes of at most L bits fill, left-aligned to 31 bits
   uint32_t sorted_rep[kMaxSymbols];    // representatives in canonical (len, id) order
@@ -209,11 +209,9 @@ __device__ __noinline__ int prepare_stream(StreamState& S, unsigned char* scratc
   S.len_offset[l1] = S.len_next[l1] = offset - c1;
   if (l0 <= 16) S.end31[l0] = (uint32_t)(end0 >> 32);
   if (l1 <= 16) S.end31[l1] = (uint32_t)(end1 >> 32);
-  // first-level prefixes behind the codes of at most kL1Bits bits get a sub-table each, as deep as their number allows
+  // first-level prefixes behind the codes of at most kL1Bits bits
   const uint32_t short_end = (uint32_t)(__shfl_sync(kAll, (kL1Bits & 1) ? end1 : end0, kL1Bits / 2) >> (63 - kL1Bits));
   const uint32_t misses = nused >= 2 ? (1u << kL1Bits) - min(short_end, 1u << kL1Bits) : 0u;
-  uint32_t sub_bits = kSubBitsMax;
-  while (sub_bits > kSubBitsMin && misses > (kTableBytes >> (sub_bits + 3))) sub_bits -= 1;
   if (lane == 0) {
     S.payload_off = payload_off;
     S.payload_size = payload_size;
@@ -222,8 +220,7 @@ __device__ __noinline__ int prepare_stream(StreamState& S, unsigned char* scratc
     S.max_len = max_len;
     S.nused = nused;
     S.only_rep = only_rep;
-    S.nsub = misses;
-    S.sub_bits = sub_bits;
+    S.misses = misses;
   }
   __syncwarp();
 
@@ -266,11 +263,9 @@ __device__ __forceinline__ void fill_tables(const StreamState* S, unsigned char*
     const StreamState& T = S[s];
     uint2 ent = make_uint2(T.only_rep, 0u);
     if (T.nused >= 2) {
-      const uint2 r = canonical_lookup(T, idx << (31 - kL1Bits), kL1Bits);
-      // else the address of the prefix's sub-table, less the offset that the prefix bits add when the lookup indexes it
-      // with prefix and sub-table bits together (32-bit wrap-around arithmetic)
-      const uint32_t sub = idx - ((1u << kL1Bits) - T.nsub);
-      ent = r.y ? r : make_uint2(T.l1_addr + kTableBytes + (sub << (T.sub_bits + 3)) - ((idx << T.sub_bits) << 3), kLongCode);
+      if (idx >= (1u << kL1Bits) - T.nsub) continue;  // looked up in the second level
+      ent = canonical_lookup(T, idx << (31 - kL1Bits), kL1Bits);
+      if (ent.y == 0) ent.y = kLongCode;  // only with damaged lengths
     }
     uint4* l1 = reinterpret_cast<uint4*>(tables + s * 2 * kTableBytes);
     l1[idx * (kL1Rep / 2) + pair] = make_uint4(ent.x, ent.y, ent.x, ent.y);
@@ -279,8 +274,8 @@ __device__ __forceinline__ void fill_tables(const StreamState* S, unsigned char*
     const uint32_t s = k / (kTableBytes / 8), i = k % (kTableBytes / 8);
     const StreamState& T = S[s];
     const uint32_t sub = i >> T.sub_bits, j = i & ((1u << T.sub_bits) - 1);
-    uint2 ent = make_uint2(0u, kLongCode);
-    if (sub < T.nsub) {
+    uint2 ent = T.nused >= 2 ? make_uint2(0u, kLongCode) : make_uint2(T.only_rep, 0u);
+    if (sub < T.nsub && T.nused >= 2) {
       const uint32_t idx = (1u << kL1Bits) - T.nsub + sub, width = kL1Bits + T.sub_bits;
       const uint2 r = canonical_lookup(T, ((idx << T.sub_bits) | j) << (31 - width), width);
       if (r.y) ent = r;
@@ -289,28 +284,35 @@ __device__ __forceinline__ void fill_tables(const StreamState* S, unsigned char*
   }
 }
 
-// Two-level table lookup of the code at the top of `hi`: {representative, length}, length kLongCode if
-// the tables do not resolve it. `l1lane` = shared address of this lane's copy of first-level entry 0.
-// The first-level entry of a prefix that belongs to longer codes holds the shared address of the
-// prefix's sub-table, which is read by a predicated load (no branch for the few lanes that need it).
+// How the lanes address the tables of all streams of a launch; the same for each, so that it takes four registers.
+struct Lookup {
+  uint32_t l1lane;      // shared address of this lane's copy of first-level entry 0 of the first stream
+  uint32_t first_long;  // first-level prefixes from this one on are looked up in the second level
+  uint32_t sub_shift;   // their prefix and sub-table bits together: hi >> sub_shift
+  uint32_t sub;         // shared address of the second level less what first_long adds to an index (wraps around)
+};
+
+// Table lookup of the code at the top of `hi`: {representative, length}, length kLongCode if the tables do not resolve
+// it. Codes are canonical, so the prefixes of longer codes are the last ones: a compare tells which level a lane reads, and
+// one load serves both. (With the second level's address in the first-level entry, its load waited for the first one in
+// nearly every warp. 1.3 G elements and four streams: 3.40 -> 3.31 ms, one chunk and one stream 19.4 -> 17.3 us.)
 // Written in PTX so that index scaling and base addition stay multiply-adds (they then run beside the
 // shifts and compares instead of competing with them for the integer pipe).
 template <int OFFSET>
-__device__ __forceinline__ uint2 lookup_code(uint32_t hi, uint32_t l1lane, uint32_t sub_shift) {
+__device__ __forceinline__ uint2 lookup_code(uint32_t hi, const Lookup& T) {
   uint2 ent;
   asm("{\n\t"
       ".reg .u32 t, a;\n\t"
       ".reg .pred q;\n\t"
-      "shr.u32 t, %2, %4;\n\t"
-      "mad.lo.u32 a, t, %5, %3;\n\t"
-      "ld.shared.v2.u32 {%0,%1}, [a+%8];\n\t"
-      "setp.gt.u32 q, %1, 63;\n\t"
-      "shr.u32 t, %2, %7;\n\t"         // prefix and sub-table index together: the entry's address allows for the prefix
-      "mad.lo.u32 a, t, 8, %0;\n\t"
-      "@q ld.shared.v2.u32 {%0,%1}, [a];\n\t"
+      "shr.u32 t, %2, %7;\n\t"
+      "setp.ge.u32 q, t, %4;\n\t"
+      "mad.lo.u32 a, t, %8, %3;\n\t"
+      "@q shr.u32 t, %2, %5;\n\t"
+      "@q mad.lo.u32 a, t, 8, %6;\n\t"
+      "ld.shared.v2.u32 {%0,%1}, [a+%9];\n\t"
       "}"
       : "=&r"(ent.x), "=&r"(ent.y)
-      : "r"(hi), "r"(l1lane), "n"(32 - kL1Bits), "n"(kL1Rep * 8), "n"(kL1Bits), "r"(sub_shift), "n"(OFFSET));
+      : "r"(hi), "r"(T.l1lane), "r"(T.first_long), "r"(T.sub_shift), "r"(T.sub), "n"(32 - kL1Bits), "n"(kL1Rep * 8), "n"(OFFSET));
   return ent;
 }
 
@@ -372,13 +374,10 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
   const int rem = PARTIAL ? (int)(n - c * kChunkElems) - 4 * (int)lane : 0;  // elements from this lane's first slot on
   const uint32_t steps = PARTIAL ? (uint32_t)(n - c * kChunkElems + 127) / 128 : kSteps;
   // the streams' tables follow each other at 2 * kTableBytes: one base address, the rest as immediate offsets
-  const uint32_t l1lane = S[0].l1_addr | ((lane & (kL1Rep - 1)) * 8u);
-  uint32_t sub_shift[KS];
+  const Lookup T{S[0].l1_addr | ((lane & (kL1Rep - 1)) * 8u), (1u << kL1Bits) - S[0].nsub, 32 - kL1Bits - S[0].sub_bits,
+                 S[0].l1_addr + kTableBytes - ((((1u << kL1Bits) - S[0].nsub) << S[0].sub_bits) << 3)};
 #pragma unroll
-  for (int s = 0; s < KS; ++s) {
-    bits[s].seek(W[s], start[s]);
-    sub_shift[s] = 32 - kL1Bits - S[s].sub_bits;
-  }
+  for (int s = 0; s < KS; ++s) bits[s].seek(W[s], start[s]);
   const uint64_t e0 = c * kChunkElems + 4 * lane;
   float4 b = load_row<PARTIAL>(base + e0, rem);
   // With one stream a step is short, and one row of base in registers ahead of its use leaves too few bytes in flight
@@ -417,16 +416,16 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
     for (int h = 0; h < 2; ++h) {
       uint2 ea[KS], eb[KS];
       uint32_t h1[KS];
-      ea[0] = lookup_code<0>(bits[0].hi, l1lane, sub_shift[0]);
-      if (KS > 1) ea[1 % KS] = lookup_code<2 * kTableBytes>(bits[1 % KS].hi, l1lane, sub_shift[1 % KS]);
-      if (KS > 2) ea[2 % KS] = lookup_code<4 * kTableBytes>(bits[2 % KS].hi, l1lane, sub_shift[2 % KS]);
-      if (KS > 3) ea[3 % KS] = lookup_code<6 * kTableBytes>(bits[3 % KS].hi, l1lane, sub_shift[3 % KS]);
+      ea[0] = lookup_code<0>(bits[0].hi, T);
+      if (KS > 1) ea[1 % KS] = lookup_code<2 * kTableBytes>(bits[1 % KS].hi, T);
+      if (KS > 2) ea[2 % KS] = lookup_code<4 * kTableBytes>(bits[2 % KS].hi, T);
+      if (KS > 3) ea[3 % KS] = lookup_code<6 * kTableBytes>(bits[3 % KS].hi, T);
 #pragma unroll
       for (int s = 0; s < KS; ++s) h1[s] = __funnelshift_l(0u, bits[s].hi, ea[s].y);  // hi << length (mod 32)
-      eb[0] = lookup_code<0>(h1[0], l1lane, sub_shift[0]);
-      if (KS > 1) eb[1 % KS] = lookup_code<2 * kTableBytes>(h1[1 % KS], l1lane, sub_shift[1 % KS]);
-      if (KS > 2) eb[2 % KS] = lookup_code<4 * kTableBytes>(h1[2 % KS], l1lane, sub_shift[2 % KS]);
-      if (KS > 3) eb[3 % KS] = lookup_code<6 * kTableBytes>(h1[3 % KS], l1lane, sub_shift[3 % KS]);
+      eb[0] = lookup_code<0>(h1[0], T);
+      if (KS > 1) eb[1 % KS] = lookup_code<2 * kTableBytes>(h1[1 % KS], T);
+      if (KS > 2) eb[2 % KS] = lookup_code<4 * kTableBytes>(h1[2 % KS], T);
+      if (KS > 3) eb[3 % KS] = lookup_code<6 * kTableBytes>(h1[3 % KS], T);
 #pragma unroll
       for (int s = 0; s < KS; ++s) {
         x[2 * h] = __fadd_rn(x[2 * h], __uint_as_float(ea[s].x));
@@ -460,10 +459,10 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
           uint2 ent[KS];
 #pragma unroll
           for (int s = 0; s < KS; ++s) bits[s].refill(W[s]);
-          ent[0] = lookup_code<0>(bits[0].hi, l1lane, sub_shift[0]);
-          if (KS > 1) ent[1 % KS] = lookup_code<2 * kTableBytes>(bits[1 % KS].hi, l1lane, sub_shift[1 % KS]);
-          if (KS > 2) ent[2 % KS] = lookup_code<4 * kTableBytes>(bits[2 % KS].hi, l1lane, sub_shift[2 % KS]);
-          if (KS > 3) ent[3 % KS] = lookup_code<6 * kTableBytes>(bits[3 % KS].hi, l1lane, sub_shift[3 % KS]);
+          ent[0] = lookup_code<0>(bits[0].hi, T);
+          if (KS > 1) ent[1 % KS] = lookup_code<2 * kTableBytes>(bits[1 % KS].hi, T);
+          if (KS > 2) ent[2 % KS] = lookup_code<4 * kTableBytes>(bits[2 % KS].hi, T);
+          if (KS > 3) ent[3 % KS] = lookup_code<6 * kTableBytes>(bits[3 % KS].hi, T);
 #pragma unroll
           for (int s = 0; s < KS; ++s) {
             if (ent[s].y > 63u) ent[s] = make_uint2(long_code<STAGED>(bits[s], S[s], W[s], status), 0u);  // consumed
@@ -593,6 +592,18 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
       return;
     }
   }
+  // Prefixes that any of the streams resolves in the second level are looked up there in all of them, in sub-tables as
+  // deep as their number allows: the lookup's addressing is then the same for all streams.
+  if (threadIdx.x < KS) {
+    uint32_t most = 0;
+#pragma unroll
+    for (int s = 0; s < KS; ++s) most = max(most, S[s].misses);
+    uint32_t sub_bits = kSubBitsMax;
+    while (sub_bits > kSubBitsMin && most > (kTableBytes >> (sub_bits + 3))) sub_bits -= 1;
+    S[threadIdx.x].nsub = most;
+    S[threadIdx.x].sub_bits = sub_bits;
+  }
+  __syncthreads();
   fill_tables<KS>(S, tables);
   __syncthreads();
 
