@@ -17,8 +17,8 @@
 //    at index*16 + lane%16): a 64-bit shared load is served half a warp at a time, so the 16 lanes of
 //    a half-warp always hit 16 different bank pairs although their indices are data dependent.
 //    Codes are canonical, so the 6-bit prefixes of longer codes are the last ones; from the first of them on a lane
-//    reads the second level instead, indexed by up to 10 more bits (the same load, no branch), which resolves codes of
-//    up to 16 bits; still longer codes are found by a canonical search behind a warp vote.
+//    reads the second level instead, indexed by up to 9 more bits (the same load, no branch), which resolves codes of
+//    up to 15 bits; still longer codes are found by a canonical search behind a warp vote.
 //  * A lane keeps a 64-bit bit buffer per stream and tops it up with one predicated word load before
 //    every fourth symbol; a lane whose four codes take more bits than it held does the step again.
 //
@@ -45,13 +45,14 @@ template <int KS>
 constexpr int kDecCtas = KS == 1 ? 2 : 1;
 constexpr int kL1Bits = 6;
 constexpr int kL1Rep = 16;
-// Second level: one sub-table per 6-bit prefix that belongs to longer codes, all of one depth: the next 10 bits if a
-// single prefix needs one (8 KB hold one table of 1024 entries; a Huffman code's long codes usually hang under one
-// prefix), down to the next 4 bits if every prefix does (64 tables of 16 entries).
-constexpr int kSubBitsMax = 10;
+// Second level: one sub-table per 6-bit prefix that belongs to longer codes, all of one depth: the next 9 bits if at most
+// two prefixes need one (8 KB hold two tables of 512 entries; a Huffman code's long codes usually hang under one
+// prefix), down to the next 4 bits if every prefix does (64 tables of 16 entries). Not 10 bits: two codes of 16 are 32,
+// and the bit buffer is shifted once per pair, by their sum modulo 32.
+constexpr int kSubBitsMax = 9;
 constexpr int kSubBitsMin = 4;
 constexpr int kL2Bits = kL1Bits + kSubBitsMax;     // longest code the two table levels resolve
-static_assert(kL2Bits <= 16, "the second code of a pair is looked up in the 32-bit upper word behind the first");
+static_assert(2 * kL2Bits < 32, "a pair of codes leaves the bit buffer with one shift of a 32-bit word");
 static_assert(((1 << kL1Bits) << (kSubBitsMin + 3)) <= 8192, "at the smallest depth every prefix gets a sub-table");
 // Length field of a table entry that does not resolve its code. As a length it takes the bit count far below zero,
 // which is how the hot loop notices: a step subtracts at most four of them per stream, and 1..4 times 2^29 (less a
@@ -345,13 +346,13 @@ __device__ __forceinline__ uint32_t long_code(LaneBits<STAGED>& B, const StreamS
 //
 // The loop body is straight-line code. A lane tops its bit buffers up once per step and then decodes its four
 // codes per stream from the upper word alone, two at a time (the second lookup takes the first code's length,
-// the buffer is shifted once per pair). Two things can go wrong for a lane in a step, both rare: a code longer
+// the buffer is shifted once per pair, by 30 bits at most). Two things can go wrong for a lane in a step, both rare: a code longer
 // than the tables resolve, and four codes that take more bits than the buffer held (32 are guaranteed, four
-// table-resolved codes can take 64). Both show as a negative bit count at the end of the step: the marker of an
+// table-resolved codes can take 60). Both show as a negative bit count at the end of the step: the marker of an
 // unresolved code is a huge length, and a lookup on too few valid bits always overdraws, because no code is a
 // prefix of another. One warp vote per step finds them, and the flagged lanes decode the step again from where it
 // started, one code at a time with a top-up before each (a top-up makes 32 bits valid, a table-resolved code
-// takes at most 16). Whatever the quick pass did to their buffers in
+// takes at most 15). Whatever the quick pass did to their buffers in
 // between stays inside the staged chunk (a top-up moves one word per step) and is discarded.
 // PARTIAL: the vector's last chunk. Only the steps that hold elements are visited, and of a step's four slots only
 // the first `have` are loaded, checked and stored. (The lane's codes end with its last element, so what the quick pass
