@@ -273,7 +273,7 @@ int lc_merge(const float* base, const void* const* streams, const uint64_t* stre
              int nbits, void* stream, uint64_t stream_capacity, float* scratch, void* workspace,
              uint64_t workspace_bytes, lc_cuda_stream_t cs);
 
-/* Copies a stream's header to the host. `stream` DEVICE, `info` HOST. Waits for `cs`. */
+/* Copies a stream's header to the host. `stream` DEVICE, at any address and on any device, `info` HOST. Waits for `cs`. */
 int lc_stream_info(const void* stream, lc_info* info, lc_cuda_stream_t cs);
 
 /* Waits for `cs`, then returns the status word of the last call that used `workspace`. */
