@@ -279,6 +279,15 @@ int lc_stream_info(const void* stream, lc_info* info, lc_cuda_stream_t cs);
 /* Waits for `cs`, then returns the status word of the last call that used `workspace`. */
 int lc_last_status(const void* workspace, lc_cuda_stream_t cs);
 
+/* lc_last_status and, if `stream` is not NULL, lc_stream_info of the stream that the call wrote, with one wait: for the
+ * caller that has enqueued the call on `cs` and needs its outcome. The device of `workspace` and `stream` must be current,
+ * as it was for that call; workspace 256-byte, stream and page 16-byte aligned. Returns the status word (the header
+ * means something only if that is LC_OK) or LC_ERR_ARG / LC_ERR_CUDA.
+ * page   HOST, NULL or LC_WAIT_PAGE_BYTES of page-locked memory (cudaHostAlloc, cudaHostRegister) that no other call uses
+ *        meanwhile: the outcome then arrives there from a kernel, which is faster than a copy of each part. */
+#define LC_WAIT_PAGE_BYTES 128
+int lc_wait(const void* workspace, const void* stream, lc_info* info, void* page, lc_cuda_stream_t cs);
+
 /*
  * Host-buffer variants: the same two passes (Algorithm 1 steps 4-6 and step 7) for callers whose state lives
  * in host memory (pinned memory makes the copies asynchronous). Every transfer is part of the call: base,

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import threading
 
 import torch
 
@@ -15,12 +16,13 @@ from . import build as _build
 
 OK, ERR_ARG, ERR_CAPACITY, ERR_NONFINITE, ERR_FORMAT, ERR_MISMATCH, ERR_TIMEOUT, ERR_CUDA, ERR_RANGE = 0, -1, -2, -3, -4, -5, -6, -7, -8
 MAX_CHAIN = 8
+WAIT_PAGE_BYTES = 128
 
 SYMBOLS = (
     "lc_version", "lc_strerror", "lc_stream_bound", "lc_workspace_bytes", "lc_compress", "lc_compress_update", "lc_compress_timed",
     "lc_recover", "lc_compress_opt", "lc_compress_cached",
     "lc_segments_layout", "lc_compress_segments", "lc_recover_segments", "lc_debug_compress_wait", "lc_merge", "lc_compress_async", "lc_shard_stats", "lc_shard_encode",
-    "lc_stream_info", "lc_last_status", "lc_host_arena_bytes", "lc_compress_host", "lc_recover_host",
+    "lc_stream_info", "lc_last_status", "lc_wait", "lc_host_arena_bytes", "lc_compress_host", "lc_recover_host",
     "lc_debug_bins", "lc_debug_codes", "lc_compress_noalloc",
 )
 NOALLOC_MAX_N = 4194304
@@ -81,6 +83,7 @@ def lib():
     L.lc_merge.argtypes = [vp, C.POINTER(vp), C.POINTER(u64), i32, u64, i32, vp, u64, vp, vp, u64, vp]
     L.lc_stream_info.argtypes = [vp, C.POINTER(LCInfo), vp]
     L.lc_last_status.argtypes = [vp, vp]
+    L.lc_wait.argtypes = [vp, vp, C.POINTER(LCInfo), vp, vp]
     L.lc_host_arena_bytes.argtypes = [u64, i32, i32]
     L.lc_host_arena_bytes.restype = u64
     L.lc_compress_host.argtypes = [vp, vp, u64, i32, vp, u64, C.POINTER(u64), vp, u64, vp]
@@ -186,14 +189,19 @@ def stream_info(stream) -> LCInfo:
     return info
 
 
-def _finished(stream, workspace, what) -> int:
-    """Waits for a compress pass on the current stream and returns its stream's size. One read of the header is enough
-    when the pass has succeeded: a pass that fails takes the magic away or never writes the size, and only then is the
-    status word read as well."""
-    info = stream_info(stream)
-    if not info.valid or info.total_bytes == 0:
-        _check(last_status(workspace), what)
-    return info.total_bytes
+_page = threading.local()  # page-locked host memory for lc_wait, from torch's pool and back to it with the thread
+
+
+def _wait(workspace, what, stream=None):
+    """Waits for the call that has just been enqueued on the current stream; raises if its status word is set. Returns
+    the header of ``stream``."""
+    page = getattr(_page, "tensor", None)
+    if page is None:
+        page = _page.tensor = torch.empty(WAIT_PAGE_BYTES, dtype=torch.uint8, pin_memory=True)
+    info = LCInfo()
+    _check(lib().lc_wait(workspace.data_ptr(), None if stream is None else stream.data_ptr(), C.byref(info), page.data_ptr(),
+                         _cs(workspace.device)), what)
+    return info
 
 
 def compress(base, cur, nbits, stream=None, workspace=None, fixed=False, mean=False):
@@ -209,7 +217,7 @@ def compress(base, cur, nbits, stream=None, workspace=None, fixed=False, mean=Fa
         compress_opt_async(base, cur, nbits, stream, workspace, (OPT_FIXED_WIDTH if fixed else 0) | (OPT_MEAN_REP if mean else 0))
     else:
         compress_async(base, cur, nbits, stream, workspace)
-    return stream[: _finished(stream, workspace, "lc_compress (device)")]
+    return stream[: _wait(workspace, "lc_compress (device)", stream).total_bytes]
 
 
 LENGTH_CACHE_BYTES = 262144
@@ -237,7 +245,7 @@ def compress_cached(base, cur, nbits, length_cache, stream=None, workspace=None,
     if workspace is None:
         workspace = alloc_workspace(n, base.device)
     compress_cached_async(base, cur, nbits, stream, workspace, length_cache, tracked_out)
-    return stream[: _finished(stream, workspace, "lc_compress_cached (device)")]
+    return stream[: _wait(workspace, "lc_compress_cached (device)", stream).total_bytes]
 
 
 def segments_layout(seg_begin, nbits):
@@ -272,7 +280,7 @@ def compress_segments(base, cur, seg_begin, nbits, streams=None, workspace=None,
         longest = max([b - a for a, b in zip(seg_begin[:-1], seg_begin[1:])] + [0])
         workspace = alloc_workspace(longest, base.device)
     compress_segments_async(base, cur, seg_begin, nbits, streams, workspace, tracked_out)
-    _check(last_status(workspace), "lc_compress_segments (device)")
+    _wait(workspace, "lc_compress_segments (device)")
     return streams, offsets
 
 
@@ -292,7 +300,7 @@ def recover_segments(base, streams_list, seg_begin, nbits, out=None, workspace=N
     if workspace is None:
         workspace = alloc_workspace(0, base.device)
     recover_segments_async(base, streams_list, seg_begin, nbits, out, workspace)
-    _check(last_status(workspace), "lc_recover_segments (device)")
+    _wait(workspace, "lc_recover_segments (device)")
     return out
 
 
@@ -307,7 +315,7 @@ def compress_update(base, cur, nbits, tracked_out=None, stream=None, workspace=N
     if tracked_out is None:
         tracked_out = torch.empty_like(base)
     compress_update_async(base, cur, nbits, stream, tracked_out, workspace)
-    return stream[: _finished(stream, workspace, "lc_compress_update (device)")], tracked_out
+    return stream[: _wait(workspace, "lc_compress_update (device)", stream).total_bytes], tracked_out
 
 
 def recover_async(base, streams, out, workspace):
@@ -327,7 +335,7 @@ def recover(base, streams, out=None, workspace=None):
     if workspace is None:
         workspace = alloc_workspace(0, base.device)
     recover_async(base, streams, out, workspace)
-    _check(last_status(workspace), "lc_recover (device)")
+    _wait(workspace, "lc_recover (device)")
     return out
 
 
@@ -391,7 +399,7 @@ def shard_encode(base, cur, nbits, whole_stats, workspace, stream=None):
     _check(lib().lc_shard_encode(base.data_ptr(), cur.data_ptr(), n, nbits, whole_stats.data_ptr(), stream.data_ptr(),
                                  stream.numel(), workspace.data_ptr(), workspace.numel(), _cs(base.device)),
            "lc_shard_encode")
-    return stream[: _finished(stream, workspace, "lc_shard_encode (device)")]
+    return stream[: _wait(workspace, "lc_shard_encode (device)", stream).total_bytes]
 
 
 def merge_async(base, streams, nbits, stream, scratch, workspace):
@@ -416,7 +424,7 @@ def merge(base, streams, nbits, stream=None, scratch=None, workspace=None):
     if workspace is None:
         workspace = alloc_workspace(n, base.device)
     merge_async(base, streams, nbits, stream, scratch, workspace)
-    return stream[: _finished(stream, workspace, "lc_merge (device)")]
+    return stream[: _wait(workspace, "lc_merge (device)", stream).total_bytes]
 
 
 def host_arena_bytes(n, nbits, k) -> int:

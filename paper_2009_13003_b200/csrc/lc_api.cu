@@ -26,6 +26,45 @@ Carved carve(void* workspace, const WorkspaceLayout& W) {
   return c;
 }
 
+// The host's form of a header.
+void parse_header(const uint8_t* h, lc_info* info) {
+  auto le = [&](int off, int bytes) {
+    uint64_t v = 0;
+    for (int b = 0; b < bytes; ++b) v |= (uint64_t)h[off + b] << (8 * b);
+    return v;
+  };
+  memset(info, 0, sizeof *info);
+  info->nbits = h[6];
+  info->fixed_width = h[7] & 1u;
+  info->shard = (h[7] >> 1) & 1u;
+  info->cached_lengths = (h[7] >> 2) & 1u;
+  info->mean_rep = (h[7] >> 3) & 1u;
+  info->n = le(8, 8);
+  info->nsym = (uint32_t)le(16, 4);
+  info->max_len = (uint32_t)le(20, 4);
+  info->nchunks = (uint32_t)le(32, 4);
+  info->payload_bits = le(40, 8);
+  info->total_bytes = le(48, 8);
+  info->payload_offset = le(56, 8);
+  info->valid = (h[0] == 'L' && h[1] == 'C' && h[2] == 'C' && h[3] == '1' && le(4, 2) == 1 && (h[7] <= 4 || h[7] == 8) &&
+                 le(24, 4) == kChunkElems && le(28, 2) == kLanes && le(30, 2) == kGroup &&
+                 le(36, 4) == kPayloadAlign)
+                    ? 1
+                    : 0;
+}
+
+// The outcome of a call for lc_wait: a stream's header (unless there is none), then the status word. One kernel that writes
+// both to mapped host memory and one wait: bound by latency. A blocking compress of 61,706 elements takes 34 us with it,
+// 40 us with a copy of each.
+constexpr uint32_t kResultWords = kHeaderBytes / 4 + 1;
+static_assert(kResultWords * 4 <= LC_WAIT_PAGE_BYTES, "size promised by the header");
+
+__global__ void result_kernel(const int32_t* status, const uint32_t* header, uint32_t* page) {
+  const uint32_t i = threadIdx.x;
+  if (i < kHeaderBytes / 4 && header) page[i] = header[i];
+  if (i == kHeaderBytes / 4) page[i] = (uint32_t)*status;
+}
+
 // lc_compress and lc_compress_update: argument checks, then memset + three kernels on `cs`.
 int compress_impl(const float* base, const float* cur, uint64_t n, int nbits, void* stream, uint64_t stream_capacity,
                   float* tracked_out, void* workspace, uint64_t workspace_bytes, const EncodeOptions& opt,
@@ -397,30 +436,29 @@ int lc_stream_info(const void* stream, lc_info* info, lc_cuda_stream_t cs) {
   uint8_t h[kHeaderBytes];
   if (cudaMemcpyAsync(h, stream, kHeaderBytes, cudaMemcpyDeviceToHost, cs) != cudaSuccess) return LC_ERR_CUDA;
   if (cudaStreamSynchronize(cs) != cudaSuccess) return LC_ERR_CUDA;
-  auto le = [&](int off, int bytes) {
-    uint64_t v = 0;
-    for (int b = 0; b < bytes; ++b) v |= (uint64_t)h[off + b] << (8 * b);
-    return v;
-  };
-  memset(info, 0, sizeof *info);
-  info->nbits = h[6];
-  info->fixed_width = h[7] & 1u;
-  info->shard = (h[7] >> 1) & 1u;
-  info->cached_lengths = (h[7] >> 2) & 1u;
-  info->mean_rep = (h[7] >> 3) & 1u;
-  info->n = le(8, 8);
-  info->nsym = (uint32_t)le(16, 4);
-  info->max_len = (uint32_t)le(20, 4);
-  info->nchunks = (uint32_t)le(32, 4);
-  info->payload_bits = le(40, 8);
-  info->total_bytes = le(48, 8);
-  info->payload_offset = le(56, 8);
-  info->valid = (h[0] == 'L' && h[1] == 'C' && h[2] == 'C' && h[3] == '1' && le(4, 2) == 1 && (h[7] <= 4 || h[7] == 8) &&
-                 le(24, 4) == kChunkElems && le(28, 2) == kLanes && le(30, 2) == kGroup &&
-                 le(36, 4) == kPayloadAlign)
-                    ? 1
-                    : 0;
+  parse_header(h, info);
   return LC_OK;
+}
+
+int lc_wait(const void* workspace, const void* stream, lc_info* info, void* page, lc_cuda_stream_t cs) {
+  if (!workspace || !aligned(workspace, 256) || !aligned(stream, 16) || (stream && !info) || !aligned(page, 16)) return LC_ERR_ARG;
+  const Control* ctl = static_cast<const Control*>(workspace);
+  uint32_t words[kResultWords] = {};
+  void* mapped = nullptr;
+  if (page && cudaHostGetDevicePointer(&mapped, page, 0) == cudaSuccess) {
+    const cudaError_t e = launch_kernel(false, result_kernel, 1, 32, 0, cs, &ctl->status, static_cast<const uint32_t*>(stream),
+                                        static_cast<uint32_t*>(mapped));
+    if (e != cudaSuccess || cudaStreamSynchronize(cs) != cudaSuccess) return LC_ERR_CUDA;
+    memcpy(words, page, sizeof words);
+  } else {
+    if (page) (void)cudaGetLastError();  // not page-locked memory: that error was this call's own
+    if (cudaMemcpyAsync(words + kHeaderBytes / 4, &ctl->status, sizeof(int32_t), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
+        (stream && cudaMemcpyAsync(words, stream, kHeaderBytes, cudaMemcpyDeviceToHost, cs) != cudaSuccess) ||
+        cudaStreamSynchronize(cs) != cudaSuccess)
+      return LC_ERR_CUDA;
+  }
+  if (stream) parse_header(reinterpret_cast<const uint8_t*>(words), info);
+  return (int32_t)words[kHeaderBytes / 4];
 }
 
 int lc_last_status(const void* workspace, lc_cuda_stream_t cs) {
