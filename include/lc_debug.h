@@ -47,6 +47,13 @@ int lc_debug_compress_wait(const float* base, const float* cur, uint64_t n, int 
                            uint64_t stream_capacity, void* workspace, uint64_t workspace_bytes, uint32_t spin_limit,
                            uint32_t first_ticket, lc_cuda_stream_t cs);
 
+/*
+ * How one launch of lc_recover_segments (at most 160 segments) is dealt out to CTAs of `warps` warps on a device that holds
+ * `slots` of them at once: segment i is decoded by the CTAs cta_begin[i] .. cta_begin[i + 1] - 1 (HOST, nseg + 1 entries).
+ * Returns the number of CTAs, 0 on bad arguments. Needs no device.
+ */
+uint32_t lc_debug_split_segments(const uint64_t* seg_begin, int nseg, uint32_t warps, uint32_t slots, uint32_t* cta_begin);
+
 #ifdef __cplusplus
 }
 #endif

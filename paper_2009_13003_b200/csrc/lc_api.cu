@@ -648,4 +648,14 @@ int lc_debug_codes(const void* workspace, uint32_t* len, uint64_t* code, lc_cuda
   return LC_OK;
 }
 
+uint32_t lc_debug_split_segments(const uint64_t* seg_begin, int nseg, uint32_t warps, uint32_t slots, uint32_t* cta_begin) {
+  if (!segments_ok(seg_begin, nseg) || nseg > (int)kSegBatch || warps == 0 || slots == 0 || !cta_begin) return 0;
+  SegBatch batch = {};
+  batch.nseg = (uint32_t)nseg;
+  for (int i = 0; i <= nseg; ++i) batch.elem_begin[i] = seg_begin[i];
+  const uint32_t ctas = split_segments(batch, warps, slots);
+  memcpy(cta_begin, batch.cta_begin, sizeof(uint32_t) * ((uint32_t)nseg + 1));
+  return ctas;
+}
+
 }  // extern "C"

@@ -251,6 +251,8 @@ struct SegBatch {
   uint64_t elem_begin[kSegBatch + 1];
   uint64_t stream_begin[kSegBatch + 1]; // segment i's stream has the bytes up to stream_begin[i + 1]
 };
+// Fills in cta_begin for CTAs of `warps` warps, `slots` of which the device holds at once; returns their number.
+uint32_t split_segments(SegBatch& batch, uint32_t warps, uint32_t slots);
 // Decodes every segment's k <= 4 streams onto its part of base, in one launch; second: later streams of the same chains.
 // The streams of segment i start at streams[j] + stream_begin[i].
 cudaError_t launch_decode_segments(const float* base, const uint8_t* const* streams, int k, SegBatch& batch, int nbits,

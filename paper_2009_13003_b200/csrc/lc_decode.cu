@@ -777,28 +777,65 @@ cudaError_t launch_segments_ks(const float* base, const uint8_t* const* streams,
   if (e != cudaSuccess) return e;
   DecodeStreams buffers;
   for (int s = 0; s < 4; ++s) buffers.ptr[s] = s < KS ? streams[s] : nullptr, buffers.bytes[s] = 0;
-  // Chunks per CTA: one per warp while all CTAs fit on the device at once, else as many more as it takes for that
-  // (a second wave of CTAs would cost their preparation again and leave the SMs idle at its end).
-  const uint64_t slots = (uint64_t)sh.sms * sh.per_sm;
-  uint64_t ctas = 0;
-  for (uint64_t per_cta = sh.warps;; per_cta += sh.warps) {
-    ctas = 0;
-    uint64_t longest = 0;
-    for (uint32_t i = 0; i < batch.nseg; ++i) {
-      const uint64_t chunks = (batch.elem_begin[i + 1] - batch.elem_begin[i] + kChunkElems - 1) / kChunkElems;
-      batch.cta_begin[i] = (uint32_t)ctas;
-      ctas += chunks ? (chunks + per_cta - 1) / per_cta : 1;  // an empty segment's stream is validated too
-      longest = chunks > longest ? chunks : longest;
-    }
-    if (ctas <= slots || per_cta >= longest) break;
-  }
-  batch.cta_begin[batch.nseg] = (uint32_t)ctas;
-  decode_segments_kernel<KS><<<(unsigned)ctas, sh.warps * 32, sh.dyn, cs>>>(base, buffers, out, status, second ? 1u : 0u, sh.stage,
+  const uint32_t ctas = split_segments(batch, sh.warps, sh.sms * sh.per_sm);
+  decode_segments_kernel<KS><<<ctas, sh.warps * 32, sh.dyn, cs>>>(base, buffers, out, status, second ? 1u : 0u, sh.stage,
                                                                            batch);
   return cudaGetLastError();
 }
 
 }  // namespace
+
+// How the CTAs are dealt out: every one takes up to r rounds (a chunk per warp) of one segment, the same r for all. While
+// all CTAs fit on the device at once, the launch takes as long as the preparation and r rounds, so the smallest such r is
+// the best of those. But every segment takes a CTA of its own, however small: with about as many segments as slots that r
+// grows to the largest segment's whole length. So the smaller r, which take several waves, are weighed against it by the
+// bound for work dealt out in order, (all preparations and rounds) / slots + the longest CTA's. 159 layers of up to 12,000
+// values and one of 25 M: 131 us with two streams and 153 with four, with one wave in every case 5177 and 8507; 130 layers,
+// 30 of them of 2.5 M: 191 and 256 us, with one wave 516 and 833. One wave that is nearly even stays.
+uint32_t split_segments(SegBatch& batch, uint32_t warps, uint32_t slots) {
+  constexpr double kPrepare = 0.5;  // of a round's time: 8 to 10 us beside 15 to 20
+  uint32_t rounds_of[kSegBatch], longest = 1, all = 0;  // 2^20 chunks a segment at most
+  for (uint32_t i = 0; i < batch.nseg; ++i) {
+    const uint32_t chunks = (uint32_t)((batch.elem_begin[i + 1] - batch.elem_begin[i] + kChunkElems - 1) / kChunkElems);
+    rounds_of[i] = chunks ? (chunks + warps - 1) / warps : 1;  // an empty segment's stream is validated too
+    all += rounds_of[i];
+    longest = max(longest, rounds_of[i]);
+  }
+  const auto ctas_with = [&](uint32_t r) {
+    uint32_t ctas = 0;
+    for (uint32_t i = 0; i < batch.nseg; ++i) ctas += (rounds_of[i] + r - 1) / r;
+    return ctas;
+  };
+  const auto time_of = [&](uint32_t r) {
+    const uint32_t ctas = ctas_with(r);
+    const double one = kPrepare + r;
+    return ctas <= slots ? one : (ctas * kPrepare + all) / slots + one;
+  };
+  // the smallest r of one wave, or `longest` if there is none; `least` rounds would fill it evenly
+  const uint32_t least = min(longest, (all + slots - 1) / slots);
+  uint32_t lo = least, fit = least;
+  while (fit < longest && ctas_with(fit) > slots) lo = fit + 1, fit = min(longest, 2 * fit);
+  while (lo < fit) {
+    const uint32_t mid = (lo + fit) / 2;
+    if (ctas_with(mid) <= slots) fit = mid;
+    else lo = mid + 1;
+  }
+  uint32_t best = fit;
+  if (fit > least + 1) {  // no split takes less than `least` rounds and one more
+    double shortest = time_of(fit);
+    for (uint32_t r = 1; r < fit; r += (r + 3) / 4) {
+      const double t = time_of(r);
+      if (t < shortest) shortest = t, best = r;
+    }
+  }
+  uint32_t ctas = 0;
+  for (uint32_t i = 0; i < batch.nseg; ++i) {
+    batch.cta_begin[i] = ctas;
+    ctas += (rounds_of[i] + best - 1) / best;
+  }
+  batch.cta_begin[batch.nseg] = ctas;
+  return ctas;
+}
 
 cudaError_t launch_decode_segments(const float* base, const uint8_t* const* streams, int k, SegBatch& batch, int nbits,
                                    float* out, int32_t* status, bool second, cudaStream_t cs) {
