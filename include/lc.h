@@ -161,8 +161,8 @@ int lc_compress_opt(const float* base, const float* cur, uint64_t n, int nbits, 
  * workspace     as for lc_compress, of lc_workspace_bytes(longest segment) bytes; one status word for the call: the
  *               first failure of any segment stays in it (lc_last_status), and the segments after a failed one are
  *               left without a valid stream (compress) or with unspecified output (recover).
- * Up to 128 segments (compress; as many of them as the workspace holds the statistics of) or 160 (recover) go through
- * one set of launches together: this is for models of tens to thousands of layers, not for millions of tiny tensors.
+ * Up to 128 segments (compress; as many of them as the workspace holds the statistics of, but one of more than some 40
+ * million elements by itself) or 160 (recover) go through one set of launches together: this is for models of tens to thousands of layers, not for millions of tiny tensors.
  * After LC_ERR_TIMEOUT of a segment, tracked_out is unspecified as a whole.
  */
 #define LC_MAX_SEGMENTS 65536

@@ -284,14 +284,26 @@ int lc_compress_segments(const float* base, const float* cur, const uint64_t* se
   Control* ctl = static_cast<Control*>(workspace);
   uint8_t* scratch = static_cast<uint8_t*>(workspace) + kScratch;
   const uint64_t capacity = (workspace_bytes - kScratch) & ~15ull;
+  const uint64_t large = tracked_out ? kSegLargeTracked : kSegLarge;
   SegGroup g;
   uint64_t off = 0;
   for (int i = 0; i < nseg;) {
     const bool first_group = i == 0;
+    if (seg_begin[i + 1] - seg_begin[i] > large) {
+      const uint64_t lo = seg_begin[i], ni = seg_begin[i + 1] - lo, slot = align_up(lc_stream_bound(ni, nbits), 256);
+      const int rc = compress_impl(base + lo, cur + lo, ni, nbits, static_cast<uint8_t*>(streams) + off, slot,
+                                   tracked_out ? tracked_out + lo : nullptr, workspace, workspace_bytes, EncodeOptions(), cs,
+                                   /*keep_status=*/!first_group);
+      if (rc != LC_OK) return rc;
+      off += slot;
+      ++i;
+      continue;
+    }
     g.first = (uint32_t)i;
     uint32_t blocks = 0, tiles = 0;
     for (g.nseg = 0; g.nseg < kSegGroup && i < nseg; ++g.nseg, ++i) {
       const uint64_t ni = seg_begin[i + 1] - seg_begin[i];
+      if (ni > large) break;
       const bool small = ni <= kChunkElems;
       const uint32_t t = small ? 0 : (uint32_t)((ni + kEncWarps * kChunkElems - 1) / (kEncWarps * kChunkElems));
       if (!small && sizeof(SegBlock) * (blocks + 1) + 8ull * (tiles + t) > capacity) break;

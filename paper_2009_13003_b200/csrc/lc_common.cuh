@@ -216,6 +216,13 @@ struct DecodeStreams {
 // A group of segments goes through three launches (statistics, tables, encode). Passed by value, within the 4 KB that
 // kernel parameters may take.
 constexpr uint32_t kSegGroup = 128;
+// Larger segments go through the passes for one vector (four launches, which end the group before them): those write a key
+// plane once, the group's encode reads base and cur a second time, and what is much larger than the L2 comes from memory
+// again: 16.5 bytes per element against 10.5, or with a tracked state 20.5 against 18.5. So the line lies higher with one.
+// Measured (4 bits, us in the group / by itself): without a tracked state 8 segments of 32 M 777 / 711, one of 32 M among
+// 120 small ones 171 / 187, of 48 M 263 / 221, 2 of 128 M 783 / 552; with one 8 of 32 M 954 / 1011, 4 of 64 M 963 / 900, one of
+// 64 M among small ones 323 / 329, 2 of 128 M 947 / 834.
+constexpr uint64_t kSegLarge = 40ull << 20, kSegLargeTracked = 64ull << 20;
 struct SegGroup {
   uint32_t nseg;
   uint32_t first;                        // number of the first of them among the segments of the call

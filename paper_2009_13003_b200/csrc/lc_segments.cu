@@ -10,7 +10,8 @@
 //   3. segments_encode_kernel: one CTA per tile of 8 chunks of the larger segments.
 // There is no key plane in global memory (the workspace is sized for the longest segment only): the encode kernel forms
 // the keys again from base and cur, which for models of this size are still in the L2, and keeps them in shared memory,
-// and it writes the tracked state from the registers it has base in.
+// and it writes the tracked state from the registers it has base in. (Segments far larger than the L2 are not brought here:
+// kSegLarge.)
 #include "lc_encode_bits.cuh"
 #include "lc_small.cuh"
 #include "lc_stats.cuh"
@@ -61,6 +62,8 @@ segments_stats_kernel(const float* base, const float* __restrict__ cur, Control*
   }
   wait_previous();
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicMax(&ctl->seg_fail, ~(group.first + s));
+  // a segment before this group that went through the passes for one vector has failed: all of the group are behind it
+  if (group.first > 0 && blockIdx.x == 0 && threadIdx.x == 0 && ctl->status != 0) atomicMax(&ctl->seg_fail, ~(group.first - 1));
 }
 
 __global__ void __launch_bounds__(kTableThreads)
@@ -410,10 +413,9 @@ cudaError_t launch_compress_segments(Control* ctl, SegBlock* blocks, unsigned lo
     if (ctas <= slots || per_cta >= longest) break;
   }
   group.cta_begin[group.nseg] = (uint32_t)ctas;
-  // overlapped launches, the first behind the caller's clear kernel
-  cudaError_t e = cudaSuccess;
-  if (ctas > 0)
-    e = launch_kernel(true, segments_stats_kernel, (unsigned)ctas, kStatsThreads, kStatsSmem, cs, base, cur, ctl, blocks, group);
+  // overlapped launches, the first behind the caller's clear kernel; one CTA at least, which looks at the status word
+  cudaError_t e = launch_kernel(true, segments_stats_kernel, (unsigned)(ctas > 0 ? ctas : 1), kStatsThreads, kStatsSmem, cs, base, cur,
+                                ctl, blocks, group);
   if (e == cudaSuccess)
     e = launch_kernel(true, segments_table_kernel, group.nseg, kTableThreads, sizeof(small::SmallShared<1>), cs, base, cur, ctl, blocks,
                       nbits, streams, tracked_out, group);
