@@ -42,9 +42,14 @@ namespace {
 using namespace enc;
 
 constexpr int kEncThreads = kEncWarps * 32;
-// 44 KB of dynamic shared memory per CTA (four CTAs per SM, beside 8 KB of tables), split evenly between the warps that work:
-// all 8 while an average chunk fits half of a 5.5 KB share (column matrix + chunk image), else 4, 2 or 1.
-constexpr uint32_t kEncSmem = 44 * 1024;
+// 48 KB of dynamic shared memory per CTA (four CTAs per SM, beside 7 KB of tables), split evenly between the warps that work:
+// all 8 while an average chunk fits half of a 6 KB share (column matrix + chunk image), else 4, 2 or 1. Up to 5.1 bits per
+// element that is all 8; with 44 KB it was up to 4.7, and 134 M elements in codes of a fixed 5 bits took 362 us instead of 322
+// (with the tracked state 498 instead of 433).
+constexpr uint32_t kEncSmem = 48 * 1024;
+// bytes of a share's half that an average chunk of `avg` bytes needs: 15 % more, for the lanes and chunks above the average
+__host__ __device__ constexpr uint64_t share_need(uint64_t avg) { return avg + avg / 7 + 64; }
+static_assert(share_need(kChunkElems * 5 / 8) <= kEncSmem / kEncWarps / 2, "codes of 5 bits throughout are coded by all warps");
 constexpr int kUpdRows = 4;  // rows of base in flight per warp in the kernel that also writes the tracked state
 constexpr uint32_t kUpdSmem = kEncWarps * kUpdRows * 512;  // its ring, behind the kEncSmem bytes of coding areas
 constexpr int kLookBack = 8;  // look-back sub-windows of 32 tile descriptors read per round
@@ -63,7 +68,6 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   __shared__ Tables tb;
   __shared__ uint32_t s_chunk_bytes[2][kEncWarps];  // [half][warp]: the pending tile and the one being coded
   __shared__ uint32_t s_tile;
-  __shared__ uint32_t s_lane_start[2][kEncThreads];  // only for chunks too large for the image area
   __shared__ unsigned long long s_tile_base, s_tile_end;
   __shared__ int s_abort;
   __shared__ uint32_t s_arrived[2];  // warps that have coded their chunk of the tile in this half
@@ -97,8 +101,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   uint16_t* lane_index = reinterpret_cast<uint16_t*>(stream + L.lane_index_off);
   uint8_t* payload = stream + L.payload_off;
   // how many warps work: as many as can each hold an average chunk (plus 15 %) twice
-  const uint64_t avg_bytes = nchunks ? ctl->payload_bits / 8 / nchunks : 0;
-  const uint64_t need = avg_bytes + avg_bytes / 7 + 64;
+  const uint64_t need = share_need(nchunks ? ctl->payload_bits / 8 / nchunks : 0);
   uint32_t active = kEncWarps;
   while (active > 1 && need > kEncSmem / active / 2) active >>= 1;
   const uint32_t image_words = kEncSmem / active / 8;  // half of the warp's share, in words
@@ -117,7 +120,8 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   // with hundreds of tiles in flight some predecessor is always late; looking back right after coding made the
   // whole CTA wait for that straggler for a third of its time. One coding phase later the predecessors' sizes
   // are there. The pending tile lives in the warps' image areas, which coding (phase A) does not touch.
-  // What the pending tile needs later is kept in shared memory (its chunk sizes, the lanes' start bits) or
+  // What the pending tile needs later is kept in shared memory (its chunk sizes; the lanes' start bits, in the image area
+  // of a chunk that has no image because it is too large) or
   // recomputed from its number: phase A has no registers to spare.
   bool p_have = false;
   uint32_t p_tile = 0, p_buf = 0;
@@ -206,7 +210,6 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     const uint32_t chunk_bits = __shfl_sync(0xffffffffu, incl, 31);
     const uint32_t chunk_bytes = valid ? (uint32_t)align_up((chunk_bits + 7) / 8, kPayloadAlign) : 0u;
     const bool staged = chunk_bytes <= image_words * 4;
-    if (!staged) s_lane_start[buf][tid] = lane_start;
     // The warp that gets here first looks up the pending tile's offset (D) while the others are still coding.
     uint32_t arrival = 0;
     if (lane == 0) {
@@ -310,7 +313,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
           for (uint32_t k = lane; k < p_chunk_bytes / 16; k += 32) dst4[k] = make_uint4(0, 0, 0, 0);
           __threadfence_block();
           __syncwarp();
-          chunk_slow(ctl->enc, ks, p_c, lane, n, reinterpret_cast<uint32_t*>(dst4), s_lane_start[p_buf][tid]);
+          chunk_slow(ctl->enc, ks, p_c, lane, n, reinterpret_cast<uint32_t*>(dst4), image[lane]);
         }
       }
       if (p_tile == ntiles - 1 && tid == 0) {
@@ -409,6 +412,8 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
       } else {
         chunk_slow(ctl->enc, ks, c, lane, n, image, lane_start);
       }
+    } else if (valid) {
+      image[lane] = lane_start;
     }
     __syncwarp();
     p_have = true;
