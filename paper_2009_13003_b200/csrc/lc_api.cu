@@ -275,7 +275,7 @@ int lc_compress_segments(const float* base, const float* cur, const uint64_t* se
   for (int i = 0; i < nseg; ++i) longest = seg_begin[i + 1] - seg_begin[i] > longest ? seg_begin[i + 1] - seg_begin[i] : longest;
   if (!workspace || !aligned(workspace, 256) || (longest > 0 && (!base || !cur)) || !aligned(base, 16) || !aligned(cur, 16))
     return LC_ERR_ARG;
-  if (tracked_out && (!aligned(tracked_out, 16) || (longest > 0 && tracked_out == cur))) return LC_ERR_ARG;
+  if (tracked_out && longest > 0 && (!aligned(tracked_out, 16) || tracked_out == cur)) return LC_ERR_ARG;  // else unused
   if (workspace_bytes < workspace_layout(longest).total) return LC_ERR_CAPACITY;
   // Of the control block only the words up to `count` are used here; the segments' blocks and scan descriptors take the
   // place of everything behind them. A group is as many segments as the workspace and the kernel parameters hold (one

@@ -75,3 +75,11 @@ def test_no_stream_behind_a_failed_segment(lc, case, failed):
             assert lc.stream_info(streams[offsets[i]:]).valid == (1 if i < min(failed) else 0), "segment %d" % i
     lc.compress_segments(base, cur, begin, 4, streams, ws)
     assert all(lc.stream_info(streams[offsets[i]:]).valid == 1 for i in range(len(SIZES)))
+
+
+def test_empty_segments_take_any_tracked_state(lc):
+    # nothing is written, so the address is not looked at, as in lc_compress_update of an empty vector
+    base = torch.zeros(16, device=DEV)
+    begin = [0, 0, 0]
+    streams, off = lc.compress_segments(base[:0], base[:0], begin, 4, tracked_out=base[1:])
+    assert all(lc.stream_info(streams[o:]).valid == 1 for o in off[:-1])
