@@ -23,6 +23,7 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 METRIC = "compress/recover GB/s of fp32 state on 1 B200, % HBM peak; compression ratio"
+SMALL_MAX_ELEMS = 32 * 4096  # up to here a compress call is one launch
 WORKLOAD = "xfmr1p3b"  # the workload the metric is quoted on; --workload picks another config for reference
 CPU_SAMPLE_ELEMS = 1 << 27  # bounded oracle sample: first 134,217,728 elements of the workload
 FALLBACK_HBM_GBS = 6650.0
@@ -627,8 +628,9 @@ def run_ours(args, rank, world, local_rank):
                   "code_bits_per_element": code_bits, "entropy_bits_per_element": entropy_bits},
         "size_model": size_model,
         "roofline": roofline, "clocks": clocks, "e2e": e2e,
-        # per step: stats, table, encode; a decode kernel per group of up to four streams
-        "gpu_launches": (3 + decode_launches) * args.steps,
+        # per step: clear, stats, table, encode (or one kernel for a small vector); a decode kernel per group of up to
+        # four streams
+        "gpu_launches": ((1 if n <= SMALL_MAX_ELEMS else 4) + decode_launches) * args.steps,
     }
     if world == 1 and not args.no_cpu_baseline:
         result["cpu_baseline"] = oracle_baseline(cfg, n)
