@@ -74,7 +74,7 @@ uint64_t lc_stream_bound(uint64_t n, int nbits);
 /* Bytes of DEVICE scratch lc_compress and lc_recover need for vectors of up to n elements: the control block
  * (status word, bucket statistics of Section 3.1.1, per-bucket code table), one descriptor per chunk for the
  * scan that places the chunks (format section 3.3), and one byte per element for the bucket keys that the
- * statistics pass hands to the encode pass; for lc_recover, the decode tables of the streams of one launch. */
+ * statistics pass hands to the encode pass; for lc_recover, the status word. */
 uint64_t lc_workspace_bytes(uint64_t n);
 
 /*
@@ -202,8 +202,7 @@ int lc_compress_cached(const float* base, const float* cur, uint64_t n, int nbit
  * k             1..LC_MAX_CHAIN.
  * n             elements in base and out; every stream's header must say the same n.
  * out           DEVICE, n fp32, 16-byte aligned; may be the same pointer as base (in-place update).
- * workspace     as for lc_compress; lc_workspace_bytes(0) is enough for any n (the status word and the decode
- *               tables of the streams live there).
+ * workspace     as for lc_compress; lc_workspace_bytes(0) is enough for any n (only the status word lives there).
  * Malformed streams set LC_ERR_FORMAT / LC_ERR_MISMATCH in the status word; `out` is then unspecified
  * but no out-of-bounds access happens.
  */

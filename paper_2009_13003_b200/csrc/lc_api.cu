@@ -278,9 +278,10 @@ int lc_compress_segments(const float* base, const float* cur, const uint64_t* se
   if (tracked_out && longest > 0 && (!aligned(tracked_out, 16) || tracked_out == cur)) return LC_ERR_ARG;  // else unused
   if (workspace_bytes < workspace_layout(longest).total) return LC_ERR_CAPACITY;
   // Of the control block only the words up to `count` are used here; the segments' blocks and scan descriptors take the
-  // place of everything behind them. A group is as many segments as the workspace and the kernel parameters hold (one
-  // always fits: a workspace for n elements has 100 KB more than a block and n elements' descriptors).
+  // place of everything behind them. A group is as many segments as the workspace and the kernel parameters hold. One
+  // always fits: a workspace for n elements has a descriptor per chunk, and more than a block besides.
   constexpr uint64_t kScratch = offsetof(Control, count);
+  static_assert(sizeof(Control) + kSpareRegionBytes >= kScratch + sizeof(SegBlock) + 16, "every group holds a segment");
   Control* ctl = static_cast<Control*>(workspace);
   uint8_t* scratch = static_cast<uint8_t*>(workspace) + kScratch;
   const uint64_t capacity = (workspace_bytes - kScratch) & ~15ull;

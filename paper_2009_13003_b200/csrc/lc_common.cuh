@@ -93,8 +93,9 @@ struct ShardStats {
 static_assert(sizeof(ShardStats) == LC_STATS_BYTES, "size promised by the header");
 static_assert(sizeof(Control) % 256 == 0, "control block must keep the planes 256-byte aligned");
 
-// A region behind the control block whose size does not depend on n. Nothing uses it at present (the decode kernel's
-// CTAs build their tables in shared memory); it stays so that the sizes lc_workspace_bytes returns stay.
+// A region behind the control block whose size does not depend on n. The per-layer compress puts the blocks and scan
+// descriptors of a group of segments over it and what follows: without it a workspace for n elements would not hold those
+// of one segment of n elements. The passes for one vector leave it alone.
 constexpr uint32_t kSpareRegionBytes = 96 * 1024;
 
 struct WorkspaceLayout {

@@ -732,7 +732,6 @@ cudaError_t decode_shape(const void* fn, uint64_t want_stage, uint32_t (&regs_of
 // With as few warps as do them in the same number of rounds all rounds are equally full; with all warps the last one can
 // be nearly empty, and takes nearly as long as the others (11.7 M elements, four streams: 19.3 chunks per SM in rounds of
 // 16 and 3.3, or of 10 and 9.3). Four warps at least: fewer take longer over the tables than they save.
-template <int KS>
 uint32_t balanced_warps(uint64_t chunks, uint64_t ctas, uint32_t most) {
   const uint64_t rounds = (chunks + ctas * most - 1) / (ctas * most);
   if (rounds == 0) return 4;
@@ -757,7 +756,7 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
                                          regs_of, sh);
   if (e != cudaSuccess) return e;
   const uint64_t chunks = chunk_end - chunk_begin, full = (uint64_t)sh.sms * sh.per_sm;
-  const uint32_t warps = balanced_warps<KS>(chunks, full, sh.warps);
+  const uint32_t warps = balanced_warps(chunks, full, sh.warps);
   uint64_t want = (chunks + warps - 1) / warps;
   if (want == 0) want = 1;  // still reports a rejected stream
   const unsigned grid = (unsigned)(want < full ? want : full);

@@ -1,4 +1,4 @@
-// Pieces shared by the two decode kernels: shared-memory access by 32-bit address, asynchronous copies, and a
+// Pieces of the decode kernels (one vector, or the segments of a vector): shared-memory access by 32-bit address, asynchronous copies, and a
 // lane's bit reader over one chunk of one stream (format section 2: a chunk is a string of bits stored in 32-bit
 // words, most significant bit first; lane t's codes are a contiguous run of that string).
 #pragma once
@@ -12,12 +12,6 @@ constexpr uint32_t kSmemPerSm = 227 * 1024;  // usable shared memory of one CTA 
 constexpr uint32_t kOverrunBytes = 512;      // padding behind the last staging area (see LaneBits::refill)
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t load_le(const uint8_t* p, int bytes) {
-  uint64_t v = 0;
-  for (int b = 0; b < bytes; ++b) v |= (uint64_t)p[b] << (8 * b);
-  return v;
-}
 
 // ---- shared-memory access by 32-bit shared address (keeps the hot loops free of generic addressing)
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
