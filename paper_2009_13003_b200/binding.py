@@ -199,7 +199,7 @@ def _wait(workspace, what, stream=None):
     the header of ``stream``."""
     page = getattr(_page, "tensor", None)
     if page is None:
-        page = _page.tensor = torch.empty(WAIT_PAGE_BYTES, dtype=torch.uint8, pin_memory=True)
+        page = _page.tensor = torch.empty(WAIT_PAGE_BYTES, dtype=torch.uint8, device="cpu", pin_memory=True)
     info = LCInfo()
     _check(lib().lc_wait(workspace.data_ptr(), None if stream is None else stream.data_ptr(), C.byref(info), page.data_ptr(),
                          _cs(workspace.device)), what)

@@ -2,6 +2,7 @@
 stream with a header. The device reports nothing of the kind here; the word is set behind the pass, on the same CUDA stream.
 """
 import ctypes as C
+import threading
 
 import numpy as np
 import pytest
@@ -63,3 +64,19 @@ def test_wait_with_and_without_a_page(lc):
             assert bytes(info) == want
             assert lc.lib().lc_wait(ws.data_ptr(), None, None, page, cs) == status
     torch.cuda.synchronize()  # no error is left behind
+
+
+def test_first_call_of_a_thread_under_a_default_device(lc):
+    base, cur = make_case(5000, 19)
+    want, got = lc.compress(base, cur, 4), []
+
+    def work():
+        with torch.device(DEV):
+            got.append(lc.compress(base, cur, 4))
+        torch.cuda.synchronize()
+
+    torch.cuda.synchronize()
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert len(got) == 1 and torch.equal(got[0], want)
