@@ -12,22 +12,23 @@
 //    area in shared memory; the lanes then pull their words from there. (Reading them straight from
 //    global memory makes every refill touch one cache line per lane.) A chunk that does not fit the
 //    staging area is decoded from global memory by the same code.
-//  * Codes are looked up in shared-memory tables whose entries hold the representative itself. The
-//    first level is indexed by the next kL1Bits bits and replicated 16 times (entry for (index, lane)
-//    at index*16 + lane%16): a 64-bit shared load is served half a warp at a time, so the 16 lanes of
-//    a half-warp always hit 16 different bank pairs although their indices are data dependent.
-//    Codes are canonical, so the 6-bit prefixes of longer codes are the last ones; from the first of them on a lane
-//    reads the second level instead, indexed by up to 9 more bits (the same load, no branch), which resolves codes of
-//    up to 15 bits; still longer codes are found by a canonical search behind a warp vote.
-//  * A lane keeps a 64-bit bit buffer per stream and tops it up with one predicated word load before
-//    every fourth symbol; a lane whose four codes take more bits than it held does the step again.
+//  * Codes are looked up in shared-memory tables whose entries hold the representative itself, 16 copies of each: a 64-bit
+//    shared load is served half a warp at a time, so 16 lanes that read copies of their own always hit 16 different bank
+//    pairs although their indices are data dependent.
+//  * Most streams take a table of one level, indexed by the next 7 bits, or by the number of leading ones of the next bits and three bits
+//    behind them (fill_one_level, decode_chunk_one_level); a lane keeps a bit position per stream and reads three words every eighth symbol.
+//  * Streams whose codes neither index resolves (by_direct, by_ones) take two levels: the next kL1Bits bits, and for the last of those prefixes,
+//    which belong to the longer codes, up to 9 more (decode_chunk_fast); a lane keeps a 64-bit buffer per stream and tops it
+//    up with one predicated word load before every fourth symbol.
+//    Both resolve codes of up to 15 bits; still longer ones are found by a canonical search behind a warp vote.
 //
 // Every read of a stream is bounds-checked against the caller's buffer size and every table is
 // validated before use, so a damaged stream yields LC_ERR_FORMAT (and unspecified output), never an
 // out-of-bounds access.
 //
-// Bound: HBM at k = 1 (8 bytes per element + the stream); at k = 4 the integer work per symbol is
-// the limit.
+// Bound: HBM at k = 1 and 2 (8 bytes per element + the streams: 1.75 and 1.72 ms for 1.3 G elements in 5 bits); at k = 4 issue slots
+// (58 % busy) and shared-memory wavefronts (61 %) side by side, 2.56 to 2.88 ms where the two levels alone took 3.0 to 3.3. Instructions per
+// element and warp at k = 4: 47, with the two levels 72.
 #include "lc_decode_bits.cuh"
 
 namespace lc {
@@ -37,10 +38,11 @@ using namespace dec;
 
 // Threads per CTA at most, and CTAs per SM that the registers must allow: with one stream 24 warps fit on an SM as two CTAs
 // of 12 (80 registers); two streams fit one CTA of 20 (96 registers: 138 M elements 240 -> 220 us against 16 warps, 11.7 M
-// elements 46 -> 31 us, because their 19.3 chunks per SM are then one round); with three and four a thread holds more state
-// and one CTA of 16 takes the SM (bounded to 96 registers, four streams spill and take 1.4 times as long).
+// elements 46 -> 31 us, because their 19.3 chunks per SM are then one round), and so do three (11.7 M elements 48 -> 41 us); with four a
+// thread holds more state and one CTA of 16 takes the SM (18 or 20 warps of 96 registers: 134 M elements 307 us instead of 290, and
+// staging areas so small that a vector of layers took 243 us instead of 155).
 template <int KS>
-constexpr int kDecThreads = KS == 1 ? 384 : KS == 2 ? 640 : 512;
+constexpr int kDecThreads = KS == 1 ? 384 : KS == 4 ? 512 : 640;
 template <int KS>
 constexpr int kDecCtas = KS == 1 ? 2 : 1;
 constexpr int kL1Bits = 6;
@@ -54,6 +56,13 @@ constexpr int kSubBitsMin = 4;
 constexpr int kL2Bits = kL1Bits + kSubBitsMax;     // longest code the two table levels resolve
 static_assert(2 * kL2Bits < 32, "a pair of codes leaves the bit buffer with one shift of a 32-bit word");
 static_assert(((1 << kL1Bits) << (kSubBitsMin + 3)) <= 8192, "at the smallest depth every prefix gets a sub-table");
+// The tables of one level have 128 entries, 16 copies each. Direct: by the next 7 bits. By leading ones (see fill_one_level): windows of
+// kOnesWindow bits in 16 classes by the number of their leading ones, 8 entries a class.
+constexpr int kDirectBits = 7;
+constexpr int kOnesWindow = 15;
+constexpr uint32_t kOneLevelEntries = 128;
+static_assert(kOneLevelEntries == 1u << kDirectBits && kOneLevelEntries == (kOnesWindow + 1) * 8, "either index");
+static_assert(2 * kOnesWindow < 32, "a pair of codes leaves a 32-bit word with one shift");
 // Length field of a table entry that does not resolve its code. As a length it takes the bit count far below zero,
 // which is how the hot loop notices: a step subtracts at most four of them per stream, and 1..4 times 2^29 (less a
 // few real lengths) leaves the sign bit of the 32-bit count set in every case.
@@ -62,6 +71,9 @@ constexpr uint32_t kLongCode = 0x20000000u;
 // a single stream of 138 M elements takes 194 us at 4, 207 at 6, 228 at 8 and 247 at 12
 template <int KS>
 constexpr int kPrefetchRows = KS == 1 ? 4 : 8;
+// the same for decode_chunk_one_level, in rows: with one stream 1.3 G elements take 1.75 ms at 4 and 2.06 at 8, with two 1.71, 1.86 at 6 and
+// 1.91 at 8; with three and four 2 to 12 make no difference
+constexpr int kAskRows = 4;
 
 // The two lookup tables of a stream are 8 KB each; the first starts on a 128-byte boundary of shared memory.
 constexpr uint32_t kTableBytes = 8192;
@@ -86,6 +98,7 @@ struct alignas(16) StreamState {
   uint32_t misses;      // first-level prefixes that belong to longer codes: the last ones (codes are canonical)
   uint32_t nsub;        // prefixes looked up in the second level: the most misses among the launch's streams
   uint32_t sub_bits;    // depth of the sub-tables, kSubBitsMin..kSubBitsMax: as many as 8 KB hold at that depth
+  uint32_t unresolved;  // windows of 15 bits whose code the table by leading ones does not resolve
   uint32_t end31[20];   // [L], L = 1..16: end of the range that codes of at most L bits fill, left-aligned to 31 bits
   uint32_t sorted_rep[kMaxSymbols];    // representatives in canonical (len, id) order
   unsigned long long first_code[64];   // first canonical code of each length
@@ -222,6 +235,7 @@ __device__ __noinline__ int prepare_stream(StreamState& S, unsigned char* scratc
     S.nused = nused;
     S.only_rep = only_rep;
     S.misses = misses;
+    S.unresolved = 0;
   }
   __syncwarp();
 
@@ -283,6 +297,102 @@ __device__ __forceinline__ void fill_tables(const StreamState* S, unsigned char*
     }
     reinterpret_cast<uint2*>(tables + s * 2 * kTableBytes + kTableBytes)[i] = ent;
   }
+}
+
+// How the codes of a launch's streams are looked up, the same for all of them.
+enum class Index { kDirect, kOnes, kTwoLevel };
+
+// The tables of one level. Direct, where no code is longer than 7 bits: entry i has the code that the 7 bits i begin with.
+//
+// By leading ones: by the number of leading ones of the next 15
+// bits and the three bits behind the zero that ends them. Codes are canonical, so a code's length grows with its leading ones, and
+// wherever the lengths of neighbouring codes differ by little (a Huffman code of buckets by exponent), three bits behind the zero
+// tell the code. That index comes out of a floating-point number: with the complement of the window as its value, the exponent
+// counts the leading ones and the top of the mantissa holds the bits behind (lookup_ones). A lookup then has one level: no compare, no
+// second address, and no uncopied entries with bank conflicts; and a table of 128 entries is filled in a fraction of the time of
+// 64 + 1024. Entry i stands for the windows whose complement v (an integer from 0 to 32767) has v + 1/2 in
+// [2^e (1 + q/8), 2^e (1 + (q + 1)/8)), e = i / 8 - 1, q = i % 8; where that is one code, the entry has it.
+template <int KS>
+__device__ __forceinline__ void fill_one_level(StreamState* S, unsigned char* tables, bool direct) {
+  static_assert(kOneLevelEntries * kL1Rep * 8 == 2 * kTableBytes, "in the place of the two levels");
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t k = threadIdx.x; k < KS * kOneLevelEntries; k += blockDim.x) {  // a warp's entries are of one stream
+    const uint32_t s = k / kOneLevelEntries, i = k % kOneLevelEntries;
+    StreamState& T = S[s];
+    uint2 ent = make_uint2(T.only_rep, 0u);
+    uint32_t missed = 0;
+    if (T.nused >= 2 && direct) {
+      ent = canonical_lookup(T, i << (31 - kDirectBits), kDirectBits);
+      if (ent.y == 0) ent.y = kLongCode;  // only with damaged lengths
+    } else if (T.nused >= 2) {
+      const uint32_t e = i / 8, q = i % 8;  // e: the exponent plus one
+      const uint32_t least = ((8 + q) << e) >> 4, end = ((9 + q) << e) >> 4;
+      const uint32_t most = end > least ? end - 1 : least;
+      const uint32_t first = (0x7fffu - most) << 16, last = (0x7fffu - least) << 16 | 0xffffu;  // windows left-aligned to 31 bits
+      const uint2 a = canonical_lookup(T, first, kOnesWindow), b = canonical_lookup(T, last, kOnesWindow);
+      const bool one = a.y != 0 && a.y == b.y && first >> (31 - a.y) == last >> (31 - a.y);
+      ent = one ? a : make_uint2(0u, kLongCode);
+      // (in the lowest classes several entries stand for one window, and one of them is looked up)
+      missed = one || ((2 * least + 1) << 3 >> e) != 8 + q ? 0u : most - least + 1;
+    }
+    missed = __reduce_add_sync(0xffffffffu, missed);
+    if (lane == 0 && missed) atomicAdd(&T.unresolved, missed);
+    uint4* row = reinterpret_cast<uint4*>(tables + s * 2 * kTableBytes) + i * (kL1Rep / 2);
+#pragma unroll
+    for (uint32_t j = 0; j < kL1Rep / 2; ++j) row[(j + lane) % (kL1Rep / 2)] = make_uint4(ent.x, ent.y, ent.x, ent.y);  // rotated: no bank conflicts
+  }
+}
+
+// Direct if no stream has a code of more than 7 bits.
+template <int KS>
+__device__ __forceinline__ bool by_direct(const StreamState* S) {
+  bool direct = true;
+#pragma unroll
+  for (int s = 0; s < KS; ++s) direct = direct && (S[s].nused < 2 || S[s].max_len <= kDirectBits);
+  return direct;
+}
+// By leading ones unless that leaves more windows of some stream unresolved than the two levels do (codes of one length
+// of 8 or 9 bits, say).
+template <int KS>
+__device__ __forceinline__ bool by_ones(const StreamState* S) {
+  bool ones = true;
+#pragma unroll
+  for (int s = 0; s < KS; ++s) {
+    const uint32_t two_level = 0x8000u - (S[s].end31[kL1Bits + S[s].sub_bits] >> 16);  // windows that the two levels leave
+    ones = ones && (S[s].nused < 2 || S[s].unresolved <= two_level);
+  }
+  return ones;
+}
+
+// {representative, length} of the code at the top of `hi`, length kLongCode if the table does not resolve it. `table`: shared
+// address of this lane's copy of entry 0, less kOnesBias by leading ones. There the float x is 1 + w 2^-23, w the top 15 bits of hi; the
+// multiply-add makes it (32767 - w + 1/2 + a bit less than 2^-9) 2^-23: the half keeps it above zero and away from the integers, where
+// rounding could matter.
+constexpr uint32_t kOnesBias = (127 - 24) * 8 * kL1Rep * 8;  // exponent field of 2^-24, the smallest value there is
+template <Index INDEX, int OFFSET>
+__device__ __forceinline__ uint2 lookup_one_level(uint32_t hi, uint32_t table) {
+  uint32_t v = hi;
+  if (INDEX == Index::kOnes) {
+    const uint32_t x = __funnelshift_r(hi, 0x3F800000u >> 15, 17);
+    v = __float_as_uint(__fmaf_rn(__uint_as_float(x), __uint_as_float(0xBF7FFFFFu) /* -(1 - 2^-24) */, __uint_as_float(0x3F807FFFu) /* 1 + 32767 * 2^-23 */));
+  }
+  uint2 ent;
+  asm("{\n\t"
+      ".reg .u32 t, a;\n\t"
+      "shr.u32 t, %2, %6;\n\t"
+      "mad.lo.u32 a, t, %4, %3;\n\t"
+      "ld.shared.v2.u32 {%0,%1}, [a+%5];\n\t"
+      "}"
+      : "=&r"(ent.x), "=&r"(ent.y)
+      : "r"(v), "r"(table), "n"(kL1Rep * 8), "n"(OFFSET), "n"(INDEX == Index::kOnes ? 20 : 32 - kDirectBits));
+  return ent;
+}
+template <Index INDEX, int KS>
+__device__ __forceinline__ void lookup_all(uint2 (&e)[KS], const uint32_t (&hi)[KS], uint32_t table) {
+  e[0] = lookup_one_level<INDEX, 0>(hi[0], table);
+  if (KS > 1) e[1 % KS] = lookup_one_level<INDEX, 2 * kTableBytes>(hi[1 % KS], table);
+  if (KS > 2) e[2 % KS] = lookup_one_level<INDEX, 4 * kTableBytes>(hi[2 % KS], table);
+  if (KS > 3) e[3 % KS] = lookup_one_level<INDEX, 6 * kTableBytes>(hi[3 % KS], table);
 }
 
 // How the lanes address the tables of all streams of a launch; the same for each, so that it takes four registers.
@@ -367,13 +477,25 @@ __device__ __forceinline__ float4 load_row(const float* p, int have) {
   return v;
 }
 
+template <bool PARTIAL>
+__device__ __forceinline__ void store_row(float* p, float x0, float x1, float x2, float x3, int have) {
+  if (!PARTIAL || have >= 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(x0, x1, x2, x3);
+  } else {
+    if (have > 0) p[0] = x0;
+    if (have > 1) p[1] = x1;
+    if (have > 2) p[2] = x2;
+  }
+}
+
 template <int KS, bool STAGED, bool PARTIAL>
 __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const Source* W, const uint32_t* start,
                                                     const float* base, float* out, uint64_t c, uint64_t n, uint32_t lane,
                                                     const float* next_rows, Status status) {
   LaneBits<STAGED> bits[KS];
-  const int rem = PARTIAL ? (int)(n - c * kChunkElems) - 4 * (int)lane : 0;  // elements from this lane's first slot on
-  const uint32_t steps = PARTIAL ? (uint32_t)(n - c * kChunkElems + 127) / 128 : kSteps;
+  const uint32_t elems = PARTIAL ? (uint32_t)min(n - c * kChunkElems, (uint64_t)kChunkElems) : kChunkElems;
+  const int rem = PARTIAL ? (int)elems - 4 * (int)lane : 0;  // elements from this lane's first slot on
+  const uint32_t steps = PARTIAL ? (elems + 127) / 128 : kSteps;
   // the streams' tables follow each other at 2 * kTableBytes: one base address, the rest as immediate offsets
   const Lookup T{S[0].l1_addr | ((lane & (kL1Rep - 1)) * 8u), (1u << kL1Bits) - S[0].nsub, 32 - kL1Bits - S[0].sub_bits,
                  S[0].l1_addr + kTableBytes - ((((1u << kL1Bits) - S[0].nsub) << S[0].sub_bits) << 3)};
@@ -474,25 +596,174 @@ __device__ __forceinline__ void decode_chunk_fast(const StreamState* S, const So
         }
       }
     }
-    if (!PARTIAL || have >= 4) {
-      *reinterpret_cast<float4*>(out + i) = make_float4(x[0], x[1], x[2], x[3]);
-    } else {
-      if (have > 0) out[i] = x[0];
-      if (have > 1) out[i + 1] = x[1];
-      if (have > 2) out[i + 2] = x[2];
-    }
+    store_row<PARTIAL>(out + i, x[0], x[1], x[2], x[3], have);
   }
 }
 static_assert(kL1Rep * 8 == 128, "first-level entries of one index span 128 bytes");
 
+// Code that a table of one level did not resolve, at bit `pos` of its chunk: canonical search. Returns {representative, length}.
+template <bool STAGED>
+__device__ __forceinline__ uint2 long_code_at(const StreamState& S, const Words<STAGED>& words, uint32_t pos, Status status) {
+  const uint32_t at = words.at(pos), w0 = words.load(at, 0), w1 = words.load(at, 1), w2 = words.load(at, 2);
+  const unsigned long long window = ((unsigned long long)__funnelshift_l(w1, w0, pos) << 32) | __funnelshift_l(w2, w1, pos);
+  uint32_t L = 1;
+  while (L < S.max_len && (S.len_count[L] == 0 || window > S.last_aligned[L])) L += 1;
+  const unsigned long long code = window >> (64 - L);
+  if (L <= S.max_len && code >= S.first_code[L] && code - S.first_code[L] < S.len_count[L])
+    return make_uint2(S.sorted_rep[S.len_offset[L] + (uint32_t)(code - S.first_code[L])], L);
+  status.set(LC_ERR_FORMAT);  // no code matches: damaged payload
+  return make_uint2(0u, L);
+}
+
+// A chunk through the tables of one level. A step is two rows (one with a single stream: see below): a lane decodes eight elements x KS
+// streams from a window of three words per stream, read anew in every step, so that all it keeps of a stream from step to step is a bit position. (A 64-bit buffer
+// that is topped up takes four registers and, with its bookkeeping, 45 instructions for four codes where this form takes 36.)
+// The window has at least 65 bits behind the position; four codes of a row that are together shorter than 32 bits leave
+// it with one funnel shift, and 33 bits are then left for the second row. A row of 32 bits or more, or with a code that the table does not
+// resolve (whose marker is a huge length), sends its lane through the row again, one code at a time, behind one vote per row.
+// Every code has at most 63 bits, so a lane of a damaged stream reads at most 1020 bytes beyond its chunk (kOverrunBytes).
+// PARTIAL: the vector's last chunk, or any chunk larger than the staging area: of each row only the slots that exist are read and written. (A
+// lane's codes end with its last element; nothing is reported for what it decodes behind it.)
+// next_chunk: floats from this chunk to the one the warp takes next, whose first rows are asked into the L2 behind this one's last; 0 if there is none.
+template <int KS, Index INDEX, bool STAGED, bool PARTIAL>
+__device__ __forceinline__ void decode_chunk_one_level(const StreamState* S, const Source* W, uint32_t (&pos)[KS], const float* base,
+                                                  float* out, uint32_t c, uint64_t n, uint32_t lane, uint64_t next_chunk,
+                                                  Status status) {
+  // With one stream the kernel is bound by HBM, and it is the steady trickle of single rows, each waited for a step before its use, that
+  // reaches the copy rate: with two rows a step 1.3 G elements took 1.87 ms instead of 1.75.
+  constexpr int R = KS == 1 ? 1 : 2;
+  const uint32_t elems = PARTIAL ? (uint32_t)min(n - (uint64_t)c * kChunkElems, (uint64_t)kChunkElems) : kChunkElems;
+  int have = (int)elems - 4 * (int)lane;  // PARTIAL: elements from this lane's first slot of the next row on
+  const uint32_t steps = PARTIAL ? (elems + 128 * R - 1) / (128 * R) : kSteps / R;
+  const uint32_t table = (S[0].l1_addr | ((lane & (kL1Rep - 1)) * 8u)) - (INDEX == Index::kOnes ? kOnesBias : 0u);
+  const float* bp = base + (uint64_t)c * kChunkElems + 4 * lane;
+  float* op = out + (uint64_t)c * kChunkElems + 4 * lane;
+  float4 b[2];  // the next two rows
+  b[0] = load_row<PARTIAL>(bp, have);
+  b[1] = load_row<PARTIAL>(bp + 128, have - 128);
+#pragma unroll 1
+  for (uint32_t j = 0; j < steps; ++j) {
+    // rows are asked into the L2 kAskRows ahead of the one that is about to be decoded; behind the last row the next chunk's, or again
+    // this step's
+    const int64_t on = j < steps - kAskRows / R ? 0 : next_chunk ? (int64_t)next_chunk - (int64_t)kChunkElems : -128 * kAskRows;
+    uint32_t hi[KS], mid[KS], lo[KS];
+#pragma unroll
+    for (int s = 0; s < KS; ++s) {
+      const Words<STAGED> words(W[s]);
+      const uint32_t at = words.at(pos[s]);
+      const uint32_t w0 = words.load(at, 0), w1 = words.load(at, 1), w2 = R > 1 ? words.load(at, 2) : 0u;
+      hi[s] = __funnelshift_l(w1, w0, pos[s]);
+      mid[s] = __funnelshift_l(w2, w1, pos[s]);
+      lo[s] = __funnelshift_l(0u, w2, pos[s]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      float4 x = b[r];
+      if (R == 1) b[0] = b[1];
+      if (j + 2 / R < steps) b[R == 1 ? 1 : r] = load_row<PARTIAL>(bp + 256, have - 256);
+      if (!PARTIAL) asm volatile("prefetch.global.L2 [%0];" ::"l"(bp + on + 128 * kAskRows));
+      uint2 e[KS];
+      uint32_t h[KS], len[KS], flags = 0;
+      lookup_all<INDEX>(e, hi, table);
+#pragma unroll
+      for (int s = 0; s < KS; ++s) {
+        x.x = __fadd_rn(x.x, __uint_as_float(e[s].x));
+        len[s] = e[s].y;
+        h[s] = __funnelshift_l(0u, hi[s], e[s].y);  // hi << length (mod 32)
+      }
+      lookup_all<INDEX>(e, h, table);
+#pragma unroll
+      for (int s = 0; s < KS; ++s) {
+        x.y = __fadd_rn(x.y, __uint_as_float(e[s].x));
+        len[s] += e[s].y;
+        h[s] = __funnelshift_l(mid[s], hi[s], len[s]);
+      }
+      lookup_all<INDEX>(e, h, table);
+#pragma unroll
+      for (int s = 0; s < KS; ++s) {
+        x.z = __fadd_rn(x.z, __uint_as_float(e[s].x));
+        len[s] += e[s].y;
+        h[s] = __funnelshift_l(0u, h[s], e[s].y);
+      }
+      lookup_all<INDEX>(e, h, table);
+#pragma unroll
+      for (int s = 0; s < KS; ++s) {
+        x.w = __fadd_rn(x.w, __uint_as_float(e[s].x));
+        len[s] += e[s].y;
+        flags |= len[s];
+      }
+      if (PARTIAL && have <= 0) flags = 0;
+      const bool again = flags >= 32u;
+      if (r + 1 < R) {
+#pragma unroll
+        for (int s = 0; s < KS; ++s) {
+          hi[s] = __funnelshift_l(mid[s], hi[s], len[s]);
+          mid[s] = __funnelshift_l(lo[s], mid[s], len[s]);
+        }
+      }
+      if (__builtin_expect(__any_sync(0xffffffffu, again), 0)) {
+        if (again) {
+          x = load_row<PARTIAL>(bp, have);
+          // one element per trip; x is rotated so that the loop needs no indexed register
+#pragma unroll 1
+          for (int i = 0; i < 4; ++i) {
+            float v = x.x;
+            if (!PARTIAL || i < have) {
+              uint2 ent[KS];
+#pragma unroll
+              for (int s = 0; s < KS; ++s) {
+                const Words<STAGED> words(W[s]);
+                const uint32_t at = words.at(pos[s]);
+                h[s] = __funnelshift_l(words.load(at, 1), words.load(at, 0), pos[s]);
+              }
+              lookup_all<INDEX>(ent, h, table);
+#pragma unroll
+              for (int s = 0; s < KS; ++s) {
+                if (ent[s].y > 63u) ent[s] = long_code_at<STAGED>(S[s], Words<STAGED>(W[s]), pos[s], status);
+                v = __fadd_rn(v, __uint_as_float(ent[s].x));
+                pos[s] += ent[s].y;
+              }
+            }
+            x.x = x.y, x.y = x.z, x.z = x.w, x.w = v;
+          }
+#pragma unroll
+          for (int s = 0; s < KS; ++s) {
+            len[s] = 0;
+            if (r + 1 < R) {  // the next row's window
+              const Words<STAGED> words(W[s]);
+              const uint32_t at = words.at(pos[s]), w1 = words.load(at, 1);
+              hi[s] = __funnelshift_l(w1, words.load(at, 0), pos[s]);
+              mid[s] = __funnelshift_l(words.load(at, 2), w1, pos[s]);
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int s = 0; s < KS; ++s) pos[s] += len[s];
+      store_row<PARTIAL>(op, x.x, x.y, x.z, x.w, have);
+      bp += 128;
+      op += 128;
+      if (PARTIAL) have -= 128;
+    }
+  }
+}
+
 // Chunk `c` of every stream: where its payload is and the lanes' bit counts. An entry that is not a valid range of the
-// payload is reported and taken as empty.
-template <int KS>
-__device__ __forceinline__ bool stage_chunk(const StreamState* S, uint64_t c, uint32_t lane, unsigned char* stage0,
-                                            uint32_t stage_bytes, Source* W, uint32_t* start, Status status) {
-  uint32_t bytes[KS];
+// payload is reported and taken as empty. The payloads are copied one behind the other into the warp's staging area of
+// KS * stage_bytes; returns whether they fit.
+// start: the lanes' first bits; ONE_LEVEL: as decode_chunk_one_level counts them, in shared memory if the payloads fit.
+//
+// ONE_LEVEL: the lanes of decode_chunk_one_level read three words a step, wherever each of them is. Lanes are as many words apart as
+// a lane's codes take, give or take a few, and if that is near a multiple of 8 words, they meet in a few banks: codes of 4.05 bits on
+// average had 4.9 wavefronts a load instead of 2.1. Such a chunk is copied with 16 bytes of space before every fourth lane (the unit on a
+// boundary twice), which makes it 2.9 to 3.4. Not always: the copy then waits for the lane starts, and the space brings lanes together that
+// are well apart without it.
+template <int KS, bool ONE_LEVEL>
+__device__ __forceinline__ bool stage_chunk(const StreamState* S, uint32_t c, uint32_t lane, unsigned char* stage0,
+                                            uint32_t stage_bytes, Source* W, uint32_t (&start)[KS], Status status) {
+  constexpr uint32_t kUnit = 16, kNear = 77;  // 0.6 words a lane
+  uint32_t bytes[KS], filled = 0;
   unsigned long long off0[KS], off1[KS];
-  bool fits = true;
   // all index loads of all streams first, so that their latencies overlap
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
@@ -501,9 +772,10 @@ __device__ __forceinline__ bool stage_chunk(const StreamState* S, uint64_t c, ui
     off0[s] = __ldg(ci + c);
     off1[s] = __ldg(ci + c + 1);
     const uint16_t* li = reinterpret_cast<const uint16_t*>(sp + S[s].lane_index_off);
-    start[s] = __ldg(li + c * kLanes + lane);
+    start[s] = __ldg(li + (uint64_t)c * kLanes + lane);
   }
-  // then the asynchronous copies of the payloads into the staging areas
+  const auto spaced = [](uint32_t bytes) { return ONE_LEVEL && ((bytes + kNear) & 1023u) <= 2 * kNear; };
+  // the asynchronous copies of the payloads into the staging areas
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
     if (off0[s] > off1[s] || off1[s] > S[s].payload_size || (off0[s] & 15) || (off1[s] & 15)) {
@@ -512,20 +784,17 @@ __device__ __forceinline__ bool stage_chunk(const StreamState* S, uint64_t c, ui
     }
     bytes[s] = (uint32_t)min(off1[s] - off0[s], (unsigned long long)kChunkElems * 8);
     const uint8_t* g = S[s].ptr + S[s].payload_off + off0[s];
-    unsigned char* st = stage0 + (size_t)s * stage_bytes;
     W[s].g = reinterpret_cast<const uint32_t*>(g);
     W[s].nw = bytes[s] >> 2;
-    W[s].sbase = smem_addr(st);
+    W[s].sbase = smem_addr(stage0) + filled;
     W[s].slim = W[s].sbase + bytes[s] + 12;
-    // 16 bytes of zero slack after the chunk must fit too
-    if (bytes[s] + 16 <= stage_bytes) {
+    filled += bytes[s] + (spaced(bytes[s]) ? 7 * kUnit : 16);  // 16 bytes of zero slack after the chunk must fit too
+    if (filled <= KS * stage_bytes && !spaced(bytes[s])) {
       for (uint32_t k = lane * 16; k < bytes[s]; k += 32 * 16) cp_async_16(W[s].sbase + k, g + k);
-      if (lane == 0) *reinterpret_cast<uint4*>(st + bytes[s]) = make_uint4(0, 0, 0, 0);
-    } else {
-      fits = false;
+      if (lane == 0) asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(W[s].sbase + bytes[s]), "r"(0) : "memory");
     }
   }
-  cp_async_commit();
+  const bool fits = filled <= KS * stage_bytes;
   // lane start offsets (exclusive scan of the lane bit counts) while the copies are in flight
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
@@ -537,39 +806,105 @@ __device__ __forceinline__ bool stage_chunk(const StreamState* S, uint64_t c, ui
       if ((int)lane >= d) incl += v;
     }
     start[s] = min(incl - lane_bits, bytes[s] * 8u);
+    if (spaced(bytes[s]) && fits) {
+      // four lanes copy the units that their codes lie in
+      const uint32_t group = lane >> 2, units = bytes[s] / kUnit;
+      const uint32_t first = __shfl_sync(0xffffffffu, start[s], lane & 28u) >> 7;
+      const uint32_t behind = __shfl_sync(0xffffffffu, start[s], (lane & 28u) + 4) >> 7;
+      const uint32_t end = group == 7 ? units : min(behind + 1, units);
+      const uint8_t* g = reinterpret_cast<const uint8_t*>(W[s].g);
+      for (uint32_t u = first + (lane & 3u); u < end; u += 4) cp_async_16(W[s].sbase + (u + group) * kUnit, g + u * kUnit);
+      start[s] += group * kUnit * 8;
+    }
+    if (ONE_LEVEL && fits) start[s] += W[s].sbase * 8;
   }
+  cp_async_commit();
   cp_async_wait_all();
   __syncwarp();
   return fits;
 }
 
-// The vector's last, partial chunk, out of line and outside the main loop: it runs once per call, in one warp, and must
-// not weigh on the registers of the others. On vectors of a few thousand chunks the whole launch waits for that warp, so
-// it runs the same straight-line steps as a whole chunk (one code at a time it took 15 us with one stream and 60 us
-// with four).
-template <int KS>
-__device__ __noinline__ void decode_last_chunk(const StreamState* S, const float* base, float* out, uint64_t c, uint64_t n,
+// A chunk that is partial (the vector's last) or larger than the staging area, out of line: it must not weigh on the registers of
+// the main loop. On vectors of a few thousand chunks the whole launch waits for the warp that has it, so it runs the same
+// straight-line steps as the others (one code at a time the last chunk took 15 us with one stream and 60 us with four). If the
+// area does not hold all streams' payloads, they take it one after the other, each over what the one before has written.
+template <int KS, Index INDEX>
+__device__ __noinline__ void decode_rare_chunk(const StreamState* S, const float* base, float* out, uint32_t c, uint64_t n,
                                                uint32_t lane, unsigned char* stage0, uint32_t stage_bytes, Status status) {
+  {
+    Source W[KS];
+    uint32_t pos[KS];
+    __syncwarp();  // the previous chunk's reads of the staging area are done
+    if (stage_chunk<KS, true>(S, c, lane, stage0, stage_bytes, W, pos, status)) {
+      decode_chunk_one_level<KS, INDEX, true, true>(S, W, pos, base, out, c, n, lane, 0, status);
+      return;
+    }
+  }
+#pragma unroll 1
+  for (int s = 0; s < KS; ++s) {
+    Source W[1];
+    uint32_t pos[1];
+    __syncwarp();
+    if (stage_chunk<1, true>(S + s, c, lane, stage0, KS * stage_bytes, W, pos, status))
+      decode_chunk_one_level<1, INDEX, true, true>(S + s, W, pos, s ? out : base, out, c, n, lane, 0, status);
+    else
+      decode_chunk_one_level<1, INDEX, false, true>(S + s, W, pos, s ? out : base, out, c, n, lane, 0, status);
+  }
+}
+
+// Any chunk through the two-level tables, likewise out of line.
+template <int KS>
+__device__ __noinline__ void decode_chunk_two_level(const StreamState* S, const float* base, float* out, uint32_t c, uint64_t n,
+                                                    uint32_t lane, unsigned char* stage0, uint32_t stage_bytes, const float* next_rows,
+                                                    Status status) {
   Source W[KS];
   uint32_t start[KS];
-  __syncwarp();  // the previous chunk's reads of the staging area are done
-  if (stage_chunk<KS>(S, c, lane, stage0, stage_bytes, W, start, status))
-    decode_chunk_fast<KS, true, true>(S, W, start, base, out, c, n, lane, base, status);
-  else
+  __syncwarp();
+  if (!stage_chunk<KS, false>(S, c, lane, stage0, stage_bytes, W, start, status))
     decode_chunk_fast<KS, false, true>(S, W, start, base, out, c, n, lane, base, status);
+  else if (((uint64_t)c + 1) * kChunkElems <= n)
+    decode_chunk_fast<KS, true, false>(S, W, start, base, out, c, n, lane, next_rows, status);
+  else
+    decode_chunk_fast<KS, true, true>(S, W, start, base, out, c, n, lane, base, status);
+}
+
+// This warp's chunks, from c on, through the tables of one level.
+template <int KS, Index INDEX>
+__device__ __forceinline__ void decode_chunks(const StreamState* S, const float* base, float* out, uint32_t c, uint32_t nwarps,
+                                              uint32_t whole_end, uint32_t chunk_end, uint64_t n, uint32_t lane, unsigned char* stage0,
+                                              uint32_t stage_bytes, Status status) {
+  for (; c < whole_end; c += nwarps) {
+    Source W[KS];
+    uint32_t pos[KS];
+    __syncwarp();  // the previous chunk's reads of the staging area are done
+    if (stage_chunk<KS, true>(S, c, lane, stage0, stage_bytes, W, pos, status))
+      decode_chunk_one_level<KS, INDEX, true, false>(S, W, pos, base, out, c, n, lane, c + nwarps < whole_end ? (uint64_t)nwarps * kChunkElems : 0, status);
+    else
+      decode_rare_chunk<KS, INDEX>(S, base, out, c, n, lane, stage0, stage_bytes, status);
+  }
+  if (c < chunk_end) decode_rare_chunk<KS, INDEX>(S, base, out, c, n, lane, stage0, stage_bytes, status);
+}
+
+// Asks a chunk's first rows into the L2.
+__device__ __forceinline__ void prefetch_rows(const float* first, uint32_t lane) {
+  if (lane == 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(first), "r"(4096u) : "memory");
 }
 
 // Chunks [chunk_begin, chunk_end) of one vector, by `ctas` CTAs of which this is number `cta`.
 // stage_bytes: bytes of staging area per warp and stream (a multiple of 16, at least 32).
 template <int KS>
 __device__ __forceinline__ void decode_vector(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
-                                              Status status, uint32_t stage_bytes, uint64_t chunk_begin,
-                                              uint64_t chunk_end, uint32_t cta, uint32_t ctas) {
+                                              Status status, uint32_t stage_bytes, uint32_t chunk_begin,
+                                              uint32_t chunk_end, uint32_t cta, uint32_t ctas) {
   // dynamic shared memory: [pad to 128 bytes | 2 tables per stream | StreamState per stream | staging areas]
   extern __shared__ __align__(16) unsigned char s_raw[];
   unsigned char* tables = s_raw + ((kTablePad - (smem_addr(s_raw) & (kTablePad - 1))) & (kTablePad - 1));
   StreamState* S = reinterpret_cast<StreamState*>(s_raw + kTablePad + KS * 2 * kTableBytes);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const uint32_t nwarps = ctas * warps;
+  const uint32_t whole_end = min(chunk_end, (uint32_t)(n / kChunkElems));  // the chunks that are full; at most 2^20 in all
+  uint32_t c = chunk_begin + cta * warps + warp;
+  if (c < whole_end) prefetch_rows(base + (uint64_t)c * kChunkElems, lane);
   static_assert(KS <= 4 && 5 * kMaxSymbols <= kTableBytes, "a warp per stream; the second level is the scratch");
   if (warp < KS) {
     const uint8_t* ptr = streams.ptr[0];
@@ -604,31 +939,34 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
     S[threadIdx.x].nsub = most;
     S[threadIdx.x].sub_bits = sub_bits;
   }
+  // what follows is the same for every thread
+  const bool direct = by_direct<KS>(S);
+  fill_one_level<KS>(S, tables, direct);
   __syncthreads();
-  fill_tables<KS>(S, tables);
-  __syncthreads();
+  const Index index = direct ? Index::kDirect : by_ones<KS>(S) ? Index::kOnes : Index::kTwoLevel;
+  if (index == Index::kTwoLevel) {
+    fill_tables<KS>(S, tables);
+    __syncthreads();
+  }
 
   unsigned char* stage0 = reinterpret_cast<unsigned char*>(S + KS) + (size_t)warp * KS * stage_bytes;
-  const uint64_t nwarps = (uint64_t)ctas * warps;
-  const uint64_t whole_end = min(chunk_end, n / kChunkElems);  // the chunks that are full
-  uint64_t c = chunk_begin + (uint64_t)cta * warps + warp;
-  for (; c < whole_end; c += nwarps) {
-    Source W[KS];
-    uint32_t start[KS];
-    __syncwarp();  // the previous chunk's reads of the staging area are done
-    const bool fits = stage_chunk<KS>(S, c, lane, stage0, stage_bytes, W, start, status);
-    // where the L2 prefetch goes on behind this chunk: the next full chunk of this warp, if there is one
-    const float* next_rows = base + (c + nwarps < whole_end ? c + nwarps : c) * kChunkElems + 4 * lane;
-    if (fits) decode_chunk_fast<KS, true, false>(S, W, start, base, out, c, n, lane, next_rows, status);
-    else decode_chunk_fast<KS, false, false>(S, W, start, base, out, c, n, lane, next_rows, status);
+  if (index == Index::kDirect) {
+    decode_chunks<KS, Index::kDirect>(S, base, out, c, nwarps, whole_end, chunk_end, n, lane, stage0, stage_bytes, status);
+  } else if (index == Index::kOnes) {
+    decode_chunks<KS, Index::kOnes>(S, base, out, c, nwarps, whole_end, chunk_end, n, lane, stage0, stage_bytes, status);
+  } else {
+    for (; c < chunk_end; c += nwarps) {
+      // where the L2 prefetch goes on behind this chunk: the next full chunk of this warp, if there is one
+      const float* next_rows = base + (uint64_t)(c + nwarps < whole_end ? c + nwarps : c) * kChunkElems + 4 * lane;
+      decode_chunk_two_level<KS>(S, base, out, c, n, lane, stage0, stage_bytes, next_rows, status);
+    }
   }
-  if (c < chunk_end) decode_last_chunk<KS>(S, base, out, c, n, lane, stage0, stage_bytes, status);
 }
 
 template <int KS>
 __global__ void __launch_bounds__(kDecThreads<KS>, kDecCtas<KS>)
 decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status, uint32_t rank,
-              uint32_t stage_bytes, uint64_t chunk_begin, uint64_t chunk_end) {
+              uint32_t stage_bytes, uint32_t chunk_begin, uint32_t chunk_end) {
   decode_vector<KS>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
 }
 
@@ -654,7 +992,7 @@ decode_segments_kernel(const float* base, const __grid_constant__ DecodeStreams 
     streams.bytes[s] = bytes;
   }
   decode_vector<KS>(base + first, streams, n, out + first, Status{status, 2 * (batch.first + lo) + second}, stage_bytes, 0,
-                    (n + kChunkElems - 1) / kChunkElems, blockIdx.x - batch.cta_begin[lo],
+                    (uint32_t)((n + kChunkElems - 1) / kChunkElems), blockIdx.x - batch.cta_begin[lo],
                     batch.cta_begin[lo + 1] - batch.cta_begin[lo]);
 }
 
@@ -672,7 +1010,7 @@ inline uint32_t ctas_on_sm(uint32_t warps, uint32_t dyn, uint32_t regs) {
   return min(min(by_regs, by_smem), by_warps);
 }
 
-// want_stage: staging bytes that hold an average chunk with some room. Among CTAs of 20 (two streams only), 16, 12 and 8 warps, takes the shape
+// want_stage: staging bytes that hold an average chunk with some room. Among CTAs of 20 (two and three streams), 16, 12 and 8 warps, takes the shape
 // that puts most warps on an SM (with four streams that is one CTA of 16 warps, with one stream several smaller ones),
 // then gives the staging areas whatever shared memory that shape leaves (chunk sizes vary around the average).
 template <int KS>
@@ -744,7 +1082,7 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
                              int32_t* status, bool second, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
   static uint32_t regs_of[kMaxDevices] = {};
   const uint64_t nchunks = (n + kChunkElems - 1) / kChunkElems;
-  // 1.03 x the largest average chunk of the streams (from the buffer sizes, which bound the payload)
+  // 1.03 x the largest average chunk of the streams and what its space may take (from the buffer sizes, which bound the payload)
   uint64_t avg = 0;
   for (int s = 0; s < KS; ++s) {
     const uint64_t index_bytes = 72 * nchunks;  // lane and chunk index entries are not staged
@@ -752,7 +1090,7 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
     avg = a > avg ? a : avg;
   }
   Shape sh;
-  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_kernel<KS>), align_up(avg + avg / 32 + 48, 16),
+  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_kernel<KS>), align_up(avg + avg / 32 + 128, 16),
                                          regs_of, sh);
   if (e != cudaSuccess) return e;
   const uint64_t chunks = chunk_end - chunk_begin, full = (uint64_t)sh.sms * sh.per_sm;
@@ -760,8 +1098,11 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
   uint64_t want = (chunks + warps - 1) / warps;
   if (want == 0) want = 1;  // still reports a rejected stream
   const unsigned grid = (unsigned)(want < full ? want : full);
-  decode_kernel<KS><<<grid, warps * 32, sh.dyn - (sh.warps - warps) * KS * sh.stage, cs>>>(base, streams, n, out, status, second ? 1u : 0u, sh.stage, chunk_begin,
-                                                         chunk_end);
+  // the staging areas of the warps left out go to the others: chunks vary (a layer of rare exponents in a vector of layers
+  // takes twice the average), and one that is read from global memory word by word holds up the launch
+  const uint32_t stage = min(sh.warps * sh.stage / warps / 16 * 16, kChunkElems * 8 + 16);
+  decode_kernel<KS><<<grid, warps * 32, sh.dyn - (sh.warps * sh.stage - warps * stage) * KS, cs>>>(base, streams, n, out, status, second ? 1u : 0u,
+                                                                                                  stage, (uint32_t)chunk_begin, (uint32_t)chunk_end);
   return cudaGetLastError();
 }
 

@@ -9,7 +9,7 @@ namespace lc {
 namespace dec {
 
 constexpr uint32_t kSmemPerSm = 227 * 1024;  // usable shared memory of one CTA on sm_100
-constexpr uint32_t kOverrunBytes = 512;      // padding behind the last staging area (see LaneBits::refill)
+constexpr uint32_t kOverrunBytes = 1024;     // padding behind the last staging area (see LaneBits::refill and decode_chunk_ones)
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -112,6 +112,25 @@ struct LaneBits {
     lo <<= len;
     cnt -= (int)len;
   }
+};
+
+// The words around a bit position of a chunk. STAGED: positions are bit addresses in shared memory, and nothing is clamped (see
+// decode_chunk_ones). Otherwise they count from the chunk's start and words beyond its end are 0.
+template <bool STAGED>
+struct Words;
+template <>
+struct Words<true> {
+  __device__ __forceinline__ explicit Words(const Source&) {}
+  __device__ __forceinline__ uint32_t at(uint32_t pos) const { return (pos >> 5) * 4u; }
+  __device__ __forceinline__ uint32_t load(uint32_t at, uint32_t i) const { return lds_u32(at + 4 * i); }
+};
+template <>
+struct Words<false> {
+  const uint32_t* g;
+  uint32_t nw;
+  __device__ __forceinline__ explicit Words(const Source& W) : g(W.g), nw(W.nw) {}
+  __device__ __forceinline__ uint32_t at(uint32_t pos) const { return pos >> 5; }
+  __device__ __forceinline__ uint32_t load(uint32_t at, uint32_t i) const { return at + i < nw ? __ldg(g + at + i) : 0u; }
 };
 
 }  // namespace dec
