@@ -347,33 +347,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
               o4[32 * (4 * q + r)] = x;
             }
           }
-        } else if (!ks.wide) {
-          // partial last chunk: four steps' loads at a time, the slots beyond the end left out
-          const uint32_t rem = (uint32_t)(n - p_c * kChunkElems);
-          const uint4* ep = reinterpret_cast<const uint4*>(plane + p_c * kChunkElems) + lane;
-          const float* b1 = base + p_c * kChunkElems;
-          float* o1 = tracked_out + p_c * kChunkElems;
-#pragma unroll 1
-          for (uint32_t q = 0; q * 512 < rem; ++q) {
-            const uint4 w4 = __ldg(ep + 32 * q);
-            const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
-            float b[4][4];
-#pragma unroll
-            for (uint32_t r = 0; r < 4; ++r)
-#pragma unroll
-              for (uint32_t e = 0; e < 4; ++e) {
-                const uint32_t i = (4 * q + r) * 128 + 4 * lane + e;
-                if (i < rem) b[r][e] = b1[i];
-              }
-#pragma unroll
-            for (uint32_t r = 0; r < 4; ++r)
-#pragma unroll
-              for (uint32_t e = 0; e < 4; ++e) {
-                const uint32_t i = (4 * q + r) * 128 + 4 * lane + e;
-                if (i < rem) o1[i] = __fadd_rn(b[r][e], __uint_as_float(s_rep[__byte_perm(w[r], 0u, 0x4440 + e)]));
-              }
-          }
-        } else {
+        } else if (ks.wide) {
           // exponents the one-byte plane does not hold: element by element
           for (uint32_t j = 0; j < kSteps; ++j) {
             for (uint32_t e = 0; e < kGroup; ++e) {
@@ -386,6 +360,33 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
           }
         }
       }
+    }
+    // The partial last chunk's, by all warps of the CTA, four rows each: by the one warp that has coded it, it took the launch
+    // 10 us longer (11.7 M elements: 35 us instead of 25).
+    if (UPDATE && p_have && !s_abort && p_tile == ntiles - 1 && n % kChunkElems != 0 && !ks.wide) {
+      const uint64_t p_c = nchunks - 1;
+      const uint32_t rem = (uint32_t)(n - p_c * kChunkElems);
+      const float* b1 = base + p_c * kChunkElems;
+      float* o1 = tracked_out + p_c * kChunkElems;
+      constexpr uint32_t kRows = kSteps / kEncWarps;
+      static_assert(kRows == 4, "a lane's plane bytes of four steps are one load");
+      const uint4 w4 = __ldg(reinterpret_cast<const uint4*>(plane + p_c * kChunkElems) + 32 * warp + lane);
+      const uint32_t w[kRows] = {w4.x, w4.y, w4.z, w4.w};
+      float b[kRows][4];
+#pragma unroll
+      for (uint32_t r = 0; r < kRows; ++r)
+#pragma unroll
+        for (uint32_t e = 0; e < 4; ++e) {
+          const uint32_t i = (kRows * warp + r) * 128 + 4 * lane + e;
+          if (i < rem) b[r][e] = b1[i];
+        }
+#pragma unroll
+      for (uint32_t r = 0; r < kRows; ++r)
+#pragma unroll
+        for (uint32_t e = 0; e < 4; ++e) {
+          const uint32_t i = (kRows * warp + r) * 128 + 4 * lane + e;
+          if (i < rem) o1[i] = __fadd_rn(b[r][e], __uint_as_float(s_rep[__byte_perm(w[r], 0u, 0x4440 + e)]));
+        }
     }
     if (!have) break;
     // The next ticket is taken now, so that the round trip overlaps the rest of this iteration. (Taking it
