@@ -275,13 +275,16 @@ def compress_segments_async(base, cur, seg_begin, nbits, streams, workspace, tra
 
 def compress_segments(base, cur, seg_begin, nbits, streams=None, workspace=None, tracked_out=None):
     """One stream per segment. Returns (streams buffer, offsets): segment i's stream starts at offsets[i]."""
-    offsets, total = segments_layout(seg_begin, nbits)
+    layout = None
     if streams is None:
-        streams = torch.empty(total, dtype=torch.uint8, device=base.device)
+        layout = segments_layout(seg_begin, nbits)
+        streams = torch.empty(layout[1], dtype=torch.uint8, device=base.device)
     if workspace is None:
         longest = max([b - a for a, b in zip(seg_begin[:-1], seg_begin[1:])] + [0])
         workspace = alloc_workspace(longest, base.device)
+    # the offsets of 62 segments take the interpreter 16 us: worked out while the GPU is busy, unless the size is needed first
     compress_segments_async(base, cur, seg_begin, nbits, streams, workspace, tracked_out)
+    offsets, _ = layout or segments_layout(seg_begin, nbits)
     _wait(workspace, "lc_compress_segments (device)")
     return streams, offsets
 
