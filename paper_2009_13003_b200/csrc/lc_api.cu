@@ -230,8 +230,8 @@ int lc_recover(const float* base, const void* const* streams, const uint64_t* st
   if (cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
   // up to four streams per launch; later launches continue in place from `out`.
   const float* src = base;
-  for (int first = 0; first < k; first += 4) {
-    const int kk = (k - first) < 4 ? (k - first) : 4;
+  for (int first = 0, kk; first < k; first += kk) {
+    kk = decode_group(k - first);
     DecodeStreams ds;
     memset(&ds, 0, sizeof ds);
     for (int j = 0; j < kk; ++j) {
@@ -353,9 +353,9 @@ int lc_recover_segments(const float* base, const void* const* streams, int k, co
     batch.elem_begin[batch.nseg] = seg_begin[i];
     batch.stream_begin[batch.nseg] = off;
     // up to four streams of every segment per launch; later launches continue in place from `out`
-    for (int first = 0; first < k; first += 4) {
+    for (int first = 0, kk; first < k; first += kk) {
       const uint8_t* group[4];
-      const int kk = (k - first) < 4 ? (k - first) : 4;
+      kk = decode_group(k - first);
       for (int j = 0; j < kk; ++j) group[j] = static_cast<const uint8_t*>(streams[first + j]);
       if (launch_decode_segments(first == 0 ? base : out, group, kk, batch, nbits, out, &ctl->status, first > 0, cs) != cudaSuccess)
         return LC_ERR_CUDA;
@@ -597,7 +597,6 @@ extern "C" int lc_recover_host(const float* base_host, const void* const* stream
   if (!pipe.create()) return LC_ERR_CUDA;
   Control* ctl = reinterpret_cast<Control*>(a);
   if (cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
-  const int groups = (k + 3) / 4;
   for (int i = 0; i < kHostSlices; ++i) {
     const uint64_t c0 = nchunks * i / kHostSlices, c1 = nchunks * (i + 1) / kHostSlices;
     const uint64_t e0 = c0 * kChunkElems, e1 = c1 * kChunkElems < n ? c1 * kChunkElems : n;
@@ -605,15 +604,15 @@ extern "C" int lc_recover_host(const float* base_host, const void* const* stream
       return LC_ERR_CUDA;
     if (cudaEventRecord(pipe.arrived[i], pipe.in) != cudaSuccess) return LC_ERR_CUDA;
     if (cudaStreamWaitEvent(cs, pipe.arrived[i], 0) != cudaSuccess) return LC_ERR_CUDA;
-    for (int g = 0; g < groups; ++g) {
-      const int first = 4 * g, kk = (k - first) < 4 ? (k - first) : 4;
+    for (int first = 0, kk; first < k; first += kk) {
+      kk = decode_group(k - first);
       DecodeStreams ds;
       memset(&ds, 0, sizeof ds);
       for (int j = 0; j < kk; ++j) {
         ds.ptr[j] = static_cast<const uint8_t*>(d_streams[first + j]);
         ds.bytes[j] = stream_bytes[first + j];
       }
-      if (launch_decode(d_x, ds, kk, n, d_x, &ctl->status, g > 0, cs, c0, c1) != cudaSuccess) return LC_ERR_CUDA;
+      if (launch_decode(d_x, ds, kk, n, d_x, &ctl->status, first > 0, cs, c0, c1) != cudaSuccess) return LC_ERR_CUDA;
     }
     if (cudaEventRecord(pipe.decoded[i], cs) != cudaSuccess) return LC_ERR_CUDA;
     if (cudaStreamWaitEvent(pipe.out, pipe.decoded[i], 0) != cudaSuccess) return LC_ERR_CUDA;

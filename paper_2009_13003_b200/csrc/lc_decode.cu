@@ -1177,6 +1177,11 @@ uint32_t split_segments(SegBatch& batch, uint32_t warps, uint32_t slots) {
   return ctas;
 }
 
+// Four at a time, but five as three and two: a launch with one stream is bound by HBM and takes as long as one with two (1.3 G elements: four
+// and one 4602 us, three and two 4023). (Eight as three, three and two, where 16 warps an SM need two rounds and 20 one: 11.7 M elements of 62
+// layers 214 us instead of 155, because the smaller staging areas do not hold the chunks of some layers.)
+int decode_group(int left) { return left <= 4 ? left : left == 5 ? 3 : 4; }
+
 cudaError_t launch_decode_segments(const float* base, const uint8_t* const* streams, int k, SegBatch& batch, int nbits,
                                    float* out, int32_t* status, bool second, cudaStream_t cs) {
   switch (k) {
