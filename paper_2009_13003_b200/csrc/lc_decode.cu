@@ -11,7 +11,7 @@
 //  * The chunk's payload of every stream is first copied, coalesced, into a warp-private staging
 //    area in shared memory; the lanes then pull their words from there. (Reading them straight from
 //    global memory makes every refill touch one cache line per lane.) A chunk that does not fit the
-//    staging area is decoded from global memory by the same code.
+//    staging area takes the streams one after the other, or is decoded from global memory by the same code.
 //  * Codes are looked up in shared-memory tables whose entries hold the representative itself, 16 copies of each: a 64-bit
 //    shared load is served half a warp at a time, so 16 lanes that read copies of their own always hit 16 different bank
 //    pairs although their indices are data dependent.
@@ -343,7 +343,8 @@ __device__ __forceinline__ void fill_one_level(StreamState* S, unsigned char* ta
   }
 }
 
-// Direct if no stream has a code of more than 7 bits.
+// Direct if no stream has a code of more than 7 bits (134 M elements, four streams: fixed 4 bits 338 us, with the two levels 411; fixed 5 bits 330
+// and 372; 20 codes of 4 and 5 bits 287 and 363).
 template <int KS>
 __device__ __forceinline__ bool by_direct(const StreamState* S) {
   bool direct = true;
@@ -352,7 +353,8 @@ __device__ __forceinline__ bool by_direct(const StreamState* S) {
   return direct;
 }
 // By leading ones unless that leaves more windows of some stream unresolved than the two levels do (codes of one length
-// of 8 or 9 bits, say).
+// of 8 or 9 bits, say: 200 of them would send every row the long way; with the two levels four streams of 134 M take 545 us). Where both
+// resolve the codes, leading ones are the faster: 134 M elements, 5 bits, four streams 289 us and 337, three 236 and 270, two 201 and 226.
 template <int KS>
 __device__ __forceinline__ bool by_ones(const StreamState* S) {
   bool ones = true;
