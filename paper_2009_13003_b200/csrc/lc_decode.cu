@@ -61,6 +61,8 @@ static_assert(((1 << kL1Bits) << (kSubBitsMin + 3)) <= 8192, "at the smallest de
 constexpr int kDirectBits = 7;
 constexpr int kOnesWindow = 15;
 constexpr uint32_t kOneLevelEntries = 128;
+constexpr uint32_t kResolved = 64;  // four codes that the table resolves are shorter
+static_assert(4 * kOnesWindow < kResolved && 4 * kOnesWindow <= 65 && 4 * kDirectBits < kResolved, "and lie within a window of three words");
 static_assert(kOneLevelEntries == 1u << kDirectBits && kOneLevelEntries == (kOnesWindow + 1) * 8, "either index");
 static_assert(2 * kOnesWindow < 32, "a pair of codes leaves a 32-bit word with one shift");
 // Length field of a table entry that does not resolve its code. As a length it takes the bit count far below zero,
@@ -623,8 +625,13 @@ __device__ __forceinline__ uint2 long_code_at(const StreamState& S, const Words<
 // streams from a window of three words per stream, read anew in every step, so that all it keeps of a stream from step to step is a bit position. (A 64-bit buffer
 // that is topped up takes four registers and, with its bookkeeping, 45 instructions for four codes where this form takes 36.)
 // The window has at least 65 bits behind the position; four codes of a row that are together shorter than 32 bits leave
-// it with one funnel shift, and 33 bits are then left for the second row. A row of 32 bits or more, or with a code that the table does not
-// resolve (whose marker is a huge length), sends its lane through the row again, one code at a time, behind one vote per row.
+// it with one funnel shift, and at least 34 bits are then left for the second row. One vote per row finds the lanes with a longer row or a
+// code that the table does not resolve (whose marker is a huge length). Rows of 32 to 60 bits were looked up from valid bits, and stand, if the
+// window had as many: always in the first of two rows, behind which the window is read anew; in the second, and with one stream, 64 less
+// the position within its word are certain. (A lookup on too few bits always overdraws, because no code is a prefix of another.)
+// Only what is left goes through the row again, one code at a time. They are rare on the whole (four streams in 6 bits: 0.3 to 1.4 % of a
+// warp's rows), but a chunk of rare exponents has nothing else, and a launch of one round waits for it. With all of them one code at a time, four
+// streams of 11.7 M elements in 62 scales took 57 us instead of 41; two of 134 M, 10 % in rare exponents, 311 instead of 226.
 // Every code has at most 63 bits, so a lane of a damaged stream reads at most 1020 bytes beyond its chunk (kOverrunBytes).
 // PARTIAL: the vector's last chunk, or any chunk larger than the staging area: of each row only the slots that exist are read and written. (A
 // lane's codes end with its last element; nothing is reported for what it decodes behind it.)
@@ -651,6 +658,7 @@ __device__ __forceinline__ void decode_chunk_one_level(const StreamState* S, con
     // this step's
     const int64_t on = j < steps - kAskRows / R ? 0 : next_chunk ? (int64_t)next_chunk - (int64_t)kChunkElems : -128 * kAskRows;
     uint32_t hi[KS], mid[KS], lo[KS];
+    bool reloaded = false;  // the second row's window, anew behind the first row: 64 bits of it are valid
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
       const Words<STAGED> words(W[s]);
@@ -697,7 +705,7 @@ __device__ __forceinline__ void decode_chunk_one_level(const StreamState* S, con
         flags |= len[s];
       }
       if (PARTIAL && have <= 0) flags = 0;
-      const bool again = flags >= 32u;
+      const bool wide = flags >= 32u;
       if (r + 1 < R) {
 #pragma unroll
         for (int s = 0; s < KS; ++s) {
@@ -705,40 +713,49 @@ __device__ __forceinline__ void decode_chunk_one_level(const StreamState* S, con
           mid[s] = __funnelshift_l(lo[s], mid[s], len[s]);
         }
       }
-      if (__builtin_expect(__any_sync(0xffffffffu, again), 0)) {
-        if (again) {
-          x = load_row<PARTIAL>(bp, have);
-          // one element per trip; x is rotated so that the loop needs no indexed register
-#pragma unroll 1
-          for (int i = 0; i < 4; ++i) {
-            float v = x.x;
-            if (!PARTIAL || i < have) {
-              uint2 ent[KS];
+      if (__builtin_expect(__any_sync(0xffffffffu, wide), 0)) {
+        if (wide) {
+          bool stands = flags < kResolved;
+          if (R == 1 || r == 1) {  // (the first of two rows has bits enough)
 #pragma unroll
-              for (int s = 0; s < KS; ++s) {
-                const Words<STAGED> words(W[s]);
-                const uint32_t at = words.at(pos[s]);
-                h[s] = __funnelshift_l(words.load(at, 1), words.load(at, 0), pos[s]);
-              }
-              lookup_all<INDEX>(ent, h, table);
-#pragma unroll
-              for (int s = 0; s < KS; ++s) {
-                if (ent[s].y > 63u) ent[s] = long_code_at<STAGED>(S[s], Words<STAGED>(W[s]), pos[s], status);
-                v = __fadd_rn(v, __uint_as_float(ent[s].x));
-                pos[s] += ent[s].y;
-              }
-            }
-            x.x = x.y, x.y = x.z, x.z = x.w, x.w = v;
+            for (int s = 0; s < KS; ++s) stands = stands && (reloaded || len[s] <= 64 - (pos[s] & 31));
           }
+          if (!stands) {
+            x = load_row<PARTIAL>(bp, have);
+            // one element per trip; x is rotated so that the loop needs no indexed register
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {
+              float v = x.x;
+              if (!PARTIAL || i < have) {
+                uint2 ent[KS];
 #pragma unroll
-          for (int s = 0; s < KS; ++s) {
-            len[s] = 0;
-            if (r + 1 < R) {  // the next row's window
-              const Words<STAGED> words(W[s]);
-              const uint32_t at = words.at(pos[s]), w1 = words.load(at, 1);
-              hi[s] = __funnelshift_l(w1, words.load(at, 0), pos[s]);
-              mid[s] = __funnelshift_l(words.load(at, 2), w1, pos[s]);
+                for (int s = 0; s < KS; ++s) {
+                  const Words<STAGED> words(W[s]);
+                  const uint32_t at = words.at(pos[s]);
+                  h[s] = __funnelshift_l(words.load(at, 1), words.load(at, 0), pos[s]);
+                }
+                lookup_all<INDEX>(ent, h, table);
+#pragma unroll
+                for (int s = 0; s < KS; ++s) {
+                  if (ent[s].y > 63u) ent[s] = long_code_at<STAGED>(S[s], Words<STAGED>(W[s]), pos[s], status);
+                  v = __fadd_rn(v, __uint_as_float(ent[s].x));
+                  pos[s] += ent[s].y;
+                }
+              }
+              x.x = x.y, x.y = x.z, x.z = x.w, x.w = v;
             }
+#pragma unroll
+            for (int s = 0; s < KS; ++s) len[s] = 0;
+          }
+          if (r + 1 < R) {  // the next row's window
+#pragma unroll
+            for (int s = 0; s < KS; ++s) {
+              const Words<STAGED> words(W[s]);
+              const uint32_t next = pos[s] + len[s], at = words.at(next), w1 = words.load(at, 1);
+              hi[s] = __funnelshift_l(w1, words.load(at, 0), next);
+              mid[s] = __funnelshift_l(words.load(at, 2), w1, next);
+            }
+            reloaded = true;
           }
         }
       }
