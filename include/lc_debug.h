@@ -54,6 +54,12 @@ int lc_debug_compress_wait(const float* base, const float* cur, uint64_t n, int 
  */
 uint32_t lc_debug_split_segments(const uint64_t* seg_begin, int nseg, uint32_t warps, uint32_t slots, uint32_t* cta_begin);
 
+/*
+ * How many warps of an SM decode side by side in a launch of lc_recover with k (1 to 4) streams whose payload has chunk_bytes bytes a
+ * chunk on average, if the kernel has `regs` registers a thread. Returns 0 on bad arguments. Needs no device.
+ */
+uint32_t lc_debug_decode_warps(int k, uint64_t chunk_bytes, uint32_t regs);
+
 #ifdef __cplusplus
 }
 #endif

@@ -23,7 +23,8 @@ SYMBOLS = (
     "lc_recover", "lc_compress_opt", "lc_compress_cached",
     "lc_segments_layout", "lc_compress_segments", "lc_recover_segments", "lc_debug_compress_wait", "lc_merge", "lc_compress_async", "lc_shard_stats", "lc_shard_encode",
     "lc_stream_info", "lc_last_status", "lc_wait", "lc_host_arena_bytes", "lc_compress_host", "lc_recover_host",
-    "lc_debug_bins", "lc_debug_codes", "lc_debug_split_segments", "lc_compress_noalloc",
+    "lc_debug_bins", "lc_debug_codes", "lc_debug_split_segments", "lc_debug_decode_warps",
+    "lc_compress_noalloc",
 )
 NOALLOC_MAX_N = 4194304
 
@@ -93,6 +94,8 @@ def lib():
     L.lc_debug_codes.argtypes = [vp, vp, vp]
     L.lc_debug_split_segments.argtypes = [C.POINTER(u64), i32, C.c_uint32, C.c_uint32, C.POINTER(C.c_uint32)]
     L.lc_debug_split_segments.restype = C.c_uint32
+    L.lc_debug_decode_warps.argtypes = [i32, u64, C.c_uint32]
+    L.lc_debug_decode_warps.restype = C.c_uint32
     _lib = L
     return L
 

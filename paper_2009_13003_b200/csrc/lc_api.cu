@@ -670,4 +670,6 @@ uint32_t lc_debug_split_segments(const uint64_t* seg_begin, int nseg, uint32_t w
   return ctas;
 }
 
+uint32_t lc_debug_decode_warps(int k, uint64_t chunk_bytes, uint32_t regs) { return decode_warps(k, chunk_bytes, regs); }
+
 }  // extern "C"

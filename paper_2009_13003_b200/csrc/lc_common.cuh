@@ -266,6 +266,8 @@ uint32_t split_segments(SegBatch& batch, uint32_t warps, uint32_t slots);
 cudaError_t launch_decode_segments(const float* base, const uint8_t* const* streams, int k, SegBatch& batch, int nbits,
                                    float* out, int32_t* status, bool second, cudaStream_t cs);
 
+// Warps on an SM in a launch with k streams whose chunks have chunk_bytes on average, by a kernel of so many registers a thread.
+uint32_t decode_warps(int k, uint64_t chunk_bytes, uint32_t regs);
 // How many streams the next launch takes, of `left` that remain of a chain.
 int decode_group(int left);
 // Decodes the chunks [chunk_begin, chunk_end) only (clipped to the vector's chunks). second: as above.

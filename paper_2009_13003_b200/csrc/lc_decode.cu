@@ -779,10 +779,14 @@ __device__ __forceinline__ void decode_chunk_one_level(const StreamState* S, con
 // average had 4.9 wavefronts a load instead of 2.1. Such a chunk is copied with 16 bytes of space before every fourth lane (the unit on a
 // boundary twice), which makes it 2.9 to 3.4. Not always: the copy then waits for the lane starts, and the space brings lanes together that
 // are well apart without it.
+constexpr uint32_t kSpaceUnit = 16, kSpaceNear = 77;  // 0.6 words a lane
+constexpr uint32_t kSpaceBytes = 7 * kSpaceUnit;
+__host__ __device__ constexpr bool spaced_chunk(uint64_t bytes) { return ((bytes + kSpaceNear) & 1023u) <= 2 * kSpaceNear; }
+
 template <int KS, bool ONE_LEVEL>
 __device__ __forceinline__ bool stage_chunk(const StreamState* S, uint32_t c, uint32_t lane, unsigned char* stage0,
                                             uint32_t stage_bytes, Source* W, uint32_t (&start)[KS], Status status) {
-  constexpr uint32_t kUnit = 16, kNear = 77;  // 0.6 words a lane
+  constexpr uint32_t kUnit = kSpaceUnit;
   uint32_t bytes[KS], filled = 0;
   unsigned long long off0[KS], off1[KS];
   // all index loads of all streams first, so that their latencies overlap
@@ -795,7 +799,7 @@ __device__ __forceinline__ bool stage_chunk(const StreamState* S, uint32_t c, ui
     const uint16_t* li = reinterpret_cast<const uint16_t*>(sp + S[s].lane_index_off);
     start[s] = __ldg(li + (uint64_t)c * kLanes + lane);
   }
-  const auto spaced = [](uint32_t bytes) { return ONE_LEVEL && ((bytes + kNear) & 1023u) <= 2 * kNear; };
+  const auto spaced = [](uint32_t bytes) { return ONE_LEVEL && spaced_chunk(bytes); };
   // the asynchronous copies of the payloads into the staging areas
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
@@ -809,7 +813,7 @@ __device__ __forceinline__ bool stage_chunk(const StreamState* S, uint32_t c, ui
     W[s].nw = bytes[s] >> 2;
     W[s].sbase = smem_addr(stage0) + filled;
     W[s].slim = W[s].sbase + bytes[s] + 12;
-    filled += bytes[s] + (spaced(bytes[s]) ? 7 * kUnit : 16);  // 16 bytes of zero slack after the chunk must fit too
+    filled += bytes[s] + (spaced(bytes[s]) ? kSpaceBytes : 16);  // 16 bytes of zero slack after the chunk must fit too
     if (filled <= KS * stage_bytes && !spaced(bytes[s])) {
       for (uint32_t k = lane * 16; k < bytes[s]; k += 32 * 16) cp_async_16(W[s].sbase + k, g + k);
       if (lane == 0) asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(W[s].sbase + bytes[s]), "r"(0) : "memory");
@@ -1031,14 +1035,54 @@ inline uint32_t ctas_on_sm(uint32_t warps, uint32_t dyn, uint32_t regs) {
   return min(min(by_regs, by_smem), by_warps);
 }
 
-// want_stage: staging bytes that hold an average chunk with some room. Among CTAs of 20 (two and three streams), 16, 12 and 8 warps, takes the shape
-// that puts most warps on an SM (with four streams that is one CTA of 16 warps, with one stream several smaller ones),
-// then gives the staging areas whatever shared memory that shape leaves (chunk sizes vary around the average).
+constexpr uint32_t kMaxStage = kChunkElems * 8 + 16;
+
+// Staging bytes a warp and stream that hold a chunk of `avg` bytes with some room (chunks vary, and the streams' areas are one), and its space
+// if such chunks are copied with space. Asked for in every case, the space took four of 16 warps from chunks of 2137 to 2206 bytes in
+// four streams, which have none: 134 M elements of 4.2 bits a code 325 us instead of 291.
+uint32_t wanted_stage(uint64_t avg) {
+  return (uint32_t)min(align_up(avg + avg / 32 + (spaced_chunk(avg) ? kSpaceBytes + 16 : 48), 16), (uint64_t)kMaxStage);
+}
+
+constexpr uint32_t tables_bytes(int ks) { return kTablePad + ks * (2 * kTableBytes + (uint32_t)sizeof(StreamState)); }
+constexpr uint32_t kMaxDyn = kSmemPerSm - 1024 - kOverrunBytes;  // room for static __shared__ and the padding
+
+// Among CTAs of `most` warps and four, eight, ... fewer, down to eight, the shape that puts most warps on an SM (with four streams that is
+// one CTA of 16 warps, with one stream several smaller ones), with the staging areas given whatever shared memory that shape leaves.
+Shape choose_shape(int ks, uint32_t want_stage, uint32_t regs, uint32_t most) {
+  const uint32_t tables = tables_bytes(ks);
+  if (want_stage > kMaxStage) want_stage = kMaxStage;
+  Shape best{};
+  for (uint32_t w = most; w >= 8; w -= 4) {
+    uint32_t st = want_stage;
+    if (tables + (uint64_t)w * ks * st > kMaxDyn) {
+      if (w > 8) continue;                               // try fewer warps first
+      st = ((kMaxDyn - tables) / (w * ks)) / 16 * 16;    // last resort: what fits; large chunks decode from global
+    }
+    const uint32_t d = tables + w * ks * st + kOverrunBytes, bps = ctas_on_sm(w, d, regs);
+    if (bps * w > best.per_sm * best.warps) {
+      best.warps = w;
+      best.stage = st;
+      best.dyn = d;
+      best.per_sm = bps;
+    }
+  }
+  if (best.per_sm == 0) return best;
+  const uint32_t budget = kSmemPerSm / best.per_sm - 1024 - 64;
+  if (budget > tables + kOverrunBytes) {
+    uint32_t st = ((budget - tables - kOverrunBytes) / (best.warps * ks)) / 16 * 16;
+    if (st > kMaxStage) st = kMaxStage;
+    const uint32_t d = tables + best.warps * ks * st + kOverrunBytes;
+    if (st > best.stage && d <= kMaxDyn + kOverrunBytes && ctas_on_sm(best.warps, d, regs) >= best.per_sm) {
+      best.stage = st;
+      best.dyn = d;
+    }
+  }
+  return best;
+}
+
 template <int KS>
-cudaError_t decode_shape(const void* fn, uint64_t want_stage, uint32_t (&regs_of)[kMaxDevices], Shape& best) {
-  constexpr uint32_t kTables = kTablePad + KS * (2 * kTableBytes + sizeof(StreamState));
-  constexpr uint32_t kMaxDyn = kSmemPerSm - 1024 - kOverrunBytes;  // room for static __shared__ and the padding
-  constexpr uint32_t kMaxStage = kChunkElems * 8 + 16;
+cudaError_t decode_shape(const void* fn, uint32_t want_stage, uint32_t (&regs_of)[kMaxDevices], Shape& best) {
   static int sms_of[kMaxDevices] = {};
   const int dev = current_device_index();
   if (dev < 0) return cudaErrorInvalidDevice;
@@ -1053,34 +1097,9 @@ cudaError_t decode_shape(const void* fn, uint64_t want_stage, uint32_t (&regs_of
     sms_of[dev] = v;
     regs_of[dev] = (uint32_t)at.numRegs;
   }
-  const uint32_t regs = regs_of[dev];
-  if (want_stage > kMaxStage) want_stage = kMaxStage;
-  best = Shape{0, 0, 0, 0, (uint32_t)sms_of[dev]};
-  for (uint32_t w = kDecThreads<KS> / 32; w >= 8; w -= 4) {
-    uint32_t st = (uint32_t)want_stage;
-    if (kTables + (uint64_t)w * KS * st > kMaxDyn) {
-      if (w > 8) continue;                               // try fewer warps first
-      st = ((kMaxDyn - kTables) / (w * KS)) / 16 * 16;   // last resort: what fits; large chunks decode from global
-    }
-    const uint32_t d = kTables + w * KS * st + kOverrunBytes, bps = ctas_on_sm(w, d, regs);
-    if (bps * w > best.per_sm * best.warps) {
-      best.warps = w;
-      best.stage = st;
-      best.dyn = d;
-      best.per_sm = bps;
-    }
-  }
+  best = choose_shape(KS, want_stage, regs_of[dev], kDecThreads<KS> / 32);
+  best.sms = (uint32_t)sms_of[dev];
   if (best.per_sm == 0) return cudaErrorLaunchOutOfResources;
-  const uint32_t budget = kSmemPerSm / best.per_sm - 1024 - 64;
-  if (budget > kTables + kOverrunBytes) {
-    uint32_t st = ((budget - kTables - kOverrunBytes) / (best.warps * KS)) / 16 * 16;
-    if (st > kMaxStage) st = kMaxStage;
-    const uint32_t d = kTables + best.warps * KS * st + kOverrunBytes;
-    if (st > best.stage && d <= kMaxDyn + kOverrunBytes && ctas_on_sm(best.warps, d, regs) >= best.per_sm) {
-      best.stage = st;
-      best.dyn = d;
-    }
-  }
   // shared-memory carve-out in percent of the SM's 228 KB: what the resident CTAs use (dynamic, static and the
   // 1 KB per CTA that the system reserves), so that whatever is left serves as L1
   const int carve = (int)(((uint64_t)best.per_sm * (best.dyn + 2048) * 100 + 228 * 1024 - 1) / (228 * 1024)) + 1;
@@ -1103,7 +1122,7 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
                              int32_t* status, bool second, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
   static uint32_t regs_of[kMaxDevices] = {};
   const uint64_t nchunks = (n + kChunkElems - 1) / kChunkElems;
-  // 1.03 x the largest average chunk of the streams and what its space may take (from the buffer sizes, which bound the payload)
+  // the largest average chunk of the streams (from the buffer sizes, which bound the payload)
   uint64_t avg = 0;
   for (int s = 0; s < KS; ++s) {
     const uint64_t index_bytes = 72 * nchunks;  // lane and chunk index entries are not staged
@@ -1111,8 +1130,7 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
     avg = a > avg ? a : avg;
   }
   Shape sh;
-  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_kernel<KS>), align_up(avg + avg / 32 + 128, 16),
-                                         regs_of, sh);
+  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_kernel<KS>), wanted_stage(avg), regs_of, sh);
   if (e != cudaSuccess) return e;
   const uint64_t chunks = chunk_end - chunk_begin, full = (uint64_t)sh.sms * sh.per_sm;
   const uint32_t warps = balanced_warps(chunks, full, sh.warps);
@@ -1134,7 +1152,7 @@ cudaError_t launch_segments_ks(const float* base, const uint8_t* const* streams,
   // the buffers are sized for nbits bits per element, which no chunk exceeds by much
   Shape sh;
   const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_segments_kernel<KS>),
-                                         align_up((uint64_t)nbits * (kChunkElems / 8) + 64, 16), regs_of, sh);
+                                         (uint32_t)align_up((uint64_t)nbits * (kChunkElems / 8) + 64, 16), regs_of, sh);
   if (e != cudaSuccess) return e;
   DecodeStreams buffers;
   for (int s = 0; s < 4; ++s) buffers.ptr[s] = s < KS ? streams[s] : nullptr, buffers.bytes[s] = 0;
@@ -1145,6 +1163,13 @@ cudaError_t launch_segments_ks(const float* base, const uint8_t* const* streams,
 }
 
 }  // namespace
+
+uint32_t decode_warps(int k, uint64_t chunk_bytes, uint32_t regs) {
+  if (k < 1 || k > 4 || regs < 16 || regs > 255) return 0;
+  const int threads = k == 1 ? kDecThreads<1> : k == 2 ? kDecThreads<2> : k == 3 ? kDecThreads<3> : kDecThreads<4>;
+  const Shape sh = choose_shape(k, wanted_stage(chunk_bytes), regs, threads / 32);
+  return sh.per_sm * sh.warps;
+}
 
 // How the CTAs are dealt out: every one takes up to r rounds (a chunk per warp) of one segment, the same r for all. While
 // all CTAs fit on the device at once, the launch takes as long as the preparation and r rounds, so the smallest such r is
