@@ -36,13 +36,15 @@ namespace {
 
 using namespace dec;
 
-// Threads per CTA at most, and CTAs per SM that the registers must allow: with one stream 24 warps fit on an SM as two CTAs
+// Warps per CTA at most, and CTAs per SM that the registers must allow: with one stream 24 warps fit on an SM as two CTAs
 // of 12 (80 registers); two streams fit one CTA of 20 (96 registers: 138 M elements 240 -> 220 us against 16 warps, 11.7 M
-// elements 46 -> 31 us, because their 19.3 chunks per SM are then one round), and so do three (11.7 M elements 48 -> 41 us); with four a
-// thread holds more state and one CTA of 16 takes the SM (18 or 20 warps of 96 registers: 134 M elements 307 us instead of 290, and
-// staging areas so small that a vector of layers took 243 us instead of 155).
+// elements 46 -> 31 us, because their 19.3 chunks per SM are then one round), and so do three (11.7 M elements 48 -> 31 us, 61,706 22 -> 17); with four
+// a thread holds more state and one CTA of 16 takes the SM (18 or 20 warps of 96 registers: 134 M elements 307 us instead of 290, and
+// staging areas so small that a vector of layers took 243 us instead of 155). With three streams there is a kernel for 16 warps of 128 registers too,
+// for flat vectors whose areas leave no room for 20 (uniform codes of 8 bits, 134 M elements 433 -> 415 us, 0.5 M 28.7 -> 26.7) and for layers
+// (62 of 11.7 M elements 48 -> 43 us, 20 of 4 M 28.7 -> 24.7).
 template <int KS>
-constexpr int kDecThreads = KS == 1 ? 384 : KS == 4 ? 512 : 640;
+constexpr int kDecWarps = KS == 1 ? 12 : KS == 4 ? 16 : 20;
 template <int KS>
 constexpr int kDecCtas = KS == 1 ? 2 : 1;
 constexpr int kL1Bits = 6;
@@ -1001,8 +1003,8 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   }
 }
 
-template <int KS>
-__global__ void __launch_bounds__(kDecThreads<KS>, kDecCtas<KS>)
+template <int KS, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, kDecCtas<KS>)
 decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status, uint32_t rank,
               uint32_t stage_bytes, uint32_t chunk_begin, uint32_t chunk_end) {
   decode_vector<KS>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
@@ -1010,8 +1012,8 @@ decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, 
 
 // Per-layer recovery: the CTAs [cta_begin[i], cta_begin[i + 1]) decode segment i. One launch instead of one per segment
 // (a segment of a few chunks occupies one SM for the 15 us that a chunk takes; 62 of them in a row took 870 us).
-template <int KS>
-__global__ void __launch_bounds__(kDecThreads<KS>, kDecCtas<KS>)
+template <int KS, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, kDecCtas<KS>)
 decode_segments_kernel(const float* base, const __grid_constant__ DecodeStreams buffers, float* out,
                        int32_t* __restrict__ status, uint32_t second, uint32_t stage_bytes,
                        const __grid_constant__ SegBatch batch) {
@@ -1094,7 +1096,7 @@ Shape choose_shape(int ks, uint32_t want_stage, uint32_t regs, uint32_t most) {
   return best;
 }
 
-template <int KS>
+template <int KS, int WARPS>
 cudaError_t decode_shape(const void* fn, uint32_t want_stage, uint32_t (&regs_of)[kMaxDevices], Shape& best) {
   static int sms_of[kMaxDevices] = {};
   const int dev = current_device_index();
@@ -1110,7 +1112,7 @@ cudaError_t decode_shape(const void* fn, uint32_t want_stage, uint32_t (&regs_of
     sms_of[dev] = v;
     regs_of[dev] = (uint32_t)at.numRegs;
   }
-  best = choose_shape(KS, want_stage, regs_of[dev], kDecThreads<KS> / 32);
+  best = choose_shape(KS, want_stage, regs_of[dev], WARPS);
   best.sms = (uint32_t)sms_of[dev];
   if (best.per_sm == 0) return cudaErrorLaunchOutOfResources;
   // shared-memory carve-out in percent of the SM's 228 KB: what the resident CTAs use (dynamic, static and the
@@ -1130,7 +1132,7 @@ uint32_t balanced_warps(uint64_t chunks, uint64_t ctas, uint32_t most) {
   return w < 4 ? 4 : (uint32_t)w;
 }
 
-template <int KS>
+template <int KS, int WARPS = kDecWarps<KS>>
 cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
                              int32_t* status, bool second, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
   static uint32_t regs_of[kMaxDevices] = {};
@@ -1142,8 +1144,12 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
     const uint64_t a = (streams.bytes[s] > index_bytes ? streams.bytes[s] - index_bytes : 0) / (nchunks ? nchunks : 1);
     avg = a > avg ? a : avg;
   }
+  // where the areas of 20 warps do not fit, the kernel for 16
+  if constexpr (KS == 3 && WARPS == 20)
+    if (choose_shape(KS, wanted_stage(avg), 96, WARPS).warps < WARPS)
+      return launch_decode_ks<KS, 16>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
   Shape sh;
-  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_kernel<KS>), wanted_stage(avg), regs_of, sh);
+  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(decode_kernel<KS, WARPS>), wanted_stage(avg), regs_of, sh);
   if (e != cudaSuccess) return e;
   const uint64_t chunks = chunk_end - chunk_begin, full = (uint64_t)sh.sms * sh.per_sm;
   const uint32_t warps = balanced_warps(chunks, full, sh.warps);
@@ -1153,24 +1159,24 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
   // the staging areas of the warps left out go to the others: chunks vary (a layer of rare exponents in a vector of layers
   // takes twice the average), and one that is read from global memory word by word holds up the launch
   const uint32_t stage = min(sh.warps * sh.stage / warps / 16 * 16, kChunkElems * 8 + 16);
-  decode_kernel<KS><<<grid, warps * 32, sh.dyn - (sh.warps * sh.stage - warps * stage) * KS, cs>>>(base, streams, n, out, status, second ? 1u : 0u,
+  decode_kernel<KS, WARPS><<<grid, warps * 32, sh.dyn - (sh.warps * sh.stage - warps * stage) * KS, cs>>>(base, streams, n, out, status, second ? 1u : 0u,
                                                                                                   stage, (uint32_t)chunk_begin, (uint32_t)chunk_end);
   return cudaGetLastError();
 }
 
-template <int KS>
+template <int KS, int WARPS = KS == 3 ? 16 : kDecWarps<KS>>
 cudaError_t launch_segments_ks(const float* base, const uint8_t* const* streams, SegBatch& batch, int nbits, float* out,
                                int32_t* status, bool second, cudaStream_t cs) {
   static uint32_t regs_of[kMaxDevices] = {};
   // the buffers are sized for nbits bits per element, which no chunk exceeds by much
   Shape sh;
-  const cudaError_t e = decode_shape<KS>(reinterpret_cast<const void*>(decode_segments_kernel<KS>),
+  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(decode_segments_kernel<KS, WARPS>),
                                          (uint32_t)align_up((uint64_t)nbits * (kChunkElems / 8) + 64, 16), regs_of, sh);
   if (e != cudaSuccess) return e;
   DecodeStreams buffers;
   for (int s = 0; s < 4; ++s) buffers.ptr[s] = s < KS ? streams[s] : nullptr, buffers.bytes[s] = 0;
   const uint32_t ctas = split_segments(batch, sh.warps, sh.sms * sh.per_sm);
-  decode_segments_kernel<KS><<<ctas, sh.warps * 32, sh.dyn, cs>>>(base, buffers, out, status, second ? 1u : 0u, sh.stage,
+  decode_segments_kernel<KS, WARPS><<<ctas, sh.warps * 32, sh.dyn, cs>>>(base, buffers, out, status, second ? 1u : 0u, sh.stage,
                                                                            batch);
   return cudaGetLastError();
 }
@@ -1179,8 +1185,8 @@ cudaError_t launch_segments_ks(const float* base, const uint8_t* const* streams,
 
 uint32_t decode_warps(int k, uint64_t chunk_bytes, uint32_t regs) {
   if (k < 1 || k > 4 || regs < 16 || regs > 255) return 0;
-  const int threads = k == 1 ? kDecThreads<1> : k == 2 ? kDecThreads<2> : k == 3 ? kDecThreads<3> : kDecThreads<4>;
-  const Shape sh = choose_shape(k, wanted_stage(chunk_bytes), regs, threads / 32);
+  const int most = k == 1 ? kDecWarps<1> : k == 2 ? kDecWarps<2> : k == 3 ? kDecWarps<3> : kDecWarps<4>;
+  const Shape sh = choose_shape(k, wanted_stage(chunk_bytes), regs, most);
   return sh.per_sm * sh.warps;
 }
 
