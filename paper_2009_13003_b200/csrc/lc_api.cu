@@ -355,7 +355,7 @@ int lc_recover_segments(const float* base, const void* const* streams, int k, co
     // up to four streams of every segment per launch; later launches continue in place from `out`
     for (int first = 0, kk; first < k; first += kk) {
       const uint8_t* group[4];
-      kk = decode_group(k - first);
+      kk = decode_group_segments(k - first, nbits);
       for (int j = 0; j < kk; ++j) group[j] = static_cast<const uint8_t*>(streams[first + j]);
       if (launch_decode_segments(first == 0 ? base : out, group, kk, batch, nbits, out, &ctl->status, first > 0, cs) != cudaSuccess)
         return LC_ERR_CUDA;

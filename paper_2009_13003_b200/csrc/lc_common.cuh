@@ -270,6 +270,7 @@ cudaError_t launch_decode_segments(const float* base, const uint8_t* const* stre
 uint32_t decode_warps(int k, uint64_t chunk_bytes, uint32_t regs);
 // How many streams the next launch takes, of `left` that remain of a chain.
 int decode_group(int left);
+int decode_group_segments(int left, int nbits);  // the same for layers coded with nbits
 // Decodes the chunks [chunk_begin, chunk_end) only (clipped to the vector's chunks). second: as above.
 cudaError_t launch_decode(const float* base, const DecodeStreams& streams, int k, uint64_t n, float* out,
                           int32_t* status, bool second, cudaStream_t cs, uint64_t chunk_begin = 0, uint64_t chunk_end = ~0ull);

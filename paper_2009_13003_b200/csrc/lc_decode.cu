@@ -1245,7 +1245,11 @@ uint32_t split_segments(SegBatch& batch, uint32_t warps, uint32_t slots) {
 // Four at a time, but five as three and two: a launch with one stream is bound by HBM and takes as long as one with two (1.3 G elements: four
 // and one 4602 us, three and two 4023). (Eight as three, three and two, where 16 warps an SM need two rounds and 20 one: 11.7 M elements of 62
 // layers 214 us instead of 155, because the smaller staging areas do not hold the chunks of some layers.)
+// Layers of up to 4 bits stay four and one: their areas, sized by nbits, let four streams have as many warps as three, and the launch with one ends
+// soonest (62 layers, 11.7 M, 3 and 4 bits: 76 and 74 us, three and two 84 and 80; 40 layers, 16 M, 94 and 93, 88 and 91). With 5 and 6 bits four
+// streams get fewer (62 layers 83 and 97, three and two 83 and 91; 40 layers 105 and 120, 92 and 101).
 int decode_group(int left) { return left <= 4 ? left : left == 5 ? 3 : 4; }
+int decode_group_segments(int left, int nbits) { return nbits <= 4 ? (left <= 4 ? left : 4) : decode_group(left); }
 
 cudaError_t launch_decode_segments(const float* base, const uint8_t* const* streams, int k, SegBatch& batch, int nbits,
                                    float* out, int32_t* status, bool second, cudaStream_t cs) {
