@@ -11,7 +11,8 @@
 //  * The chunk's payload of every stream is first copied, coalesced, into a warp-private staging
 //    area in shared memory; the lanes then pull their words from there. (Reading them straight from
 //    global memory makes every refill touch one cache line per lane.) A chunk that does not fit the
-//    staging area takes the streams one after the other, or is decoded from global memory by the same code.
+//    staging area takes the streams one after the other with tables of one level, and what then does not fit, or any with two levels, is
+//    decoded from global memory by the same code.
 //  * Codes are looked up in shared-memory tables whose entries hold the representative itself, 16 copies of each: a 64-bit
 //    shared load is served half a warp at a time, so 16 lanes that read copies of their own always hit 16 different bank
 //    pairs although their indices are data dependent.
@@ -645,7 +646,7 @@ __device__ __forceinline__ uint2 long_code_at(const StreamState& S, const Words<
 // Only what is left goes through the row again, one code at a time. They are rare on the whole (four streams in 6 bits: 0.3 to 1.4 % of a
 // warp's rows), but a chunk of rare exponents has nothing else, and a launch of one round waits for it. With all of them one code at a time, four
 // streams of 11.7 M elements in 62 scales took 57 us instead of 41; two of 134 M, 10 % in rare exponents, 311 instead of 226.
-// Every code has at most 63 bits, so a lane of a damaged stream reads at most 1020 bytes beyond its chunk (kOverrunBytes).
+// Every code has at most 63 bits, so a lane of a damaged stream reads at most 1013 bytes beyond its chunk (kOverrunBytes).
 // PARTIAL: the vector's last chunk, or any chunk larger than the staging area: of each row only the slots that exist are read and written. (A
 // lane's codes end with its last element; nothing is reported for what it decodes behind it.)
 // next_chunk: floats from this chunk to the one the warp takes next, whose first rows are asked into the L2 behind this one's last; 0 if there is none.

@@ -9,7 +9,10 @@ namespace lc {
 namespace dec {
 
 constexpr uint32_t kSmemPerSm = 227 * 1024;  // usable shared memory of one CTA on sm_100
-constexpr uint32_t kOverrunBytes = 1024;     // padding behind the last staging area (see LaneBits::refill and decode_chunk_ones)
+constexpr uint32_t kOverrunBytes = 1024;     // padding behind the last staging area (see LaneBits::refill and decode_chunk_one_level)
+// A lane starts within its chunk (stage_chunk sees to it) and has 128 codes of at most 63 bits: the last begins behind 127 of them, and three words
+// are read there.
+static_assert((kChunkElems / kLanes - 1) * 63 / 8 + 1 + 12 <= kOverrunBytes, "a damaged stream's lanes read stale shared memory, never beyond it");
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -115,7 +118,7 @@ struct LaneBits {
 };
 
 // The words around a bit position of a chunk. STAGED: positions are bit addresses in shared memory, and nothing is clamped (see
-// decode_chunk_ones). Otherwise they count from the chunk's start and words beyond its end are 0.
+// decode_chunk_one_level). Otherwise they count from the chunk's start and words beyond its end are 0.
 template <bool STAGED>
 struct Words;
 template <>
