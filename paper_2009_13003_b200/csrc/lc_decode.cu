@@ -792,10 +792,12 @@ __device__ __forceinline__ void decode_chunk_one_level(const StreamState* S, con
 // a lane's codes take, give or take a few, and if that is near a multiple of 8 words, they meet in a few banks: codes of 4.05 bits on
 // average had 4.9 wavefronts a load instead of 2.1. Such a chunk is copied with 16 bytes of space before every fourth lane (the unit on a
 // boundary twice), which makes it 2.9 to 3.4. Not always: the copy then waits for the lane starts, and the space brings lanes together that
-// are well apart without it.
-constexpr uint32_t kSpaceUnit = 16, kSpaceNear = 77;  // 0.6 words a lane
+// are well apart without it. So a chunk has space from 19 bytes below a multiple of 1024 to 38 above (0.15 and 0.3 words a lane). 134 M elements,
+// four streams: chunks about 30 above, log-normal deltas, 323 us with space and 339 without; but 48 above 363 and 287, 32 below (5.9 bits) 382 and
+// 353, 74 below 294 and 276.
+constexpr uint32_t kSpaceUnit = 16, kSpaceBelow = 19, kSpaceAbove = 38;
 constexpr uint32_t kSpaceBytes = 7 * kSpaceUnit;
-__host__ __device__ constexpr bool spaced_chunk(uint64_t bytes) { return ((bytes + kSpaceNear) & 1023u) <= 2 * kSpaceNear; }
+__host__ __device__ constexpr bool spaced_chunk(uint64_t bytes) { return ((bytes + kSpaceBelow) & 1023u) <= kSpaceBelow + kSpaceAbove; }
 
 template <int KS, bool ONE_LEVEL>
 __device__ __forceinline__ bool stage_chunk(const StreamState* S, uint32_t c, uint32_t lane, unsigned char* stage0,

@@ -13,7 +13,7 @@ from test_gpu_parity import DEV, assert_recover_parity
 pytestmark = pytest.mark.gpu
 
 # "long tail" with chunks of its rarest bucket: larger than the staging area
-CASES = ["twenty of four and five bits", "up to seven bits", "four bits on average", "up to eight bits", "long tail",
+CASES = ["twenty of four and five bits", "up to seven bits", "two bits on average", "up to eight bits", "long tail",
          "two hundred of seven and eight bits"]
 
 
