@@ -28,8 +28,8 @@
 // out-of-bounds access.
 //
 // Bound: HBM at k = 1 and 2 (8 bytes per element + the streams: 1.75 and 1.72 ms for 1.3 G elements in 5 bits); at k = 4 issue slots
-// (58 % busy) and shared-memory wavefronts (61 %) side by side, 2.56 to 2.88 ms where the two levels alone took 3.0 to 3.3. Instructions per
-// element and warp at k = 4: 47, with the two levels 72.
+// (58 % busy) and shared-memory wavefronts (62 %) side by side, 2.5 to 2.8 ms where the two levels alone took 3.0 to 3.3. A launch of 2^26 elements in
+// four streams executes 49 instructions per element and warp, with the two levels 72.
 #include "lc_decode_bits.cuh"
 
 namespace lc {
@@ -975,10 +975,11 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   }
   // Prefixes that any of the streams resolves in the second level are looked up there in all of them, in sub-tables as
   // deep as their number allows: the lookup's addressing is then the same for all streams.
-  uint32_t most = 0, sub_bits = kSubBitsMax;  // these and what follows are the same for every thread
+  uint32_t most = 0;  // this and what follows are the same for every thread
 #pragma unroll
   for (int s = 0; s < KS; ++s) most = max(most, S[s].misses);
-  while (sub_bits > kSubBitsMin && most > (kTableBytes >> (sub_bits + 3))) sub_bits -= 1;
+  static_assert(kTableBytes / 8 == 1u << 10 && kSubBitsMax == 9 && kSubBitsMin == 4, "sub-tables of 10 - ceil(log2 most) bits fill the second level");
+  const uint32_t sub_bits = __clz(max(most, 2u) - 1) - 22;  // 9 to 4
   if (threadIdx.x < KS) {
     S[threadIdx.x].nsub = most;
     S[threadIdx.x].sub_bits = sub_bits;
