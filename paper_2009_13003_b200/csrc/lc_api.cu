@@ -89,7 +89,8 @@ int compress_impl(const float* base, const float* cur, uint64_t n, int nbits, vo
   // outcome of the pass that produced `cur`; the table pass then leaves the vector alone if it is set)
   // The four kernels are launched so that each may begin before the one ahead of it has ended.
   const uint64_t control = opt.mean_rep ? sizeof(Control) : offsetof(Control, enc);  // the sums of the variant lie behind enc
-  cudaError_t e = launch_clear(c.ctl, control, c.tiles, align_up(8 * W.nchunks, 16), keep_status, cs);
+  const uint64_t groups = scan_group_words(W.nchunks);
+  cudaError_t e = launch_clear(c.ctl, control, c.tiles - groups, 8 * groups + align_up(8 * W.nchunks, 16), keep_status, cs);
   if (e != cudaSuccess) return LC_ERR_CUDA;
   if ((e = launch_stats(base, cur, n, c.ctl, c.plane, cs, opt.mean_rep, true)) != cudaSuccess) return LC_ERR_CUDA;
   if ((e = launch_table(c.ctl, n, nbits, static_cast<uint8_t*>(stream), true, opt.fixed_width, nullptr, opt.length_cache, cs,
@@ -417,7 +418,8 @@ int lc_shard_encode(const float* base, const float* cur, uint64_t n, int nbits, 
   if (workspace_bytes < W.total || stream_capacity < lc_stream_bound(n, nbits)) return LC_ERR_CAPACITY;
   const Carved c = carve(workspace, W);
   // the statistics of a shard may be coded more than once: the encode pass's scan starts from zero each time
-  if (cudaMemsetAsync(c.tiles, 0, 8 * W.nchunks, cs) != cudaSuccess) return LC_ERR_CUDA;
+  const uint64_t groups = scan_group_words(W.nchunks);
+  if (cudaMemsetAsync(c.tiles - groups, 0, 8 * (groups + W.nchunks), cs) != cudaSuccess) return LC_ERR_CUDA;
   if (launch_table(c.ctl, n, nbits, static_cast<uint8_t*>(stream), true, false,
                    static_cast<const ShardStats*>(whole_stats), nullptr, cs) != cudaSuccess)
     return LC_ERR_CUDA;

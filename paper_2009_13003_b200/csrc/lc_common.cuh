@@ -52,10 +52,16 @@ constexpr uint32_t kUnitsPerChunk = kChunkElems / kUnitElems;
 // ---- encode pass ----------------------------------------------------------------------------------
 constexpr uint32_t kEncWarps = 8;  // warps per CTA of the encode pass (one chunk per warp at a time)
 
-// Chunk descriptor of the decoupled look-back scan of the encode pass: flag in the top two bits, bytes below.
+// Tile descriptor of the scan of the encode pass: flag in the top two bits, bytes below.
 constexpr uint64_t kTileFlagShift = 62;
 constexpr uint64_t kTileInvalid = 0, kTileAggregate = 1, kTilePrefix = 2, kTileAbort = 3;
 constexpr uint64_t kTileValueMask = (1ull << kTileFlagShift) - 1;
+// The encode pass for one vector also adds the tiles of kScanGroupChunks chunks up in a word of their own: how many of them have a
+// size yet (at most 256) above kGroupCountShift, their bytes below, and from the group's first tile, once it knows its offset, that offset
+// and flag kTilePrefix. All of it by atomic additions, so that their order does not matter: a word is complete when all tiles are in it.
+constexpr uint32_t kScanGroupChunks = 256;
+constexpr uint64_t kGroupCountShift = 53;
+constexpr uint64_t kGroupValueMask = (1ull << kGroupCountShift) - 1;
 
 // Entry of the per-key encode table written by the table kernel.
 struct EncEntry {
@@ -95,8 +101,13 @@ static_assert(sizeof(Control) % 256 == 0, "control block must keep the planes 25
 
 // A region behind the control block whose size does not depend on n. The per-layer compress puts the blocks and scan
 // descriptors of a group of segments over it and what follows: without it a workspace for n elements would not hold those
-// of one segment of n elements. The passes for one vector leave it alone.
+// of one segment of n elements. The passes for one vector keep the group words of their scan at its end, in front of the tiles'
+// descriptors, so that one range is cleared.
 constexpr uint32_t kSpareRegionBytes = 96 * 1024;
+__host__ __device__ constexpr inline uint64_t scan_group_words(uint64_t nchunks) {  // an even number
+  return align_up((nchunks + kScanGroupChunks - 1) / kScanGroupChunks, 2);
+}
+static_assert(8 * scan_group_words(1ull << 20) <= kSpareRegionBytes, "the groups of the largest vector");
 
 struct WorkspaceLayout {
   uint64_t control_off, spare_off, tiles_off, plane_off, total;
@@ -204,6 +215,7 @@ cudaError_t launch_stats(const float* base, const float* cur, uint64_t n, Contro
 //        kept buckets, representatives and code then come from them, the table's counts from ctl's own
 cudaError_t launch_table(Control* ctl, uint64_t n, int nbits, uint8_t* stream, bool wide_ok, bool fixed,
                          const ShardStats* whole, uint8_t* length_cache, cudaStream_t cs, bool mean = false, bool overlap = false);
+// tiles: one word per chunk, behind scan_group_words(chunks) others; zero
 // tracked_out: nullptr, or where to write base + quantized delta (may be base itself)
 cudaError_t launch_encode(Control* ctl, unsigned long long* tiles, const uint8_t* plane, const float* base,
                           const float* cur, uint64_t n, uint8_t* stream, float* tracked_out, const EncodeOptions& opt,

@@ -8,15 +8,14 @@
 //   A. every lane codes its 128 elements into its own column of a warp-private word matrix in shared
 //      memory (word k of lane t at k*32 + t: plain stores, no bank conflicts, no atomics). Two elements are looked up at
 //      once in a table of pairs whose index is formed for all four elements of a step together (lc_encode_bits.cuh),
-//      and the step's codes are appended as one, so a step of four elements costs two lookups and one append. With a
-//      lookup per element and an append per two the pass took 0.99 ms for 1.3 G elements
-//      (5 bits), now 0.775 ms;
+//      and the step's codes are appended as one, so a step of four elements costs two lookups and one append. The table's entries
+//      are spread so that lookups meet little in banks (268 M elements 173 -> 166 us);
 //   B. a warp shuffle scan of the lane bit counts gives every lane its bit offset in the chunk (the
 //      lane index of the stream) and the chunk its size, which is published at once;
-//   C. the lanes' words are shifted to their bit offsets and ORed into the chunk image (shared memory);
+//   C. the lanes' words are shifted to their bit offsets and written to the chunk image (shared memory);
 //   D. the tile's byte offset comes from an exclusive scan over all tiles, done across CTAs with a
-//      decoupled look-back over per-tile descriptors (per-chunk descriptors were tried: with thousands
-//      of chunks in flight every look-back walks too far back);
+//      decoupled look-back over per-tile descriptors and words that sum up groups of 32 tiles (per-chunk descriptors were tried: with
+//      thousands of chunks in flight every look-back walks too far back, and so it does over 592 tiles in flight);
 //   E. the chunk image is copied to the payload with coalesced 16-byte stores.
 // The loop is software-pipelined: D and E of a tile run after A and B of the CTA's next tile (whose C follows
 // once E has freed the image area), and D is done by whichever warp finishes coding first (see the loop). Tiles are handed out by an atomic ticket, so
@@ -33,7 +32,10 @@
 // exponent field >= 128, for which the one-byte key plane is not enough and keys come from base and cur.
 //
 // Bound: reads 1 byte and writes about 0.5 bytes per element, so this pass is limited by the integer work per element,
-// not by HBM: logic, shifts, permutes and compares issue at 64 lanes per clock and SM, half the rate of multiply-adds.
+// not by HBM: logic, shifts, permutes and compares issue at 64 lanes per clock and SM, half the rate of multiply-adds. 268 M elements in 5 bits take
+// 147 us (Gaussian deltas 143), 62 for the bytes alone; with lookups and appends left out 100. Tried and not kept: warps that wait for each other through
+// barriers in shared memory instead of the block's (147), one vote for two rows (148; Gaussian 163), an append of nine instructions instead of ten that
+// counts all bits (148), and one of seven that splits a code with a 64-bit multiply-add (174 instead of 169).
 #include "lc_encode_bits.cuh"
 
 namespace lc {
@@ -52,7 +54,7 @@ __host__ __device__ constexpr uint64_t share_need(uint64_t avg) { return avg + a
 static_assert(share_need(kChunkElems * 5 / 8) <= kEncSmem / kEncWarps / 2, "codes of 5 bits throughout are coded by all warps");
 constexpr int kUpdRows = 4;  // rows of base in flight per warp in the kernel that also writes the tracked state
 constexpr uint32_t kUpdSmem = kEncWarps * kUpdRows * 512;  // its ring, behind the kEncSmem bytes of coding areas
-constexpr int kLookBack = 8;  // look-back sub-windows of 32 tile descriptors read per round
+constexpr int kGroupWindows = 2;  // sub-windows of 32 group words that a round of the look-back reads
 
 // UPDATE: the kernel also writes the tracked state of Algorithm 1 step 7, tracked_out = base + quantized delta
 // (fp32, the representative of the zero bucket, +0, added like any other): inside the coding loop for the chunks
@@ -64,13 +66,15 @@ __global__ void __launch_bounds__(kEncThreads, UPDATE ? 3 : 4)
 encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles, const uint8_t* __restrict__ plane,
               const float* base, const float* __restrict__ cur, uint64_t n, uint8_t* __restrict__ stream,
               float* tracked_out, uint32_t spin_limit, uint32_t ticket_bias, uint32_t two_pass_scan) {
-  extern __shared__ __align__(16) uint32_t s_dyn[];
+  extern __shared__ __align__(128) uint32_t s_dyn[];  // rows that straddle lines cost the asynchronous copies of UPDATE 5 %
   __shared__ Tables tb;
-  __shared__ uint32_t s_chunk_bytes[2][kEncWarps];  // [half][warp]: the pending tile and the one being coded
-  __shared__ uint32_t s_tile;
-  __shared__ unsigned long long s_tile_base, s_tile_end;
-  __shared__ int s_abort;
-  __shared__ uint32_t s_arrived[2];  // warps that have coded their chunk of the tile in this half
+  // What warps hand each other in iteration i of the loop. A warp may reach the next iteration's barrier while another is still behind this one's, so
+  // the words alternate: those read behind the iteration's barrier by i % 2, those that the next iteration reads too by i % 3.
+  __shared__ uint32_t s_chunk_bytes[3][kEncWarps];
+  __shared__ uint32_t s_arrived[3];  // warps that have coded their chunk
+  __shared__ uint32_t s_tile[2];     // the tile to be coded next
+  __shared__ unsigned long long s_tile_base[2], s_tile_end[2];  // of the pending tile
+  __shared__ int s_abort[2];
   __shared__ uint32_t s_rep[UPDATE ? 256 : 1];  // UPDATE: representative (bit pattern) by plane byte
 
   wait_previous();
@@ -78,10 +82,13 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   // The table pass may have rejected the vector, or another CTA may already have given up waiting: leave, all
   // threads together (one thread reads the word; a thread-by-thread test could split the CTA if the word changed
   // in between, and the warps that stayed would wait at barriers for the ones that left).
-  if (tid == 0) s_abort = ctl->status;
+  if (tid == 0) {
+    s_abort[0] = ctl->status;
+    s_tile[0] = atomicAdd(&ctl->ticket, 1u) + ticket_bias;
+    s_arrived[0] = s_arrived[1] = s_arrived[2] = 0;
+  }
   __syncthreads();
-  if (s_abort != 0) return;
-  __syncthreads();  // everybody has read s_abort before thread 0 reuses it below
+  if (s_abort[0] != 0) return;
   for (uint32_t b = tid; b < 256; b += kEncThreads) {
     const EncEntry e = ctl->enc[((b & 1u) << 8) | (b >> 1)];
     tb.full[b] = make_uint2(e.code_lo, e.len);
@@ -96,7 +103,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   const bool long_codes = ctl->max_len > 32;
   const KeySource ks{plane, base, cur, ctl->wide != 0};
   const StreamLayout L = stream_layout(n, nsym);
-  const uint64_t nchunks = L.nchunks;
+  const uint32_t nchunks = (uint32_t)L.nchunks, whole = (uint32_t)(n / kChunkElems);  // at most 2^20 chunks
   unsigned long long* chunk_index = reinterpret_cast<unsigned long long*>(stream + L.chunk_index_off);
   uint16_t* lane_index = reinterpret_cast<uint16_t*>(stream + L.lane_index_off);
   uint8_t* payload = stream + L.payload_off;
@@ -111,9 +118,11 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   const uint32_t neg_base = (uint32_t)(-tb.base) & 0xffffu, neg_base2 = neg_base << 16 | neg_base;
   const bool use_pair = tb.use_pair != 0;
 
-  auto fast_chunk = [&](uint64_t cc) { return cc < nchunks && (cc + 1) * kChunkElems <= n && !long_codes && !ks.wide; };
+  auto fast_chunk = [&](uint32_t cc) { return cc < whole && !long_codes && !ks.wide; };
 
-  const uint64_t ntiles = (nchunks + active - 1) / active;
+  const uint32_t ntiles = (nchunks + active - 1) / active;
+  const uint32_t group_tiles = kScanGroupChunks / active;
+  unsigned long long* groups = tiles - scan_group_words(nchunks);
 
   // The loop is software-pipelined over tiles: a tile's offset is looked up, and its image copied out, only
   // after the *next* tile has been coded. Every earlier tile needs its size before this one can be placed, and
@@ -123,22 +132,15 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   // What the pending tile needs later is kept in shared memory (its chunk sizes; the lanes' start bits, in the image area
   // of a chunk that has no image because it is too large) or
   // recomputed from its number: phase A has no registers to spare.
+  // There is one barrier an iteration, behind coding: the first warp that gets there takes the next ticket and looks up the pending tile's
+  // offset while the others are still coding, the last one publishes the tile's size.
   bool p_have = false;
-  uint32_t p_tile = 0, p_buf = 0;
-
-  if (tid == 0) {
-    s_tile = atomicAdd(&ctl->ticket, 1u) + ticket_bias;
-    s_abort = 0;
-    s_arrived[0] = s_arrived[1] = 0;
-  }
+  uint32_t p_tile = 0, parity = 0, buf = 0, p_buf = 2;
+  uint32_t tile = s_tile[0];
   while (true) {
-    __syncthreads();  // the ticket taken during the previous iteration is visible; that iteration is done
-                      // with the other half of s_chunk_bytes
-    const uint64_t tile = s_tile;
     const bool have = tile < ntiles;
     if (!have && !p_have) break;
-    const uint32_t buf = p_buf ^ 1u;
-    const uint64_t c = tile * active + warp;
+    const uint32_t c = tile * active + warp;
     const bool valid = have && warp < active && c < nchunks;
     bool fast = valid && fast_chunk(c);
 
@@ -146,15 +148,15 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     // appends, which depend on each other through the bit accumulator.
     uint32_t lane_bits = 0;
     if (fast) {
-      const uint4* ep = reinterpret_cast<const uint4*>(plane + c * kChunkElems) + lane;
+      const uint4* ep = reinterpret_cast<const uint4*>(plane + (uint64_t)c * kChunkElems) + lane;
       const uint32_t col0 = smem_addr(column) + lane * 4;
       ColumnPacker pk{0u, 0u, col0, col0 + lane_words * 128};
       // UPDATE: the tracked state of this chunk is written here, where its plane bytes are in registers; the
       // memory traffic of the update then runs under the coding, which is bound by instruction issue. A chunk on
       // this path never reads base for its coding (not even when it is coded again the slow way), so base may be
       // overwritten at once. Row j of base is requested while row j - 1 is coded.
-      const float4* b4 = reinterpret_cast<const float4*>(base + c * kChunkElems) + lane;
-      float4* o4 = reinterpret_cast<float4*>(tracked_out + c * kChunkElems) + lane;
+      const float4* b4 = reinterpret_cast<const float4*>(base + (uint64_t)c * kChunkElems) + lane;
+      float4* o4 = reinterpret_cast<float4*>(tracked_out + (uint64_t)c * kChunkElems) + lane;
       // Rows of base come through a ring of kUpdRows 512-byte slots per warp behind the coding areas, filled by
       // cp.async four rows ahead: that many loads in flight per lane would not fit the registers, and the kernel's
       // L1 is too small to help. A lane reads back only the 16 bytes it copied itself, so no barrier is needed.
@@ -191,7 +193,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
       else code_rows<false>(pk, tb, neg_base2, load, row);
       lane_bits = finish_column(pk, col0);
     } else if (valid && !long_codes && !ks.wide) {
-      lane_bits = code_partial(&tb, reinterpret_cast<const uint4*>(plane + c * kChunkElems) + lane, (uint32_t)(n - c * kChunkElems),
+      lane_bits = code_partial(&tb, reinterpret_cast<const uint4*>(plane + (uint64_t)c * kChunkElems) + lane, (uint32_t)(n - (uint64_t)c * kChunkElems),
                                lane, smem_addr(column) + lane * 4, lane_words);
       fast = true;
     }
@@ -210,96 +212,128 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     const uint32_t chunk_bits = __shfl_sync(0xffffffffu, incl, 31);
     const uint32_t chunk_bytes = valid ? (uint32_t)align_up((chunk_bits + 7) / 8, kPayloadAlign) : 0u;
     const bool staged = chunk_bytes <= image_words * 4;
-    // The warp that gets here first looks up the pending tile's offset (D) while the others are still coding.
     uint32_t arrival = 0;
     if (lane == 0) {
       s_chunk_bytes[buf][warp] = chunk_bytes;
+      __threadfence_block();
       arrival = atomicAdd(&s_arrived[buf], 1u);
     }
     arrival = __shfl_sync(0xffffffffu, arrival, 0);
+    if (arrival == kEncWarps - 1 && have && !two_pass_scan) {
+      uint32_t bytes = 0;
+      if (lane < kEncWarps) bytes = *reinterpret_cast<volatile uint32_t*>(&s_chunk_bytes[buf][lane]);
+      bytes = __reduce_add_sync(0xffffffffu, bytes);
+      if (lane == 0) {
+        st_tile(&tiles[tile], (kTileAggregate << kTileFlagShift) | bytes);
+        atomicAdd(&groups[tile / group_tiles], (1ull << kGroupCountShift) | bytes);
+      }
+    }
 
-    // ---- D: exclusive prefix of the pending tile by decoupled look-back
-    if (p_have && arrival == 0) {
-      unsigned long long part = 0;  // this lane's share of the sum
-      bool abort = false;
-      if (two_pass_scan) {
-        // the chunk index is already there (encode_scan_kernel): the tile starts where its first chunk starts
-        if (lane == 0) part = chunk_index[(uint64_t)p_tile * active];
-      } else if (p_tile > 0) {
-        long long look = (long long)p_tile - 1;
-        uint32_t spins = 0;
-        bool done = false;
-        while (!done && !abort) {
-          // a round reads the kLookBack * 32 descriptors before `look` at once: the nearest tile that
-          // already knows its prefix is about one coding phase of tickets back
-          unsigned long long st[kLookBack];
+    // ---- D: the next ticket, and the offset of the pending tile: the sum over the tiles before it. Those of its own group (32 with
+    // eight warps) it reads one by one, behind them the group words up to the nearest that knows its offset. (Tiles one by one all the way, 592
+    // and more back, took three dependent rounds of 256 words, and the other seven warps waited for them: 268 M elements 164 us, so 158.)
+    if (arrival == 0) {
+      uint32_t next = 0;
+      if (have && lane == 0) next = atomicAdd(&ctl->ticket, 1u) + ticket_bias;
+      if (p_have) {
+        unsigned long long part = 0;  // this lane's share of the groups before
+        uint32_t own_bytes = 0;       // the tiles before it in its group, 256 chunks at most
+        bool abort = false;
+        const uint32_t group = p_tile / group_tiles, before = p_tile % group_tiles;
+        if (two_pass_scan) {
+          // the chunk index is already there (encode_scan_kernel): the tile starts where its first chunk starts
+          if (lane == 0) part = chunk_index[p_tile * active];
+        } else {
+          int look = (int)group - 1;
+          bool own = before == 0, done = group == 0;
+          uint32_t spins = 0;
+          while (!abort && !(own && done)) {
+            unsigned long long st[kGroupWindows];
 #pragma unroll
-          for (int u = 0; u < kLookBack; ++u) {
-            const long long idx = look - 32 * u - lane;
-            st[u] = (kTilePrefix << kTileFlagShift);  // tiles before the first: prefix 0
-            if (idx >= 0) st[u] = ld_tile(&tiles[idx]);
-          }
-          bool retry = false;
+            for (int u = 0; u < kGroupWindows; ++u) {
+              const int idx = look - 32 * u - (int)lane;
+              st[u] = kTilePrefix << kTileFlagShift | (unsigned long long)group_tiles << kGroupCountShift;  // before the first: prefix 0
+              if (!done && idx >= 0) st[u] = ld_tile(&groups[idx]);
+            }
+            bool retry = false;
+            if (!own) {
+              uint32_t sum = 0;
+              uint32_t missing = 0;  // 1: a tile without a size, 2: an aborted one
+              for (uint32_t i = lane; i < before; i += 32) {
+                const unsigned long long t = ld_tile(&tiles[group * group_tiles + i]);
+                const uint32_t flag = (uint32_t)(t >> kTileFlagShift);
+                sum += (uint32_t)t;
+                missing |= flag == kTileAggregate ? 0u : flag == kTileAbort ? 2u : 1u;
+              }
+              missing = __reduce_or_sync(0xffffffffu, missing);
+              if (missing & 2u) abort = true;
+              else if (missing) retry = true;
+              else own_bytes = __reduce_add_sync(0xffffffffu, sum), own = true;
+            }
 #pragma unroll
-          for (int u = 0; u < kLookBack; ++u) {
-            if (done || abort || retry) continue;
-            const uint32_t flag = (uint32_t)(st[u] >> kTileFlagShift);
-            const uint32_t m_prefix = __ballot_sync(0xffffffffu, flag == kTilePrefix);
-            const uint32_t m_other = __ballot_sync(0xffffffffu, flag != kTilePrefix && flag != kTileAggregate);
-            const int first_prefix = m_prefix ? __ffs(m_prefix) - 1 : 32;
-            const uint32_t relevant = first_prefix < 32 ? (0xffffffffu >> (31 - first_prefix)) : 0xffffffffu;
-            if (m_other & relevant) {
-              // a tile without a size yet, or an aborted one
-              if (__ballot_sync(0xffffffffu, flag == kTileAbort) & relevant) abort = true;
-              else retry = true;  // poll again from `look`, which already skips the complete sub-windows
-            } else {
-              if ((int)lane <= first_prefix) part += st[u] & kTileValueMask;
-              if (first_prefix < 32) done = true;
-              else look -= 32;
+            for (int u = 0; u < kGroupWindows; ++u) {
+              if (done || abort || retry) continue;
+              const uint32_t flag = (uint32_t)(st[u] >> kTileFlagShift);
+              const bool complete = ((uint32_t)(st[u] >> kGroupCountShift) & 511u) == group_tiles && (flag & 1u) == 0;
+              const uint32_t m_prefix = __ballot_sync(0xffffffffu, complete && flag == kTilePrefix);
+              const uint32_t m_other = __ballot_sync(0xffffffffu, !complete);
+              const int first_prefix = m_prefix ? __ffs(m_prefix) - 1 : 32;
+              const uint32_t relevant = first_prefix < 32 ? (0xffffffffu >> (31 - first_prefix)) : 0xffffffffu;
+              if (m_other & relevant) {
+                // a group with a tile that has no size yet, or an aborted one
+                if (__ballot_sync(0xffffffffu, (flag & 1u) != 0) & relevant) abort = true;
+                else retry = true;  // poll again from `look`, which already skips the complete sub-windows
+              } else {
+                if ((int)lane <= first_prefix) part += st[u] & kGroupValueMask;
+                if (first_prefix < 32) done = true;
+                else look -= 32;
+              }
+            }
+            if (retry) {
+              if (++spins > spin_limit) abort = true;
+              else __nanosleep(40);
             }
           }
-          if (retry) {
-            if (++spins > spin_limit) abort = true;
-            else __nanosleep(40);
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) part += __shfl_xor_sync(0xffffffffu, part, d);
+        if (lane == 0) {
+          if (abort) {
+            set_status(&ctl->status, LC_ERR_TIMEOUT);
+            st_tile(&tiles[p_tile], kTileAbort << kTileFlagShift);
+            st_tile(&groups[group], kTileAbort << kTileFlagShift);  // what is still added to it leaves the lower flag bit
+            s_abort[parity] = 1;
+          } else {
+            unsigned long long p_tile_bytes = 0;
+#pragma unroll
+            for (int w = 0; w < (int)kEncWarps; ++w) p_tile_bytes += s_chunk_bytes[p_buf][w];
+            // added, not stored: sizes of the group's tiles may still be on their way
+            if (before == 0 && !two_pass_scan) atomicAdd(&groups[group], (kTilePrefix << kTileFlagShift) | part);
+            s_abort[parity] = 0;
+            s_tile_base[parity] = part + own_bytes;
+            s_tile_end[parity] = part + own_bytes + p_tile_bytes;
           }
         }
       }
-#pragma unroll
-      for (int d = 16; d > 0; d >>= 1) part += __shfl_xor_sync(0xffffffffu, part, d);
-      if (lane == 0) {
-        if (abort) {
-          set_status(&ctl->status, LC_ERR_TIMEOUT);
-          st_tile(&tiles[p_tile], kTileAbort << kTileFlagShift);
-          s_abort = 1;
-        } else {
-          unsigned long long p_tile_bytes = 0;
-#pragma unroll
-          for (int w = 0; w < (int)kEncWarps; ++w) p_tile_bytes += s_chunk_bytes[p_buf][w];
-          if (p_tile > 0 && !two_pass_scan)
-            st_tile(&tiles[p_tile], (kTilePrefix << kTileFlagShift) | (part + p_tile_bytes));
-          s_abort = 0;
-          s_tile_base = part;
-          s_tile_end = part + p_tile_bytes;
-        }
-      }
+      if (have && lane == 0) s_tile[parity ^ 1] = next;
     }
-    __syncthreads();  // all chunk sizes of the new tile, and the pending tile's offset, are known
-    if (tid == 0) {
-      s_arrived[p_buf] = 0;  // the other half's counter, for the next iteration
-      if (have && !two_pass_scan) {
-        unsigned long long tile_bytes = 0;
-#pragma unroll
-        for (int w = 0; w < (int)kEncWarps; ++w) tile_bytes += s_chunk_bytes[buf][w];
-        const unsigned long long flag = tile == 0 ? kTilePrefix : kTileAggregate;
-        st_tile(&tiles[tile], (flag << kTileFlagShift) | tile_bytes);
-      }
+    __syncthreads();  // the pending tile's offset and the next ticket are known
+    if (tid == 0) s_arrived[p_buf] = 0;  // used again behind the next barrier
+    const uint32_t next_tile = have ? s_tile[parity ^ 1] : ntiles;
+    // The next chunk's plane bytes are asked into the L2, a line per lane (268 M elements 158 -> 147 us; with the tracked state, where rows of base
+    // are what counts, 782 either way).
+    {
+      const uint32_t next_c = next_tile * active + warp;
+      if (!UPDATE && warp < active && next_c < nchunks)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(plane + (uint64_t)next_c * kChunkElems + lane * 128));
     }
+    const bool p_write = p_have && !s_abort[parity];
 
     // ---- E: write the pending tile's chunks and their index entries
-    if (p_have && !s_abort) {
-      unsigned long long chunk_off = s_tile_base;
+    if (p_write) {
+      unsigned long long chunk_off = s_tile_base[parity];
       for (uint32_t w = 0; w < warp; ++w) chunk_off += s_chunk_bytes[p_buf][w];
-      const uint64_t p_c = (uint64_t)p_tile * active + warp;
+      const uint32_t p_c = p_tile * active + warp;
       const uint32_t p_chunk_bytes = s_chunk_bytes[p_buf][warp];
       const bool p_staged = p_chunk_bytes <= image_words * 4;
       if (warp < active && p_c < nchunks) {
@@ -317,19 +351,19 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
         }
       }
       if (p_tile == ntiles - 1 && tid == 0) {
-        const unsigned long long payload_bytes = s_tile_end;
+        const unsigned long long payload_bytes = s_tile_end[parity];
         chunk_index[nchunks] = payload_bytes;
         *reinterpret_cast<unsigned long long*>(stream + 48) = L.payload_off + payload_bytes;
       }
     }
     // ---- tracked state of the pending tile's chunks (everything that reads base for coding them is done)
-    if (UPDATE && p_have && !s_abort) {
-      const uint64_t p_c = (uint64_t)p_tile * active + warp;
+    if (UPDATE && p_write) {
+      const uint32_t p_c = p_tile * active + warp;
       if (warp < active && p_c < nchunks && !fast_chunk(p_c)) {  // the others were updated while they were coded
-        if ((p_c + 1) * kChunkElems <= n && !ks.wide) {
-          const uint4* ep = reinterpret_cast<const uint4*>(plane + p_c * kChunkElems) + lane;
-          const float4* b4 = reinterpret_cast<const float4*>(base + p_c * kChunkElems) + lane;
-          float4* o4 = reinterpret_cast<float4*>(tracked_out + p_c * kChunkElems) + lane;
+        if (p_c < whole && !ks.wide) {
+          const uint4* ep = reinterpret_cast<const uint4*>(plane + (uint64_t)p_c * kChunkElems) + lane;
+          const float4* b4 = reinterpret_cast<const float4*>(base + (uint64_t)p_c * kChunkElems) + lane;
+          float4* o4 = reinterpret_cast<float4*>(tracked_out + (uint64_t)p_c * kChunkElems) + lane;
 #pragma unroll 2
           for (int q = 0; q < 8; ++q) {
             const uint4 w4 = __ldg(ep + 32 * q);  // plane bytes of steps 4q .. 4q+3
@@ -351,7 +385,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
           // exponents the one-byte plane does not hold: element by element
           for (uint32_t j = 0; j < kSteps; ++j) {
             for (uint32_t e = 0; e < kGroup; ++e) {
-              const uint64_t i = p_c * kChunkElems + 128ull * j + 4 * lane + e;
+              const uint64_t i = (uint64_t)p_c * kChunkElems + 128ull * j + 4 * lane + e;
               if (i >= n) continue;
               const uint32_t sym = ctl->enc[ks.key(p_c, j, lane, e)].sym;
               const uint32_t rep = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * sym + 4);
@@ -363,7 +397,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     }
     // The partial last chunk's, by all warps of the CTA, four rows each: by the one warp that has coded it, it took the launch
     // 10 us longer (11.7 M elements: 35 us instead of 25).
-    if (UPDATE && p_have && !s_abort && p_tile == ntiles - 1 && n % kChunkElems != 0 && !ks.wide) {
+    if (UPDATE && p_write && p_tile == ntiles - 1 && n % kChunkElems != 0 && !ks.wide) {
       const uint64_t p_c = nchunks - 1;
       const uint32_t rem = (uint32_t)(n - p_c * kChunkElems);
       const float* b1 = base + p_c * kChunkElems;
@@ -389,28 +423,16 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
         }
     }
     if (!have) break;
-    // The next ticket is taken now, so that the round trip overlaps the rest of this iteration. (Taking it
-    // earlier would only make the tile look late to its successors: its size cannot appear before it is coded.)
-    if (tid == 0) s_tile = atomicAdd(&ctl->ticket, 1u) + ticket_bias;
     __syncwarp();  // the warp's image area is free again
 
     // ---- C: assemble the new tile's chunk image in shared memory
     if (valid && staged) {
-      uint4* im4 = reinterpret_cast<uint4*>(image);
-      for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) im4[k] = make_uint4(0, 0, 0, 0);
-      __syncwarp();
       if (fast) {
-        const uint32_t nw = (lane_bits + 31) >> 5, r = lane_start & 31;
-        uint32_t* out = image + (lane_start >> 5);
-        uint32_t prev = 0;
-        for (uint32_t k = 0; k < nw; ++k) {
-          const uint32_t w = column[k * 32 + lane];
-          atomicOr(out + k, __funnelshift_r(w, prev, r));
-          prev = w;
-        }
-        const uint32_t tail = r ? prev << (32 - r) : 0u;
-        if (tail) atomicOr(out + nw, tail);
+        assemble_chunk(column, lane, lane_bits, lane_start, image, chunk_bytes);
       } else {
+        uint4* im4 = reinterpret_cast<uint4*>(image);
+        for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) im4[k] = make_uint4(0, 0, 0, 0);
+        __syncwarp();
         chunk_slow(ctl->enc, ks, c, lane, n, image, lane_start);
       }
     } else if (valid) {
@@ -418,8 +440,11 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     }
     __syncwarp();
     p_have = true;
-    p_tile = (uint32_t)tile;
+    p_tile = tile;
     p_buf = buf;
+    buf = buf == 2 ? 0 : buf + 1;
+    parity ^= 1;
+    tile = next_tile;
   }
 }
 
@@ -445,7 +470,7 @@ encode_sizes_kernel(const Control* __restrict__ ctl, unsigned long long* __restr
   for (uint64_t c = warp0; c < nchunks; c += nwarps) {
     uint32_t bits = 0;
     if (!ks.wide && (c + 1) * kChunkElems <= n) {
-      const uint4* ep = reinterpret_cast<const uint4*>(plane + c * kChunkElems) + lane;
+      const uint4* ep = reinterpret_cast<const uint4*>(plane + (uint64_t)c * kChunkElems) + lane;
       uint4 v[kSteps / 4];
 #pragma unroll
       for (uint32_t q = 0; q < kSteps / 4; ++q) v[q] = __ldg(ep + 32 * q);

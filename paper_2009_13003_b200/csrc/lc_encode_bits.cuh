@@ -13,11 +13,17 @@ constexpr uint32_t kEntryLenMask = 255u;
 constexpr uint32_t kEntryMaxLen = 24;
 constexpr uint32_t kEntryLong = 100u;      // length of an entry without a code: it takes every sum of two beyond 32
 constexpr uint32_t kSingleMaxLen = 16;     // codes in `single`: two of them make one append of at most 32 bits
-constexpr int kPairSpan = 32;              // values a byte takes in the index of a pair
+constexpr uint32_t kPairSpan = 32;         // values a byte takes in the index of a pair
+// Words from one value of a pair's second element to the next. An odd number above 32: the bank then depends on both elements. With 32 it
+// was the first element's value, of which a vector has a dozen that are frequent: 4.6 to 5.4 wavefronts a lookup, with 37 it
+// is 2.7 to 3.1 (counted for Gaussian, Laplace, log-normal and Student deltas in 4 to 6 bits; 33 3.8 to 4.1, 35 2.8 to 3.2, 39 to 45 as 37).
+constexpr uint32_t kPairStride = 37;
+constexpr uint32_t kPairWords = (kPairSpan - 1) * kPairStride + kPairSpan;
+static_assert(4 * kPairWords < 65536, "two byte offsets in one word");
 
 struct Tables {
   union {
-    uint32_t pair[kPairSpan * kPairSpan];  // both codes of two neighbouring elements
+    uint32_t pair[kPairWords];  // both codes of two neighbouring elements
     uint32_t single[256];                  // by plane byte
   };
   uint2 full[256];     // by plane byte: {code, length} for codes of up to 32 bits
@@ -92,7 +98,7 @@ __device__ __forceinline__ void build_tables(Tables& tb, uint32_t sym0_len, Kept
       const auto escapes = [&](uint32_t v) { return all == 0 ? false : v == 0 ? lowest <= (uint32_t)base && lowest <= highest : v == 31 && highest > (uint32_t)base + 31; };
       const uint2 f0 = tb.full[min(base + v0, 255u)], f1 = tb.full[min(base + v1, 255u)];
       const uint32_t len = f0.y + f1.y;
-      tb.pair[k] = escapes(v0) || escapes(v1) || f0.y > 32 || f1.y > 32 ? kEntryLong : make_entry(f0.x << (f1.y & 31) | f1.x, len, kEntryMaxLen);
+      tb.pair[v1 * kPairStride + v0] = escapes(v0) || escapes(v1) || f0.y > 32 || f1.y > 32 ? kEntryLong : make_entry(f0.x << (f1.y & 31) | f1.x, len, kEntryMaxLen);
     }
   } else {
     tb.single[b] = make_entry(tb.full[b].x, my_len, kSingleMaxLen);
@@ -230,7 +236,7 @@ struct ColumnPacker {
 __device__ __forceinline__ uint2 lookup_pairs(const Tables& tb, uint32_t word, uint32_t neg_base) {
   const uint32_t v0 = __viaddmin_s16x2_relu(__byte_perm(word, 0u, 0x4240), neg_base, 0x001f001fu);  // elements 0, 2
   const uint32_t v1 = __viaddmin_s16x2_relu(__byte_perm(word, 0u, 0x4341), neg_base, 0x001f001fu);  // elements 1, 3
-  const uint32_t at = (v1 * kPairSpan + v0) * 4u;  // byte offsets of the two entries, one in each half
+  const uint32_t at = (v1 * kPairStride + v0) * 4u;  // byte offsets of the two entries, one in each half
   const volatile char* t = reinterpret_cast<const volatile char*>(tb.pair);  // volatile: one row ahead of the use
   return make_uint2(*reinterpret_cast<const volatile uint32_t*>(t + (at & 0xffffu)),
                     *reinterpret_cast<const volatile uint32_t*>(t + (at >> 16)));
@@ -239,9 +245,9 @@ __device__ __forceinline__ uint2 lookup_pairs(const Tables& tb, uint32_t word, u
 // together, send the warp the long way.
 __device__ __forceinline__ void put_pairs(ColumnPacker& pk, const Tables& tb, uint32_t word, uint2 e) {
   const uint32_t len = (e.x + e.y) & kEntryLenMask;
-  if (__any_sync(0xffffffffu, len > 32)) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) pk.put_full(tb.full[__byte_perm(word, 0u, 0x4440 + k)]);
+  if (__builtin_expect(__any_sync(0xffffffffu, len > 32), 0)) {
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) pk.put_full(tb.full[(word >> (8 * k)) & 255u]);
   } else {
     pk.put_two(e.x, e.y, len);
   }
@@ -254,9 +260,9 @@ __device__ __forceinline__ uint4 lookup_singles(const Tables& tb, uint32_t word)
 }
 __device__ __forceinline__ void put_singles(ColumnPacker& pk, const Tables& tb, uint32_t word, uint4 e) {
   const uint32_t l0 = (e.x + e.y) & kEntryLenMask, l1 = (e.z + e.w) & kEntryLenMask;
-  if (__any_sync(0xffffffffu, max(l0, l1) > 32)) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) pk.put_full(tb.full[__byte_perm(word, 0u, 0x4440 + k)]);
+  if (__builtin_expect(__any_sync(0xffffffffu, max(l0, l1) > 32), 0)) {
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) pk.put_full(tb.full[(word >> (8 * k)) & 255u]);
   } else {
     pk.put_two(e.x, e.y, l0);
     pk.put_two(e.z, e.w, l1);
@@ -315,6 +321,53 @@ __device__ __forceinline__ uint32_t finish_column(const ColumnPacker& pk, uint32
   if (pk.nb >= 32 || (pk.nb > 0 && pk.dst >= pk.lim)) return 0xffffffffu;
   if (pk.nb > 0) asm volatile("st.shared.u32 [%0], %1;" ::"r"(pk.dst), "r"(pk.w) : "memory");
   return ((pk.dst - col0) >> 7) * 32 + pk.nb;
+}
+
+// ORs a lane's `bits` bits from its column into the zeroed chunk image at `image` (shared or global memory), from bit `start` on.
+__device__ __forceinline__ void or_column(const uint32_t* column, uint32_t lane, uint32_t bits, uint32_t start, uint32_t* image) {
+  const uint32_t words = (bits + 31) >> 5, r = start & 31;
+  uint32_t* out = image + (start >> 5);
+  uint32_t prev = 0;
+  for (uint32_t k = 0; k < words; ++k) {
+    const uint32_t w = column[k * 32 + lane];
+    atomicOr(out + k, __funnelshift_r(w, prev, r));
+    prev = w;
+  }
+  const uint32_t tail = r ? prev << (32 - r) : 0u;
+  if (tail) atomicOr(out + words, tail);
+}
+
+// Assembles a chunk's image in shared memory (`chunk_bytes` of it, 16-byte aligned) from the columns; the whole warp.
+// Where every lane has 32 bits or more, a lane ends in another word than it begins in: it gets the bits of its first word that belong
+// to the lane before out of that lane's register and writes every word that it completes with a plain store, and nothing has to be
+// zeroed first. Otherwise (a partial chunk, codes of almost no bits) the lanes OR their words into the zeroed image.
+__device__ __forceinline__ void assemble_chunk(const uint32_t* column, uint32_t lane, uint32_t bits, uint32_t start, uint32_t* image,
+                                               uint32_t chunk_bytes) {
+  if (__any_sync(0xffffffffu, bits < 32)) {
+    uint4* im4 = reinterpret_cast<uint4*>(image);
+    for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) im4[k] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    or_column(column, lane, bits, start, image);
+    return;
+  }
+  const uint32_t r = start & 31, first = start >> 5, end = start + bits;
+  const uint32_t whole = (end >> 5) - first;  // words that the lane completes, its first among them: 1 or more
+  const uint32_t* col = column + lane;
+  // what it leaves of the next word (a column is zero behind its bits, and may end before that word does)
+  const uint32_t partial = __funnelshift_r(whole < (bits + 31) >> 5 ? col[whole * 32] : 0u, col[(whole - 1) * 32], r);
+  const uint32_t carry = __shfl_up_sync(0xffffffffu, partial, 1);
+  uint32_t* out = image + first;
+  uint32_t prev = col[0];
+  out[0] = prev >> r | (r ? carry : 0u);
+#pragma unroll 4
+  for (uint32_t k = 1; k < whole; ++k) {
+    const uint32_t w = col[k * 32];
+    out[k] = __funnelshift_r(w, prev, r);
+    prev = w;
+  }
+  // the last lane's partial word, and zeros up to the end
+  const uint32_t rest = __shfl_sync(0xffffffffu, partial, 31), at = __shfl_sync(0xffffffffu, end >> 5, 31) + lane;
+  if (at < chunk_bytes / 4) image[at] = lane == 0 ? rest : 0u;
 }
 
 // Phase A for the vector's partial last chunk of `rem` elements: as for a whole chunk, with the slots beyond the end

@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kSegThreads, 3)
 segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ blocks, unsigned long long* __restrict__ tiles,
                        const float* base, const float* cur, uint8_t* __restrict__ streams, float* tracked_out,
                        uint32_t lane_words, uint32_t image_bytes, uint32_t spin_limit, const __grid_constant__ SegGroup group) {
-  extern __shared__ __align__(16) unsigned char s_dyn[];
+  extern __shared__ __align__(128) unsigned char s_dyn[];
   __shared__ Tables tb;
   __shared__ uint32_t s_rep[256];  // representative (bit pattern) by plane byte
   __shared__ uint32_t s_bytes[kEncWarps];
@@ -262,20 +262,8 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
 
   // ---- C: assemble the chunk's image (in the place of the plane bytes, which have been read)
   if (staged) {
-    uint4* im4 = reinterpret_cast<uint4*>(image);
     __syncwarp();
-    for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) im4[k] = make_uint4(0, 0, 0, 0);
-    __syncwarp();
-    const uint32_t nw = (lane_bits + 31) >> 5, r = lane_start & 31;
-    uint32_t* out = image + (lane_start >> 5);
-    uint32_t prev = 0;
-    for (uint32_t k = 0; k < nw; ++k) {
-      const uint32_t w = column[k * 32 + lane];
-      atomicOr(out + k, __funnelshift_r(w, prev, r));
-      prev = w;
-    }
-    const uint32_t tail = r ? prev << (32 - r) : 0u;
-    if (tail) atomicOr(out + nw, tail);
+    assemble_chunk(column, lane, lane_bits, lane_start, image, chunk_bytes);
   }
 
   // ---- D: the tile's offset: exclusive prefix over the segment's tiles by decoupled look-back (bounded), one warp
@@ -339,16 +327,7 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
       for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) dst4[k] = make_uint4(0, 0, 0, 0);
       __threadfence_block();
       __syncwarp();
-      const uint32_t nw = (lane_bits + 31) >> 5, r = lane_start & 31;
-      uint32_t* out = reinterpret_cast<uint32_t*>(dst4) + (lane_start >> 5);
-      uint32_t prev = 0;
-      for (uint32_t k = 0; k < nw; ++k) {
-        const uint32_t w = column[k * 32 + lane];
-        atomicOr(out + k, __funnelshift_r(w, prev, r));
-        prev = w;
-      }
-      const uint32_t tail = r ? prev << (32 - r) : 0u;
-      if (tail) atomicOr(out + nw, tail);
+      or_column(column, lane, lane_bits, lane_start, reinterpret_cast<uint32_t*>(dst4));
     } else {
       for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) dst4[k] = make_uint4(0, 0, 0, 0);
       __threadfence_block();
