@@ -19,18 +19,19 @@ table_kernel(Control* __restrict__ ctl, uint64_t n, int nbits, uint8_t* __restri
   begin_next();
   wait_previous();
   const uint32_t tid = threadIdx.x, key = key_of_position(tid);
-  // an earlier pass of the same call has failed (lc_merge: a stream was rejected): leave no stream behind
-  if (ctl->status != 0) {  // nothing in this kernel has written the word yet: the same for every thread
-    clear_header(stream);
-    return;
-  }
-  // The statistics that decide the table: this vector's own, or those of the whole vector it is a shard of.
+  // The statistics that decide the table: this vector's own, or those of the whole vector it is a shard of. (Read together with the status word.)
+  const int32_t status = *reinterpret_cast<const volatile int32_t*>(&ctl->status);
   KeyStats my;
   my.local = ctl->count[key];
   my.count = whole ? whole->count[key] : my.local;
   my.inv_min = whole ? whole->inv_min[key] : ctl->inv_min[key];
   my.max_bits = whole ? whole->max_bits[key] : ctl->max_bits[key];
   my.mant_sum = mean ? ctl->mant_sum[key] : 0ull;
+  // an earlier pass of the same call has failed (lc_merge: a stream was rejected): leave no stream behind
+  if (status != 0) {  // nothing in this kernel has written the word yet: the same for every thread
+    clear_header(stream);
+    return;
+  }
   const int err = table_pass(T, my, TableArgs{n, nbits, wide_ok != 0, fixed != 0, whole != nullptr, mean != 0, cache}, stream);
   if (err) {
     clear_header(stream);
