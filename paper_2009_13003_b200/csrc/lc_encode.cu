@@ -28,7 +28,7 @@
 // the key plane.
 //
 // The vector's partial last chunk takes a masked form of A. Rare cases take a compact two-pass path (lengths, then bits
-// ORed in place): codes longer than 32 bits, a lane or chunk that outgrows its shared-memory area, and vectors with an
+// ORed in place): codes longer than 32 bits, a lane or chunk that outgrows its shared-memory area, and chunks with an
 // exponent field >= 128, for which the one-byte key plane is not enough and keys come from base and cur.
 //
 // Bound: reads 1 byte and writes about 0.5 bytes per element, so this pass is limited by the integer work per element,
@@ -75,6 +75,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   __shared__ uint32_t s_tile[2];     // the tile to be coded next
   __shared__ unsigned long long s_tile_base[2], s_tile_end[2];  // of the pending tile
   __shared__ int s_abort[2];
+  __shared__ uint32_t s_any_wide;               // the vector has elements that the plane does not identify
   __shared__ uint32_t s_rep[UPDATE ? 256 : 1];  // UPDATE: representative (bit pattern) by plane byte
 
   wait_previous();
@@ -89,19 +90,19 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   }
   __syncthreads();
   if (s_abort[0] != 0) return;
+  if (tid == 0) s_any_wide = ctl->wide;
   for (uint32_t b = tid; b < 256; b += kEncThreads) {
-    const EncEntry e = ctl->enc[((b & 1u) << 8) | (b >> 1)];
+    const EncEntry e = ctl->enc[key_of_byte(b)];
     tb.full[b] = make_uint2(e.code_lo, e.len);
     // the table pass has written the stream's symbol table: entry of symbol s at 64 + 16 s, representative at +4
     if (UPDATE) s_rep[b] = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
   }
   __syncthreads();
   static_assert(kEncThreads == 256, "a thread per plane byte");
-  build_tables(tb, ctl->enc[0].len, [&](uint32_t b) { return ctl->enc[((b & 1u) << 8) | (b >> 1)].sym != 0; });
+  build_tables(tb, ctl->enc[0].len, [&](uint32_t b) { return ctl->enc[key_of_byte(b)].sym != 0; });
 
   const uint32_t nsym = ctl->nsym;
   const bool long_codes = ctl->max_len > 32;
-  const KeySource ks{plane, base, cur, ctl->wide != 0};
   const StreamLayout L = stream_layout(n, nsym);
   const uint32_t nchunks = (uint32_t)L.nchunks, whole = (uint32_t)(n / kChunkElems);  // at most 2^20 chunks
   unsigned long long* chunk_index = reinterpret_cast<unsigned long long*>(stream + L.chunk_index_off);
@@ -118,7 +119,9 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
   const uint32_t neg_base = (uint32_t)(-tb.base) & 0xffffu, neg_base2 = neg_base << 16 | neg_base;
   const bool use_pair = tb.use_pair != 0;
 
-  auto fast_chunk = [&](uint32_t cc) { return cc < whole && !long_codes && !ks.wide; };
+  // wide_chunk: keys from base and cur. The tracked state of a chunk that is neither that nor long_codes is written while it is coded.
+  auto wide_chunk = [&](uint32_t cc) { return s_any_wide != 0 && has_escape(plane, cc, lane); };
+  auto keys = [&](bool wide) { return KeySource{plane, base, cur, wide}; };
 
   const uint32_t ntiles = (nchunks + active - 1) / active;
   const uint32_t group_tiles = kScanGroupChunks / active;
@@ -142,7 +145,8 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     if (!have && !p_have) break;
     const uint32_t c = tile * active + warp;
     const bool valid = have && warp < active && c < nchunks;
-    bool fast = valid && fast_chunk(c);
+    const bool wide = valid && wide_chunk(c);
+    bool fast = valid && c < whole && !long_codes && !wide;
 
     // ---- A: code the lane's elements into its column. Lookups run one row (4 elements) ahead of the
     // appends, which depend on each other through the bit accumulator.
@@ -192,13 +196,13 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
       if (use_pair) code_rows<true>(pk, tb, neg_base2, load, row);
       else code_rows<false>(pk, tb, neg_base2, load, row);
       lane_bits = finish_column(pk, col0);
-    } else if (valid && !long_codes && !ks.wide) {
+    } else if (valid && !long_codes && !wide) {
       lane_bits = code_partial(&tb, reinterpret_cast<const uint4*>(plane + (uint64_t)c * kChunkElems) + lane, (uint32_t)(n - (uint64_t)c * kChunkElems),
                                lane, smem_addr(column) + lane * 4, lane_words);
       fast = true;
     }
     if (fast && __any_sync(0xffffffffu, lane_bits == 0xffffffffu)) fast = false;  // some lane outgrew its column: redo the chunk the slow way
-    if (!fast && valid) lane_bits = chunk_slow(ctl->enc, ks, c, lane, n, nullptr, 0);
+    if (!fast && valid) lane_bits = chunk_slow(ctl->enc, keys(wide), c, lane, n, nullptr, 0);
 
     // ---- B: lane offsets, lane index, chunk size; the tile's size is published as early as possible
     if (valid) lane_index[c * kLanes + lane] = (uint16_t)lane_bits;
@@ -347,7 +351,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
           for (uint32_t k = lane; k < p_chunk_bytes / 16; k += 32) dst4[k] = make_uint4(0, 0, 0, 0);
           __threadfence_block();
           __syncwarp();
-          chunk_slow(ctl->enc, ks, p_c, lane, n, reinterpret_cast<uint32_t*>(dst4), image[lane]);
+          chunk_slow(ctl->enc, keys(wide_chunk(p_c)), p_c, lane, n, reinterpret_cast<uint32_t*>(dst4), image[lane]);
         }
       }
       if (p_tile == ntiles - 1 && tid == 0) {
@@ -359,8 +363,9 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     // ---- tracked state of the pending tile's chunks (everything that reads base for coding them is done)
     if (UPDATE && p_write) {
       const uint32_t p_c = p_tile * active + warp;
-      if (warp < active && p_c < nchunks && !fast_chunk(p_c)) {  // the others were updated while they were coded
-        if (p_c < whole && !ks.wide) {
+      const bool p_wide = warp < active && p_c < nchunks && wide_chunk(p_c);
+      if (warp < active && p_c < nchunks && (p_c >= whole || long_codes || p_wide)) {  // the others were updated while they were coded
+        if (p_c < whole && !p_wide) {
           const uint4* ep = reinterpret_cast<const uint4*>(plane + (uint64_t)p_c * kChunkElems) + lane;
           const float4* b4 = reinterpret_cast<const float4*>(base + (uint64_t)p_c * kChunkElems) + lane;
           float4* o4 = reinterpret_cast<float4*>(tracked_out + (uint64_t)p_c * kChunkElems) + lane;
@@ -381,10 +386,11 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
               o4[32 * (4 * q + r)] = x;
             }
           }
-        } else if (ks.wide) {
+        } else if (p_wide) {
           // exponents the one-byte plane does not hold: element by element
           for (uint32_t j = 0; j < kSteps; ++j) {
             for (uint32_t e = 0; e < kGroup; ++e) {
+              const KeySource ks = keys(true);
               const uint64_t i = (uint64_t)p_c * kChunkElems + 128ull * j + 4 * lane + e;
               if (i >= n) continue;
               const uint32_t sym = ctl->enc[ks.key(p_c, j, lane, e)].sym;
@@ -397,7 +403,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     }
     // The partial last chunk's, by all warps of the CTA, four rows each: by the one warp that has coded it, it took the launch
     // 10 us longer (11.7 M elements: 35 us instead of 25).
-    if (UPDATE && p_write && p_tile == ntiles - 1 && n % kChunkElems != 0 && !ks.wide) {
+    if (UPDATE && p_write && p_tile == ntiles - 1 && n % kChunkElems != 0 && !wide_chunk(nchunks - 1)) {
       const uint64_t p_c = nchunks - 1;
       const uint32_t rem = (uint32_t)(n - p_c * kChunkElems);
       const float* b1 = base + p_c * kChunkElems;
@@ -433,7 +439,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
         uint4* im4 = reinterpret_cast<uint4*>(image);
         for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) im4[k] = make_uint4(0, 0, 0, 0);
         __syncwarp();
-        chunk_slow(ctl->enc, ks, c, lane, n, image, lane_start);
+        chunk_slow(ctl->enc, keys(wide), c, lane, n, image, lane_start);
       }
     } else if (valid) {
       image[lane] = lane_start;
@@ -462,14 +468,15 @@ encode_sizes_kernel(const Control* __restrict__ ctl, unsigned long long* __restr
                     uint64_t nchunks) {
   __shared__ uint8_t s_len[256];  // code length by plane byte (lengths are at most 63)
   if (ctl->status != 0) return;  // nothing in this kernel writes the word: the same for every thread
-  for (uint32_t b = threadIdx.x; b < 256; b += kEncThreads) s_len[b] = (uint8_t)ctl->enc[((b & 1u) << 8) | (b >> 1)].len;
+  for (uint32_t b = threadIdx.x; b < 256; b += kEncThreads) s_len[b] = (uint8_t)ctl->enc[key_of_byte(b)].len;
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31;
-  const KeySource ks{plane, base, cur, ctl->wide != 0};
+  const bool any_wide = ctl->wide != 0;
   const uint64_t warp0 = (uint64_t)blockIdx.x * kEncWarps + (threadIdx.x >> 5), nwarps = (uint64_t)gridDim.x * kEncWarps;
   for (uint64_t c = warp0; c < nchunks; c += nwarps) {
     uint32_t bits = 0;
-    if (!ks.wide && (c + 1) * kChunkElems <= n) {
+    const bool wide = any_wide && has_escape(plane, (uint32_t)c, lane);
+    if (!wide && (c + 1) * kChunkElems <= n) {
       const uint4* ep = reinterpret_cast<const uint4*>(plane + (uint64_t)c * kChunkElems) + lane;
       uint4 v[kSteps / 4];
 #pragma unroll
@@ -482,7 +489,7 @@ encode_sizes_kernel(const Control* __restrict__ ctl, unsigned long long* __restr
           bits += s_len[w[r] & 255u] + s_len[(w[r] >> 8) & 255u] + s_len[(w[r] >> 16) & 255u] + s_len[w[r] >> 24];
       }
     } else {
-      bits = chunk_slow(ctl->enc, ks, c, lane, n, nullptr, 0);
+      bits = chunk_slow(ctl->enc, KeySource{plane, base, cur, wide}, c, lane, n, nullptr, 0);
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, d);

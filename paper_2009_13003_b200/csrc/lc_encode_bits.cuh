@@ -117,8 +117,7 @@ struct KeySource {
       const uint64_t i = c * kChunkElems + 128ull * j + 4 * lane + e;
       return __float_as_uint(__fsub_rn(cur[i], base[i])) >> 23;
     }
-    const uint32_t b = plane[c * kChunkElems + (j >> 2) * 512 + lane * 16 + (j & 3) * 4 + e];
-    return ((b & 1u) << 8) | (b >> 1);
+    return key_of_byte(plane[c * kChunkElems + (j >> 2) * 512 + lane * 16 + (j & 3) * 4 + e]);
   }
 };
 
@@ -142,6 +141,19 @@ struct OrPacker {
   }
 };
 
+// Whether a chunk has elements that the plane does not identify (byte 0), in a vector that has some; the whole warp. Out of line: rare.
+static __device__ __noinline__ bool has_escape(const uint8_t* plane, uint32_t c, uint32_t lane) {
+  const uint4* p = reinterpret_cast<const uint4*>(plane + (uint64_t)c * kChunkElems) + lane;
+  uint32_t zero = 0;
+#pragma unroll
+  for (uint32_t q = 0; q < kSteps / 4; ++q) {
+    const uint4 v = __ldg(p + 32 * q);
+    const auto of = [](uint32_t x) { return (x - 0x01010101u) & ~x & 0x80808080u; };  // not zero if one of x's bytes is
+    zero |= of(v.x) | of(v.y) | of(v.z) | of(v.w);
+  }
+  return __any_sync(0xffffffffu, zero != 0);
+}
+
 // Slow, compact path (see the header). With dst == nullptr it only returns the lane's bit count;
 // otherwise it ORs the lane's bits into the zeroed chunk image at dst, starting at bit lane_start.
 // The plane bytes of four steps are read as one 16-byte vector, the way the fast path reads them. Codes come from the per-key table in global memory:
@@ -164,8 +176,7 @@ static __device__ __noinline__ uint32_t chunk_slow(const EncEntry* __restrict__ 
         if (i >= n) continue;
         uint32_t key;
         if (from_plane) {
-          const uint32_t b = (words[r] >> (8 * e)) & 255u;
-          key = ((b & 1u) << 8) | (b >> 1);
+          key = key_of_byte((words[r] >> (8 * e)) & 255u);
         } else {
           key = ks.key(c, j, lane, e);
         }

@@ -135,7 +135,7 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
                        uint32_t lane_words, uint32_t image_bytes, uint32_t spin_limit, const __grid_constant__ SegGroup group) {
   extern __shared__ __align__(128) unsigned char s_dyn[];
   __shared__ Tables tb;
-  __shared__ uint32_t s_rep[256];  // representative (bit pattern) by plane byte
+  __shared__ uint32_t s_rep[256];  // representative (bit pattern) by the low byte of a slot, which is plane byte ^ 1
   __shared__ uint32_t s_bytes[kEncWarps];
   __shared__ uint32_t s_tile;
   __shared__ unsigned long long s_prefix;
@@ -156,13 +156,13 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
   uint8_t* stream = streams + group.stream_begin[s];
   const bool wide = B.wide != 0, long_codes = B.max_len > 32;
   for (uint32_t b = tid; b < 256; b += kSegThreads) {
-    const EncEntry e = B.enc[((b & 1u) << 8) | (b >> 1)];
+    const EncEntry e = B.enc[key_of_byte(b)];
     tb.full[b] = make_uint2(e.code_lo, e.len);
-    s_rep[b] = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
+    s_rep[b ^ 1] = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
   }
   __syncthreads();
   static_assert(kSegThreads == 256, "a thread per plane byte");
-  build_tables(tb, B.enc[0].len, [&](uint32_t b) { return B.enc[((b & 1u) << 8) | (b >> 1)].sym != 0; });
+  build_tables(tb, B.enc[0].len, [&](uint32_t b) { return B.enc[key_of_byte(b)].sym != 0; });
 
   const StreamLayout L = stream_layout(n, nsym);
   const uint32_t first_tile = group.tile_begin[s], last_tile = group.tile_begin[s + 1] - 1;
@@ -197,7 +197,7 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
         const uint32_t k1 = slot_of(__float_as_uint(__fsub_rn(c4[r].y, b4[r].y)));
         const uint32_t k2 = slot_of(__float_as_uint(__fsub_rn(c4[r].z, b4[r].z)));
         const uint32_t k3 = slot_of(__float_as_uint(__fsub_rn(c4[r].w, b4[r].w)));
-        w[r] = __byte_perm(__byte_perm(k0, k1, 0x0040), __byte_perm(k2, k3, 0x0040), 0x5410);
+        w[r] = __byte_perm(__byte_perm(k0, k1, 0x0040), __byte_perm(k2, k3, 0x0040), 0x5410) ^ kPlaneFlip;  // all exponent fields are below 128
         if (tracked_out) {
           const uint32_t i = (4 * q + r) * 128 + 4 * lane, have = i < rem ? rem - i : 0u;
           float4 x;

@@ -26,10 +26,16 @@ __device__ __forceinline__ float4 ld_stream(const float4* p) {
 
 // Slot of a delta's bucket in the shared-memory tables: (exponent field << 1) | sign. The two signs of one
 // exponent are neighbours and 8 consecutive exponents fill the 16 bank pairs of a 64-bit access exactly once,
-// so the few hot buckets of a vector (neighbouring exponents, both signs) rarely meet in a bank. The low byte
-// of the slot is the element's byte in the key plane.
+// so the few hot buckets of a vector (neighbouring exponents, both signs) rarely meet in a bank.
 __device__ __forceinline__ uint32_t slot_of(uint32_t bits) { return ((bits >> 22) & 0x1FEu) | (bits >> 31); }
 __device__ __forceinline__ uint32_t key_of_slot(uint32_t slot) { return ((slot & 1u) << 8) | (slot >> 1); }
+
+// The plane bytes of four elements from their slots: slot ^ 1, and 0 where that is 256 or more; two at a time, in 16-bit halves.
+__device__ __forceinline__ uint32_t plane_word(uint32_t k0, uint32_t k1, uint32_t k2, uint32_t k3) {
+  const uint32_t lo = __vmins2(__byte_perm(k0, k1, 0x5410) ^ 0x00010001u, 0x01000100u);
+  const uint32_t hi = __vmins2(__byte_perm(k2, k3, 0x5410) ^ 0x00010001u, 0x01000100u);
+  return __byte_perm(lo, hi, 0x6420);
+}
 
 template <bool MEAN>
 struct Acc {
@@ -99,11 +105,8 @@ __device__ __forceinline__ void stats_units(Acc<MEAN>& acc, const float* __restr
         const uint32_t d2 = __float_as_uint(__fsub_rn(c[r].z, b[r].z));
         const uint32_t d3 = __float_as_uint(__fsub_rn(c[r].w, b[r].w));
         const uint32_t k0 = slot_of(d0), k1 = slot_of(d1), k2 = slot_of(d2), k3 = slot_of(d3);
+        if (PLANE) ew[r] = plane_word(k0, k1, k2, k3);
         acc.add4(d0, d1, d2, d3, k0, k1, k2, k3);
-        // plane byte = low byte of the slot; gather the four into one word, element e in byte e.
-        const uint32_t lo = __byte_perm(k0, k1, 0x0040);
-        const uint32_t hi = __byte_perm(k2, k3, 0x0040);
-        ew[r] = __byte_perm(lo, hi, 0x5410);
       }
     } else {
       // ragged tail: the last units of the vector, element by element.
@@ -117,7 +120,7 @@ __device__ __forceinline__ void stats_units(Acc<MEAN>& acc, const float* __restr
             d = __float_as_uint(__fsub_rn(cur[i], base[i]));
             acc.add(d);
           }
-          word |= (slot_of(d) & 255u) << (8 * e);
+          word |= (min(slot_of(d) ^ 1u, 256u) & 255u) << (8 * e);
         }
         ew[r] = word;
       }
