@@ -639,7 +639,7 @@ __device__ __forceinline__ uint2 long_code_at(const StreamState& S, const Words<
   return make_uint2(0u, L);
 }
 
-// A chunk through the tables of one level. A step is two rows (one with a single stream: see below): a lane decodes eight elements x KS
+// A chunk through the tables of one level. A step is two rows (or one: see R): a lane decodes eight elements x KS
 // streams from a window of three words per stream, read anew in every step, so that all it keeps of a stream from step to step is a bit position. (A 64-bit buffer
 // that is topped up takes four registers and, with its bookkeeping, 45 instructions for four codes where this form takes 36.)
 // The window has at least 65 bits behind the position; four codes of a row that are together shorter than 32 bits leave
@@ -654,13 +654,12 @@ __device__ __forceinline__ uint2 long_code_at(const StreamState& S, const Words<
 // PARTIAL: the vector's last chunk, or any chunk larger than the staging area: of each row only the slots that exist are read and written. (A
 // lane's codes end with its last element; nothing is reported for what it decodes behind it.)
 // next_chunk: floats from this chunk to the one the warp takes next, whose first rows are asked into the L2 behind this one's last; 0 if there is none.
-template <int KS, Index INDEX, bool STAGED, bool PARTIAL>
+// R: rows a step. Two, but one with a single stream in a launch of many rounds: that is bound by HBM, and it is the steady trickle of single rows, each waited
+// for a step before its use, that reaches the copy rate (two_rows).
+template <int KS, int R, Index INDEX, bool STAGED, bool PARTIAL>
 __device__ __forceinline__ void decode_chunk_one_level(const StreamState* S, const Source* W, uint32_t (&pos)[KS], const float* base,
                                                   float* out, uint32_t c, uint64_t n, uint32_t lane, uint64_t next_chunk,
                                                   Status status) {
-  // With one stream the kernel is bound by HBM, and it is the steady trickle of single rows, each waited for a step before its use, that
-  // reaches the copy rate: with two rows a step 1.3 G elements took 1.87 ms instead of 1.75.
-  constexpr int R = KS == 1 ? 1 : 2;
   const uint32_t elems = PARTIAL ? (uint32_t)min(n - (uint64_t)c * kChunkElems, (uint64_t)kChunkElems) : kChunkElems;
   int have = (int)elems - 4 * (int)lane;  // PARTIAL: elements from this lane's first slot of the next row on
   const uint32_t steps = PARTIAL ? (elems + 128 * R - 1) / (128 * R) : kSteps / R;
@@ -885,7 +884,7 @@ __device__ __noinline__ void decode_rare_chunk(const StreamState* S, const float
     uint32_t pos[KS];
     __syncwarp();  // the previous chunk's reads of the staging area are done
     if (stage_chunk<KS, true>(S, c, lane, stage0, stage_bytes, W, pos, status)) {
-      decode_chunk_one_level<KS, INDEX, true, true>(S, W, pos, base, out, c, n, lane, 0, status);
+      decode_chunk_one_level<KS, 2, INDEX, true, true>(S, W, pos, base, out, c, n, lane, 0, status);
       return;
     }
   }
@@ -895,9 +894,9 @@ __device__ __noinline__ void decode_rare_chunk(const StreamState* S, const float
     uint32_t pos[1];
     __syncwarp();
     if (stage_chunk<1, true>(S + s, c, lane, stage0, KS * stage_bytes, W, pos, status))
-      decode_chunk_one_level<1, INDEX, true, true>(S + s, W, pos, s ? out : base, out, c, n, lane, 0, status);
+      decode_chunk_one_level<1, 2, INDEX, true, true>(S + s, W, pos, s ? out : base, out, c, n, lane, 0, status);
     else
-      decode_chunk_one_level<1, INDEX, false, true>(S + s, W, pos, s ? out : base, out, c, n, lane, 0, status);
+      decode_chunk_one_level<1, 2, INDEX, false, true>(S + s, W, pos, s ? out : base, out, c, n, lane, 0, status);
   }
 }
 
@@ -918,7 +917,7 @@ __device__ __noinline__ void decode_chunk_two_level(const StreamState* S, const 
 }
 
 // This warp's chunks, from c on, through the tables of one level.
-template <int KS, Index INDEX>
+template <int KS, int R, Index INDEX>
 __device__ __forceinline__ void decode_chunks(const StreamState* S, const float* base, float* out, uint32_t c, uint32_t nwarps,
                                               uint32_t whole_end, uint32_t chunk_end, uint64_t n, uint32_t lane, unsigned char* stage0,
                                               uint32_t stage_bytes, Status status) {
@@ -927,7 +926,7 @@ __device__ __forceinline__ void decode_chunks(const StreamState* S, const float*
     uint32_t pos[KS];
     __syncwarp();  // the previous chunk's reads of the staging area are done
     if (stage_chunk<KS, true>(S, c, lane, stage0, stage_bytes, W, pos, status))
-      decode_chunk_one_level<KS, INDEX, true, false>(S, W, pos, base, out, c, n, lane, c + nwarps < whole_end ? (uint64_t)nwarps * kChunkElems : 0, status);
+      decode_chunk_one_level<KS, R, INDEX, true, false>(S, W, pos, base, out, c, n, lane, c + nwarps < whole_end ? (uint64_t)nwarps * kChunkElems : 0, status);
     else
       decode_rare_chunk<KS, INDEX>(S, base, out, c, n, lane, stage0, stage_bytes, status);
   }
@@ -941,7 +940,7 @@ __device__ __forceinline__ void prefetch_rows(const float* first, uint32_t lane)
 
 // Chunks [chunk_begin, chunk_end) of one vector, by `ctas` CTAs of which this is number `cta`.
 // stage_bytes: bytes of staging area per warp and stream (a multiple of 16, at least 32).
-template <int KS>
+template <int KS, int R>
 __device__ __forceinline__ void decode_vector(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
                                               Status status, uint32_t stage_bytes, uint32_t chunk_begin,
                                               uint32_t chunk_end, uint32_t cta, uint32_t ctas) {
@@ -1002,9 +1001,9 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   unsigned char* stage0 = reinterpret_cast<unsigned char*>(S + KS) + (size_t)warp * KS * stage_bytes;
   wait_previous();  // the launch before this one, if it is a chain's, has written `base`
   if (index == Index::kDirect) {
-    decode_chunks<KS, Index::kDirect>(S, base, out, c, nwarps, whole_end, chunk_end, n, lane, stage0, stage_bytes, status);
+    decode_chunks<KS, R, Index::kDirect>(S, base, out, c, nwarps, whole_end, chunk_end, n, lane, stage0, stage_bytes, status);
   } else if (index == Index::kOnes) {
-    decode_chunks<KS, Index::kOnes>(S, base, out, c, nwarps, whole_end, chunk_end, n, lane, stage0, stage_bytes, status);
+    decode_chunks<KS, R, Index::kOnes>(S, base, out, c, nwarps, whole_end, chunk_end, n, lane, stage0, stage_bytes, status);
   } else {
     for (; c < chunk_end; c += nwarps) {
       // where the L2 prefetch goes on behind this chunk: the next full chunk of this warp, if there is one
@@ -1014,16 +1013,16 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   }
 }
 
-template <int KS, int WARPS>
+template <int KS, int WARPS, int R>
 __global__ void __launch_bounds__(32 * WARPS, kDecCtas<KS>)
 decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status, uint32_t rank,
               uint32_t stage_bytes, uint32_t chunk_begin, uint32_t chunk_end) {
-  decode_vector<KS>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
+  decode_vector<KS, R>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
 }
 
 // Per-layer recovery: the CTAs [cta_begin[i], cta_begin[i + 1]) decode segment i. One launch instead of one per segment
 // (a segment of a few chunks occupies one SM for the 15 us that a chunk takes; 62 of them in a row took 870 us).
-template <int KS, int WARPS>
+template <int KS, int WARPS, int R>
 __global__ void __launch_bounds__(32 * WARPS, kDecCtas<KS>)
 decode_segments_kernel(const float* base, const __grid_constant__ DecodeStreams buffers, float* out,
                        int32_t* __restrict__ status, uint32_t second, uint32_t stage_bytes,
@@ -1042,7 +1041,7 @@ decode_segments_kernel(const float* base, const __grid_constant__ DecodeStreams 
     streams.ptr[s] = buffers.ptr[s] + off;
     streams.bytes[s] = bytes;
   }
-  decode_vector<KS>(base + first, streams, n, out + first, Status{status, 2 * (batch.first + lo) + second}, stage_bytes, 0,
+  decode_vector<KS, R>(base + first, streams, n, out + first, Status{status, 2 * (batch.first + lo) + second}, stage_bytes, 0,
                     (uint32_t)((n + kChunkElems - 1) / kChunkElems), blockIdx.x - batch.cta_begin[lo],
                     batch.cta_begin[lo + 1] - batch.cta_begin[lo]);
 }
@@ -1132,6 +1131,11 @@ cudaError_t decode_shape(const void* fn, uint32_t want_stage, uint32_t (&regs_of
   return cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, carve < 100 ? carve : 100);
 }
 
+// One stream: two rows a step while the warps on the device have two and a half chunks each at most. A launch of few rounds waits for its lanes' chains, which
+// are shorter that way; one of many rounds for HBM. One row and two: 61,706 elements blocking 26.9 and 25.4 us, 11.7 M 28.0 and 24.8, 21 M (1.4 rounds)
+// 47.3 and 42.3, 32 M (2.2) 57.5 and 52.6, 43 M (3.0) 69.5 and 72.1, 87 M 129.5 and 138.0, 1.3 G 1750 and 1870.
+constexpr bool two_rows(uint64_t chunks, uint64_t warps) { return 2 * chunks <= 5 * warps; }
+
 // A warp decodes whole chunks, so `chunks` of them take a whole number of rounds over the CTAs that fit on the device.
 // With as few warps as do them in the same number of rounds all rounds are equally full; with all warps the last one can
 // be nearly empty, and takes nearly as long as the others (11.7 M elements, four streams: 19.3 chunks per SM in rounds of
@@ -1145,7 +1149,7 @@ uint32_t balanced_warps(uint64_t chunks, uint64_t ctas, uint32_t most) {
 
 // second: this launch goes on from what the one before it recovers, and may begin beside its end: tables and first rows do not wait for it (11.7 M
 // elements, eight streams: 81.0 -> 76.0 us).
-template <int KS, int WARPS = kDecWarps<KS>>
+template <int KS, int WARPS = kDecWarps<KS>, int R = 2>
 cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
                              int32_t* status, bool second, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
   static uint32_t regs_of[kMaxDevices] = {};
@@ -1162,9 +1166,11 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
     if (choose_shape(KS, wanted_stage(avg), 96, WARPS).warps < WARPS)
       return launch_decode_ks<KS, 16>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
   Shape sh;
-  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(decode_kernel<KS, WARPS>), wanted_stage(avg), regs_of, sh);
+  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(decode_kernel<KS, WARPS, R>), wanted_stage(avg), regs_of, sh);
   if (e != cudaSuccess) return e;
   const uint64_t chunks = chunk_end - chunk_begin, full = (uint64_t)sh.sms * sh.per_sm;
+  if constexpr (KS == 1 && R == 2)
+    if (!two_rows(chunks, full * sh.warps)) return launch_decode_ks<KS, WARPS, 1>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
   const uint32_t warps = balanced_warps(chunks, full, sh.warps);
   uint64_t want = (chunks + warps - 1) / warps;
   if (want == 0) want = 1;  // still reports a rejected stream
@@ -1172,23 +1178,27 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
   // the staging areas of the warps left out go to the others: chunks vary (a layer of rare exponents in a vector of layers
   // takes twice the average), and one that is read from global memory word by word holds up the launch
   const uint32_t stage = min(sh.warps * sh.stage / warps / 16 * 16, kChunkElems * 8 + 16);
-  return launch_kernel(second, decode_kernel<KS, WARPS>, grid, warps * 32, sh.dyn - (sh.warps * sh.stage - warps * stage) * KS, cs, base, streams, n, out,
+  return launch_kernel(second, decode_kernel<KS, WARPS, R>, grid, warps * 32, sh.dyn - (sh.warps * sh.stage - warps * stage) * KS, cs, base, streams, n, out,
                        status, second ? 1u : 0u, stage, (uint32_t)chunk_begin, (uint32_t)chunk_end);
 }
 
-template <int KS, int WARPS = KS == 3 ? 16 : kDecWarps<KS>>
+template <int KS, int WARPS = KS == 3 ? 16 : kDecWarps<KS>, int R = 2>
 cudaError_t launch_segments_ks(const float* base, const uint8_t* const* streams, SegBatch& batch, int nbits, float* out,
                                int32_t* status, bool second, cudaStream_t cs) {
   static uint32_t regs_of[kMaxDevices] = {};
   // the buffers are sized for nbits bits per element, which no chunk exceeds by much
   Shape sh;
-  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(decode_segments_kernel<KS, WARPS>),
+  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(decode_segments_kernel<KS, WARPS, R>),
                                          (uint32_t)align_up((uint64_t)nbits * (kChunkElems / 8) + 64, 16), regs_of, sh);
   if (e != cudaSuccess) return e;
+  if constexpr (KS == 1 && R == 2) {
+    const uint64_t chunks = (batch.elem_begin[batch.nseg] - batch.elem_begin[0]) / kChunkElems;  // about
+    if (!two_rows(chunks, (uint64_t)sh.sms * sh.per_sm * sh.warps)) return launch_segments_ks<KS, WARPS, 1>(base, streams, batch, nbits, out, status, second, cs);
+  }
   DecodeStreams buffers;
   for (int s = 0; s < 4; ++s) buffers.ptr[s] = s < KS ? streams[s] : nullptr, buffers.bytes[s] = 0;
   const uint32_t ctas = split_segments(batch, sh.warps, sh.sms * sh.per_sm);
-  return launch_kernel(second, decode_segments_kernel<KS, WARPS>, ctas, sh.warps * 32, sh.dyn, cs, base, buffers, out, status, second ? 1u : 0u, sh.stage,
+  return launch_kernel(second, decode_segments_kernel<KS, WARPS, R>, ctas, sh.warps * 32, sh.dyn, cs, base, buffers, out, status, second ? 1u : 0u, sh.stage,
                        batch);
 }
 
