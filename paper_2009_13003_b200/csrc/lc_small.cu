@@ -7,11 +7,10 @@
 // registers through statistics, coding and the tracked state. Warp w takes the chunk's steps 2w and 2w + 1, so the codes
 // of a thread are one contiguous piece of its lane's sub-stream: a scan over warps and lanes of the pieces' bit counts
 // places them, and each thread ORs its piece into the chunk's image in shared memory, which leaves with 16-byte stores.
-// In a cluster, the CTAs read each other's statistics and chunk sizes from shared memory, each derives the same table, and
-// two hardware barriers take the place of kernel boundaries and of the encode pass's look-back. Same bytes as the general
-// path. GPU time of a call: 9.4 us at 1000 elements (18 us with one warp coding alone and the earlier table pass), 12.4 us
-// at 16,000 and 15.1 us at 61,706 (25.5 us in the general path). What the CTAs read of each other decides the latter:
-// reading all 512 keys of 15 CTAs, every CTA in the same order, made it 26.9 us.
+// In a cluster, the CTAs add their statistics to each other's in shared memory and read each other's chunk sizes there, each derives the same table, and
+// hardware barriers take the place of kernel boundaries and of the encode pass's look-back. Same bytes as the general
+// path. GPU time of a call: about 8 us at 1000 elements (18 us with one warp coding alone and the earlier table pass), 12.8 us at 61,706 (25.5 us in the general
+// path; 14.8 us with the CTAs reading each other's statistics of the keys that occur, 26.9 of all 512).
 #include "lc_small.cuh"
 
 namespace lc {
@@ -27,6 +26,7 @@ small_compress_kernel(Control* ctl, const float* base, const float* cur, uint32_
                       float* tracked_out, int keep_status) {
   extern __shared__ __align__(16) unsigned char s_small[];
   SmallShared<M>& S = *reinterpret_cast<SmallShared<M>*>(s_small);
+  begin_next();
   const uint32_t tid = threadIdx.x;
   const bool first = !CLUSTER || cluster_rank() == 0;
   const int earlier = keep_status ? ctl->status : 0;  // the same for every thread: nothing here has written it yet

@@ -7,7 +7,7 @@
 // with the fronts of both queues in registers). Ranks, tree depths (pointer jumping), codes
 // (a sum over the symbols that come before) and sums are computed by all symbols at once; the stream's header and table
 // leave as 16-byte stores. With those steps in one thread, 64-bit shared-memory atomics and byte stores the pass took 10.5 us
-// for 8 symbols, 14 us for 16 and 28-36 us for 64; now 7.0, 8.3 and 13.4 us (cold caches, about 3 us of each the launch).
+// for 8 symbols, 14 us for 16 and 28-36 us for 64; in cycles of the pass alone it now takes 6000 (3 us) for 8, 6600 for 16 and 12,000 for 64.
 #pragma once
 #include "lc_common.cuh"
 
@@ -47,7 +47,7 @@ struct TableShared {
   unsigned long long part[4][kTableThreads / 32];
   uint32_t rep[kMaxSymbols], key[kMaxSymbols], len[kMaxSymbols];                 // by symbol
   uint32_t up[2 * kMaxSymbols];  // by tree node: depth below the node in the low half << 16 | that node
-  uint32_t ballot[kTableThreads / 32], flags[kTableThreads / 32];
+  uint32_t warps[kTableThreads / 32];  // candidates of a warp's keys in the low half, what is wrong with the keys above
   uint16_t sym_of_key[kKeys], place[kMaxSymbols];  // place: by symbol, among the leaves
   uint32_t nsym, max_len, wide;
   unsigned long long payload_bits;
@@ -119,10 +119,7 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
   const bool bad = (key & 255u) == 255u && my.count != 0;
   const bool big = (key & 255u) >= 128u && (my.count != 0 || my.local != 0);
   const uint32_t flags = (__any_sync(kAll, bad) ? 1u : 0u) | (__any_sync(kAll, big) ? 2u : 0u);
-  if (lane == 0) {
-    T.ballot[warp] = ballot;
-    T.flags[warp] = flags;
-  }
+  if (lane == 0) T.warps[warp] = __popc(ballot) | flags << 16;
   T.sym_of_key[tid] = 0;
   T.len[tid] = 0;
   T.code[tid] = 0;
@@ -136,10 +133,10 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
   uint32_t rank = __popc(ballot & ((1u << lane) - 1)), ncand = 0, all_flags = 0;
 #pragma unroll
   for (uint32_t w = 0; w < kTableThreads / 32; ++w) {
-    const uint32_t b = __popc(T.ballot[w]);
-    if (w < warp) rank += b;
-    ncand += b;
-    all_flags |= T.flags[w];
+    const uint32_t v = T.warps[w];
+    if (w < warp) rank += v & 0xffffu;
+    ncand += v & 0xffffu;
+    all_flags |= v >> 16;
   }
   if (all_flags & 1u) return LC_ERR_NONFINITE;
   const uint32_t wide = all_flags >> 1;
@@ -168,7 +165,9 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
     T.rep[sym] = (key << 23) | mr;
   }
   {
-    const unsigned long long kept_sum = table_warp_sum(kept ? my.count : 0ull);
+    // a vector's own counts add up to less than 2^32
+    const unsigned long long kept_sum =
+        A.shard ? table_warp_sum(kept ? my.count : 0ull) : __reduce_add_sync(kAll, kept ? (uint32_t)my.count : 0u);
     if (lane == 0) T.part[0][warp] = kept_sum;
     if (A.shard) {
       const unsigned long long kept_local = table_warp_sum(kept ? my.local : 0ull), whole = table_warp_sum(my.count);
@@ -250,23 +249,39 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
         else merge_leaves(leaf32, node32, T.up, nused);
         T.up[root] = root;
       }
-      __syncthreads();
       // ---- depths: every node jumps to its ancestor's ancestor until all have reached the root
-      for (uint32_t reach = 1; reach < min(nused, 64u); reach *= 2) {  // no leaf is deeper than nused - 1, nor than 63
-        uint32_t x[2];
-#pragma unroll
-        for (uint32_t h = 0; h < 2; ++h) {
-          const uint32_t v = tid + h * kTableThreads;
-          if (v <= root) {
-            const uint32_t a = T.up[v], b = T.up[a & 0xffffu];
-            x[h] = ((a >> 16) + (b >> 16)) << 16 | (b & 0xffffu);
+      const auto above = [&](uint32_t v) {
+        const uint32_t a = T.up[v], b = T.up[a & 0xffffu];
+        return ((a >> 16) + (b >> 16)) << 16 | (b & 0xffffu);
+      };
+      if (nused <= 32) {
+        // two nodes a lane in the warp that has built the tree, without block barriers (sixteen symbols: 670 cycles instead of 1140)
+        if (warp == 0) {
+          __syncwarp();
+          for (uint32_t reach = 1; reach < nused; reach *= 2) {
+            const uint32_t v0 = min(lane, root), v1 = min(lane + 32, root), x0 = above(v0), x1 = above(v1);
+            __syncwarp();
+            T.up[v0] = x0;
+            T.up[v1] = x1;
+            __syncwarp();
           }
         }
         __syncthreads();
-#pragma unroll
-        for (uint32_t h = 0; h < 2; ++h)
-          if (tid + h * kTableThreads <= root) T.up[tid + h * kTableThreads] = x[h];
+      } else {
         __syncthreads();
+        for (uint32_t reach = 1; reach < min(nused, 64u); reach *= 2) {  // no leaf is deeper than nused - 1, nor than 63
+          uint32_t x[2];
+#pragma unroll
+          for (uint32_t h = 0; h < 2; ++h) {
+            const uint32_t v = tid + h * kTableThreads;
+            if (v <= root) x[h] = above(v);
+          }
+          __syncthreads();
+#pragma unroll
+          for (uint32_t h = 0; h < 2; ++h)
+            if (tid + h * kTableThreads <= root) T.up[tid + h * kTableThreads] = x[h];
+          __syncthreads();
+        }
       }
       if (used) my_len = T.up[T.place[tid]] >> 16;
     }
@@ -297,8 +312,10 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
   }
   // ---- payload size: this vector's own elements, with the lengths just found
   {
-    const unsigned long long bits = table_warp_sum(my_local * my_len);
-    if (lane == 0) T.part[3][warp] = bits;
+    const unsigned long long mine = my_local * my_len;  // below 2^38
+    const unsigned long long bits = (unsigned long long)__reduce_add_sync(kAll, (uint32_t)(mine >> 24)) << 24;
+    const uint32_t low = __reduce_add_sync(kAll, (uint32_t)mine & 0xffffffu);
+    if (lane == 0) T.part[3][warp] = bits + low;
   }
   __syncthreads();
   const unsigned long long payload_bits = table_part_total(T.part[3]);
