@@ -71,9 +71,10 @@ __device__ __forceinline__ uint32_t cluster_ld(uint32_t a) {
 // One vector of n <= (CTAs) * M * kChunkElems elements; all threads of the CTA or cluster. dbg: nullptr, or the control
 // block that receives the statistics and the code table (lc_debug_*). Returns 0 or the error that makes the vector
 // unencodable, the same everywhere.
-template <int M, bool CLUSTER>
+// gate: table_pass's; nothing is written to the stream, or to tracked_out, before it.
+template <int M, bool CLUSTER, class Gate = NoGate>
 __device__ __forceinline__ int small_vector(SmallShared<M>& S, const float* base, const float* cur, uint32_t n, int nbits,
-                                            uint8_t* stream, float* tracked_out, Control* dbg) {
+                                            uint8_t* stream, float* tracked_out, Control* dbg, Gate gate = Gate()) {
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t rank = CLUSTER ? cluster_rank() : 0u, ctas = CLUSTER ? cluster_size() : 1u;
   const uint32_t chunk0 = rank * M;  // this CTA's first chunk
@@ -188,7 +189,7 @@ __device__ __forceinline__ int small_vector(SmallShared<M>& S, const float* base
   }
 
   // ---- table pass, in every CTA (its barriers also end the histogram's use); header and symbol table by the first
-  const int err = table_pass(S.T, my, TableArgs{n, nbits, true, false, false, false, nullptr}, stream, rank == 0);
+  const int err = table_pass(S.T, my, TableArgs{n, nbits, true, false, false, false, nullptr}, stream, rank == 0, gate);
   if (err) return err;
   if (n == 0) return LC_OK;
   {

@@ -103,11 +103,17 @@ __device__ __forceinline__ void clear_header(uint8_t* stream) {
   if (threadIdx.x < 4) reinterpret_cast<uint4*>(stream)[threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
 }
 
+struct NoGate {
+  __device__ __forceinline__ bool operator()() const { return true; }
+};
+
+// gate(): called by all threads before the first write to the stream; false, the same for all, ends the pass with LC_ERR_ARG.
 // `my`: the statistics of key_of_position(threadIdx.x). Returns 0, or the error that makes the vector unencodable, the
 // same for all threads; on success the stream's header (but for its total size), table and padding are written (unless
 // !write), and T is complete and visible to all threads.
+template <class Gate = NoGate>
 __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, const TableArgs& A, uint8_t* __restrict__ stream,
-                                          bool write = true) {
+                                          bool write = true, Gate gate = Gate()) {
   constexpr uint32_t kAll = 0xffffffffu;
   constexpr unsigned long long kNone = ~0ull;  // weight behind the end of a queue
   const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -321,6 +327,7 @@ __device__ __forceinline__ int table_pass(TableShared& T, const KeyStats& my, co
   const unsigned long long payload_bits = table_part_total(T.part[3]);
 
   // ---- outputs
+  if (!gate()) return LC_ERR_ARG;
   if (tid == 0) {
     T.rep[0] = 0;
     T.nsym = nsym;
