@@ -161,19 +161,19 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
   const uint32_t tile = s_tile;
   const uint32_t s = find_segment(group.tile_begin, group.nseg, tile);
   const SegBlock& B = blocks[group.block[s]];
-  const uint32_t nsym = B.nsym;
+  static_assert(kSegThreads == 256, "a thread per plane byte");
+  const EncEntry e = B.enc[key_of_byte(tid)];
+  const uint32_t nsym = B.nsym, sym0_len = B.enc[0].len;
   if (nsym == 0) return;  // failed: the same word for every thread
   const uint64_t lo = group.elem_begin[s], n = group.elem_begin[s + 1] - lo;
   uint8_t* stream = streams + group.stream_begin[s];
   const bool wide = B.wide != 0, long_codes = B.max_len > 32;
-  for (uint32_t b = tid; b < 256; b += kSegThreads) {
-    const EncEntry e = B.enc[key_of_byte(b)];
-    tb.full[b] = make_uint2(e.code_lo, e.len);
-    s_rep[b ^ 1] = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
-  }
+  const uint32_t rep = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
+  tb.full[tid] = make_uint2(e.code_lo, e.len);
   __syncthreads();
-  static_assert(kSegThreads == 256, "a thread per plane byte");
-  build_tables(tb, B.enc[0].len, [&](uint32_t b) { return B.enc[key_of_byte(b)].sym != 0; });
+  build_tables(tb, sym0_len, [&](uint32_t) { return e.sym != 0; });
+  s_rep[tid ^ 1] = rep;
+  __syncthreads();
 
   const StreamLayout L = stream_layout(n, nsym);
   const uint32_t first_tile = group.tile_begin[s], last_tile = group.tile_begin[s + 1] - 1;
