@@ -237,7 +237,8 @@ int lc_recover(const float* base, const void* const* streams, const uint64_t* st
     if (!streams[j] || !aligned(streams[j], 16)) return LC_ERR_ARG;
   if (workspace_bytes < workspace_layout(0).total) return LC_ERR_CAPACITY;
   Control* ctl = static_cast<Control*>(workspace);
-  if (cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
+  bool clear = n <= (uint64_t)kClearChunks * kChunkElems;  // by the first launch
+  if (!clear && cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
   // up to four streams per launch; later launches continue in place from `out`.
   const float* src = base;
   for (int first = 0, kk; first < k; first += kk) {
@@ -248,7 +249,13 @@ int lc_recover(const float* base, const void* const* streams, const uint64_t* st
       ds.ptr[j] = static_cast<const uint8_t*>(streams[first + j]);
       ds.bytes[j] = stream_bytes[first + j];
     }
-    if (launch_decode(src, ds, kk, n, out, &ctl->status, first > 0, cs) != cudaSuccess) return LC_ERR_CUDA;
+    cudaError_t e = launch_decode(src, ds, kk, n, out, &ctl->status, first > 0, cs, 0, ~0ull, clear);
+    if (clear && e == cudaErrorNotSupported) {
+      if (cudaMemsetAsync(&ctl->status, 0, sizeof(int32_t), cs) != cudaSuccess) return LC_ERR_CUDA;
+      e = launch_decode(src, ds, kk, n, out, &ctl->status, first > 0, cs);
+    }
+    if (e != cudaSuccess) return LC_ERR_CUDA;
+    clear = false;
     src = out;
   }
   return LC_OK;

@@ -940,7 +940,8 @@ __device__ __forceinline__ void prefetch_rows(const float* first, uint32_t lane)
 
 // Chunks [chunk_begin, chunk_end) of one vector, by `ctas` CTAs of which this is number `cta`.
 // stage_bytes: bytes of staging area per warp and stream (a multiple of 16, at least 32).
-template <int KS, int R>
+// CLEAR: the CTAs are one cluster, whose first clears the status word; none writes to it before.
+template <int KS, int R, bool CLEAR>
 __device__ __forceinline__ void decode_vector(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
                                               Status status, uint32_t stage_bytes, uint32_t chunk_begin,
                                               uint32_t chunk_end, uint32_t cta, uint32_t ctas) {
@@ -950,6 +951,10 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   StreamState* S = reinterpret_cast<StreamState*>(s_raw + kTablePad + KS * 2 * kTableBytes);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const uint32_t nwarps = ctas * warps;
+  if (CLEAR) {
+    if (cta == 0 && threadIdx.x == 0) *status.word = 0;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  }
   begin_next();  // the next group of a chain may prepare its tables on the SMs that this launch leaves
   const uint32_t whole_end = min(chunk_end, (uint32_t)(n / kChunkElems));  // the chunks that are full; at most 2^20 in all
   uint32_t c = chunk_begin + cta * warps + warp;
@@ -969,6 +974,7 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
     }
   }
   __syncthreads();
+  if (CLEAR) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 #pragma unroll
   for (int s = 0; s < KS; ++s) {
     const int err = S[s].err;
@@ -1013,11 +1019,11 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   }
 }
 
-template <int KS, int WARPS, int R>
+template <int KS, int WARPS, int R, bool CLEAR>
 __global__ void __launch_bounds__(32 * WARPS, kDecCtas<KS>)
 decode_kernel(const float* base, DecodeStreams streams, uint64_t n, float* out, int32_t* __restrict__ status, uint32_t rank,
               uint32_t stage_bytes, uint32_t chunk_begin, uint32_t chunk_end) {
-  decode_vector<KS, R>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
+  decode_vector<KS, R, CLEAR>(base, streams, n, out, Status{status, rank}, stage_bytes, chunk_begin, chunk_end, blockIdx.x, gridDim.x);
 }
 
 // Per-layer recovery: the CTAs [cta_begin[i], cta_begin[i + 1]) decode segment i. One launch instead of one per segment
@@ -1041,7 +1047,7 @@ decode_segments_kernel(const float* base, const __grid_constant__ DecodeStreams 
     streams.ptr[s] = buffers.ptr[s] + off;
     streams.bytes[s] = bytes;
   }
-  decode_vector<KS, R>(base + first, streams, n, out + first, Status{status, 2 * (batch.first + lo) + second}, stage_bytes, 0,
+  decode_vector<KS, R, false>(base + first, streams, n, out + first, Status{status, 2 * (batch.first + lo) + second}, stage_bytes, 0,
                     (uint32_t)((n + kChunkElems - 1) / kChunkElems), blockIdx.x - batch.cta_begin[lo],
                     batch.cta_begin[lo + 1] - batch.cta_begin[lo]);
 }
@@ -1147,9 +1153,13 @@ uint32_t balanced_warps(uint64_t chunks, uint64_t ctas, uint32_t most) {
   return w < 4 ? 4 : (uint32_t)w;
 }
 
+constexpr unsigned kMaxClearCtas = 8;  // a portable cluster size
+static_assert(kClearChunks <= 4 * kMaxClearCtas, "four warps a CTA at least");
+
 // second: this launch goes on from what the one before it recovers, and may begin beside its end: tables and first rows do not wait for it (11.7 M
 // elements, eight streams: 81.0 -> 76.0 us).
-template <int KS, int WARPS = kDecWarps<KS>, int R = 2>
+// CLEAR: see decode_vector; at most kClearChunks chunks. cudaErrorNotSupported, with nothing launched: the device has no room for the cluster.
+template <int KS, bool CLEAR, int WARPS = kDecWarps<KS>, int R = 2>
 cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, uint64_t n, float* out,
                              int32_t* status, bool second, uint64_t chunk_begin, uint64_t chunk_end, cudaStream_t cs) {
   static uint32_t regs_of[kMaxDevices] = {};
@@ -1164,13 +1174,14 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
   // where the areas of 20 warps do not fit, the kernel for 16
   if constexpr (KS == 3 && WARPS == 20)
     if (choose_shape(KS, wanted_stage(avg), 96, WARPS).warps < WARPS)
-      return launch_decode_ks<KS, 16>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+      return launch_decode_ks<KS, CLEAR, 16>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
   Shape sh;
-  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(decode_kernel<KS, WARPS, R>), wanted_stage(avg), regs_of, sh);
+  const auto kernel = decode_kernel<KS, WARPS, R, CLEAR>;
+  const cudaError_t e = decode_shape<KS, WARPS>(reinterpret_cast<const void*>(kernel), wanted_stage(avg), regs_of, sh);
   if (e != cudaSuccess) return e;
   const uint64_t chunks = chunk_end - chunk_begin, full = (uint64_t)sh.sms * sh.per_sm;
-  if constexpr (KS == 1 && R == 2)
-    if (!two_rows(chunks, full * sh.warps)) return launch_decode_ks<KS, WARPS, 1>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+  if constexpr (KS == 1 && R == 2 && !CLEAR)
+    if (!two_rows(chunks, full * sh.warps)) return launch_decode_ks<KS, CLEAR, WARPS, 1>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
   const uint32_t warps = balanced_warps(chunks, full, sh.warps);
   uint64_t want = (chunks + warps - 1) / warps;
   if (want == 0) want = 1;  // still reports a rejected stream
@@ -1178,8 +1189,37 @@ cudaError_t launch_decode_ks(const float* base, const DecodeStreams& streams, ui
   // the staging areas of the warps left out go to the others: chunks vary (a layer of rare exponents in a vector of layers
   // takes twice the average), and one that is read from global memory word by word holds up the launch
   const uint32_t stage = min(sh.warps * sh.stage / warps / 16 * 16, kChunkElems * 8 + 16);
-  return launch_kernel(second, decode_kernel<KS, WARPS, R>, grid, warps * 32, sh.dyn - (sh.warps * sh.stage - warps * stage) * KS, cs, base, streams, n, out,
-                       status, second ? 1u : 0u, stage, (uint32_t)chunk_begin, (uint32_t)chunk_end);
+  const size_t dyn = sh.dyn - (sh.warps * sh.stage - warps * stage) * KS;
+  if constexpr (CLEAR) {
+    static int room_of[kMaxDevices] = {};  // by device ordinal: 0 not looked at yet, 1 room, 2 none
+    const int dev = current_device_index();
+    if (dev < 0) return cudaErrorInvalidDevice;
+    unsigned ctas = 1;  // a power of two, so that every size is one the hardware schedules
+    while (ctas < grid) ctas *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    cfg.blockDim = dim3(warps * 32);
+    cfg.stream = cs;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (room_of[dev] == 0) {
+      int fit = 0;
+      at[0].val.clusterDim = {kMaxClearCtas, 1, 1};
+      cfg.gridDim = dim3(kMaxClearCtas);
+      cfg.dynamicSmemBytes = kMaxDyn;
+      room_of[dev] = cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) == cudaSuccess && fit > 0 ? 1 : 2;
+      (void)cudaGetLastError();
+    }
+    if (room_of[dev] == 2 || ctas > kMaxClearCtas) return cudaErrorNotSupported;
+    at[0].val.clusterDim = {ctas, 1, 1};
+    cfg.gridDim = dim3(ctas);
+    cfg.dynamicSmemBytes = dyn;
+    return cudaLaunchKernelEx(&cfg, kernel, base, streams, n, out, status, 0u, stage, (uint32_t)chunk_begin, (uint32_t)chunk_end);
+  } else {
+    return launch_kernel(second, kernel, grid, warps * 32, dyn, cs, base, streams, n, out, status, second ? 1u : 0u, stage, (uint32_t)chunk_begin,
+                         (uint32_t)chunk_end);
+  }
 }
 
 template <int KS, int WARPS = KS == 3 ? 16 : kDecWarps<KS>, int R = 2>
@@ -1284,16 +1324,20 @@ cudaError_t launch_decode_segments(const float* base, const uint8_t* const* stre
 }
 
 cudaError_t launch_decode(const float* base, const DecodeStreams& streams, int k, uint64_t n, float* out,
-                          int32_t* status, bool second, cudaStream_t cs, uint64_t chunk_begin, uint64_t chunk_end) {
-  if (k < 1 || k > 4) return cudaErrorInvalidValue;
+                          int32_t* status, bool second, cudaStream_t cs, uint64_t chunk_begin, uint64_t chunk_end, bool clear) {
+  if (k < 1 || k > 4 || (clear && (second || n > (uint64_t)kClearChunks * kChunkElems))) return cudaErrorInvalidValue;
   const uint64_t all_chunks = (n + kChunkElems - 1) / kChunkElems;
   if (chunk_end > all_chunks) chunk_end = all_chunks;
   if (chunk_begin > chunk_end) chunk_begin = chunk_end;
   switch (k) {
-    case 1: return launch_decode_ks<1>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
-    case 2: return launch_decode_ks<2>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
-    case 3: return launch_decode_ks<3>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
-    case 4: return launch_decode_ks<4>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+    case 1: return clear ? launch_decode_ks<1, true>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs)
+                         : launch_decode_ks<1, false>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+    case 2: return clear ? launch_decode_ks<2, true>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs)
+                         : launch_decode_ks<2, false>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+    case 3: return clear ? launch_decode_ks<3, true>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs)
+                         : launch_decode_ks<3, false>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
+    case 4: return clear ? launch_decode_ks<4, true>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs)
+                         : launch_decode_ks<4, false>(base, streams, n, out, status, second, chunk_begin, chunk_end, cs);
     default: return cudaErrorInvalidValue;
   }
 }
