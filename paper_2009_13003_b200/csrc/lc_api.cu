@@ -99,7 +99,7 @@ int compress_impl(const float* base, const float* cur, uint64_t n, int nbits, vo
   // The four kernels are launched so that each may begin before the one ahead of it has ended.
   const uint64_t control = opt.mean_rep ? sizeof(Control) : offsetof(Control, enc);  // the sums of the variant lie behind enc
   const uint64_t groups = scan_group_words(W.nchunks);
-  cudaError_t e = launch_clear(c.ctl, control, c.tiles - groups, 8 * groups + align_up(8 * W.nchunks, 16), keep_status, cs);
+  cudaError_t e = launch_clear(c.ctl, control, c.tiles - groups, 8 * groups + align_up(8 * W.nchunks, 16), keep_status, cs, /*overlap=*/keep_status);
   if (e != cudaSuccess) return LC_ERR_CUDA;
   if ((e = launch_stats(base, cur, n, c.ctl, c.plane, cs, opt.mean_rep, true)) != cudaSuccess) return LC_ERR_CUDA;
   if ((e = launch_table(c.ctl, n, nbits, static_cast<uint8_t*>(stream), true, opt.fixed_width, nullptr, opt.length_cache, cs,

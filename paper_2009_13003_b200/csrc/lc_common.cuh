@@ -199,8 +199,9 @@ constexpr uint64_t kLengthCacheBytes = 512ull * kLengthCacheRow;
 constexpr uint64_t kSmallMaxElems = 32 * kChunkElems;
 
 // Zeroes two ranges (16-byte aligned, multiples of 16 bytes; the first word of `a` is kept if keep_first) with a kernel, the
-// first of a chain of overlapped launches: unlike a memset it lets the next kernel begin beside it.
-cudaError_t launch_clear(void* a, uint64_t a_bytes, void* b, uint64_t b_bytes, bool keep_first, cudaStream_t cs);
+// first of a chain of overlapped launches: unlike a memset it lets the next kernel begin beside it. overlap: the launch ahead is one of this library's, and
+// this one goes on as soon as that has ended (lc_merge, 0.3 M elements, two streams: 57.0 -> 53.7 us blocking, 20 M, four: 149.6 -> 147.9 queued).
+cudaError_t launch_clear(void* a, uint64_t a_bytes, void* b, uint64_t b_bytes, bool keep_first, cudaStream_t cs, bool overlap = false);
 
 // ---- launchers (each defined next to its kernel) ---------------------------------------------------
 // the whole compress pass of a small vector (0 < n <= kSmallMaxElems) in one launch; tracked_out may be null.

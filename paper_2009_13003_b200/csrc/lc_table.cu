@@ -61,16 +61,17 @@ __device__ __forceinline__ void clear_range(uint4* p, uint64_t count, bool keep_
 }
 
 __global__ void __launch_bounds__(256) clear_kernel(uint4* a, uint64_t a_count, uint4* b, uint64_t b_count, uint32_t keep_first) {
-  begin_next();
+  wait_previous();
+  begin_next();  // only now: the statistics pass reads what the launch before this one writes
   clear_range(a, a_count, keep_first != 0);
   clear_range(b, b_count, false);
 }
 
 }  // namespace
 
-cudaError_t launch_clear(void* a, uint64_t a_bytes, void* b, uint64_t b_bytes, bool keep_first, cudaStream_t cs) {
+cudaError_t launch_clear(void* a, uint64_t a_bytes, void* b, uint64_t b_bytes, bool keep_first, cudaStream_t cs, bool overlap) {
   const uint64_t items = (a_bytes > b_bytes ? a_bytes : b_bytes) / 16, ctas = (items + 255) / 256;
-  return launch_kernel(false, clear_kernel, (unsigned)(ctas < 1 ? 1 : ctas > 148 ? 148 : ctas), 256, 0, cs, static_cast<uint4*>(a),
+  return launch_kernel(overlap, clear_kernel, (unsigned)(ctas < 1 ? 1 : ctas > 148 ? 148 : ctas), 256, 0, cs, static_cast<uint4*>(a),
                        a_bytes / 16, static_cast<uint4*>(b), b_bytes / 16, keep_first ? 1u : 0u);
 }
 
