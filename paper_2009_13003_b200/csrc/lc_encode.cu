@@ -28,7 +28,7 @@
 // the key plane.
 //
 // The vector's partial last chunk takes a masked form of A. Rare cases take a compact two-pass path (lengths, then bits
-// ORed in place): codes longer than 32 bits, a lane or chunk that outgrows its shared-memory area, and chunks with an
+// ORed in place; chunk_slow): codes longer than 32 bits, a lane or chunk that outgrows its shared-memory area, and chunks with an
 // exponent field >= 128, for which the one-byte key plane is not enough and keys come from base and cur.
 //
 // Bound: reads 1 byte and writes about 0.5 bytes per element, so this pass is limited by the integer work per element,
@@ -49,6 +49,7 @@ constexpr int kEncThreads = kEncWarps * 32;
 // element that is all 8; with 44 KB it was up to 4.7, and 134 M elements in codes of a fixed 5 bits took 362 us instead of 322
 // (with the tracked state 498 instead of 433).
 constexpr uint32_t kEncSmem = 48 * 1024;
+constexpr uint32_t kEncDyn = kTablesBytes + kEncSmem;
 // bytes of a share's half that an average chunk of `avg` bytes needs: 15 % more, for the lanes and chunks above the average
 __host__ __device__ constexpr uint64_t share_need(uint64_t avg) { return avg + avg / 7 + 64; }
 static_assert(share_need(kChunkElems * 5 / 8) <= kEncSmem / kEncWarps / 2, "codes of 5 bits throughout are coded by all warps");
@@ -66,8 +67,9 @@ __global__ void __launch_bounds__(kEncThreads, UPDATE ? 3 : 4)
 encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles, const uint8_t* __restrict__ plane,
               const float* base, const float* __restrict__ cur, uint64_t n, uint8_t* __restrict__ stream,
               float* tracked_out, uint32_t spin_limit, uint32_t ticket_bias, uint32_t two_pass_scan) {
-  extern __shared__ __align__(128) uint32_t s_dyn[];  // rows that straddle lines cost the asynchronous copies of UPDATE 5 %
-  __shared__ Tables tb;
+  extern __shared__ __align__(128) uint32_t s_all[];
+  Tables& tb = shared_tables();
+  uint32_t* s_dyn = s_all + kTablesBytes / 4;  // rows that straddle lines cost the asynchronous copies of UPDATE 5 %
   // What warps hand each other in iteration i of the loop. A warp may reach the next iteration's barrier while another is still behind this one's, so
   // the words alternate: those read behind the iteration's barrier by i % 2, those that the next iteration reads too by i % 3.
   __shared__ uint32_t s_chunk_bytes[3][kEncWarps];
@@ -96,6 +98,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     s_tile[0] = atomicAdd(&ctl->ticket, 1u) + ticket_bias;
     s_arrived[0] = s_arrived[1] = s_arrived[2] = 0;
   }
+  if (tid == 0) tb.long_codes = long_codes;
   tb.full[tid] = make_uint2(e.code_lo, e.len);
   __syncthreads();
   if (s_abort[0] != 0) return;
@@ -547,13 +550,13 @@ cudaError_t launch_encode(Control* ctl, unsigned long long* tiles, const uint8_t
   const int v = tracked_out ? 1 : 0;
   if (blocks_per_sm[dev][v] == 0) {
     const void* fn = v ? reinterpret_cast<const void*>(encode_kernel<true>) : reinterpret_cast<const void*>(encode_kernel<false>);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncSmem + (v ? kUpdSmem : 0));
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kEncDyn + (v ? kUpdSmem : 0));
     if (e != cudaSuccess) return e;
     int nsm = 0;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     int bps = 0;
-    e = v ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, encode_kernel<true>, kEncThreads, kEncSmem + kUpdSmem)
-          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, encode_kernel<false>, kEncThreads, kEncSmem);
+    e = v ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, encode_kernel<true>, kEncThreads, kEncDyn + kUpdSmem)
+          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, encode_kernel<false>, kEncThreads, kEncDyn);
     if (e != cudaSuccess) return e;
     sms[dev] = nsm;
     blocks_per_sm[dev][v] = bps > 0 ? bps : 1;
@@ -570,9 +573,9 @@ cudaError_t launch_encode(Control* ctl, unsigned long long* tiles, const uint8_t
   const uint32_t two = opt.two_pass_scan ? 1u : 0u;
   overlap = overlap && !opt.two_pass_scan;
   if (v)
-    return launch_kernel(overlap, encode_kernel<true>, grid, kEncThreads, kEncSmem + kUpdSmem, cs, ctl, tiles, plane, base, cur, n, stream,
+    return launch_kernel(overlap, encode_kernel<true>, grid, kEncThreads, kEncDyn + kUpdSmem, cs, ctl, tiles, plane, base, cur, n, stream,
                          tracked_out, opt.spin_limit, opt.ticket_bias, two);
-  return launch_kernel(overlap, encode_kernel<false>, grid, kEncThreads, kEncSmem, cs, ctl, tiles, plane, base, cur, n, stream,
+  return launch_kernel(overlap, encode_kernel<false>, grid, kEncThreads, kEncDyn, cs, ctl, tiles, plane, base, cur, n, stream,
                        static_cast<float*>(nullptr), opt.spin_limit, opt.ticket_bias, two);
 }
 

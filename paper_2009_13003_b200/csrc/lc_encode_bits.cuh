@@ -31,7 +31,15 @@ struct Tables {
   uint32_t best, below, above;
   int32_t base;        // see build_tables
   uint32_t use_pair;
+  uint32_t long_codes;  // set by the kernel: some code is longer than 32 bits
 };
+// They lie at the start of the dynamic shared memory, so that the out-of-line functions below need no pointer to them (as one more argument it cost the
+// encode pass's main loop registers: 268 M elements 158 us instead of 148).
+constexpr uint32_t kTablesBytes = (uint32_t)((sizeof(Tables) + 127) / 128 * 128);
+__device__ __forceinline__ Tables& shared_tables() {
+  extern __shared__ __align__(128) unsigned char s_tables[];
+  return *reinterpret_cast<Tables*>(s_tables);
+}
 
 __device__ __forceinline__ uint32_t make_entry(uint32_t code, uint32_t len, uint32_t longest) {
   return len > longest ? kEntryLong : (len ? code << (32 - len) : 0u) | len;
@@ -154,12 +162,44 @@ static __device__ __noinline__ bool has_escape(const uint8_t* plane, uint32_t c,
   return __any_sync(0xffffffffu, zero != 0);
 }
 
+// A whole chunk from the CTA's tables: with dst == nullptr returns the lane's bits, otherwise ORs them into the zeroed chunk image at `dst`. Plane bytes
+// as the fast path reads them.
+__device__ __forceinline__ uint32_t chunk_from_tables(const Tables& tb, const uint4* ep, uint32_t* dst, uint32_t lane_start) {
+  uint32_t bits = 0;
+  OrPacker pk{0ull, lane_start & 31u, dst ? dst + (lane_start >> 5) : nullptr};
+  uint4 v = ep[0];
+#pragma unroll 1
+  for (uint32_t q = 0; q < kSteps / 4; ++q) {
+    const uint4 nxt = ep[32 * (q + 1 < kSteps / 4 ? q + 1 : q)];
+    const uint32_t words[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (uint32_t r = 0; r < 4; ++r) {
+      uint2 f[kGroup];
+#pragma unroll
+      for (uint32_t e = 0; e < kGroup; ++e) {
+        f[e] = tb.full[__byte_perm(words[r], 0u, 0x4440 + e)];
+        bits += f[e].y;
+      }
+      if (dst) {
+#pragma unroll
+        for (uint32_t e = 0; e < kGroup; ++e) pk.put(f[e].x, f[e].y);
+      }
+    }
+    v = nxt;
+  }
+  if (dst) pk.flush();
+  return bits;
+}
+
 // Slow, compact path (see the header). With dst == nullptr it only returns the lane's bit count;
 // otherwise it ORs the lane's bits into the zeroed chunk image at dst, starting at bit lane_start.
-// The plane bytes of four steps are read as one 16-byte vector, the way the fast path reads them. Codes come from the per-key table in global memory:
-// passing the CTA's shared tables in as well was measured to cost the kernel's main loop 4 %.
+// The plane bytes of four steps are read as one 16-byte vector, the way the fast path reads them. Codes come from the per-key table in global memory.
 static __device__ __noinline__ uint32_t chunk_slow(const EncEntry* __restrict__ enc, KeySource ks, uint64_t c,
                                             uint32_t lane, uint64_t n, uint32_t* dst, uint32_t lane_start) {
+  // A whole chunk that outgrew its columns or its image. (A vector of layers has some where exponents are rare, and a launch of one round of chunks waits for them:
+  // 11.7 M elements in 62 layers, that have such a chunk, 88 us in 4 bits and 107 in 5 by the loop below, 62 and 70 so; 46.5 and 48 without one.)
+  if ((c + 1) * kChunkElems <= n && !ks.wide && !shared_tables().long_codes)
+    return chunk_from_tables(shared_tables(), reinterpret_cast<const uint4*>(ks.plane + c * kChunkElems) + lane, dst, lane_start);
   OrPacker pk{0ull, lane_start & 31u, dst ? dst + (lane_start >> 5) : nullptr};
   uint32_t bits = 0;
   const bool from_plane = !ks.wide;

@@ -144,8 +144,9 @@ __global__ void __launch_bounds__(kSegThreads, 3)
 segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ blocks, unsigned long long* __restrict__ tiles,
                        const float* base, const float* cur, uint8_t* __restrict__ streams, float* tracked_out,
                        uint32_t lane_words, uint32_t image_bytes, uint32_t spin_limit, const __grid_constant__ SegGroup group) {
-  extern __shared__ __align__(128) unsigned char s_dyn[];
-  __shared__ Tables tb;
+  extern __shared__ __align__(128) unsigned char s_all[];
+  Tables& tb = shared_tables();
+  unsigned char* s_dyn = s_all + kTablesBytes;
   __shared__ uint32_t s_rep[256];  // representative (bit pattern) by the low byte of a slot, which is plane byte ^ 1
   __shared__ uint32_t s_bytes[kEncWarps];
   __shared__ uint32_t s_tile;
@@ -169,6 +170,7 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
   uint8_t* stream = streams + group.stream_begin[s];
   const bool wide = B.wide != 0, long_codes = B.max_len > 32;
   const uint32_t rep = *reinterpret_cast<const uint32_t*>(stream + kHeaderBytes + kTableEntryBytes * e.sym + 4);
+  if (tid == 0) tb.long_codes = long_codes;
   tb.full[tid] = make_uint2(e.code_lo, e.len);
   __syncthreads();
   build_tables(tb, sym0_len, [&](uint32_t) { return e.sym != 0; });
@@ -393,7 +395,7 @@ cudaError_t launch_compress_segments(Control* ctl, SegBlock* blocks, unsigned lo
     if (e == cudaSuccess) e = cudaFuncSetAttribute(segments_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(small::SmallShared<1>));
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(segments_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(kEncWarps * (seg_lane_words(kMaxNbits) * 128 + seg_image_bytes(kMaxNbits))));
+                               (int)(kTablesBytes + kEncWarps * (seg_lane_words(kMaxNbits) * 128 + seg_image_bytes(kMaxNbits))));
     if (e != cudaSuccess) return e;
     sms_of[dev] = v;
   }
@@ -423,7 +425,7 @@ cudaError_t launch_compress_segments(Control* ctl, SegBlock* blocks, unsigned lo
   const uint32_t ntiles = group.tile_begin[group.nseg];
   if (e == cudaSuccess && ntiles > 0) {
     const uint32_t lane_words = seg_lane_words(nbits), image_bytes = seg_image_bytes(nbits);
-    e = launch_kernel(true, segments_encode_kernel, ntiles, kSegThreads, kEncWarps * (lane_words * 128 + image_bytes), cs, ctl, blocks,
+    e = launch_kernel(true, segments_encode_kernel, ntiles, kSegThreads, kTablesBytes + kEncWarps * (lane_words * 128 + image_bytes), cs, ctl, blocks,
                       tiles, base, cur, streams, tracked_out, lane_words, image_bytes, EncodeOptions().spin_limit, group);
   }
   return e;
