@@ -44,7 +44,7 @@ namespace {
 using namespace enc;
 
 constexpr int kEncThreads = kEncWarps * 32;
-// 48 KB of dynamic shared memory per CTA (four CTAs per SM, beside 7 KB of tables), split evenly between the warps that work:
+// 48 KB of shared memory per CTA for coding (four CTAs per SM, beside 8 KB of tables), split evenly between the warps that work:
 // all 8 while an average chunk fits half of a 6 KB share (column matrix + chunk image), else 4, 2 or 1. Up to 5.1 bits per
 // element that is all 8; with 44 KB it was up to 4.7, and 134 M elements in codes of a fixed 5 bits took 362 us instead of 322
 // (with the tracked state 498 instead of 433).
