@@ -979,8 +979,8 @@ __device__ __forceinline__ void decode_vector(const float* base, const DecodeStr
   for (int s = 0; s < KS; ++s) {
     const int err = S[s].err;
     if (err) {  // the same words for every thread
+      wait_previous();  // the launch before this one may clear the word; and the order of the launches reaches back to the first
       if (threadIdx.x == 0) status.set(err);
-      wait_previous();  // the order of the launches reaches back to the first
       return;
     }
   }

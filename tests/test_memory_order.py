@@ -1,0 +1,26 @@
+"""Orders of memory accesses that no run shows reliably, looked up in the kernels' source. CPU only."""
+import os
+import re
+
+from conftest import ROOT
+
+
+def body(file, head):
+    """The brace-matched body, without comments, of the first function whose declaration contains `head`."""
+    text = re.sub(r"//.*", "", open(os.path.join(ROOT, "paper_2009_13003_b200", "csrc", file)).read())
+    begin = text.index("{", text.index(head))
+    depth = 0
+    for i in range(begin, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        if depth == 0:
+            return text[begin: i + 1]
+    raise AssertionError(head)
+
+
+def test_a_rejected_stream_is_reported_behind_the_launch_before():
+    # The launch before a chain's later one may be the one that clears the status word: an error set ahead of
+    # wait_previous() could be cleared again. Only that clearing itself, in the first launch, is ahead of it.
+    text = body("lc_decode.cu", "void decode_vector(")
+    ahead = text[: text.index("wait_previous()")]
+    assert re.findall(r"status\s*\.\s*\w+[^;]*;", ahead) == ["status.word = 0;"]
+    assert "status.set(err)" in text[len(ahead):]
