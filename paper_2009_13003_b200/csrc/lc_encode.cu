@@ -232,6 +232,8 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
     }
     arrival = __shfl_sync(0xffffffffu, arrival, 0);
     if (arrival == kEncWarps - 1 && have && !two_pass_scan) {
+      __threadfence_block();  // lane 0 has seen the other warps arrive; behind this and the warp's barrier all lanes see their sizes
+      __syncwarp();
       uint32_t bytes = 0;
       if (lane < kEncWarps) bytes = *reinterpret_cast<volatile uint32_t*>(&s_chunk_bytes[buf][lane]);
       bytes = __reduce_add_sync(0xffffffffu, bytes);

@@ -24,3 +24,14 @@ def test_a_rejected_stream_is_reported_behind_the_launch_before():
     ahead = text[: text.index("wait_previous()")]
     assert re.findall(r"status\s*\.\s*\w+[^;]*;", ahead) == ["status.word = 0;"]
     assert "status.set(err)" in text[len(ahead):]
+
+
+def test_the_last_warp_to_arrive_reads_the_sizes_behind_a_fence():
+    # Every warp writes its chunk's size, then (behind a fence) adds itself to the count; lane 0 of the last one sees the
+    # count, other lanes read the sizes.
+    text = body("lc_encode.cu", "encode_kernel(Control*")
+    write, count = text.index("s_chunk_bytes[buf][warp] = chunk_bytes"), text.index("atomicAdd(&s_arrived[buf]")
+    read = text.index("&s_chunk_bytes[buf][lane]")
+    assert write < text.index("__threadfence_block()", write) < count
+    branch = text[text.index("arrival == kEncWarps - 1", count): read]
+    assert 0 < branch.find("__threadfence_block()") < branch.find("__syncwarp()")
