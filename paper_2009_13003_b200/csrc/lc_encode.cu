@@ -210,7 +210,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
       fast = true;
     }
     if (fast && __any_sync(0xffffffffu, lane_bits == 0xffffffffu)) fast = false;  // some lane outgrew its column: redo the chunk the slow way
-    if (!fast && valid) lane_bits = chunk_slow(ctl->enc, keys(wide), c, lane, n, nullptr, 0);
+    if (!fast && valid) lane_bits = chunk_slow<true>(ctl->enc, keys(wide), c, lane, n, nullptr, 0);
 
     // ---- B: lane offsets, lane index, chunk size; the tile's size is published as early as possible
     if (valid) lane_index[c * kLanes + lane] = (uint16_t)lane_bits;
@@ -361,7 +361,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
           for (uint32_t k = lane; k < p_chunk_bytes / 16; k += 32) dst4[k] = make_uint4(0, 0, 0, 0);
           __threadfence_block();
           __syncwarp();
-          chunk_slow(ctl->enc, keys(wide_chunk(p_c)), p_c, lane, n, reinterpret_cast<uint32_t*>(dst4), image[lane]);
+          chunk_slow<true>(ctl->enc, keys(wide_chunk(p_c)), p_c, lane, n, reinterpret_cast<uint32_t*>(dst4), image[lane]);
         }
       }
       if (p_tile == ntiles - 1 && tid == 0) {
@@ -449,7 +449,7 @@ encode_kernel(Control* __restrict__ ctl, unsigned long long* __restrict__ tiles,
         uint4* im4 = reinterpret_cast<uint4*>(image);
         for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) im4[k] = make_uint4(0, 0, 0, 0);
         __syncwarp();
-        chunk_slow(ctl->enc, keys(wide), c, lane, n, image, lane_start);
+        chunk_slow<true>(ctl->enc, keys(wide), c, lane, n, image, lane_start);
       }
     } else if (valid) {
       image[lane] = lane_start;
@@ -499,7 +499,7 @@ encode_sizes_kernel(const Control* __restrict__ ctl, unsigned long long* __restr
           bits += s_len[w[r] & 255u] + s_len[(w[r] >> 8) & 255u] + s_len[(w[r] >> 16) & 255u] + s_len[w[r] >> 24];
       }
     } else {
-      bits = chunk_slow(ctl->enc, KeySource{plane, base, cur, wide}, c, lane, n, nullptr, 0);
+      bits = chunk_slow<false>(ctl->enc, KeySource{plane, base, cur, wide}, c, lane, n, nullptr, 0);
     }
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) bits += __shfl_xor_sync(0xffffffffu, bits, d);

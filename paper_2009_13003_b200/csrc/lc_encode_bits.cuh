@@ -194,12 +194,15 @@ __device__ __forceinline__ uint32_t chunk_from_tables(const Tables& tb, const ui
 // Slow, compact path (see the header). With dst == nullptr it only returns the lane's bit count;
 // otherwise it ORs the lane's bits into the zeroed chunk image at dst, starting at bit lane_start.
 // The plane bytes of four steps are read as one 16-byte vector, the way the fast path reads them. Codes come from the per-key table in global memory.
+// TABLES: the kernel keeps the CTA's code tables at the start of its dynamic shared memory (one launched without them has nothing there to read).
+template <bool TABLES>
 static __device__ __noinline__ uint32_t chunk_slow(const EncEntry* __restrict__ enc, KeySource ks, uint64_t c,
                                             uint32_t lane, uint64_t n, uint32_t* dst, uint32_t lane_start) {
   // A whole chunk that outgrew its columns or its image. (A vector of layers has some where exponents are rare, and a launch of one round of chunks waits for them:
   // 11.7 M elements in 62 layers, that have such a chunk, 88 us in 4 bits and 107 in 5 by the loop below, 62 and 70 so; 46.5 and 48 without one.)
-  if ((c + 1) * kChunkElems <= n && !ks.wide && !shared_tables().long_codes)
-    return chunk_from_tables(shared_tables(), reinterpret_cast<const uint4*>(ks.plane + c * kChunkElems) + lane, dst, lane_start);
+  if constexpr (TABLES)
+    if ((c + 1) * kChunkElems <= n && !ks.wide && !shared_tables().long_codes)
+      return chunk_from_tables(shared_tables(), reinterpret_cast<const uint4*>(ks.plane + c * kChunkElems) + lane, dst, lane_start);
   OrPacker pk{0ull, lane_start & 31u, dst ? dst + (lane_start >> 5) : nullptr};
   uint32_t bits = 0;
   const bool from_plane = !ks.wide;

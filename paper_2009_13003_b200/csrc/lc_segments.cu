@@ -247,7 +247,7 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
     }
     if (__any_sync(0xffffffffu, lane_bits == 0xffffffffu)) fast = false;  // some lane outgrew its column
   }
-  if (!fast && valid) lane_bits = chunk_slow(B.enc, ks, c, lane, n, nullptr, 0);
+  if (!fast && valid) lane_bits = chunk_slow<true>(B.enc, ks, c, lane, n, nullptr, 0);
 
   // ---- B: lane offsets, lane index, chunk size
   if (valid) reinterpret_cast<uint16_t*>(stream + L.lane_index_off)[c * kLanes + lane] = (uint16_t)lane_bits;
@@ -356,7 +356,7 @@ segments_encode_kernel(Control* __restrict__ ctl, const SegBlock* __restrict__ b
       for (uint32_t k = lane; k < chunk_bytes / 16; k += 32) dst4[k] = make_uint4(0, 0, 0, 0);
       __threadfence_block();
       __syncwarp();
-      chunk_slow(B.enc, ks, c, lane, n, reinterpret_cast<uint32_t*>(dst4), lane_start);
+      chunk_slow<true>(B.enc, ks, c, lane, n, reinterpret_cast<uint32_t*>(dst4), lane_start);
     }
   }
   if (tile == last_tile && tid == 0) {

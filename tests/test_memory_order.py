@@ -1,6 +1,8 @@
-"""Orders of memory accesses that no run shows reliably, looked up in the kernels' source. CPU only."""
+"""What memory the kernels touch and in which order, where no run shows it reliably: looked up in their source. CPU only."""
 import os
 import re
+
+import pytest
 
 from conftest import ROOT
 
@@ -35,3 +37,11 @@ def test_the_last_warp_to_arrive_reads_the_sizes_behind_a_fence():
     assert write < text.index("__threadfence_block()", write) < count
     branch = text[text.index("arrival == kEncWarps - 1", count): read]
     assert 0 < branch.find("__threadfence_block()") < branch.find("__syncwarp()")
+
+
+@pytest.mark.parametrize("file,head", [("lc_encode.cu", "encode_kernel(Control*"), ("lc_encode.cu", "encode_sizes_kernel(const Control*"),
+                                       ("lc_segments.cu", "segments_encode_kernel(Control*")])
+def test_only_kernels_with_code_tables_send_the_slow_path_to_them(file, head):
+    # The tables lie at the start of the dynamic shared memory, of which encode_sizes_kernel is launched with none.
+    text = body(file, head)
+    assert set(re.findall(r"\bchunk_slow(\S*?)\(", text)) == {"<true>" if "shared_tables()" in text else "<false>"}
