@@ -283,7 +283,10 @@ int lc_last_status(const void* workspace, lc_cuda_stream_t cs);
  * as it was for that call; workspace 256-byte, stream and page 16-byte aligned. Returns the status word (the header
  * means something only if that is LC_OK) or LC_ERR_ARG / LC_ERR_CUDA.
  * page   HOST, NULL or LC_WAIT_PAGE_BYTES of page-locked memory (cudaHostAlloc, cudaHostRegister) that no other call uses
- *        meanwhile: the outcome then arrives there from a kernel, which is faster than a copy of each part. */
+ *        meanwhile: the outcome then arrives there from a kernel, which is faster than a copy of each part. The calling
+ *        thread looks at it for some milliseconds, and only then waits for `cs`; it waits for `cs` at once if the device's
+ *        flags ask for yielding or blocking (cudaSetDeviceFlags). With a page the call may return while that kernel,
+ *        the last thing that it has enqueued, is still ending: `cs` need not be idle yet (cudaStreamQuery). */
 #define LC_WAIT_PAGE_BYTES 128
 int lc_wait(const void* workspace, const void* stream, lc_info* info, void* page, lc_cuda_stream_t cs);
 

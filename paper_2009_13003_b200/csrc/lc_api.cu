@@ -62,7 +62,20 @@ void parse_header(const uint8_t* h, lc_info* info) {
 constexpr uint32_t kResultWords = kHeaderBytes / 4 + 1;
 static_assert(kResultWords * 4 <= LC_WAIT_PAGE_BYTES, "size promised by the header");
 constexpr uint32_t kNoResult = 0x80000000u;     // no status
-constexpr uint32_t kPollsPerQuery = 1u << 12;  // looks at the word between looks at the stream, which would not get there if a kernel failed
+constexpr uint32_t kPolls = 1u << 18;           // looks at the word, some milliseconds, before the stream is waited for: by then 3 us more are nothing
+
+// Between two looks at a word in memory: leaves the core's other thread the execution units.
+inline void pause_core() {
+#if defined(__x86_64__)
+  asm volatile("pause" ::: "memory");
+#endif
+}
+
+// Whether a thread that waits for the current device is meant to keep its core (cudaSetDeviceFlags).
+bool may_poll() {
+  unsigned flags = 0;
+  return cudaGetDeviceFlags(&flags) == cudaSuccess && (flags & (cudaDeviceScheduleYield | cudaDeviceScheduleBlockingSync)) == 0;
+}
 
 __global__ void result_kernel(const int32_t* status, const uint32_t* header, uint32_t* page) {
   const uint32_t i = threadIdx.x;
@@ -483,12 +496,10 @@ int lc_wait(const void* workspace, const void* stream, lc_info* info, void* page
     const cudaError_t e = launch_kernel(true, result_kernel, 1, 32, 0, cs, &ctl->status, static_cast<const uint32_t*>(stream),
                                         static_cast<uint32_t*>(mapped));
     if (e != cudaSuccess) return LC_ERR_CUDA;
-    for (uint32_t polls = 1; *word == kNoResult; ++polls) {
-      if (polls % kPollsPerQuery) continue;
-      const cudaError_t q = cudaStreamQuery(cs);
-      if (q == cudaErrorNotReady) continue;
-      if (q != cudaSuccess || *word == kNoResult) return LC_ERR_CUDA;
-    }
+    if (may_poll())
+      for (uint32_t polls = 0; *word == kNoResult && polls < kPolls; ++polls) pause_core();
+    // not polled for, or long in coming, or a kernel ahead of it has failed
+    if (*word == kNoResult && (cudaStreamSynchronize(cs) != cudaSuccess || *word == kNoResult)) return LC_ERR_CUDA;
     std::atomic_thread_fence(std::memory_order_acquire);
     memcpy(words, page, sizeof words);
   } else {
