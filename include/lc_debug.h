@@ -47,6 +47,11 @@ int lc_debug_compress_wait(const float* base, const float* cur, uint64_t n, int 
                            uint64_t stream_capacity, void* workspace, uint64_t workspace_bytes, uint32_t spin_limit,
                            uint32_t first_ticket, lc_cuda_stream_t cs);
 
+/* The same for lc_compress_update, whose encode pass is a kernel of its own. */
+int lc_debug_update_wait(const float* base, const float* cur, uint64_t n, int nbits, void* stream,
+                         uint64_t stream_capacity, float* tracked_out, void* workspace, uint64_t workspace_bytes,
+                         uint32_t spin_limit, uint32_t first_ticket, lc_cuda_stream_t cs);
+
 /*
  * How one launch of lc_recover_segments (at most 160 segments) is dealt out to CTAs of `warps` warps on a device that holds
  * `slots` of them at once: segment i is decoded by the CTAs cta_begin[i] .. cta_begin[i + 1] - 1 (HOST, nseg + 1 entries).

@@ -21,7 +21,7 @@ WAIT_PAGE_BYTES = 128
 SYMBOLS = (
     "lc_version", "lc_strerror", "lc_stream_bound", "lc_workspace_bytes", "lc_compress", "lc_compress_update", "lc_compress_timed",
     "lc_recover", "lc_compress_opt", "lc_compress_cached",
-    "lc_segments_layout", "lc_compress_segments", "lc_recover_segments", "lc_debug_compress_wait", "lc_merge", "lc_compress_async", "lc_shard_stats", "lc_shard_encode",
+    "lc_segments_layout", "lc_compress_segments", "lc_recover_segments", "lc_debug_compress_wait", "lc_debug_update_wait", "lc_merge", "lc_compress_async", "lc_shard_stats", "lc_shard_encode",
     "lc_stream_info", "lc_last_status", "lc_wait", "lc_host_arena_bytes", "lc_compress_host", "lc_recover_host",
     "lc_debug_bins", "lc_debug_codes", "lc_debug_split_segments", "lc_debug_decode_warps",
     "lc_compress_noalloc",
@@ -76,6 +76,7 @@ def lib():
     L.lc_compress_segments.argtypes = [vp, vp, C.POINTER(u64), i32, i32, vp, u64, vp, vp, u64, vp]
     L.lc_recover_segments.argtypes = [vp, C.POINTER(vp), i32, C.POINTER(u64), i32, i32, vp, vp, u64, vp]
     L.lc_debug_compress_wait.argtypes = [vp, vp, u64, i32, vp, u64, vp, u64, C.c_uint32, C.c_uint32, vp]
+    L.lc_debug_update_wait.argtypes = [vp, vp, u64, i32, vp, u64, vp, vp, u64, C.c_uint32, C.c_uint32, vp]
     L.lc_compress_timed.argtypes = [vp, vp, u64, i32, vp, u64, vp, u64, vp, C.POINTER(C.c_float)]
     L.lc_recover.argtypes = [vp, C.POINTER(vp), C.POINTER(u64), i32, u64, vp, vp, u64, vp]
     L.lc_compress_async.argtypes = [vp, vp, u64, i32, vp, u64, vp, u64, vp, vp, vp]
@@ -173,6 +174,14 @@ def debug_compress_wait(base, cur, nbits, stream, workspace, spin_limit, first_t
                                       stream.numel(), workspace.data_ptr(), workspace.numel(), spin_limit,
                                       first_ticket, _cs(base.device))
     _check(rc, "lc_debug_compress_wait")
+
+
+def debug_update_wait(base, cur, nbits, stream, tracked_out, workspace, spin_limit, first_ticket):
+    """lc_debug_update_wait: lc_compress_update with the look-back's poll limit and first tile number given."""
+    rc = lib().lc_debug_update_wait(base.data_ptr(), cur.data_ptr(), base.numel(), nbits, stream.data_ptr(),
+                                    stream.numel(), tracked_out.data_ptr(), workspace.data_ptr(), workspace.numel(),
+                                    spin_limit, first_ticket, _cs(base.device))
+    _check(rc, "lc_debug_update_wait")
 
 
 def compress_timed(base, cur, nbits, stream, workspace):

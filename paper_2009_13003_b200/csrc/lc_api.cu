@@ -213,6 +213,17 @@ int lc_debug_compress_wait(const float* base, const float* cur, uint64_t n, int 
   return compress_impl(base, cur, n, nbits, stream, stream_capacity, nullptr, workspace, workspace_bytes, opt, cs);
 }
 
+int lc_debug_update_wait(const float* base, const float* cur, uint64_t n, int nbits, void* stream,
+                         uint64_t stream_capacity, float* tracked_out, void* workspace, uint64_t workspace_bytes,
+                         uint32_t spin_limit, uint32_t first_ticket, lc_cuda_stream_t cs) {
+  const int rc = check_tracked_out(cur, n, tracked_out);
+  if (rc != LC_OK) return rc;
+  EncodeOptions opt;
+  opt.spin_limit = spin_limit;
+  opt.ticket_bias = first_ticket;
+  return compress_impl(base, cur, n, nbits, stream, stream_capacity, tracked_out, workspace, workspace_bytes, opt, cs);
+}
+
 int lc_compress_timed(const float* base, const float* cur, uint64_t n, int nbits, void* stream,
                       uint64_t stream_capacity, void* workspace, uint64_t workspace_bytes, lc_cuda_stream_t cs,
                       float* kernel_ms) {
