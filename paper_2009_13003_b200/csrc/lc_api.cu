@@ -87,7 +87,7 @@ __global__ void result_kernel(const int32_t* status, const uint32_t* header, uin
   if (i == kHeaderBytes / 4) *reinterpret_cast<volatile uint32_t*>(page + i) = st;  // last: the host looks at it
 }
 
-// lc_compress and lc_compress_update: argument checks, then memset + three kernels on `cs`.
+// lc_compress, lc_compress_update and their variants: argument checks, then one launch (a small vector), or four and more, on `cs`.
 int compress_impl(const float* base, const float* cur, uint64_t n, int nbits, void* stream, uint64_t stream_capacity,
                   float* tracked_out, void* workspace, uint64_t workspace_bytes, const EncodeOptions& opt,
                   cudaStream_t cs, bool keep_status = false) {
@@ -99,7 +99,7 @@ int compress_impl(const float* base, const float* cur, uint64_t n, int nbits, vo
   if (workspace_bytes < W.total || stream_capacity < lc_stream_bound(n, nbits)) return LC_ERR_CAPACITY;
   const Carved c = carve(workspace, W);
 
-  // a small vector with the default options: one CTA or cluster does everything in one launch (no memset either)
+  // a small vector with the default options: one CTA or cluster does everything in one launch
   if (n > 0 && n <= kSmallMaxElems && !opt.two_pass_scan && !opt.fixed_width && !opt.mean_rep && !opt.length_cache &&
       opt.ticket_bias == 0 && opt.spin_limit == EncodeOptions().spin_limit) {
     const cudaError_t e = launch_small_compress(c.ctl, base, cur, n, nbits, static_cast<uint8_t*>(stream), tracked_out, keep_status, cs);

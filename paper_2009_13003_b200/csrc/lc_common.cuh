@@ -149,9 +149,10 @@ static __device__ __noinline__ void set_status_ranked(int32_t* status, uint32_t 
 // `overlap` may start once every CTA of the one before it in the stream has called begin_next(), and may touch what that
 // kernel (and those before it) wrote only behind wait_previous(). Every kernel of such a chain calls wait_previous(), so
 // that the guarantee reaches back to the first; the first of a call is launched without `overlap`, i.e. behind everything
-// the caller has enqueued. Without the attribute both are no-ops. With a memset and plain launches instead, a compress of
-// 11.7 M elements took 52 us on the GPU, with this 45 us. (Recovery has only a memset ahead of its kernel; there the launch of
-// a clearing kernel costs the host more than the overlap gains.)
+// the caller has enqueued (but lc_wait's kernel, its call's only one, which touches nothing ahead of wait_previous()). Without the
+// attribute both are no-ops. With a memset and plain launches instead, a compress of 11.7 M elements took 52 us on the GPU, with
+// this 45 us. (The first launch of a recovery has a memset ahead of it, beyond kClearChunks chunks; there the launch of a clearing
+// kernel costs the host more than the overlap gains.)
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void begin_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

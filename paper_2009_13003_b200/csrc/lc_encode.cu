@@ -470,8 +470,8 @@ constexpr int kScanThreads = 1024;
 
 // Size in bytes of every chunk (format section 3.3: the chunk's bits rounded up to 16 bytes), one warp per chunk,
 // into sizes[c]. Whole chunks whose keys the one-byte plane identifies take their code lengths from a 256-byte
-// table in shared memory, 16 plane bytes per load; the vector's partial last chunk and vectors with exponent
-// fields >= 128 go through the slow path's counting mode.
+// table in shared memory, 16 plane bytes per load; the vector's partial last chunk and chunks that hold byte 0 while the
+// vector has exponent fields >= 128 go through the slow path's counting mode.
 __global__ void __launch_bounds__(kEncThreads)
 encode_sizes_kernel(const Control* __restrict__ ctl, unsigned long long* __restrict__ sizes,
                     const uint8_t* __restrict__ plane, const float* base, const float* __restrict__ cur, uint64_t n,

@@ -1,7 +1,7 @@
 // Small vectors: the whole compress pass (Algorithm 1 steps 4-6, optionally step 7) in one launch and without a
 // workspace: one CTA for a vector of one chunk, one cluster of CTAs for a vector of up to 32.
 //
-// For such a vector the three kernels of the general path and the memset before them are all launch latency; layers of
+// For such a vector the four kernels of the general path are all launch latency; layers of
 // a few hundred elements are common in per-layer use, and so are whole models of some ten thousand. Bound: latency, so every
 // part of the pass is spread over all 16 warps. A thread loads its eight elements of a chunk once and keeps base and delta in
 // registers through statistics, coding and the tracked state. Warp w takes the chunk's steps 2w and 2w + 1, so the codes
@@ -38,7 +38,7 @@ small_compress_kernel(Control* ctl, const float* base, const float* cur, uint32_
   if (!first) return;
   if (err) clear_header(stream);
   if (tid == 0) {
-    // what the memset of the general path clears, as far as later readers look at it
+    // what the general path clears and its table pass writes, as far as later readers look at it
     ctl->status = err;  // barriers (of the cluster) lie between the reads above and this
     ctl->ticket = 0;
     ctl->nsym = err ? 0 : S.T.nsym;
